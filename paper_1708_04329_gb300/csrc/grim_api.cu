@@ -549,14 +549,10 @@ int grim_filter(const grim_index* idx, const char* reads, const uint64_t* offset
     return sc;
   }
 
-  // what the final sort and split work from
-  const int32_t* lists = cand;
-  const uint64_t* lists_off = cand_off;
-  uint64_t n_lists = n_cand;
-  bool list_mode = cand_mode;
-
+  // the passing records (sorted between this buffer and the other one)
+  RecordsView found = ra, other = rb;
   if (cand_mode) {
-    launch_candidates(v, rv, cand, cand_off, ra, ctl, st, "candidates", {false, 0}, 0, true);
+    launch_candidates(v, rv, cand, cand_off, ra, ctl, st);
   } else {
     // all bins: coarse-then-exact when the index allows it and every read
     // needs enough of its tokens present for super-bins to fail early;
@@ -592,23 +588,18 @@ int grim_filter(const grim_index* idx, const char* reads, const uint64_t* offset
         // survivors bounds the total from above
         *n_out = n_surv * f;
         return GRIM_E_OVERFLOW;
-      } else {
-        int32_t* icand = reinterpret_cast<int32_t*>(ws + L.cand);
-        uint64_t* ioff = reinterpret_cast<uint64_t*>(ws + L.cand_off);
-        const RecordsView surv = sort_records(ra, rb, n_surv, read_bits + cbits, ws + L.hist, st);
-        expand_survivors(surv.keys, n_surv, cbits, f, n_reads, icand, ioff, st);
-        lists = icand;
-        lists_off = ioff;
-        n_lists = n_surv * f;
-        list_mode = true;
       }
       // restart the record and work counters for the next pass
       CK(cudaMemsetAsync(ctl, 0, offsetof(Ctl, blocks), st));
+      if (two) {  // the survivors stay in ra; their passing members go to rb
+        launch_refine(v, rv, ra.keys, n_surv, cbits, f, rb, bin_bits, ctl, st);
+        found = rb;
+        other = ra;
+      }
     }
     path_used = two ? GRIM_PATH_TWO_LEVEL : GRIM_PATH_EXACT;
-    if (two) launch_candidates(v, rv, lists, lists_off, ra, ctl, st, "candidates_refine");
-    else launch_exhaustive(v, rv, ra, bin_bits, h.max_d, ctl, st, "exhaustive", {false, 0},
-                           shape);
+    if (!two)
+      launch_exhaustive(v, rv, ra, bin_bits, h.max_d, ctl, st, "exhaustive", {false, 0}, shape);
   }
   CK(cudaGetLastError());
   CK(cudaMemcpyAsync(&h, ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
@@ -619,8 +610,8 @@ int grim_filter(const grim_index* idx, const char* reads, const uint64_t* offset
   *n_out = h.n_rec;
   if (h.n_rec > cap) return GRIM_E_OVERFLOW;
   const uint32_t key_bits =
-      list_mode ? bit_length(n_lists ? n_lists - 1 : 0) : bin_bits + read_bits;
-  sort_and_emit(ra, rb, h.n_rec, key_bits, ws + L.hist, list_mode, bin_bits, lists, lists_off,
+      cand_mode ? bit_length(n_cand ? n_cand - 1 : 0) : bin_bits + read_bits;
+  sort_and_emit(found, other, h.n_rec, key_bits, ws + L.hist, cand_mode, bin_bits, cand, cand_off,
                 n_reads, out_read, out_bin, out_count, st);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(st));

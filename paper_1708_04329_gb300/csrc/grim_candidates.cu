@@ -55,7 +55,6 @@ struct CandArgs {
   RecordsView rec;
   Ctl* ctl;
   Live live;
-  bool check_ids;  // caller's lists: an id outside [0, num_bins) is an error
 };
 
 constexpr int kWarps = 8;
@@ -323,7 +322,6 @@ __global__ void __launch_bounds__(kWarps * 32, cand_ctas_per_sm(WPB)) k_candidat
   const uint64_t n_chunks = c_end > c_begin ? (c_end - c_begin + chunk - 1) / chunk : 0;
 
   uint32_t cur = 0xFFFFFFFFu, K = 0, thr = 0, nh = 0;  // the read whose planes are built
-  const bool check = a.check_ids;
   const uint32_t last_row = (uint32_t)(a.ix.bm_rows - 1);
   const uint32_t num_bins = (uint32_t)a.ix.num_bins;  // bins are uint32 (checked at build)
   bool bad = false;  // this lane saw a candidate id outside [0, num_bins)
@@ -372,7 +370,7 @@ __global__ void __launch_bounds__(kWarps * 32, cand_ctas_per_sm(WPB)) k_candidat
 #pragma unroll
           for (int u = 0; u < U; ++u) {
             const bool in = off + u * CPW + slot < n;
-            bad |= check && in && bc[u] >= num_bins;
+            bad |= in && bc[u] >= num_bins;
             const uint32_t row = min(bc[u], last_row);
             if (in) load_words<WL>(a.ix.bm + (uint64_t)row * WPB + sub * WL, v[u]);
           }
@@ -396,8 +394,6 @@ __global__ void __launch_bounds__(kWarps * 32, cand_ctas_per_sm(WPB)) k_candidat
 #pragma unroll
           for (int u = 0; u < U; ++u)
             sums[u] = off + u * CPW + slot < n ? plane_sum<WPB, WL>(v[u], P, K, xplanes, sub, nh) : 0u;
-          // bins past num_bins exist only as zero padding of the table
-          // (members of the last super-bin); they never pass
           if constexpr (G == 32) {
             // a lane group is the whole warp (512-byte vectors): one
             // full-warp reduction per candidate, and lane u emits candidate u
@@ -442,8 +438,101 @@ __global__ void __launch_bounds__(kWarps * 32, cand_ctas_per_sm(WPB)) k_candidat
   if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) atomicOr(&a.ctl->status, kStatusBadCand);
 }
 
+// Exact check of the coarse pass's survivors, one (survivor, member bin) item
+// at a time by a whole warp: lane j looks up the read's tokens j, j + 32, ...
+// in the member's vector and a ballot counts the misses; the item ends once
+// they exceed D'.  The tokens are in the all-bins order (rarest first), so
+// most members end after one or two of these rounds.  Survivors come in the
+// order the coarse pass found them: an item needs only its read's token row,
+// so nothing is gained by sorting them by read first (the bit planes of
+// k_candidates pay for themselves over a list, not over two members).
+// Measured on GB300 against sorting the survivors, expanding them into lists
+// and checking those with k_candidates: 6.4M survivors of 100 bp reads on the
+// 3.1 Gbp tables 3.0 -> 1.8 ms; 2,383 survivors of a 1 Mbp genome 540 -> 25 us
+// (19 chunks of short lists there, each one warp's serial work).  The chain of
+// loads (token, then word of the vector) bounds it, so kRefineItems items run
+// side by side in a warp.
+constexpr int kRefineItems = 4;
+
+__global__ void __launch_bounds__(kWarps * 32, 4) k_refine(IndexView ix, ReadsView rv,
+                                                           const unsigned long long* __restrict__ keys,
+                                                           uint64_t n_surv, uint32_t cbits, uint32_t f,
+                                                           RecordsView rec, uint32_t bin_bits,
+                                                           Ctl* ctl, Live live) {
+  constexpr int U = kRefineItems;
+  if (*(volatile uint32_t*)&ctl->status) return;
+  if (gated_off(ctl, live)) return;
+  if (live.on) n_surv = ctl->n_surv;
+  const uint32_t lane = threadIdx.x & 31;
+  const uint64_t warp = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
+  const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  const uint64_t n_items = n_surv * f;
+  for (uint64_t base = warp * 32; base < n_items; base += n_warps * 32) {
+    // lane i: the batch's item i
+    const uint64_t i = base + lane;
+    uint32_t r = 0, bin = 0, m = 0, found = 0;  // found: sum + 1 of a passing item
+    bool in = i < n_items;
+    if (in) {
+      const uint64_t sv = i / f;
+      const unsigned long long key = keys[sv];
+      r = (uint32_t)(key >> cbits);
+      const uint64_t b = (key & ((1ull << cbits) - 1ull)) * f + (i - sv * f);
+      in = b < ix.num_bins;  // the last super-bin may have fewer members
+      bin = (uint32_t)b;
+      m = in ? rv.meta[r] : 0u;
+    }
+    const uint32_t todo = __ballot_sync(0xFFFFFFFFu, in);
+    for (int k = 0; k < 32; k += U) {
+      uint32_t live_items = (todo >> k) & ((1u << U) - 1u);
+      if (!live_items) continue;
+      const uint16_t* tok[U];
+      const uint32_t* vec[U];
+      uint32_t ntok[U], dmax[U], misses[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const uint32_t mu = __shfl_sync(0xFFFFFFFFu, m, k + u);
+        tok[u] = rv.tokens + (uint64_t)__shfl_sync(0xFFFFFFFFu, r, k + u) * rv.copies * rv.ts + lane;
+        vec[u] = ix.bm + (uint64_t)__shfl_sync(0xFFFFFFFFu, bin, k + u) * ix.wpb;
+        ntok[u] = mu & 0xFFu;
+        dmax[u] = mu >> 8;
+        misses[u] = 0;
+      }
+      for (uint32_t j = 0; live_items; j += 32) {
+        uint32_t t[U], w[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          t[u] = (live_items >> u & 1u) && j + lane < ntok[u] ? tok[u][j] : rowPad(ix.r4);
+#pragma unroll
+        for (int u = 0; u < U; ++u) w[u] = t[u] < ix.r4 ? __ldg(vec[u] + (t[u] >> 5)) : 0u;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const bool miss = t[u] != rowPad(ix.r4) && !((w[u] >> (t[u] & 31u)) & 1u);
+          misses[u] += __popc(__ballot_sync(0xFFFFFFFFu, miss));
+          if (misses[u] > dmax[u]) {
+            live_items &= ~(1u << u);
+          } else if ((live_items >> u & 1u) && j + 32 >= ntok[u]) {  // every token looked up
+            live_items &= ~(1u << u);
+            if (lane == (uint32_t)(k + u)) found = ntok[u] - misses[u] + 1u;
+          }
+        }
+      }
+    }
+    const uint32_t bal = __ballot_sync(0xFFFFFFFFu, found != 0);
+    if (bal) {
+      unsigned long long first = 0;
+      if (lane == 0) first = atomicAdd(&ctl->n_rec, (unsigned long long)__popc(bal));
+      first = __shfl_sync(0xFFFFFFFFu, first, 0);
+      const unsigned long long pos = first + __popc(bal & ((1u << lane) - 1u));
+      if (found && pos < rec.cap) {
+        rec.keys[pos] = ((unsigned long long)r << bin_bits) | bin;
+        rec.counts[pos] = (uint8_t)(found - 1u);
+      }
+    }
+  }
+}
+
 template <int WPB, int U>
-void launch_u(const CandArgs& a, cudaStream_t st, const char* name) {
+void launch_u(const CandArgs& a, cudaStream_t st) {
   const size_t smem = (size_t)kWarps * warp_smem_words(a.ix.r4, WPB) * sizeof(uint32_t);
   cudaFuncSetAttribute(k_candidates<WPB, U>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int dev = 0, sms = 0, per_sm = 0;
@@ -453,32 +542,46 @@ void launch_u(const CandArgs& a, cudaStream_t st, const char* name) {
   if (per_sm < 1) per_sm = 1;
   // persistent: warps that find no chunk left exit at once
   const uint64_t grid = (uint64_t)sms * per_sm;
-  ProfScope ps(name, st);
+  ProfScope ps("candidates", st);
   k_candidates<WPB, U><<<(unsigned)grid, kWarps * 32, smem, st>>>(a);
 }
 
 template <int WPB>
-void launch_t(const CandArgs& a, cudaStream_t st, const char* name, uint32_t unroll) {
-  if (unroll >= 8) launch_u<WPB, 8>(a, st, name);
-  else if (unroll >= 4) launch_u<WPB, 4>(a, st, name);
-  else if (unroll >= 2) launch_u<WPB, 2>(a, st, name);
-  else launch_u<WPB, 1>(a, st, name);
+void launch_t(const CandArgs& a, cudaStream_t st, uint32_t unroll) {
+  if (unroll >= 8) launch_u<WPB, 8>(a, st);
+  else if (unroll >= 4) launch_u<WPB, 4>(a, st);
+  else if (unroll >= 2) launch_u<WPB, 2>(a, st);
+  else launch_u<WPB, 1>(a, st);
 }
 
 }  // namespace
 
+void launch_refine(const IndexView& ix, const ReadsView& rv, const unsigned long long* keys,
+                   uint64_t n_surv, uint32_t cbits, uint32_t f, RecordsView rec, uint32_t bin_bits,
+                   Ctl* ctl, cudaStream_t st, Live live) {
+  if (n_surv == 0) return;
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const uint64_t need = (n_surv * f + 32 * kWarps - 1) / (32 * kWarps);
+  const uint64_t most = (uint64_t)(sms > 0 ? sms : 1) * 4;
+  ProfScope ps("candidates_refine", st);
+  k_refine<<<(unsigned)(need < most ? need : most), kWarps * 32, 0, st>>>(
+      ix, rv, keys, n_surv, cbits, f, rec, bin_bits, ctl, live);
+}
+
 void launch_candidates(const IndexView& ix, const ReadsView& rv, const int32_t* cand,
                        const uint64_t* cand_off, RecordsView rec, Ctl* ctl, cudaStream_t st,
-                       const char* prof_name, Live live, uint32_t unroll, bool check_ids) {
+                       Live live, uint32_t unroll) {
   if (unroll == 0) unroll = kDefaultCandUnroll;
   if (rv.n_reads == 0) return;
-  CandArgs a{ix, rv, cand, cand_off, rec, ctl, live, check_ids};
+  CandArgs a{ix, rv, cand, cand_off, rec, ctl, live};
   switch (ix.wpb) {
-    case 1: launch_t<1>(a, st, prof_name, unroll); break;
-    case 2: launch_t<2>(a, st, prof_name, unroll); break;
-    case 8: launch_t<8>(a, st, prof_name, unroll); break;
-    case 32: launch_t<32>(a, st, prof_name, unroll); break;
-    case 128: launch_t<128>(a, st, prof_name, unroll); break;
+    case 1: launch_t<1>(a, st, unroll); break;
+    case 2: launch_t<2>(a, st, unroll); break;
+    case 8: launch_t<8>(a, st, unroll); break;
+    case 32: launch_t<32>(a, st, unroll); break;
+    case 128: launch_t<128>(a, st, unroll); break;
     default: break;  // q outside 2..6 is rejected by grim_build
   }
 }

@@ -19,24 +19,18 @@ constexpr uint32_t kSortThreads = 256;
 constexpr uint32_t kSortItems = 16;  // per thread per pass
 constexpr uint32_t kSortTile = kSortThreads * kSortItems;
 
-// Live record counts: *n_live (capped at n) when n_live is set, else n; a
-// gate (ctl, path) makes the kernel a no-op unless the batch took that path.
+// Live record counts: *n_live (capped at n) when n_live is set, else n.
 __device__ __forceinline__ uint64_t live_n(const unsigned long long* n_live, uint64_t n) {
   if (!n_live) return n;
   const uint64_t v = *n_live;
   return v < n ? v : n;
 }
-__device__ __forceinline__ bool gate_off(const Ctl* c, uint32_t gate) {
-  return c && gate && c->path != gate;
-}
 
 __global__ void __launch_bounds__(kSortThreads) k_rs_hist(const unsigned long long* __restrict__ keys,
                                                           uint64_t n, uint32_t shift,
                                                           uint32_t* __restrict__ hist, uint32_t nb,
-                                                          const unsigned long long* n_live,
-                                                          const Ctl* gc, uint32_t gate) {
+                                                          const unsigned long long* n_live) {
   __shared__ uint32_t cnt[256];
-  if (gate_off(gc, gate)) return;
   n = live_n(n_live, n);
   if ((uint64_t)blockIdx.x * kSortTile >= n) return;  // past the live records
   cnt[threadIdx.x] = 0;
@@ -61,10 +55,8 @@ __device__ __forceinline__ uint64_t hist_at(uint32_t i, uint32_t nb_live, uint64
 }
 
 __global__ void __launch_bounds__(1024) k_rs_scan(uint32_t* __restrict__ h, uint64_t nb, uint64_t n,
-                                                  const unsigned long long* n_live, const Ctl* gc,
-                                                  uint32_t gate) {
+                                                  const unsigned long long* n_live) {
   __shared__ uint32_t s_warp[32];
-  if (gate_off(gc, gate)) return;
   n = live_n(n_live, n);
   const uint32_t nb_live = (uint32_t)((n + kSortTile - 1) / kSortTile);
   if (nb_live == 0) return;
@@ -108,12 +100,10 @@ __global__ void __launch_bounds__(1024) k_rs_scan(uint32_t* __restrict__ h, uint
 __global__ void __launch_bounds__(kSortThreads) k_rs_scatter(
     const unsigned long long* __restrict__ kin, const uint8_t* __restrict__ cin,
     unsigned long long* __restrict__ kout, uint8_t* __restrict__ cout, uint64_t n, uint32_t shift,
-    const uint32_t* __restrict__ hist, uint32_t nb, const unsigned long long* n_live, const Ctl* gc,
-    uint32_t gate) {
+    const uint32_t* __restrict__ hist, uint32_t nb, const unsigned long long* n_live) {
   constexpr uint32_t kW = kSortThreads / 32;
   __shared__ uint32_t s_base[256];
   __shared__ uint32_t s_wcnt[kW][256];
-  if (gate_off(gc, gate)) return;
   n = live_n(n_live, n);
   if ((uint64_t)blockIdx.x * kSortTile >= n) return;  // past the live records
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -152,9 +142,8 @@ __global__ void k_emit(const unsigned long long* __restrict__ keys,
                        const uint64_t* __restrict__ cand_off, uint32_t n_reads,
                        uint32_t* __restrict__ out_read, uint32_t* __restrict__ out_bin,
                        uint8_t* __restrict__ out_count, const unsigned long long* n_live,
-                       const uint32_t* n_reads_live, const Ctl* gc, uint32_t gate) {
+                       const uint32_t* n_reads_live) {
   const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  if (gate_off(gc, gate)) return;
   if (i >= live_n(n_live, n)) return;
   if (n_reads_live) n_reads = *n_reads_live;
   const unsigned long long key = keys[i];
@@ -178,36 +167,6 @@ __global__ void k_emit(const unsigned long long* __restrict__ keys,
   out_count[i] = counts[i];
 }
 
-// Survivors of the coarse pass (keys read << cbits | super-bin, sorted) become
-// candidate lists of the members of each surviving super-bin: candidates
-// f*i .. f*i+f-1 are bins f*s .. f*s+f-1, and read r's list starts at f times
-// the number of survivors of reads before r.
-__global__ void k_expand(const unsigned long long* __restrict__ keys, uint64_t n_surv,
-                         uint32_t cbits, uint32_t f, uint32_t n_reads, int32_t* __restrict__ cand,
-                         uint64_t* __restrict__ cand_off, const Ctl* lc, uint32_t gate) {
-  const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  if (lc) {
-    if (gate_off(lc, gate)) return;
-    n_surv = lc->n_surv;
-    n_reads = lc->live_reads;
-  }
-  const unsigned long long mask = cbits >= 64 ? ~0ull : ((1ull << cbits) - 1ull);
-  if (i < n_surv) {
-    const uint32_t s = (uint32_t)(keys[i] & mask);
-    for (uint32_t k = 0; k < f; ++k) cand[f * i + k] = (int32_t)(f * s + k);
-  }
-  if (i <= n_reads) {
-    const unsigned long long target = (unsigned long long)i << cbits;
-    uint64_t lo = 0, hi = n_surv;  // first survivor with key >= target
-    while (lo < hi) {
-      const uint64_t mid = (lo + hi) / 2;
-      if (keys[mid] < target) lo = mid + 1;
-      else hi = mid;
-    }
-    cand_off[i] = f * lo;
-  }
-}
-
 }  // namespace
 
 uint64_t sort_workspace_bytes(uint64_t cap) {
@@ -215,18 +174,8 @@ uint64_t sort_workspace_bytes(uint64_t cap) {
   return 256ull * (nb ? nb : 1) * sizeof(uint32_t);
 }
 
-void expand_survivors(const unsigned long long* keys, uint64_t n_surv, uint32_t cbits, uint32_t f,
-                      uint32_t n_reads, int32_t* cand, uint64_t* cand_off, cudaStream_t st,
-                      const Ctl* live_ctl, uint32_t gate) {
-  const uint64_t n = n_surv > (uint64_t)n_reads + 1 ? n_surv : (uint64_t)n_reads + 1;
-  ProfScope ps("expand", st);
-  k_expand<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(keys, n_surv, cbits, f, n_reads, cand,
-                                                       cand_off, live_ctl, gate);
-}
-
 RecordsView sort_records(RecordsView a, RecordsView b, uint64_t n, uint32_t key_bits, void* hist,
-                         cudaStream_t st, const unsigned long long* n_live, const Ctl* gate_ctl,
-                         uint32_t gate) {
+                         cudaStream_t st, const unsigned long long* n_live) {
   if (n == 0) return a;
   const uint32_t nb = (uint32_t)((n + kSortTile - 1) / kSortTile);
   uint32_t* h = static_cast<uint32_t*>(hist);
@@ -236,16 +185,16 @@ RecordsView sort_records(RecordsView a, RecordsView b, uint64_t n, uint32_t key_
     const uint32_t shift = 8 * p;
     {
       ProfScope ps("sort_hist", st);
-      k_rs_hist<<<nb, kSortThreads, 0, st>>>(src.keys, n, shift, h, nb, n_live, gate_ctl, gate);
+      k_rs_hist<<<nb, kSortThreads, 0, st>>>(src.keys, n, shift, h, nb, n_live);
     }
     {
       ProfScope ps("sort_scan", st);
-      k_rs_scan<<<1, 1024, 0, st>>>(h, nb, n, n_live, gate_ctl, gate);
+      k_rs_scan<<<1, 1024, 0, st>>>(h, nb, n, n_live);
     }
     {
       ProfScope ps("sort_scatter", st);
       k_rs_scatter<<<nb, kSortThreads, 0, st>>>(src.keys, src.counts, dst.keys, dst.counts, n,
-                                                shift, h, nb, n_live, gate_ctl, gate);
+                                                shift, h, nb, n_live);
     }
     RecordsView t = src;
     src = dst;
@@ -258,15 +207,13 @@ void sort_and_emit(RecordsView a, RecordsView b, uint64_t n, uint32_t key_bits, 
                    bool candidate_mode, uint32_t bin_bits, const int32_t* cand,
                    const uint64_t* cand_off, uint32_t n_reads, uint32_t* out_read,
                    uint32_t* out_bin, uint8_t* out_count, cudaStream_t st,
-                   const unsigned long long* n_live, const uint32_t* n_reads_live,
-                   const Ctl* gate_ctl, uint32_t gate) {
+                   const unsigned long long* n_live, const uint32_t* n_reads_live) {
   if (n == 0) return;
-  const RecordsView src = sort_records(a, b, n, key_bits, hist, st, n_live, gate_ctl, gate);
+  const RecordsView src = sort_records(a, b, n, key_bits, hist, st, n_live);
   ProfScope ps("emit", st);
   k_emit<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(src.keys, src.counts, n, candidate_mode,
                                                       bin_bits, cand, cand_off, n_reads, out_read,
-                                                      out_bin, out_count, n_live, n_reads_live,
-                                                      gate_ctl, gate);
+                                                      out_bin, out_count, n_live, n_reads_live);
 }
 
 }  // namespace grim

@@ -453,6 +453,13 @@ __global__ void __launch_bounds__(NT, 1) k_exhaustive(ExhArgs a) {
         if (lane == 0 && tot) base = atomicAdd(&a.ctl->n_rec, (unsigned long long)tot);
         base = __shfl_sync(0xFFFFFFFFu, base, 0);
         unsigned long long pos = base + incl - cnt;
+        // past the capacity (count-only calls: always) records are only
+        // counted, not walked bit by bit: 500 reads against 6.55M bins at
+        // q = 4, six budgets, 9.5e9 passing pairs: 15.6 -> 10.4 ms
+        if (base >= a.rec.cap) {
+#pragma unroll
+          for (int w = 0; w < 4; ++w) pm[w] = 0;
+        }
 #pragma unroll
         for (int w = 0; w < 4; ++w) {
           uint32_t m = pm[w];

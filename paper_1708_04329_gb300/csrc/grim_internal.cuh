@@ -165,14 +165,18 @@ void launch_exhaustive(const IndexView& ix, const ReadsView& rv, RecordsView rec
                        const char* prof_name = "exhaustive", Live live = {false, 0},
                        ExhShape shape = {0, 0, 0, 0});
 // unroll: candidate gathers in flight per lane group (1, 2, 4 or 8; 0 =
-// default).  check_ids: the lists are the caller's; an id outside
-// [0, num_bins) sets kStatusBadCand (and is not gathered).  Internal lists
-// (survivor members) may hold zero-padding bins past num_bins: they are
-// gathered and never pass.
+// default).  An id outside [0, num_bins) sets kStatusBadCand.
 void launch_candidates(const IndexView& ix, const ReadsView& rv, const int32_t* cand,
                        const uint64_t* cand_off, RecordsView rec, Ctl* ctl, cudaStream_t st,
-                       const char* prof_name = "candidates", Live live = {false, 0},
-                       uint32_t unroll = 0, bool check_ids = false);
+                       Live live = {false, 0}, uint32_t unroll = 0);
+// The exact check of the coarse pass's survivors (keys read << cbits |
+// super-bin, in any order): the members of each surviving super-bin of f
+// bins against the bin-major table; passing (read, bin) pairs become records
+// with keys read << bin_bits | bin.  With `live` on, the survivor count is
+// read from ctl->n_surv and n_surv only sizes the launch.
+void launch_refine(const IndexView& ix, const ReadsView& rv, const unsigned long long* keys,
+                   uint64_t n_surv, uint32_t cbits, uint32_t f, RecordsView rec, uint32_t bin_bits,
+                   Ctl* ctl, cudaStream_t st, Live live = {false, 0});
 
 // Radix sort of n (key, count) records by the low key_bits bits of the key,
 // followed by the split into the caller's (read, bin, count) arrays.
@@ -180,17 +184,12 @@ uint64_t sort_workspace_bytes(uint64_t cap);
 // n_live (nullable): the record count is read on the device from *n_live,
 // capped at n; n then only sizes the launches
 RecordsView sort_records(RecordsView a, RecordsView b, uint64_t n, uint32_t key_bits, void* hist,
-                         cudaStream_t st, const unsigned long long* n_live = nullptr,
-                         const Ctl* gate_ctl = nullptr, uint32_t gate = 0);
-void expand_survivors(const unsigned long long* keys, uint64_t n_surv, uint32_t cbits, uint32_t f,
-                      uint32_t n_reads, int32_t* cand, uint64_t* cand_off, cudaStream_t st,
-                      const Ctl* live_ctl = nullptr, uint32_t gate = 0);
+                         cudaStream_t st, const unsigned long long* n_live = nullptr);
 void sort_and_emit(RecordsView a, RecordsView b, uint64_t n, uint32_t key_bits, void* hist,
                    bool candidate_mode, uint32_t bin_bits, const int32_t* cand,
                    const uint64_t* cand_off, uint32_t n_reads, uint32_t* out_read,
                    uint32_t* out_bin, uint8_t* out_count, cudaStream_t st,
-                   const unsigned long long* n_live = nullptr, const uint32_t* n_reads_live = nullptr,
-                   const Ctl* gate_ctl = nullptr, uint32_t gate = 0);
+                   const unsigned long long* n_live = nullptr, const uint32_t* n_reads_live = nullptr);
 
 // ---------------------------------------------------------------------------
 // per-kernel timing (grim_profile): wraps one launch in events on `st`
@@ -222,7 +221,7 @@ inline uint32_t token_stride(const IndexView& v) {
 }
 
 struct Layout {
-  uint64_t tok, meta, keys_a, keys_b, cnt_a, cnt_b, hist, cand, cand_off, total;
+  uint64_t tok, meta, keys_a, keys_b, cnt_a, cnt_b, hist, spare, total;
 };
 
 // Survivors of the coarse pass get their own capacity: reads from repeat
@@ -238,8 +237,8 @@ inline uint64_t record_capacity(uint32_t n_reads, uint64_t cap, uint32_t coarse_
   return s > cap ? s : cap;
 }
 
-// coarse_factor > 0: room for the coarse pass's survivors and for the
-// candidate lists they expand into (coarse_factor per survivor)
+// coarse_factor > 0: room for the coarse pass's survivors, and per survivor
+// the coarse_factor words that grim_filter_workspace_size has always counted
 // Token copies per read: the all-bins kernel's 256-bin tiles (q = 6) read
 // one of 4 block-rotated copies per lane group (see k_tokenise).
 inline uint32_t token_copies(const IndexView& v, bool cand_mode) {
@@ -265,9 +264,8 @@ inline Layout layout(const IndexView& v, uint32_t n_reads, uint64_t cap, uint32_
   o = align256(o + rcap);
   L.hist = o;
   o = align256(o + sort_workspace_bytes(rcap));
-  L.cand = o;
+  L.spare = o;
   o = align256(o + (coarse_factor ? rcap * coarse_factor * sizeof(int32_t) : 0));
-  L.cand_off = o;
   o = align256(o + (coarse_factor ? ((uint64_t)n_reads + 1) * sizeof(uint64_t) : 0));
   L.total = o;
   return L;

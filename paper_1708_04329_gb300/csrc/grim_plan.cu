@@ -155,8 +155,7 @@ int capture(grim_plan* p) {
                   p->ctl, st, live, d.max_e, d.max_bases);
   if (p->cand_mode) {
     launch_check_candidates(B.cand_off, d.max_reads, d.max_cand, p->ctl, st, live);
-    launch_candidates(v, rv, B.cand, B.cand_off, ra, p->ctl, st, "candidates", live,
-                      d.cand_unroll, true);
+    launch_candidates(v, rv, B.cand, B.cand_off, ra, p->ctl, st, live, d.cand_unroll);
     k_plan_control<<<1, 1, 0, st>>>(p->ctl, kCtlFinal, 0, 0, 0, 0);
     sort_and_emit(ra, rb, d.cap, bit_length(d.max_cand ? d.max_cand - 1 : 0), ws + L.hist, true,
                   bin_bits, B.cand, B.cand_off, d.max_reads, B.out_read,
@@ -165,37 +164,25 @@ int capture(grim_plan* p) {
     bool forced = false;
     all_bins_path(idx, &forced);
     k_plan_control<<<1, 1, 0, st>>>(p->ctl, kCtlDecide, p->f != 0, has_exact, rcap, forced);
-    int32_t* icand = reinterpret_cast<int32_t*>(ws + L.cand);
-    uint64_t* ioff = reinterpret_cast<uint64_t*>(ws + L.cand_off);
     const uint32_t cbits =
         idx->cv.num_bins > 1 ? bit_length(idx->cv.num_bins - 1) : 0;
+    // both paths leave their records in rb: the coarse pass's survivors are
+    // in ra while their members are checked
     if (p->f) {
       const Live coarse{true, kPathCoarse};
       launch_exhaustive(idx->cv, rv, ra, cbits, max_d, p->ctl, st, "exhaustive_coarse", coarse,
                         idx->shape);
       k_plan_control<<<1, 1, 0, st>>>(p->ctl, kCtlAfterCoarse, 1, has_exact, rcap, 0);
-      const RecordsView surv = sort_records(ra, rb, rcap, read_bits + cbits, ws + L.hist, st,
-                                            &p->ctl->n_surv, p->ctl, kPathCoarse);
-      expand_survivors(surv.keys, rcap, cbits, p->f, d.max_reads, icand, ioff, st, p->ctl,
-                       kPathCoarse);
-      launch_candidates(v, rv, icand, ioff, ra, p->ctl, st, "candidates_refine", coarse,
-                        d.cand_unroll);
+      launch_refine(v, rv, ra.keys, rcap, cbits, p->f, rb, bin_bits, p->ctl, st, coarse);
     }
     if (has_exact) {
       const Live exact{true, kPathExact};
-      launch_exhaustive(v, rv, ra, bin_bits, max_d, p->ctl, st, "exhaustive", exact, idx->shape);
+      launch_exhaustive(v, rv, rb, bin_bits, max_d, p->ctl, st, "exhaustive", exact, idx->shape);
     }
     k_plan_control<<<1, 1, 0, st>>>(p->ctl, kCtlFinal, 0, 0, 0, 0);
-    if (p->f) {
-      sort_and_emit(ra, rb, d.cap, bit_length(rcap * p->f - 1), ws + L.hist, true, bin_bits, icand,
-                    ioff, d.max_reads, B.out_read, B.out_bin, B.out_count, st,
-                    &p->ctl->n_final, &p->ctl->live_reads, p->ctl, kPathCoarse);
-    }
-    if (has_exact) {
-      sort_and_emit(ra, rb, d.cap, bin_bits + read_bits, ws + L.hist, false, bin_bits, nullptr,
-                    nullptr, d.max_reads, B.out_read, B.out_bin, B.out_count, st,
-                    &p->ctl->n_final, &p->ctl->live_reads, p->ctl, kPathExact);
-    }
+    sort_and_emit(rb, ra, d.cap, bin_bits + read_bits, ws + L.hist, false, bin_bits, nullptr,
+                  nullptr, d.max_reads, B.out_read, B.out_bin, B.out_count, st, &p->ctl->n_final,
+                  &p->ctl->live_reads);
   }
   cudaMemcpyAsync(p->result, p->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st);
   e = cudaStreamEndCapture(st, &p->graph);

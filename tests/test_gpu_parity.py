@@ -587,3 +587,18 @@ def test_survivor_overflow_takes_the_exact_pass():
     st = grim.grim_last_filter_stats()
     assert st["survivors"] == n_surv and st["all_bins_path"] == grim.GRIM_PATH_TWO_LEVEL
     idx.close()
+
+
+@pytest.mark.parametrize("q,factor,n", [(4, 3, 1), (5, 2, 15), (5, 2, 16), (5, 2, 17), (5, 64, 1),
+                                        (6, 16, 2), (6, 5, 33)])
+def test_survivor_check_batches(q, factor, n):
+    """Survivors are checked in warp batches of 32 (survivor, member) items:
+    counts below, at and past a batch, factors that cut a survivor across two
+    batches, and a last super-bin with fewer members."""
+    from paper_1708_04329_gb300 import synth
+
+    g = synth.genome(20 * 64 * 37 + 11, seed=q * 7 + n)
+    rs = synth.reads(g, n, seed=n, lengths=(60, 100), probs=(0.5, 0.5), e=3, max_edits=3)
+    ix = build(g, 37, q, 100, layouts=6, coarse_factor=factor)
+    assert_same(gpu_filter(ix, rs, cap=200_000), oracle.filter(oracle.bin_vectors(g, 37, q, 100), rs))
+    ix.close()
