@@ -9,7 +9,8 @@
 // Each 8-bit pass is a per-block digit histogram, one exclusive scan over
 // all blocks' histograms, and a stable scatter (per-warp ranks from
 // __match_any_sync, then warp order, then round order).  A last kernel splits
-// the keys into the caller's read / bin / count arrays.
+// the keys into the caller's read / bin / count arrays.  Short lists skip the
+// radix sort: one kernel places each record by counting the smaller keys.
 #include "grim_internal.cuh"
 
 namespace grim {
@@ -136,35 +137,78 @@ __global__ void __launch_bounds__(kSortThreads) k_rs_scatter(
   }
 }
 
-__global__ void k_emit(const unsigned long long* __restrict__ keys,
-                       const uint8_t* __restrict__ counts, uint64_t n, bool cand_mode,
-                       uint32_t bin_bits, const int32_t* __restrict__ cand,
-                       const uint64_t* __restrict__ cand_off, uint32_t n_reads,
-                       uint32_t* __restrict__ out_read, uint32_t* __restrict__ out_bin,
-                       uint8_t* __restrict__ out_count, const unsigned long long* n_live,
-                       const uint32_t* n_reads_live) {
-  const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  if (i >= live_n(n_live, n)) return;
-  if (n_reads_live) n_reads = *n_reads_live;
-  const unsigned long long key = keys[i];
+// One record into the caller's arrays at position i.
+struct EmitArgs {
+  bool cand_mode;
+  uint32_t bin_bits;
+  const int32_t* cand;
+  const uint64_t* cand_off;
+  uint32_t n_reads;
+  uint32_t* out_read;
+  uint32_t* out_bin;
+  uint8_t* out_count;
+};
+__device__ __forceinline__ void emit_record(const EmitArgs& e, uint64_t i, unsigned long long key,
+                                            uint8_t count, uint32_t n_reads) {
   uint32_t r, b;
-  if (cand_mode) {
-    b = (uint32_t)cand[key];
+  if (e.cand_mode) {
+    b = (uint32_t)e.cand[key];
     // largest r with cand_off[r] <= key
     uint32_t lo = 0, hi = n_reads - 1;
     while (lo < hi) {
       const uint32_t mid = lo + (hi - lo + 1) / 2;
-      if (cand_off[mid] <= key) lo = mid;
+      if (e.cand_off[mid] <= key) lo = mid;
       else hi = mid - 1;
     }
     r = lo;
   } else {
-    r = (uint32_t)(key >> bin_bits);
-    b = (uint32_t)(key & ((bin_bits >= 64) ? ~0ull : ((1ull << bin_bits) - 1ull)));
+    r = (uint32_t)(key >> e.bin_bits);
+    b = (uint32_t)(key & ((e.bin_bits >= 64) ? ~0ull : ((1ull << e.bin_bits) - 1ull)));
   }
-  out_read[i] = r;
-  out_bin[i] = b;
-  out_count[i] = counts[i];
+  e.out_read[i] = r;
+  e.out_bin[i] = b;
+  e.out_count[i] = count;
+}
+
+__global__ void k_emit(const unsigned long long* __restrict__ keys,
+                       const uint8_t* __restrict__ counts, uint64_t n, EmitArgs e,
+                       const unsigned long long* n_live, const uint32_t* n_reads_live) {
+  const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+  if (i >= live_n(n_live, n)) return;
+  emit_record(e, i, keys[i], counts[i], n_reads_live ? *n_reads_live : e.n_reads);
+}
+
+// Short pass lists: a record's place is the number of smaller keys, counted
+// outright.  kRankSplit threads share a record and the block walks all keys
+// through shared memory, so sorting and splitting n records is one launch of
+// n^2 compares instead of the radix sort's three launches per key byte.
+// Measured on GB300 (rank against radix with two-byte keys, events around each
+// launch, us): 64 records 7 / 31, 2,048 9.5 / 61, 8,192 27 / 77, 16,384 75 /
+// 78, 32,768 273 / 86: the line is drawn where the compares still hide behind
+// the launches they replace.
+constexpr uint64_t kRankMax = 8192;
+constexpr uint32_t kRankThreads = 256;
+constexpr uint32_t kRankSplit = 16;    // threads per record
+constexpr uint32_t kRankChunk = 2048;  // keys in shared memory at a time
+__global__ void __launch_bounds__(kRankThreads) k_rank_emit(
+    const unsigned long long* __restrict__ keys, const uint8_t* __restrict__ counts, uint32_t n,
+    EmitArgs e) {
+  __shared__ unsigned long long s_key[kRankChunk];
+  const uint32_t i = (blockIdx.x * kRankThreads + threadIdx.x) / kRankSplit;
+  const uint32_t part = threadIdx.x % kRankSplit;
+  const unsigned long long key = i < n ? keys[i] : 0ull;
+  uint32_t rank = 0;
+  for (uint32_t c0 = 0; c0 < n; c0 += kRankChunk) {
+    const uint32_t m = min(kRankChunk, n - c0);
+    __syncthreads();
+    for (uint32_t j = threadIdx.x; j < m; j += kRankThreads) s_key[j] = keys[c0 + j];
+    __syncthreads();
+#pragma unroll 8
+    for (uint32_t j = part; j < m; j += kRankSplit) rank += s_key[j] < key;
+  }
+#pragma unroll
+  for (uint32_t d = 1; d < kRankSplit; d <<= 1) rank += __shfl_xor_sync(0xFFFFFFFFu, rank, d);
+  if (i < n && part == 0) emit_record(e, rank, key, counts[i], e.n_reads);
 }
 
 }  // namespace
@@ -209,11 +253,17 @@ void sort_and_emit(RecordsView a, RecordsView b, uint64_t n, uint32_t key_bits, 
                    uint32_t* out_bin, uint8_t* out_count, cudaStream_t st,
                    const unsigned long long* n_live, const uint32_t* n_reads_live) {
   if (n == 0) return;
+  const EmitArgs e{candidate_mode, bin_bits, cand, cand_off, n_reads, out_read, out_bin, out_count};
+  if (!n_live && n <= kRankMax) {
+    ProfScope ps("rank_emit", st);
+    k_rank_emit<<<(unsigned)((n * kRankSplit + kRankThreads - 1) / kRankThreads), kRankThreads, 0,
+                  st>>>(a.keys, a.counts, (uint32_t)n, e);
+    return;
+  }
   const RecordsView src = sort_records(a, b, n, key_bits, hist, st, n_live);
   ProfScope ps("emit", st);
-  k_emit<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(src.keys, src.counts, n, candidate_mode,
-                                                      bin_bits, cand, cand_off, n_reads, out_read,
-                                                      out_bin, out_count, n_live, n_reads_live);
+  k_emit<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(src.keys, src.counts, n, e, n_live,
+                                                      n_reads_live);
 }
 
 }  // namespace grim

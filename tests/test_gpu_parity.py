@@ -602,3 +602,23 @@ def test_survivor_check_batches(q, factor, n):
     ix = build(g, 37, q, 100, layouts=6, coarse_factor=factor)
     assert_same(gpu_filter(ix, rs, cap=200_000), oracle.filter(oracle.bin_vectors(g, 37, q, 100), rs))
     ix.close()
+
+
+@pytest.mark.parametrize("n", [1, 15, 16, 17, 2047, 2048, 2049, 8191, 8192, 8193])
+def test_pass_list_order_by_length(n):
+    """Pass lists placed by counting smaller keys and by radix sort: one
+    record, a block's edge, a shared-memory chunk's edge and the line between
+    the two, with unsorted duplicate candidates that all pass (T <= 0)."""
+    rng = np.random.default_rng(n)
+    g = rng.choice(np.frombuffer(b"ACGT", np.uint8), 60_000)
+    nr = max(1, n // 50)
+    at = rng.integers(0, len(g) - 40, nr)
+    rs = Reads([g[p:p + 40].tobytes().decode() for p in at], [20] * nr)
+    cand = rng.integers(0, 1200, n).astype(np.int32)
+    off = np.sort(rng.integers(0, n + 1, nr + 1)).astype(np.uint64)
+    off[0], off[-1] = 0, n
+    ix = build(g, 50, 5, 40, layouts=2)
+    got = gpu_filter(ix, rs, off, cand, cap=n)
+    assert len(got[0]) == n
+    assert_same(got, oracle.filter(oracle.bin_vectors(g, 50, 5, 40), rs, cand_off=off, cand=cand))
+    ix.close()
