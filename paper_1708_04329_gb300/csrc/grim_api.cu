@@ -534,7 +534,7 @@ int grim_filter(const grim_index* idx, const char* reads, const uint64_t* offset
   const uint32_t read_bits = n_reads > 1 ? bit_length((uint64_t)n_reads - 1) : 0;
 
   CK(cudaMemsetAsync(ctl, 0, sizeof(Ctl), st));
-  launch_tokenise(reads, offsets, lens, e, v, rv, tokens, meta, ctl, st);
+  launch_tokenise(reads, offsets, lens, e, v, rv, tokens, meta, ctl, st, cand_mode);
   if (cand_mode) launch_check_candidates(cand_off, n_reads, n_cand, ctl, st);
   else if (!idx->shape.read_switch) launch_block_spread(lens, n_reads, v.q, ctl, st);
   CK(cudaGetLastError());

@@ -14,14 +14,17 @@
 //       sum = sum_k 2^k * popcount(v & P_k)
 //   -- every position counts, repeats included, with a handful of AND +
 //   POPC per 32 bits instead of one bit test per token.
-// * A bin vector (4^q bits) is gathered by G lanes with 16-byte loads
-//   (q = 5: 8 lanes x 16 B = 128 B, four candidates per warp step; q = 6:
-//   32 lanes x 16 B = 512 B).  The U vectors of a step are reduced over the
-//   lane group together (a butterfly that halves the sums at each exchange;
-//   for a whole-warp group, one redux.sync per vector), compared with
+// * Up to q = 5 a bin vector (4^q bits) is gathered by G lanes with 16-byte
+//   loads (q = 5: 8 lanes x 16 B = 128 B, four candidates per warp step).  The
+//   U vectors of a step are reduced over the lane group together (a butterfly
+//   that halves the sums at each exchange), compared with
 //   T = (L-q+1) - q*e, and one ballot places the passes.
-// * The path is a random 128/512-byte gather per (read, bin) pair: bound by
+// * At q = 6 (512-byte vectors) k_candidates_lookup looks up the read's tokens
+//   instead, few lines of a vector at a time.
+// * The path is random reads of 128-byte lines per (read, bin) pair: bound by
 //   HBM, not by arithmetic.
+#include <math.h>
+
 #include "grim_internal.cuh"
 
 namespace grim {
@@ -59,39 +62,34 @@ struct CandArgs {
 
 constexpr int kWarps = 8;
 // gathers in flight per lane group when the caller leaves it to the library
-// (the autotuner's choice on GB300 for both 128- and 512-byte vectors)
+// (the autotuner's choice on GB300 for 128-byte vectors)
 constexpr uint32_t kDefaultCandUnroll = 2;
+// and candidates in flight per warp for the look-ups in 512-byte vectors
+// (98.9M candidates through a plan, ms at 1 / 2 / 4 / 8: e = 7 4.4 / 5.4 / 4.4 /
+// 4.35, e = 0 3.4 / 4.9 / 3.4 / 3.2)
+constexpr uint32_t kDefaultLookupUnroll = 8;
 constexpr int kRegPlanes = 2;  // bit planes held in registers: multiplicities up to 3
 
 // Multiplicities of 4 and more (bits kRegPlanes.. of a token's count) are
-// rare.  Up to 128-byte vectors they are kept as further bit planes in shared
-// memory (xplanes[k - kRegPlanes][word]).  For 512-byte vectors those planes
-// would take 3 KB a warp beside the 4 KB histogram and limit the kernel to
-// 32 warps per SM; instead the read's tokens of multiplicity >= 4 are listed
-// (token | (mult & ~3) << 16; at most 255 / 4 < 64 of them) and added one by
-// one, which makes room for 48 warps.
-template <int WPB> __host__ __device__ constexpr bool heavy_list() { return WPB >= 128; }
-constexpr uint32_t kMaxHeavy = 64;
-
-// per-warp shared memory: the multiplicity histogram, then the higher bit
-// planes or the list of heavy tokens
+// rare; they are kept as further bit planes in shared memory
+// (xplanes[k - kRegPlanes][word]).
+// per-warp shared memory: the multiplicity histogram, then the higher planes
 __host__ __device__ constexpr uint32_t hist_words_of(uint32_t r4) { return r4 >= 4 ? r4 / 4 : 1; }
 __host__ __device__ constexpr uint32_t warp_smem_words(uint32_t r4, uint32_t wpb) {
-  return hist_words_of(r4) + (wpb >= 128 ? kMaxHeavy : (8 - kRegPlanes) * wpb);
+  return hist_words_of(r4) + (8 - kRegPlanes) * wpb;
 }
 
 // The read's multiplicity histogram (byte t = how many of its positions hold
 // token t) and its bit planes P_k = {t : bit k of mult(t)} for this lane's WL
 // words of a bin vector: planes below kRegPlanes in registers, the rest in
-// shared memory, or (heavy_list) the heavy tokens in xplanes[0, *nh).
-// Returns K, the number of planes in use, and the read's threshold in *thr.
+// shared memory.  Returns K, the number of planes in use, and the read's threshold in *thr.
 // Warp-collective.
 template <int WPB, int WL>
 __device__ __forceinline__ uint32_t build_planes(const ReadsView& rv, uint32_t r, uint32_t r4,
                                                  uint32_t* hist, uint32_t* xplanes, uint32_t lane,
                                                  uint32_t sub, uint32_t (&P)[kRegPlanes][WL],
-                                                 uint32_t* thr, uint32_t* nh) {
-  constexpr int kPlanesBuilt = heavy_list<WPB>() ? kRegPlanes : 8;
+                                                 uint32_t* thr) {
+  constexpr int kPlanesBuilt = 8;
   const uint32_t hist_words = hist_words_of(r4);
   // the warp has finished reading the previous read's histogram
   __syncwarp();
@@ -141,51 +139,17 @@ __device__ __forceinline__ uint32_t build_planes(const ReadsView& rv, uint32_t r
       }
     }
   }
-  if constexpr (heavy_list<WPB>()) {
-    uint32_t count = 0;
-    if (K > (uint32_t)kRegPlanes) {
-      // list the tokens of multiplicity >= 4 with the part of their count
-      // above the register planes; each lane takes its histogram words
-      uint32_t mine = 0;
-      for (uint32_t i = lane; i < hist_words; i += 32) {
-        const uint32_t h = hist[i];
-        mine += ((h & 0xFCu) != 0) + ((h & 0xFC00u) != 0) + ((h & 0xFC0000u) != 0) +
-                ((h & 0xFC000000u) != 0);
-      }
-      uint32_t incl = mine;
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-        if (lane >= (uint32_t)d) incl += t;
-      }
-      count = __shfl_sync(0xFFFFFFFFu, incl, 31);
-      uint32_t pos = incl - mine;
-      for (uint32_t i = lane; i < hist_words; i += 32) {
-        const uint32_t h = hist[i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint32_t mult = (h >> (8 * j)) & 0xFFu;
-          if (mult >= 4 && pos < kMaxHeavy) xplanes[pos++] = (4 * i + j) | ((mult & ~3u) << 16);
-        }
-      }
-      __syncwarp();
-    }
-    *nh = min(count, kMaxHeavy);
-  }
   *thr = ntok - dmax;  // pass iff sum >= (L-q+1) - min(q*e, L-q+1)
   return K;
 }
 
-// sum_k 2^k popc(v & P_k) over this lane's WL words (with heavy_list: the
-// two register planes, then the listed heavy tokens that fall in this
-// lane's words, nh of them)
+// sum_k 2^k popc(v & P_k) over this lane's WL words
 template <int WPB, int WL>
 __device__ __forceinline__ uint32_t plane_sum(const uint32_t (&v)[WL],
                                               const uint32_t (&P)[kRegPlanes][WL], uint32_t K,
-                                              const uint32_t* xplanes, uint32_t sub, uint32_t nh) {
-  static_assert(!heavy_list<WPB>() || (WL == 4 && kRegPlanes == 2), "heavy list layout");
+                                              const uint32_t* xplanes, uint32_t sub) {
   if constexpr (WL == 4 && kRegPlanes == 2) {
-    if (heavy_list<WPB>() || K <= 2) {
+    if (K <= 2) {
       // the eight masked words (four of weight 1, four of weight 2) summed
       // bit-wise with a carry-save tree first: 4 POPC instead of 8
       const uint32_t a0 = v[0] & P[0][0], a1 = v[1] & P[0][1], a2 = v[2] & P[0][2],
@@ -198,19 +162,7 @@ __device__ __forceinline__ uint32_t plane_sum(const uint32_t (&v)[WL],
       const uint32_t s4 = b1 ^ b2 ^ b3, c4 = (b1 & b2) | (b3 & (b1 ^ b2));   // weights 2, 4
       const uint32_t s5 = s3 ^ s4, c5 = s3 & s4;                              // weights 2, 4
       const uint32_t s6 = c3 ^ c4 ^ c5, c6 = (c3 & c4) | (c5 & (c3 ^ c4));   // weights 4, 8
-      uint32_t sum = __popc(s2) + 2u * __popc(s5) + 4u * __popc(s6) + 8u * __popc(c6);
-      if constexpr (heavy_list<WPB>()) {
-        for (uint32_t i = 0; i < nh; ++i) {
-          const uint32_t ent = xplanes[i];
-          const uint32_t t = ent & 0xFFFFu, wi = t >> 5;  // token, word of the vector
-          if (wi / WL == sub) {
-            const uint32_t w = wi % WL;
-            const uint32_t word = w == 0 ? v[0] : w == 1 ? v[1] : w == 2 ? v[2] : v[3];
-            sum += ((word >> (t & 31u)) & 1u) * (ent >> 16);
-          }
-        }
-      }
-      return sum;
+      return __popc(s2) + 2u * __popc(s5) + 4u * __popc(s6) + 8u * __popc(c6);
     }
   }
   uint32_t sum = 0;
@@ -293,21 +245,19 @@ __device__ __forceinline__ uint32_t read_of(const uint64_t* __restrict__ cand_of
   return lo;
 }
 
-// CTAs per SM.  Up to 128-byte vectors: eight (64 warps, 32 registers a
-// thread); the gathers are latency-bound, and the extra warps outweigh a few
-// spilled words.  512-byte vectors (q = 6): six (40 registers), where the
-// spills of the 32-register layout cost more than the warps gain.
-__host__ __device__ constexpr int cand_ctas_per_sm(int wpb) { return wpb >= 128 ? 6 : 8; }
+// CTAs per SM: eight (64 warps, 32 registers a thread); the gathers are
+// latency-bound, and the extra warps outweigh a few spilled words.
+constexpr int kCandCtasPerSm = 8;
 
 template <int WPB, int U>
-__global__ void __launch_bounds__(kWarps * 32, cand_ctas_per_sm(WPB)) k_candidates(CandArgs a) {
+__global__ void __launch_bounds__(kWarps * 32, kCandCtasPerSm) k_candidates(CandArgs a) {
   using C = Cfg<WPB>;
   constexpr int WL = C::WL, G = C::G, CPW = C::CPW;
   extern __shared__ uint32_t s_warp[];
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t r4 = a.ix.r4;
   uint32_t* hist = s_warp + warp * warp_smem_words(r4, WPB);  // byte t = multiplicity of token t
-  uint32_t* xplanes = hist + hist_words_of(r4);  // higher planes or heavy tokens
+  uint32_t* xplanes = hist + hist_words_of(r4);  // higher planes
   const uint32_t sub = lane % G;     // this lane's slice of a bin vector
   const uint32_t slot = lane / G;    // which of the warp's CPW candidates
   if (*(volatile uint32_t*)&a.ctl->status) return;
@@ -321,7 +271,7 @@ __global__ void __launch_bounds__(kWarps * 32, cand_ctas_per_sm(WPB)) k_candidat
       c_end > c_begin ? chunk_size(c_end - c_begin, (uint64_t)gridDim.x * kWarps) : kChunkMin;
   const uint64_t n_chunks = c_end > c_begin ? (c_end - c_begin + chunk - 1) / chunk : 0;
 
-  uint32_t cur = 0xFFFFFFFFu, K = 0, thr = 0, nh = 0;  // the read whose planes are built
+  uint32_t cur = 0xFFFFFFFFu, K = 0, thr = 0;  // the read whose planes are built
   const uint32_t last_row = (uint32_t)(a.ix.bm_rows - 1);
   const uint32_t num_bins = (uint32_t)a.ix.num_bins;  // bins are uint32 (checked at build)
   bool bad = false;  // this lane saw a candidate id outside [0, num_bins)
@@ -356,7 +306,7 @@ __global__ void __launch_bounds__(kWarps * 32, cand_ctas_per_sm(WPB)) k_candidat
         load_ids<U, CPW>(seg, 0, n, slot, bc);
         if (r != cur) {
           cur = r;
-          K = build_planes<WPB, WL>(a.rv, r, r4, hist, xplanes, lane, sub, P, &thr, &nh);
+          K = build_planes<WPB, WL>(a.rv, r, r4, hist, xplanes, lane, sub, P, &thr);
         }
         // U independent gathers in flight per lane group; the ids of the
         // next step are fetched before this step's vectors are used
@@ -393,20 +343,8 @@ __global__ void __launch_bounds__(kWarps * 32, cand_ctas_per_sm(WPB)) k_candidat
           uint32_t sums[U];
 #pragma unroll
           for (int u = 0; u < U; ++u)
-            sums[u] = off + u * CPW + slot < n ? plane_sum<WPB, WL>(v[u], P, K, xplanes, sub, nh) : 0u;
-          if constexpr (G == 32) {
-            // a lane group is the whole warp (512-byte vectors): one
-            // full-warp reduction per candidate, and lane u emits candidate u
-            uint32_t total = 0, id = 0;
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-              const uint32_t t = __reduce_add_sync(0xFFFFFFFFu, sums[u]);
-              total = lane == (uint32_t)u ? t : total;
-              id = lane == (uint32_t)u ? bc[u] : id;
-            }
-            const uint32_t c = off + lane;
-            emit(lane < (uint32_t)U && c < n && id < num_bins && total >= thr, c, total);
-          } else if constexpr (U > 1 && U <= G) {
+            sums[u] = off + u * CPW + slot < n ? plane_sum<WPB, WL>(v[u], P, K, xplanes, sub) : 0u;
+          if constexpr (U > 1 && U <= G) {
             // the U sums reduced over the lane group at once: each lane ends
             // with the total of candidate uq, held by G/U lanes
             const uint32_t total = reduce_scatter<G, U>(sums, sub);
@@ -531,6 +469,198 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_refine(IndexView ix, ReadsVi
   }
 }
 
+// Candidate lists over large vectors (q = 6, 512 bytes), by token look-ups.
+// A random 512-byte row costs DRAM its bytes (13.7e9 rows/s), and half of one
+// half (27e9; a single 128-byte line 38e9), so the bin is ruled out from as
+// few lines as possible: the tokeniser groups a read's tokens by line,
+// fullest line first, and lane j looks up token 32*s + j of the first
+// `stage` groups of 32 -- as many as leave more than D' misses expected -- in
+// U candidates at once; one redux per candidate counts the tokens present.
+// Only a bin that could still pass has the rest of its tokens looked up.
+// Measured on GB300 (300k reads of 150 bp, e = 7, 98.9M candidates): 3.83 ms,
+// 0.97 of the two-line rate; ANDing whole vectors with bit planes of the read
+// took 9.48 ms at 91 warp instructions a candidate.  The same look-ups over
+// 128-byte vectors (q = 5, mixed reads) lost to the planes, 9.8 against 8.6
+// ms: one line is read either way, and a quarter warp per vector issues less.
+constexpr int kStageMax = 4;
+
+struct StageTokens {
+  const char* at[kStageMax];  // the token's word in row 0, or a zero word
+  uint32_t step[kStageMax];   // bytes from row to row (0 for the zero word)
+  uint32_t bit[kStageMax];    // token & 31
+};
+
+// alive bits (candidate k of the batch) after the first S groups of tokens.
+// At the most groups, reads with large budgets leave many bins alive, so lane
+// k keeps candidate k's tokens present and the rest of the check goes on from
+// there; with fewer groups almost every bin ends here and starts over if not.
+template <int S, int U>
+__device__ __forceinline__ uint32_t stage_scan(const StageTokens& st, uint32_t ids, uint32_t n,
+                                               uint32_t need, uint32_t lane, uint32_t& present) {
+  uint32_t alive = 0;
+  for (uint32_t k = 0; k < n; k += U) {
+    uint32_t w[U][S];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint32_t row = __shfl_sync(0xFFFFFFFFu, ids, k + u);
+#pragma unroll
+      for (int s = 0; s < S; ++s)
+        w[u][s] = __ldg(reinterpret_cast<const uint32_t*>(st.at[s] + (uint64_t)row * st.step[s]));
+    }
+    uint32_t a = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      uint32_t c = 0;
+#pragma unroll
+      for (int s = 0; s < S; ++s) c += (w[u][s] >> st.bit[s]) & 1u;
+      c = __reduce_add_sync(0xFFFFFFFFu, c);
+      if (c >= need) a |= 1u << u;
+      if (S == kStageMax) present = lane == k + u ? c : present;
+    }
+    alive |= a << k;
+  }
+  return alive;
+}
+
+template <int U>
+__global__ void __launch_bounds__(kWarps * 32, 6) k_candidates_lookup(CandArgs a, uint32_t miss256) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t r4 = a.ix.r4, wpb = a.ix.wpb;
+  if (*(volatile uint32_t*)&a.ctl->status) return;
+  if (gated_off(a.ctl, a.live)) return;
+  const uint32_t n_reads = live_reads(a.ctl, a.live, a.rv.n_reads);
+  if (n_reads == 0) return;
+  const uint64_t c_begin = a.cand_off[0], c_end = a.cand_off[n_reads];
+  if (c_end <= c_begin) return;
+  const uint64_t chunk = chunk_size(c_end - c_begin, (uint64_t)gridDim.x * kWarps);
+  const uint64_t n_chunks = (c_end - c_begin + chunk - 1) / chunk;
+  const uint32_t num_bins = (uint32_t)a.ix.num_bins;
+  // a word of the control block that stays zero: what a q-gram with a
+  // non-base, or a lane past the read's tokens, looks up
+  const char* zero = reinterpret_cast<const char*>(a.ctl->pad);
+
+  uint32_t cur = 0xFFFFFFFFu, ntok = 0, dmax = 0, stage = 0, need = 0;
+  const uint16_t* tok = nullptr;
+  StageTokens st;
+  bool bad = false;
+  uint32_t cj_next = 0;
+  if (lane == 0) cj_next = atomicAdd(&a.ctl->item, 1u);
+  for (;;) {
+    const uint32_t cj = __shfl_sync(0xFFFFFFFFu, cj_next, 0);
+    if (cj >= n_chunks) break;
+    if (lane == 0) cj_next = atomicAdd(&a.ctl->item, 1u);
+    const uint64_t base = c_begin + (uint64_t)cj * chunk;
+    const uint32_t clen = (uint32_t)min(chunk, c_end - base);
+    uint32_t r = read_of(a.cand_off, n_reads, base, lane);
+    uint32_t c1 = (uint32_t)min(a.cand_off[r + 1] - base, (uint64_t)clen);
+    uint32_t p = 0;
+    while (p < clen) {
+      const uint32_t c1_next = r + 2 <= n_reads && c1 < clen
+                                   ? (uint32_t)min(a.cand_off[r + 2] - base, (uint64_t)clen)
+                                   : c1;
+      uint32_t id_next = p + lane < c1 ? (uint32_t)__ldg(a.cand + base + p + lane) : 0u;
+      if (c1 > p && r != cur) {
+        cur = r;
+        const uint32_t m = a.rv.meta[r];
+        ntok = m & 0xFFu;
+        dmax = (m >> 8) & 0xFFu;
+        tok = a.rv.tokens + (uint64_t)r * a.rv.copies * a.rv.ts;
+        // groups of 32 tokens that leave D' + 6 misses expected
+        stage = min(min(((dmax + 6u) * 8u + miss256 - 1u) / miss256, (ntok + 31u) / 32u),
+                    (uint32_t)kStageMax);
+#pragma unroll
+        for (int s = 0; s < kStageMax; ++s) {
+          const uint32_t t = s * 32u + lane < ntok ? tok[s * 32u + lane] : rowPad(r4);
+          const bool on = t < r4 && (uint32_t)s < stage;
+          st.at[s] = on ? reinterpret_cast<const char*>(a.ix.bm + (t >> 5)) : zero;
+          st.step[s] = on ? wpb * 4u : 0u;
+          st.bit[s] = t & 31u;
+        }
+        const uint32_t n1 = min(stage * 32u, ntok);
+        need = n1 > dmax ? n1 - dmax : 0u;  // fewer of these present: more than D' misses
+      }
+      for (; p < c1; p += 32) {
+        const uint32_t n = min(c1 - p, 32u);
+        const uint32_t id = id_next;
+        if (p + 32u + lane < c1) id_next = (uint32_t)__ldg(a.cand + base + p + 32u + lane);
+        const bool ok = lane < n && id < num_bins;
+        bad |= lane < n && !ok;
+        const uint32_t row = ok ? id : 0u;
+        uint32_t alive, present = 0;
+        switch (stage) {
+          case 1: alive = stage_scan<1, U>(st, row, n, need, lane, present); break;
+          case 2: alive = stage_scan<2, U>(st, row, n, need, lane, present); break;
+          case 3: alive = stage_scan<3, U>(st, row, n, need, lane, present); break;
+          default: alive = stage_scan<kStageMax, U>(st, row, n, need, lane, present); break;
+        }
+        alive &= __ballot_sync(0xFFFFFFFFu, ok);
+        // the few bins left: all their tokens, four bins side by side
+        uint32_t found = 0;  // sum + 1 of this lane's candidate
+        while (alive) {
+          constexpr int V = 4;
+          const uint32_t* vec[V];
+          uint32_t k[V], misses[V], on = 0;
+#pragma unroll
+          for (int v = 0; v < V; ++v) {
+            k[v] = alive ? (uint32_t)__ffs(alive) - 1u : 0u;
+            if (alive) on |= 1u << v;
+            alive &= alive - 1u;
+            vec[v] = a.ix.bm + (uint64_t)__shfl_sync(0xFFFFFFFFu, row, k[v]) * wpb;
+            misses[v] = 0;
+            if (stage == (uint32_t)kStageMax)
+              misses[v] = min(kStageMax * 32u, ntok) - __shfl_sync(0xFFFFFFFFu, present, k[v]);
+          }
+          for (uint32_t j = stage == (uint32_t)kStageMax ? kStageMax * 32u : 0u; on && j < ntok;
+               j += 32) {
+            const uint32_t t = j + lane < ntok ? tok[j + lane] : rowPad(r4);
+            uint32_t w[V];
+#pragma unroll
+            for (int v = 0; v < V; ++v)
+              w[v] = t < r4 && (on >> v & 1u) ? __ldg(vec[v] + (t >> 5)) : 0u;
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+              const bool miss = t != rowPad(r4) && !((w[v] >> (t & 31u)) & 1u);
+              misses[v] += __popc(__ballot_sync(0xFFFFFFFFu, miss));
+              if (misses[v] > dmax) on &= ~(1u << v);
+            }
+          }
+#pragma unroll
+          for (int v = 0; v < V; ++v)
+            if ((on >> v & 1u) && lane == k[v]) found = ntok - misses[v] + 1u;
+        }
+        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, found != 0);
+        if (bal) {
+          unsigned long long first = 0;
+          if (lane == 0) first = atomicAdd(&a.ctl->n_rec, (unsigned long long)__popc(bal));
+          first = __shfl_sync(0xFFFFFFFFu, first, 0);
+          const unsigned long long pos = first + __popc(bal & ((1u << lane) - 1u));
+          if (found && pos < a.rec.cap) {
+            a.rec.keys[pos] = base + p + lane;
+            a.rec.counts[pos] = (uint8_t)(found - 1u);
+          }
+        }
+      }
+      p = c1;
+      ++r;
+      c1 = c1_next;
+    }
+  }
+  if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) atomicOr(&a.ctl->status, kStatusBadCand);
+}
+
+template <int U>
+void launch_lookup(const CandArgs& a, cudaStream_t st) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  // share of a window's tokens that a random one misses, in 1/256
+  const double grams = (double)a.ix.B + a.ix.ext - a.ix.q + 1;
+  const double miss = exp(-grams / (double)a.ix.r4);
+  const uint32_t miss256 = miss * 256.0 < 16.0 ? 16u : (uint32_t)(miss * 256.0);
+  ProfScope ps("candidates", st);
+  k_candidates_lookup<U><<<(unsigned)(sms > 0 ? sms : 1) * 6u, kWarps * 32, 0, st>>>(a, miss256);
+}
+
 template <int WPB, int U>
 void launch_u(const CandArgs& a, cudaStream_t st) {
   const size_t smem = (size_t)kWarps * warp_smem_words(a.ix.r4, WPB) * sizeof(uint32_t);
@@ -573,7 +703,7 @@ void launch_refine(const IndexView& ix, const ReadsView& rv, const unsigned long
 void launch_candidates(const IndexView& ix, const ReadsView& rv, const int32_t* cand,
                        const uint64_t* cand_off, RecordsView rec, Ctl* ctl, cudaStream_t st,
                        Live live, uint32_t unroll) {
-  if (unroll == 0) unroll = kDefaultCandUnroll;
+  if (unroll == 0) unroll = ix.wpb > 32 ? kDefaultLookupUnroll : kDefaultCandUnroll;
   if (rv.n_reads == 0) return;
   CandArgs a{ix, rv, cand, cand_off, rec, ctl, live};
   switch (ix.wpb) {
@@ -581,7 +711,12 @@ void launch_candidates(const IndexView& ix, const ReadsView& rv, const int32_t* 
     case 2: launch_t<2>(a, st, unroll); break;
     case 8: launch_t<8>(a, st, unroll); break;
     case 32: launch_t<32>(a, st, unroll); break;
-    case 128: launch_t<128>(a, st, unroll); break;
+    case 128:
+      if (unroll >= 8) launch_lookup<8>(a, st);
+      else if (unroll >= 4) launch_lookup<4>(a, st);
+      else if (unroll >= 2) launch_lookup<2>(a, st);
+      else launch_lookup<1>(a, st);
+      break;
     default: break;  // q outside 2..6 is rejected by grim_build
   }
 }

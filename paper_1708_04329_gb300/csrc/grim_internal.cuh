@@ -123,14 +123,23 @@ void launch_row_popcount(const uint32_t* tm, uint32_t rows, uint64_t words_per_r
 
 void launch_reverse_complement(const char* reads, const uint64_t* offsets, const uint32_t* lens,
                                uint32_t n_reads, char* out, cudaStream_t st);
+// order: how each token row is written (the sums do not depend on it).
+enum class TokenOrder : uint32_t {
+  kPosition,  // as they come in the read
+  kRarest,    // rarest first (IndexView::presence), repeats last
+  kCyclic,    // rarest first within row classes, 4 block-rotated copies (256-bin tiles)
+  kLines,     // grouped by the 128-byte line of a bin vector that holds them, fullest line first
+};
 // max_e: reads with a larger budget are an argument error (graph launches
 // fix the counter depth from it); 0xFFFF = no limit.  max_bases: size of the
 // reads buffer when known (a read ending past it fails the batch with
-// kStatusArg), else ~0.  rv.copies token copies per read are written.
+// kStatusArg), else ~0.  rv.copies token copies per read are written.  The
+// order is chosen from the mode: lists (`cand_mode`) or all bins.
 void launch_tokenise(const char* reads, const uint64_t* offsets, const uint32_t* lens,
                      const uint16_t* e, const IndexView& ix, ReadsView rv, uint16_t* tokens,
-                     uint32_t* meta, Ctl* ctl, cudaStream_t st, Live live = {false, 0},
-                     uint32_t max_e = 0xFFFFu, uint64_t max_bases = ~0ull);
+                     uint32_t* meta, Ctl* ctl, cudaStream_t st, bool cand_mode,
+                     Live live = {false, 0}, uint32_t max_e = 0xFFFFu,
+                     uint64_t max_bases = ~0ull);
 // ctl->blk_max / blk_lo: the most 16-token blocks of a read of the batch, and
 // 32 - the fewest
 void launch_block_spread(const uint32_t* lens, uint32_t n_reads, uint32_t q, Ctl* ctl,

@@ -152,7 +152,7 @@ int capture(grim_plan* p) {
   if (p->hio) k_copy_in<<<dim3(64, kCopySegs), 256, 0, st>>>(p->copy, p->ctl);
   launch_tokenise(B.reads, B.offsets, B.lens, B.e, v, rv,
                   reinterpret_cast<uint16_t*>(ws + L.tok), reinterpret_cast<uint32_t*>(ws + L.meta),
-                  p->ctl, st, live, d.max_e, d.max_bases);
+                  p->ctl, st, p->cand_mode, live, d.max_e, d.max_bases);
   if (p->cand_mode) {
     launch_check_candidates(B.cand_off, d.max_reads, d.max_cand, p->ctl, st, live);
     launch_candidates(v, rv, B.cand, B.cand_off, ra, p->ctl, st, live, d.cand_unroll);

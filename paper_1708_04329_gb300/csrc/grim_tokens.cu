@@ -31,12 +31,18 @@ constexpr uint32_t kMaxStride = 256;  // token stride: <= 255 tokens rounded up 
 // warp's 16 groups cover the four bank groups four times each.  Every block
 // holds the same tokens in every copy, so the per-block early exit and every
 // sum are unchanged.
+//
+// Candidate lists at q = 6 (TokenOrder::kLines): q-grams with a non-base
+// first (misses that need no look-up), then the tokens grouped by the
+// 128-byte line of a 512-byte bin vector that holds them (token >> 10), the
+// line with the most tokens first, so that the list kernel's first look-ups
+// touch as few lines of a vector as can rule the bin out.
 __global__ void __launch_bounds__(kTokWarps * 32) k_tokenise(
     const char* __restrict__ reads, const uint64_t* __restrict__ offsets,
     const uint32_t* __restrict__ lens, const uint16_t* __restrict__ e, uint32_t n_reads, uint32_t q,
     uint32_t max_read_len, uint32_t r4, uint32_t ts, const uint32_t* __restrict__ presence,
     uint16_t* __restrict__ tokens, uint32_t* __restrict__ meta, Ctl* ctl, Live live,
-    uint32_t max_e, uint64_t max_bases, uint32_t copies) {
+    uint32_t max_e, uint64_t max_bases, uint32_t copies, TokenOrder order) {
   __shared__ unsigned long long s_key[kTokWarps][kMaxStride];
   __shared__ uint16_t s_row[kTokWarps][kMaxStride];
   __shared__ uint16_t s_seq[kTokWarps][kMaxStride];
@@ -77,7 +83,7 @@ __global__ void __launch_bounds__(kTokWarps * 32) k_tokenise(
     }
     const bool clean = (flags & 4u) == 0;
     const uint32_t row = clean ? v : rowInvalid(r4);
-    if (!presence && copies == 1) {  // no order wanted (candidate lists): positions as they are
+    if (order == TokenOrder::kPosition) {
       out[j] = (uint16_t)row;
       continue;
     }
@@ -85,7 +91,35 @@ __global__ void __launch_bounds__(kTokWarps * 32) k_tokenise(
     s_seq[warp][j] = (uint16_t)row;  // the order without a presence table
   }
   __syncwarp();
-  for (uint32_t j = lane; j < ntok && (presence || copies > 1); j += 32) {
+  if (order == TokenOrder::kLines) {
+    // tokens per line (class 4: not a token), then each line's first position
+    uint32_t cnt[5] = {0, 0, 0, 0, 0};
+    for (uint32_t j0 = 0; j0 < ntok; j0 += 32) {
+      const uint32_t c = j0 + lane < ntok ? s_row[warp][j0 + lane] >> 10 : 5u;
+#pragma unroll
+      for (uint32_t k = 0; k < 5; ++k) cnt[k] += __popc(__ballot_sync(0xFFFFFFFFu, c == k));
+    }
+    uint32_t at[5];
+    at[4] = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      at[k] = cnt[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (cnt[i] > cnt[k] || (cnt[i] == cnt[k] && i < k)) at[k] += cnt[i];
+    }
+    for (uint32_t j0 = 0; j0 < ntok; j0 += 32) {
+      const uint32_t c = j0 + lane < ntok ? s_row[warp][j0 + lane] >> 10 : 5u;
+#pragma unroll
+      for (uint32_t k = 0; k < 5; ++k) {
+        const uint32_t m = __ballot_sync(0xFFFFFFFFu, c == k);
+        if (c == k) out[at[k] + __popc(m & ((1u << lane) - 1u))] = s_row[warp][j0 + lane];
+        at[k] += __popc(m);
+      }
+    }
+  }
+  const bool ranked = order == TokenOrder::kRarest || order == TokenOrder::kCyclic;
+  for (uint32_t j = lane; j < ntok && ranked; j += 32) {
     // a clean token whose value already occurred earlier in the read misses
     // exactly the bins its first occurrence misses: it adds no new bins to
     // the dead set, so repeats go after every distinct token (1024-bin
@@ -100,7 +134,7 @@ __global__ void __launch_bounds__(kTokWarps * 32) k_tokenise(
     s_key[warp][j] = ((unsigned long long)repeat << 48) | (rare << 8) | j;
   }
   __syncwarp();
-  if (presence && copies == 1) {
+  if (order == TokenOrder::kRarest) {
     // rank = number of smaller keys (keys are distinct: position breaks ties)
     for (uint32_t j = lane; j < ntok; j += 32) {
       const unsigned long long mine = s_key[warp][j];
@@ -108,7 +142,7 @@ __global__ void __launch_bounds__(kTokWarps * 32) k_tokenise(
       for (uint32_t i = 0; i < ntok; ++i) rank += s_key[warp][i] < mine;
       out[rank] = s_row[warp][j];
     }
-  } else if (copies > 1) {
+  } else if (order == TokenOrder::kCyclic) {
     if (presence) {
       // rank of each token within its row class, and the size of each class
       uint32_t cnt = 0;  // 4 byte counters: tokens of class c counted by this lane
@@ -236,16 +270,23 @@ void launch_reverse_complement(const char* reads, const uint64_t* offsets, const
 
 void launch_tokenise(const char* reads, const uint64_t* offsets, const uint32_t* lens,
                      const uint16_t* e, const IndexView& ix, ReadsView rv, uint16_t* tokens,
-                     uint32_t* meta, Ctl* ctl, cudaStream_t st, Live live, uint32_t max_e,
-                     uint64_t max_bases) {
+                     uint32_t* meta, Ctl* ctl, cudaStream_t st, bool cand_mode, Live live,
+                     uint32_t max_e, uint64_t max_bases) {
   const uint32_t copies = rv.copies;
+  // lists read whole token rows in any order up to 128-byte vectors; larger
+  // ones (q = 6) are looked up line by line
+  const TokenOrder order = cand_mode ? (ix.wpb > 32 ? TokenOrder::kLines : TokenOrder::kPosition)
+                           : copies > 1   ? TokenOrder::kCyclic
+                           : ix.presence ? TokenOrder::kRarest
+                                         : TokenOrder::kPosition;
   if (rv.n_reads == 0) return;
   const uint32_t threads = kTokWarps * 32;
   uint64_t grid = ((uint64_t)rv.n_reads * 32 + threads - 1) / threads;
   ProfScope ps("tokenise", st);
   k_tokenise<<<(unsigned)grid, threads, 0, st>>>(reads, offsets, lens, e, rv.n_reads, ix.q,
                                                  ix.max_read_len, ix.r4, rv.ts, ix.presence, tokens,
-                                                 meta, ctl, live, max_e, max_bases, copies);
+                                                 meta, ctl, live, max_e, max_bases, copies,
+                                                 order);
 }
 
 void launch_block_spread(const uint32_t* lens, uint32_t n_reads, uint32_t q, Ctl* ctl,

@@ -622,3 +622,31 @@ def test_pass_list_order_by_length(n):
     assert len(got[0]) == n
     assert_same(got, oracle.filter(oracle.bin_vectors(g, 50, 5, 40), rs, cand_off=off, cand=cand))
     ix.close()
+
+
+@pytest.mark.parametrize("L", [6, 36, 37, 38, 69, 70, 101, 150, 250, 260])
+def test_q6_list_lookups(L):
+    """q = 6 lists are ruled out from the first groups of 32 tokens: reads of
+    one token, at and past a group's edge and of 255 tokens, budgets from 0
+    to T <= 0, reads with non-bases and of one repeated base, lists of 0, 1,
+    31, 32, 33 and 100 candidates, duplicates and all bins of a repeat."""
+    rng = np.random.default_rng(L)
+    g = rng.choice(np.frombuffer(b"ACGT", np.uint8), 40_000)
+    g[20_000:22_000] = np.tile(g[:125], 16)
+    g[30_000:30_400] = ord("A")
+    at = [20_010, 5, 30_050, 1234, 20_300, 39_000 - L, 777, 15_000]
+    reads = [g[p:p + L].tobytes().decode() for p in at] * 2
+    reads[1] = "N" + reads[1][1:]
+    reads[3] = reads[3][:L // 2] + "n" * (L - L // 2)
+    e = [0, 1, 2, L // 20, 5, 7, L // 6, 300] + [7] * 8
+    counts = [0, 1, 31, 32, 33, 100, 400, 64, 400, 1, 0, 5, 32, 96, 97, 400]
+    nb = -(-len(g) // 100)
+    cand = np.concatenate([rng.integers(0, nb, c) for c in counts]).astype(np.int32)
+    off = np.concatenate([[0], np.cumsum(counts)]).astype(np.uint64)
+    cand[off[6].astype(int):off[7].astype(int)] = np.arange(400) % nb
+    rs = Reads(reads, e)
+    ix = build(g, 100, 6, 260, layouts=2)
+    want = oracle.filter(oracle.bin_vectors(g, 100, 6, 260), rs, cand_off=off, cand=cand)
+    assert len(want[0]) > 64
+    assert_same(gpu_filter(ix, rs, off, cand, cap=2000), want)
+    ix.close()
