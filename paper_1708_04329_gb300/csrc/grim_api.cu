@@ -345,51 +345,53 @@ int grim_build_ex(const char* ref, uint64_t len, uint32_t B, uint32_t q, uint32_
     return code;
   };
   cudaError_t e;
-  // packed reference (one spare word at the end of each array for the
-  // two-word reads of the token extraction)
-  const uint64_t n32 = (len + 31) / 32;
-  uint32_t *codes = nullptr, *invalid = nullptr;
-  e = scratch_alloc(reinterpret_cast<void**>(&codes), (2 * n32 + 2) * sizeof(uint32_t), st);
-  if (e != cudaSuccess) return fail(cuda_fail(e));
-  e = scratch_alloc(reinterpret_cast<void**>(&invalid), (n32 + 2) * sizeof(uint32_t), st);
-  if (e != cudaSuccess) {
-    cudaFreeAsync(codes, st);
-    return fail(cuda_fail(e));
-  }
-  cudaMemsetAsync(codes + 2 * n32, 0, 2 * sizeof(uint32_t), st);
-  cudaMemsetAsync(invalid + n32, 0xFF, 2 * sizeof(uint32_t), st);
-  launch_pack_ref(ref, len, codes, invalid, st);
-  // q >= 5: the token-major tables are bit transposes of the bin-major one
-  // (a scratch copy when the index keeps no bin-major table)
-  const bool transpose = v.q >= 5 && (ix->tm || ix->ctm);
+  // one pass from the letters to every table it can write; the other tables
+  // of q >= 5 are bit transposes of the bin-major one (a scratch copy when the
+  // index keeps none), those of q < 5 come from the packed reference
+  const uint32_t fused = build_fused_layouts(v, f);
+  const bool from_bm_tm = v.q >= 5 && ix->tm && !(fused & GRIM_LAYOUT_TOKEN_MAJOR);
+  const bool from_bm_ctm = v.q >= 5 && ix->ctm && !(fused & GRIM_LAYOUT_COARSE);
   uint32_t* bm = ix->bm;
-  if (!bm && transpose) {
+  if (!bm && (from_bm_tm || from_bm_ctm)) {
     e = scratch_alloc(reinterpret_cast<void**>(&bm), bm_bins * v.wpb * sizeof(uint32_t), st);
+    if (e != cudaSuccess) return fail(cuda_fail(e));
+  }
+  if (bm && bm_bins > v.num_bins)
+    cudaMemsetAsync(bm + v.num_bins * v.wpb, 0, (bm_bins - v.num_bins) * v.wpb * sizeof(uint32_t),
+                    st);
+  uint32_t *codes = nullptr, *invalid = nullptr;
+  if (fused) {
+    launch_build_fused(ref, v, cv, f, bm, from_bm_tm ? nullptr : ix->tm,
+                       from_bm_ctm ? nullptr : ix->ctm, st);
+  } else {
+    // packed reference (one spare word at the end of each array for the
+    // two-word reads of the token extraction)
+    const uint64_t n32 = (len + 31) / 32;
+    e = scratch_alloc(reinterpret_cast<void**>(&codes), (2 * n32 + 2) * sizeof(uint32_t), st);
+    if (e == cudaSuccess)
+      e = scratch_alloc(reinterpret_cast<void**>(&invalid), (n32 + 2) * sizeof(uint32_t), st);
     if (e != cudaSuccess) {
-      cudaFreeAsync(codes, st);
-      cudaFreeAsync(invalid, st);
+      if (codes) cudaFreeAsync(codes, st);
+      if (bm != ix->bm) cudaFreeAsync(bm, st);
       return fail(cuda_fail(e));
     }
+    cudaMemsetAsync(codes + 2 * n32, 0, 2 * sizeof(uint32_t), st);
+    cudaMemsetAsync(invalid + n32, 0xFF, 2 * sizeof(uint32_t), st);
+    launch_pack_ref(ref, len, codes, invalid, st);
+    if (bm) launch_build_bin_major(codes, invalid, v, bm, st);
+    if (v.q < 5) {
+      if (ix->tm) launch_build_token_major(codes, invalid, v, ix->tm, st);
+      if (ix->ctm) launch_build_token_major(codes, invalid, cv, ix->ctm, st);
+    }
+    cudaFreeAsync(codes, st);
+    cudaFreeAsync(invalid, st);
   }
-  if (bm) {
-    if (bm_bins > v.num_bins)
-      cudaMemsetAsync(bm + v.num_bins * v.wpb, 0, (bm_bins - v.num_bins) * v.wpb * sizeof(uint32_t),
-                      st);
-    launch_build_bin_major(codes, invalid, v, bm, st);
-  }
-  if (transpose) {
-    if (ix->tm) launch_tm_from_bm(bm, v, v.wpb, 1, ix->tm, st);
-    if (ix->ctm) launch_tm_from_bm(bm, cv, v.wpb, f, ix->ctm, st);
-  } else {
-    if (ix->tm) launch_build_token_major(codes, invalid, v, ix->tm, st);
-    if (ix->ctm) launch_build_token_major(codes, invalid, cv, ix->ctm, st);
-  }
+  if (from_bm_tm) launch_tm_from_bm(bm, v, v.wpb, 1, ix->tm, st);
+  if (from_bm_ctm) launch_tm_from_bm(bm, cv, v.wpb, f, ix->ctm, st);
   if (bm != ix->bm) cudaFreeAsync(bm, st);
   // token presence from the table the all-bins filter sweeps first
   if (ix->ctm) launch_row_popcount(ix->ctm, cv.r4, cv.wpad, ix->presence, st);
   else if (ix->tm) launch_row_popcount(ix->tm, v.r4, v.wpad, ix->presence, st);
-  cudaFreeAsync(codes, st);
-  cudaFreeAsync(invalid, st);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   prof_collect();

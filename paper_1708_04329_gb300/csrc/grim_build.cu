@@ -1,12 +1,15 @@
 // Index build (§GRIM-Filter: the reference is scanned once and every bin's
 // bit vector is set from the tokens that occur in it; Fig. 2):
-//   k_pack_ref          ASCII -> 2-bit codes + not-a-base mask
+//   k_build_fused       q = 5, 6: ASCII straight to bin-major vectors and, at
+//                       q = 5, both token-major tables in one pass
+//   k_pack_ref          ASCII -> 2-bit codes + not-a-base mask (the kernels below)
 //   k_build_bin_major   one warp per bin, bit vector in shared memory
 //   k_build_token_major one CTA per 1024-bin tile, the tile's [4^q rows x tile
 //                       words] bitmap in shared memory (q <= 4)
 //   k_tm_from_bm        q = 5, 6: token-major (and coarse token-major) tiles
 //                       as bit transposes of the bin-major vectors, ORed over
-//                       the members of each super-bin for the coarse table
+//                       the members of each super-bin for the coarse table,
+//                       where k_build_fused does not write them
 #include "grim_internal.cuh"
 
 namespace grim {
@@ -216,6 +219,194 @@ __global__ void k_row_popcount(const uint32_t* __restrict__ tm, uint64_t words,
   }
 }
 
+// 16 bases (bytes, first base lowest) to a code word (first base in the top
+// bits) and a not-a-base mask.  A letter is a base iff folding its case and
+// looking its 2-bit code up in "ACGT" gives it back.
+__device__ __forceinline__ void pack16(const uint4& v, uint32_t& code, uint32_t& inv) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  code = inv = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t u = w[i] & 0xDFDFDFDFu;
+    const uint32_t c = ((u >> 1) ^ (u >> 2)) & 0x03030303u;
+    uint32_t sel = (c | (c >> 4)) & 0x00FF00FFu;
+    sel = (sel | (sel >> 8)) & 0xFFFFu;  // the four codes as byte selectors
+    const uint32_t x = __byte_perm(0x54474341u, 0u, sel) ^ u;
+    // the four codes side by side, the first in the top two bits of a byte
+    code = (code << 8) | ((c * 0x40100401u) >> 24);
+    if (x) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if ((x >> (8 * k)) & 0xFFu) inv |= 1u << (4 * i + k);
+    }
+  }
+}
+
+// The whole build of a tile of kFusedBins bins by one CTA (q = 5, 6), from the
+// reference's letters:
+//   1. the tile's letters become 2-bit codes and a not-a-base mask in shared
+//      memory (SWAR, 16 letters a thread and load);
+//   2. each warp walks the cores (B positions) of its run of 32 bins and the
+//      k + 1 cores after it, and sets the tokens starting in a core in a
+//      vector of its own: P, those of the first `rem` positions, then A, all
+//      of them.  A q-gram lies inside bin b's window iff it starts in
+//      [bB, bB + B + ext - q], which with ext - q + 1 = k B + rem is
+//      A(b) | ... | A(b + k) | P(b + k + 1): every token is set once, not once
+//      for each of the bins whose windows overlap there;
+//   3. (q = 5) the run's 32 vectors, one word a lane, are a 32 x 32 bit
+//      transpose away from the token rows; both token-major tables leave
+//      through shared memory in row pieces of 64 and 64 / f bytes.
+// Bound by shared-memory atomics (one per token) and the letters and tables
+// themselves (8.1 GB for the 3.1 Gbp index at q = 5).
+constexpr uint32_t kFusedBins = 512, kFusedWarps = kFusedBins / 32, kFusedMaxK = 3;
+constexpr uint32_t kFusedGroups = kFusedBins / 32;  // tile words of a token row
+
+struct FusedArgs {
+  const char* ref;
+  uint64_t n, num_bins, wpad, cwpad;
+  uint32_t B, q, k, rem;
+  uint32_t code_words;  // code words of the tile in shared memory (16 bases each)
+  uint32_t f;           // coarse factor (ctm set: 2, 4, 8 or 16)
+  uint32_t* bm;
+  uint32_t* tm;
+  uint32_t* ctm;
+};
+
+// shared memory, in words: row pieces / vectors of the tile (q = 5), then
+// codes and mask, later the coarse row pieces, then a vector per warp
+__host__ __device__ constexpr uint32_t fused_rows_words(uint32_t wpl) {
+  return wpl == 1 ? 1024u * kFusedGroups + 32u : 0u;
+}
+__host__ __device__ constexpr uint32_t fused_code_words(uint32_t wpl, uint32_t code_words) {
+  const uint32_t c = code_words + (code_words + 1) / 2 + 2;
+  const uint32_t coarse = wpl == 1 ? 1024u * (kFusedGroups / 2) + 32u : 0u;
+  return c > coarse ? c : coarse;
+}
+
+template <uint32_t WPL>  // words of a vector per lane: 1 (q = 5) or 4 (q = 6)
+__global__ void __launch_bounds__(kFusedWarps * 32, 2) k_build_fused(FusedArgs a) {
+  extern __shared__ uint32_t s_fused[];
+  uint32_t* s_rows = s_fused;
+  uint32_t* s_code = s_fused + fused_rows_words(WPL);
+  uint16_t* inv16 = reinterpret_cast<uint16_t*>(s_code + a.code_words);  // 16 positions each
+  uint32_t* s_vec = s_code + fused_code_words(WPL, a.code_words);
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint64_t bin0 = (uint64_t)blockIdx.x * kFusedBins;
+  const uint64_t p0 = bin0 * a.B;  // a multiple of 512: 16-byte aligned in an aligned reference
+  // 1. letters -> codes; positions past the reference are not bases
+  bool any = false;
+  const bool aligned = (reinterpret_cast<uintptr_t>(a.ref) & 15u) == 0;
+  for (uint32_t i = tid; i < a.code_words; i += kFusedWarps * 32) {
+    const uint64_t p = p0 + 16ull * i;
+    uint32_t code = 0, inv = 0xFFFFu;
+    if (aligned && p + 16 <= a.n) {
+      pack16(__ldg(reinterpret_cast<const uint4*>(a.ref + p)), code, inv);
+    } else if (p < a.n) {
+      uint32_t w[4] = {0, 0, 0, 0};
+      for (uint32_t j = 0; j < 16 && p + j < a.n; ++j)
+        w[j >> 2] |= (uint32_t)(uint8_t)a.ref[p + j] << (8 * (j & 3));
+      pack16(make_uint4(w[0], w[1], w[2], w[3]), code, inv);  // 0 is not a base
+    }
+    s_code[i] = code;
+    inv16[i] = (uint16_t)inv;
+    any |= inv != 0;
+  }
+  uint32_t* v = s_vec + warp * 32 * WPL;
+#pragma unroll
+  for (uint32_t w = 0; w < WPL; ++w) v[w * 32 + lane] = 0;
+  any = __syncthreads_or(any);
+
+  // 2. tokens starting at tile positions [lo, hi) into the warp's vector
+  const uint32_t sh = 32u - 2u * a.q, qmask = (1u << a.q) - 1u;
+  auto set_tokens = [&](uint32_t lo, uint32_t hi) {
+    for (uint32_t p = lo + lane; p < hi; p += 32) {
+      const uint32_t* c = s_code + (p >> 4);
+      const uint32_t t = __funnelshift_l(c[1], c[0], 2u * p) >> sh;
+      if (any) {
+        const uint16_t* m = inv16 + (p >> 4);
+        if ((((uint32_t)m[0] | ((uint32_t)m[1] << 16)) >> (p & 15u)) & qmask) continue;
+      }
+      atomicOr(v + (t >> 5), 1u << (t & 31u));
+    }
+  };
+  uint32_t pend[kFusedMaxK + 1][WPL];  // bins c - k .. c so far (newest first)
+#pragma unroll
+  for (uint32_t i = 0; i <= kFusedMaxK; ++i)
+#pragma unroll
+    for (uint32_t w = 0; w < WPL; ++w) pend[i][w] = 0;
+  const uint32_t first = warp * 32;
+  for (uint32_t c = first; c <= first + 32 + a.k; ++c) {
+    const uint32_t lo = c * a.B;
+    set_tokens(lo, lo + a.rem);
+    __syncwarp();
+    // core c's first positions complete bin c - k - 1
+    const uint32_t done = c - a.k - 1;
+    if (c >= first + a.k + 1) {
+#pragma unroll
+      for (uint32_t w = 0; w < WPL; ++w) {
+        uint32_t x = v[w * 32 + lane];
+#pragma unroll
+        for (uint32_t i = 0; i <= kFusedMaxK; ++i)
+          if (i == a.k) x |= pend[i][w];
+        if (a.bm && bin0 + done < a.num_bins)
+          a.bm[(bin0 + done) * (32 * WPL) + w * 32 + lane] = x;
+        if (WPL == 1) s_rows[done * 32 + lane] = x;
+      }
+    }
+    if (c == first + 32 + a.k) break;
+    set_tokens(lo + a.rem, lo + a.B);
+    __syncwarp();
+#pragma unroll
+    for (uint32_t w = 0; w < WPL; ++w) {
+      const uint32_t x = v[w * 32 + lane];
+      v[w * 32 + lane] = 0;
+#pragma unroll
+      for (uint32_t i = kFusedMaxK; i > 0; --i) pend[i][w] = pend[i - 1][w] | x;
+      pend[0][w] = x;
+    }
+    __syncwarp();
+  }
+  if (WPL != 1 || (!a.tm && !a.ctm)) return;
+
+  // 3. token rows: the coarse table's from the ORs of f vectors, then the bins'
+  __syncthreads();  // vectors complete, codes no longer read
+  uint32_t* s_coarse = s_code;
+  const uint32_t cgroups = a.ctm ? kFusedGroups / a.f : 0u;  // row words of the tile's super-bins
+  uint32_t x[32];
+  if (warp < cgroups) {
+#pragma unroll
+    for (uint32_t k = 0; k < 32; ++k) {
+      uint32_t w = 0;
+      for (uint32_t m = 0; m < a.f; ++m) w |= s_rows[((warp * 32 + k) * a.f + m) * 32 + lane];
+      x[k] = w;
+    }
+    transpose32(x);
+#pragma unroll
+    for (uint32_t j = 0; j < 32; ++j) s_coarse[(32u * lane + j) * cgroups + warp + lane] = x[j];
+  }
+#pragma unroll
+  for (uint32_t k = 0; k < 32; ++k) x[k] = s_rows[(first + k) * 32 + lane];
+  transpose32(x);
+  __syncthreads();  // every vector is in registers
+  if (a.tm) {
+#pragma unroll
+    for (uint32_t j = 0; j < 32; ++j) s_rows[(32u * lane + j) * kFusedGroups + warp + lane] = x[j];
+  }
+  __syncthreads();
+  const uint64_t col0 = (uint64_t)blockIdx.x * kFusedGroups;
+  if (a.tm && col0 < a.wpad)
+    for (uint32_t i = tid; i < 1024u * kFusedGroups; i += kFusedWarps * 32) {
+      const uint32_t t = i / kFusedGroups, col = i % kFusedGroups;
+      a.tm[(uint64_t)t * a.wpad + col0 + col] = s_rows[i + (t >> 5)];
+    }
+  const uint64_t ccol0 = (uint64_t)blockIdx.x * cgroups;
+  if (cgroups && ccol0 < a.cwpad)
+    for (uint32_t i = tid; i < 1024u * cgroups; i += kFusedWarps * 32) {
+      const uint32_t t = i / cgroups, col = i % cgroups;
+      a.ctm[(uint64_t)t * a.cwpad + ccol0 + col] = s_coarse[i + (t >> 5)];
+    }
+}
+
 }  // namespace
 
 void launch_tm_from_bm(const uint32_t* bm, const IndexView& unit_view, uint32_t wpb, uint32_t f,
@@ -241,6 +432,63 @@ void launch_row_popcount(const uint32_t* tm, uint32_t rows, uint64_t words_per_r
                          uint32_t* presence, cudaStream_t st) {
   ProfScope ps("row_popcount", st);
   k_row_popcount<<<rows, 512, 0, st>>>(tm, words_per_row, presence);
+}
+
+namespace {
+uint64_t fused_tile_words(const IndexView& v) {  // code words of a tile
+  const uint32_t span = v.ext - v.q + 1;
+  return ((uint64_t)(kFusedBins + span / v.B) * v.B + span % v.B + v.q + 15) / 16 + 1;
+}
+size_t fused_smem(const IndexView& v) {
+  const uint32_t wpl = v.wpb / 32;
+  return sizeof(uint32_t) * (fused_rows_words(wpl) +
+                             fused_code_words(wpl, (uint32_t)fused_tile_words(v)) +
+                             kFusedWarps * 32 * wpl);
+}
+}  // namespace
+
+uint32_t build_fused_layouts(const IndexView& v, uint32_t f) {
+  if (v.q < 5 || (v.ext - v.q + 1) / v.B > kFusedMaxK || fused_tile_words(v) > 65536 ||
+      fused_smem(v) > 227 * 1024)
+    return 0;
+  uint32_t can = GRIM_LAYOUT_BIN_MAJOR;
+  if (v.q == 5) can |= GRIM_LAYOUT_TOKEN_MAJOR;
+  // whole row words of super-bins in a tile
+  if (v.q == 5 && f > 1 && kFusedGroups % f == 0) can |= GRIM_LAYOUT_COARSE;
+  return can;
+}
+
+void launch_build_fused(const char* ref, const IndexView& v, const IndexView& cv, uint32_t f,
+                        uint32_t* bm, uint32_t* tm, uint32_t* ctm, cudaStream_t st) {
+  const uint32_t span = v.ext - v.q + 1;
+  FusedArgs a{};
+  a.ref = ref;
+  a.n = v.n;
+  a.num_bins = v.num_bins;
+  a.wpad = v.wpad;
+  a.cwpad = cv.wpad;
+  a.B = v.B;
+  a.q = v.q;
+  a.k = span / v.B;
+  a.rem = span % v.B;
+  a.code_words = (uint32_t)fused_tile_words(v);
+  a.f = f;
+  a.bm = bm;
+  a.tm = tm;
+  a.ctm = ctm;
+  // tiles up to the padded ends of the rows (their vectors are zero there)
+  uint64_t grid = (v.num_bins + kFusedBins - 1) / kFusedBins;
+  if (tm) grid = v.num_bins_pad / kFusedBins;
+  if (ctm && cv.num_bins_pad * f / kFusedBins > grid) grid = cv.num_bins_pad * f / kFusedBins;
+  const size_t smem = fused_smem(v);
+  ProfScope ps("build_fused", st);
+  if (v.q == 5) {
+    cudaFuncSetAttribute(k_build_fused<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_build_fused<1><<<(unsigned)grid, kFusedWarps * 32, smem, st>>>(a);
+  } else {
+    cudaFuncSetAttribute(k_build_fused<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_build_fused<4><<<(unsigned)grid, kFusedWarps * 32, smem, st>>>(a);
+  }
 }
 
 void launch_pack_ref(const char* ref, uint64_t n, uint32_t* codes, uint32_t* invalid,

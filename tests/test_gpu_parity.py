@@ -650,3 +650,44 @@ def test_q6_list_lookups(L):
     assert len(want[0]) > 64
     assert_same(gpu_filter(ix, rs, off, cand, cap=2000), want)
     ix.close()
+
+
+@pytest.mark.parametrize("q,B,mrl,factor,n,layouts,shift", [
+    (5, 200, 100, 2, 512 * 200, 7, 0),          # one whole tile, windows of two cores
+    (5, 200, 100, 2, 512 * 200 + 1, 7, 1),      # one base into the next; unaligned reference
+    (5, 100, 105, 4, 3 * 512 * 100 - 7, 7, 0),  # ext - q + 1 = B: no partial core
+    (5, 100, 250, 8, 60_000, 7, 0),             # windows of four cores
+    (5, 90, 250, 16, 100_003, 7, 3),
+    (5, 61, 250, 2, 40_000, 7, 0),              # more cores than the one-pass build takes
+    (5, 173, 101, 3, 120_000, 7, 0),            # a factor whose super-bins do not fill row words
+    (5, 200, 100, 2, 300_000, 1, 0),            # single tables
+    (5, 200, 100, 2, 300_000, 4, 0),
+    (5, 200, 5, 2, 4, 7, 0),                    # shorter than q
+    (5, 900, 100, 2, 500_000, 7, 0),            # a tile past shared memory
+    (6, 100, 150, 16, 512 * 100 + 37, 7, 0),
+    (6, 128, 250, 4, 90_001, 5, 2)])
+def test_one_pass_build_shapes(q, B, mrl, factor, n, layouts, shift):
+    """Tables of the one-pass build at its tile and window edges, against the
+    oracle, with lower case and runs of non-bases; shapes it leaves to the
+    other kernels beside them."""
+    from paper_1708_04329_gb300 import grim
+
+    rng = np.random.default_rng(n + B)
+    g = rng.choice(np.frombuffer(b"ACGTacgt", np.uint8), n)
+    for p in rng.integers(0, n, 5):
+        g[p:p + int(rng.integers(1, 12))] = ord("N")
+    if n > 60_000:
+        g[n // 2:n // 2 + 700] = ord("-")
+    dev = torch.zeros(n + shift, dtype=torch.uint8, device="cuda")
+    dev[shift:] = torch.from_numpy(g).cuda()
+    idx = grim.grim_build_ex(dev[shift:], B, q, mrl, layouts, factor)
+    oix = oracle.bin_vectors(g, B, q, mrl)
+    tm, bm = _gpu_tables(idx, q)
+    if bm is not None:
+        assert np.array_equal(bm.view(np.uint8).reshape(oix.num_bins, -1), oix.vecs)
+    if tm is not None:
+        assert np.array_equal(tm, oracle.token_major(oix))
+    if layouts & 4:
+        coarse = oracle.token_major(oracle.bin_vectors(g, factor * B, q, mrl))
+        assert np.array_equal(idx.coarse_token_major().cpu().numpy().view(np.uint32), coarse)
+    idx.close()
