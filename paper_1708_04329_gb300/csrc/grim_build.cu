@@ -201,14 +201,21 @@ __global__ void __launch_bounds__(1024) k_tm_from_bm(const uint32_t* __restrict_
   }
 }
 
-// One CTA per token row: the number of set bits, i.e. how many (super-)bins
-// hold the token.
-__global__ void k_row_popcount(const uint32_t* __restrict__ tm, uint64_t words,
-                               uint32_t* __restrict__ presence) {
+// The number of set bits of each token row, i.e. how many (super-)bins hold
+// the token: one CTA per row, 16 bytes a load (rows are whole 128-byte lines),
+// four loads in flight a thread (0.17 ms for 1 GB; 0.45 with 4-byte loads).
+__global__ void __launch_bounds__(512) k_row_popcount(const uint32_t* __restrict__ tm,
+                                                      uint64_t words,
+                                                      uint32_t* __restrict__ presence) {
   __shared__ unsigned long long part[32];
-  const uint32_t* row = tm + (uint64_t)blockIdx.x * words;
+  const uint4* row = reinterpret_cast<const uint4*>(tm + (uint64_t)blockIdx.x * words);
+  const uint64_t n = words / 4;
   unsigned long long c = 0;
-  for (uint64_t i = threadIdx.x; i < words; i += blockDim.x) c += __popc(__ldg(row + i));
+#pragma unroll 4
+  for (uint64_t i = threadIdx.x; i < n; i += blockDim.x) {
+    const uint4 v = __ldg(row + i);
+    c += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+  }
   for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xFFFFFFFFu, c, o);
   if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = c;
   __syncthreads();
@@ -224,21 +231,22 @@ __global__ void k_row_popcount(const uint32_t* __restrict__ tm, uint64_t words,
 // looking its 2-bit code up in "ACGT" gives it back.
 __device__ __forceinline__ void pack16(const uint4& v, uint32_t& code, uint32_t& inv) {
   const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-  code = inv = 0;
+  uint32_t x[4], m[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const uint32_t u = w[i] & 0xDFDFDFDFu;
     const uint32_t c = ((u >> 1) ^ (u >> 2)) & 0x03030303u;
     uint32_t sel = (c | (c >> 4)) & 0x00FF00FFu;
-    sel = (sel | (sel >> 8)) & 0xFFFFu;  // the four codes as byte selectors
-    const uint32_t x = __byte_perm(0x54474341u, 0u, sel) ^ u;
-    // the four codes side by side, the first in the top two bits of a byte
-    code = (code << 8) | ((c * 0x40100401u) >> 24);
-    if (x) {
+    sel |= sel >> 8;  // the four codes as byte selectors (low 16 bits)
+    x[i] = __byte_perm(0x54474341u, 0u, sel & 0xFFFFu) ^ u;
+    m[i] = c * 0x40100401u;  // top byte: the four codes side by side, the first on top
+  }
+  code = __byte_perm(__byte_perm(m[3], m[2], 0x0073u), __byte_perm(m[1], m[0], 0x0073u), 0x5410u);
+  inv = 0;
+  if (x[0] | x[1] | x[2] | x[3]) {
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if ((x >> (8 * k)) & 0xFFu) inv |= 1u << (4 * i + k);
-    }
+    for (int k = 0; k < 16; ++k)
+      if ((x[k >> 2] >> (8 * (k & 3))) & 0xFFu) inv |= 1u << k;
   }
 }
 
@@ -256,8 +264,11 @@ __device__ __forceinline__ void pack16(const uint4& v, uint32_t& code, uint32_t&
 //   3. (q = 5) the run's 32 vectors, one word a lane, are a 32 x 32 bit
 //      transpose away from the token rows; both token-major tables leave
 //      through shared memory in row pieces of 64 and 64 / f bytes.
-// Bound by shared-memory atomics (one per token) and the letters and tables
-// themselves (8.1 GB for the 3.1 Gbp index at q = 5).
+// Bound by instruction issue (about 250 warp instructions a bin, 71% of the
+// issue slots; the shared atomics take 23% of their pipe), not by its 8.1 GB
+// of letters and tables at 3.1 Gbp, B = 200, q = 5: 4.3 ms there.  Packing the
+// reference, setting each bin's bits from the codes and two transposes from
+// DRAM took 16.0 ms.
 constexpr uint32_t kFusedBins = 512, kFusedWarps = kFusedBins / 32, kFusedMaxK = 3;
 constexpr uint32_t kFusedGroups = kFusedBins / 32;  // tile words of a token row
 
@@ -283,7 +294,8 @@ __host__ __device__ constexpr uint32_t fused_code_words(uint32_t wpl, uint32_t c
   return c > coarse ? c : coarse;
 }
 
-template <uint32_t WPL>  // words of a vector per lane: 1 (q = 5) or 4 (q = 6)
+// WPL: words of a vector per lane, 1 (q = 5) or 4 (q = 6); K >= k
+template <uint32_t WPL, uint32_t K>
 __global__ void __launch_bounds__(kFusedWarps * 32, 2) k_build_fused(FusedArgs a) {
   extern __shared__ uint32_t s_fused[];
   uint32_t* s_rows = s_fused;
@@ -316,52 +328,87 @@ __global__ void __launch_bounds__(kFusedWarps * 32, 2) k_build_fused(FusedArgs a
   for (uint32_t w = 0; w < WPL; ++w) v[w * 32 + lane] = 0;
   any = __syncthreads_or(any);
 
-  // 2. tokens starting at tile positions [lo, hi) into the warp's vector
-  const uint32_t sh = 32u - 2u * a.q, qmask = (1u << a.q) - 1u;
-  auto set_tokens = [&](uint32_t lo, uint32_t hi) {
-    for (uint32_t p = lo + lane; p < hi; p += 32) {
+  // 2. tokens starting at tile positions [lo, lo + len) into the warp's
+  // vector: a lane takes `per` consecutive positions, whose per + q - 1 <= 16
+  // bases it aligns into one register, so a token costs two shifts for its
+  // bit, a shift and a mask for its word, and the atomic
+  constexpr uint32_t kQ = WPL == 1 ? 5u : 6u, kMost = 17u - kQ;  // positions per lane
+  constexpr uint32_t kBitShift = 32u - 2u * kQ, kWordMask = ((1u << (2u * kQ - 5u)) - 1u) << 2;
+  const uint32_t v_base = (uint32_t)__cvta_generic_to_shared(v);
+  auto set_tokens = [&](uint32_t lo, uint32_t len, uint32_t per) {
+    for (uint32_t at = lane * per; at < len; at += 32u * per) {
+      const uint32_t p = lo + at;
+      uint32_t ok = (1u << min(per, len - at)) - 1u;
       const uint32_t* c = s_code + (p >> 4);
-      const uint32_t t = __funnelshift_l(c[1], c[0], 2u * p) >> sh;
+      const uint32_t x = __funnelshift_l(c[1], c[0], 2u * p);
       if (any) {
-        const uint16_t* m = inv16 + (p >> 4);
-        if ((((uint32_t)m[0] | ((uint32_t)m[1] << 16)) >> (p & 15u)) & qmask) continue;
+        const uint16_t* m16 = inv16 + (p >> 4);
+        const uint32_t m = ((uint32_t)m16[0] | ((uint32_t)m16[1] << 16)) >> (p & 15u);
+        uint32_t bad = m;
+#pragma unroll
+        for (uint32_t i = 1; i < kQ; ++i) bad |= m >> i;
+        ok &= ~bad;
       }
-      atomicOr(v + (t >> 5), 1u << (t & 31u));
+      auto set = [&](uint32_t i) {
+        asm volatile(
+            "{\n.reg .pred p;\nsetp.ne.u32 p, %2, 0;\n@p red.shared.or.b32 [%0], %1;\n}" ::"r"(
+                v_base + ((x >> (kBitShift + 3u - 2u * i)) & kWordMask)),
+            "r"(1u << ((x >> (kBitShift - 2u * i)) & 31u)), "r"(ok & (1u << i))
+            : "memory");
+      };
+#pragma unroll
+      for (uint32_t i = 0; i < 4; ++i) set(i);
+      if (per > 4) {
+#pragma unroll
+        for (uint32_t i = 4; i < 8; ++i) set(i);
+      }
+      if (per > 8) {
+#pragma unroll
+        for (uint32_t i = 8; i < kMost; ++i) set(i);
+      }
     }
   };
-  uint32_t pend[kFusedMaxK + 1][WPL];  // bins c - k .. c so far (newest first)
+  const uint32_t rest = a.B - a.rem;
+  const uint32_t per_p = max(1u, min(kMost, (a.rem + 31u) / 32u));
+  const uint32_t per_r = min(kMost, (rest + 31u) / 32u);
+  uint32_t pend[K + 1][WPL];  // bins c - k .. c so far (newest first)
 #pragma unroll
-  for (uint32_t i = 0; i <= kFusedMaxK; ++i)
+  for (uint32_t i = 0; i <= K; ++i)
 #pragma unroll
     for (uint32_t w = 0; w < WPL; ++w) pend[i][w] = 0;
   const uint32_t first = warp * 32;
-  for (uint32_t c = first; c <= first + 32 + a.k; ++c) {
-    const uint32_t lo = c * a.B;
-    set_tokens(lo, lo + a.rem);
+  // this run's bins in the bin-major table
+  const uint32_t rows = a.bm && bin0 + first < a.num_bins
+                            ? (uint32_t)min((uint64_t)32u, a.num_bins - bin0 - first)
+                            : 0u;
+  uint32_t* out = a.bm + (bin0 + first) * (32 * WPL) + lane;
+  uint32_t lo = first * a.B;
+  for (uint32_t c = 0; c <= 32 + a.k; ++c, lo += a.B) {
+    set_tokens(lo, a.rem, per_p);
     __syncwarp();
     // core c's first positions complete bin c - k - 1
-    const uint32_t done = c - a.k - 1;
-    if (c >= first + a.k + 1) {
+    if (c > a.k) {
+      const uint32_t done = c - a.k - 1;
 #pragma unroll
       for (uint32_t w = 0; w < WPL; ++w) {
         uint32_t x = v[w * 32 + lane];
 #pragma unroll
-        for (uint32_t i = 0; i <= kFusedMaxK; ++i)
+        for (uint32_t i = 0; i <= K; ++i)
           if (i == a.k) x |= pend[i][w];
-        if (a.bm && bin0 + done < a.num_bins)
-          a.bm[(bin0 + done) * (32 * WPL) + w * 32 + lane] = x;
-        if (WPL == 1) s_rows[done * 32 + lane] = x;
+        if (done < rows) out[w * 32] = x;
+        if (WPL == 1) s_rows[(first + done) * 32 + lane] = x;
       }
+      out += 32 * WPL;
+      if (done == 31) break;
     }
-    if (c == first + 32 + a.k) break;
-    set_tokens(lo + a.rem, lo + a.B);
+    set_tokens(lo + a.rem, rest, per_r);
     __syncwarp();
 #pragma unroll
     for (uint32_t w = 0; w < WPL; ++w) {
       const uint32_t x = v[w * 32 + lane];
       v[w * 32 + lane] = 0;
 #pragma unroll
-      for (uint32_t i = kFusedMaxK; i > 0; --i) pend[i][w] = pend[i - 1][w] | x;
+      for (uint32_t i = K; i > 0; --i) pend[i][w] = pend[i - 1][w] | x;
       pend[0][w] = x;
     }
     __syncwarp();
@@ -393,18 +440,24 @@ __global__ void __launch_bounds__(kFusedWarps * 32, 2) k_build_fused(FusedArgs a
     for (uint32_t j = 0; j < 32; ++j) s_rows[(32u * lane + j) * kFusedGroups + warp + lane] = x[j];
   }
   __syncthreads();
+  // a thread keeps its column and steps down the rows
+  static_assert(kFusedWarps * 32 == 32 * kFusedGroups, "one pass covers 32 token rows");
   const uint64_t col0 = (uint64_t)blockIdx.x * kFusedGroups;
-  if (a.tm && col0 < a.wpad)
-    for (uint32_t i = tid; i < 1024u * kFusedGroups; i += kFusedWarps * 32) {
-      const uint32_t t = i / kFusedGroups, col = i % kFusedGroups;
-      a.tm[(uint64_t)t * a.wpad + col0 + col] = s_rows[i + (t >> 5)];
-    }
+  if (a.tm && col0 < a.wpad) {
+    uint32_t* dst = a.tm + (uint64_t)(tid / kFusedGroups) * a.wpad + col0 + tid % kFusedGroups;
+#pragma unroll 8
+    for (uint32_t j = 0; j < 32; ++j, dst += 32 * a.wpad)
+      *dst = s_rows[tid + j * (32 * kFusedGroups + 1)];
+  }
   const uint64_t ccol0 = (uint64_t)blockIdx.x * cgroups;
-  if (cgroups && ccol0 < a.cwpad)
-    for (uint32_t i = tid; i < 1024u * cgroups; i += kFusedWarps * 32) {
-      const uint32_t t = i / cgroups, col = i % cgroups;
-      a.ctm[(uint64_t)t * a.cwpad + ccol0 + col] = s_coarse[i + (t >> 5)];
-    }
+  if (cgroups && ccol0 < a.cwpad) {
+    const uint32_t per = kFusedWarps * 32 / cgroups;  // rows of a pass: 32 f
+    uint32_t t = tid / cgroups;
+    uint32_t* dst = a.ctm + (uint64_t)t * a.cwpad + ccol0 + tid % cgroups;
+#pragma unroll 4
+    for (uint32_t i = tid; i < 1024u * cgroups; i += kFusedWarps * 32, t += per, dst += per * a.cwpad)
+      *dst = s_coarse[i + (t >> 5)];
+  }
 }
 
 }  // namespace
@@ -482,13 +535,12 @@ void launch_build_fused(const char* ref, const IndexView& v, const IndexView& cv
   if (ctm && cv.num_bins_pad * f / kFusedBins > grid) grid = cv.num_bins_pad * f / kFusedBins;
   const size_t smem = fused_smem(v);
   ProfScope ps("build_fused", st);
-  if (v.q == 5) {
-    cudaFuncSetAttribute(k_build_fused<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_build_fused<1><<<(unsigned)grid, kFusedWarps * 32, smem, st>>>(a);
-  } else {
-    cudaFuncSetAttribute(k_build_fused<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_build_fused<4><<<(unsigned)grid, kFusedWarps * 32, smem, st>>>(a);
-  }
+  auto run = [&](auto kernel) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    kernel<<<(unsigned)grid, kFusedWarps * 32, smem, st>>>(a);
+  };
+  if (v.q == 5) run(a.k <= 1 ? k_build_fused<1, 1> : k_build_fused<1, kFusedMaxK>);
+  else run(a.k <= 1 ? k_build_fused<4, 1> : k_build_fused<4, kFusedMaxK>);
 }
 
 void launch_pack_ref(const char* ref, uint64_t n, uint32_t* codes, uint32_t* invalid,
