@@ -102,7 +102,7 @@ void* g_alloc_ctx = nullptr;
 // Validate an index's parameters and allocate its tables (contents not yet
 // written): token-major [4^q][num_bins_pad/32], bin-major padded with zero
 // vectors to whole super-bins, coarse token-major over super-bins of f bins,
-// and the per-token presence counts.
+// and the per-token presence counts and ranks.
 int index_alloc(uint64_t len, uint32_t B, uint32_t q, uint32_t max_read_len, uint32_t layouts,
                 uint32_t f, grim_index** out) {
   *out = nullptr;
@@ -165,18 +165,18 @@ int index_alloc(uint64_t len, uint32_t B, uint32_t q, uint32_t max_read_len, uin
     if (e != cudaSuccess) return fail(e);
   }
   if (layouts & (GRIM_LAYOUT_COARSE | GRIM_LAYOUT_TOKEN_MAJOR)) {
-    e = table(&ix->presence, (uint64_t)v.r4 * sizeof(uint32_t));
+    e = table(&ix->presence, (uint64_t)v.r4 * (sizeof(uint32_t) + sizeof(uint16_t)));
     if (e != cudaSuccess) return fail(e);
   }
   ix->coarse_pays = coarse_density(B, q, v.ext, f) <= kCoarseDensityMax;
   v.tm = ix->tm;
   v.bm = ix->bm;
   v.bm_rows = bm_bins;
-  v.presence = ix->presence;
+  v.rank = ix->presence ? reinterpret_cast<uint16_t*>(ix->presence + v.r4) : nullptr;
   ix->v = v;
   cv.tm = ix->ctm;
   cv.bm = nullptr;
-  cv.presence = ix->presence;
+  cv.rank = v.rank;
   ix->cv = cv;
   *out = ix;
   return GRIM_OK;
@@ -390,8 +390,8 @@ int grim_build_ex(const char* ref, uint64_t len, uint32_t B, uint32_t q, uint32_
   if (from_bm_ctm) launch_tm_from_bm(bm, cv, v.wpb, f, ix->ctm, st);
   if (bm != ix->bm) cudaFreeAsync(bm, st);
   // token presence from the table the all-bins filter sweeps first
-  if (ix->ctm) launch_row_popcount(ix->ctm, cv.r4, cv.wpad, ix->presence, st);
-  else if (ix->tm) launch_row_popcount(ix->tm, v.r4, v.wpad, ix->presence, st);
+  if (ix->ctm) launch_presence(ix->ctm, cv.r4, cv.wpad, ix->presence, index_rank(ix), st);
+  else if (ix->tm) launch_presence(ix->tm, v.r4, v.wpad, ix->presence, index_rank(ix), st);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   prof_collect();
@@ -538,7 +538,6 @@ int grim_filter(const grim_index* idx, const char* reads, const uint64_t* offset
   CK(cudaMemsetAsync(ctl, 0, sizeof(Ctl), st));
   launch_tokenise(reads, offsets, lens, e, v, rv, tokens, meta, ctl, st, cand_mode);
   if (cand_mode) launch_check_candidates(cand_off, n_reads, n_cand, ctl, st);
-  else if (!idx->shape.read_switch) launch_block_spread(lens, n_reads, v.q, ctl, st);
   CK(cudaGetLastError());
   // input errors end the call before the filter runs; the batch's largest
   // miss budget sizes the all-bins kernel's counters

@@ -226,6 +226,23 @@ __global__ void __launch_bounds__(512) k_row_popcount(const uint32_t* __restrict
   }
 }
 
+// A token's rank among the tokens of its class (token % classes): how many of
+// them fewer (super-)bins hold, ties by value.
+__global__ void __launch_bounds__(128) k_token_ranks(const uint32_t* __restrict__ presence,
+                                                     uint32_t rows, uint32_t classes,
+                                                     uint16_t* __restrict__ rank) {
+  __shared__ uint32_t s_p[4096];  // q <= 6
+  for (uint32_t i = threadIdx.x; i < rows; i += 128) s_p[i] = presence[i];
+  __syncthreads();
+  const uint32_t t = blockIdx.x * 128 + threadIdx.x;
+  if (t >= rows) return;
+  const uint32_t mine = s_p[t];
+  uint32_t r = 0;
+  for (uint32_t i = t % classes; i < rows; i += classes)
+    r += s_p[i] < mine || (s_p[i] == mine && i < t);
+  rank[t] = (uint16_t)r;
+}
+
 // 16 bases (bytes, first base lowest) to a code word (first base in the top
 // bits) and a not-a-base mask.  A letter is a base iff folding its case and
 // looking its 2-bit code up in "ACGT" gives it back.
@@ -481,10 +498,14 @@ void launch_tm_from_bm(const uint32_t* bm, const IndexView& unit_view, uint32_t 
   }
 }
 
-void launch_row_popcount(const uint32_t* tm, uint32_t rows, uint64_t words_per_row,
-                         uint32_t* presence, cudaStream_t st) {
-  ProfScope ps("row_popcount", st);
-  k_row_popcount<<<rows, 512, 0, st>>>(tm, words_per_row, presence);
+void launch_presence(const uint32_t* tm, uint32_t rows, uint64_t words_per_row, uint32_t* presence,
+                     uint16_t* rank, cudaStream_t st) {
+  {
+    ProfScope ps("row_popcount", st);
+    k_row_popcount<<<rows, 512, 0, st>>>(tm, words_per_row, presence);
+  }
+  ProfScope ps("token_ranks", st);
+  k_token_ranks<<<(rows + 127) / 128, 128, 0, st>>>(presence, rows, rows > 1024 ? 4u : 1u, rank);
 }
 
 namespace {

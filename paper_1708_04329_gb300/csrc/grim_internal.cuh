@@ -82,10 +82,12 @@ struct IndexView {
   uint32_t B, q, ext, max_read_len, r4, wpb;
   const uint32_t* tm;  // token-major [r4][wpad]
   const uint32_t* bm;  // bin-major [num_bins][wpb]
-  // [r4] number of (super-)bins holding each token, or null; the tokeniser
-  // orders each read's tokens by it so that the all-bins kernels apply the
-  // rarest tokens first and every bin of a tile fails as early as possible
-  const uint32_t* presence;
+  // [r4] each token's rank by the number of (super-)bins holding it, rarest
+  // first (at q = 6: its rank within its row class, token & 3), or null for an
+  // index of lists alone; the tokeniser orders each read's tokens by it so
+  // that the all-bins kernels apply the rarest tokens first and every bin of a
+  // tile fails as early as possible
+  const uint16_t* rank;
 };
 
 // Reads after tokenising: token j of read r (copy k) at
@@ -124,16 +126,17 @@ void launch_build_token_major(const uint32_t* codes, const uint32_t* invalid, co
 // bin-major table bm [units * f][wpb]; q >= 5
 void launch_tm_from_bm(const uint32_t* bm, const IndexView& unit_view, uint32_t wpb, uint32_t f,
                        uint32_t* tm, cudaStream_t st);
-// presence[t] = popcount of row t of a token-major table
-void launch_row_popcount(const uint32_t* tm, uint32_t rows, uint64_t words_per_row,
-                         uint32_t* presence, cudaStream_t st);
+// presence[t] = popcount of row t of a token-major table, and the tokens'
+// ranks by it (IndexView::rank)
+void launch_presence(const uint32_t* tm, uint32_t rows, uint64_t words_per_row, uint32_t* presence,
+                     uint16_t* rank, cudaStream_t st);
 
 void launch_reverse_complement(const char* reads, const uint64_t* offsets, const uint32_t* lens,
                                uint32_t n_reads, char* out, cudaStream_t st);
 // order: how each token row is written (the sums do not depend on it).
 enum class TokenOrder : uint32_t {
   kPosition,  // as they come in the read
-  kRarest,    // rarest first (IndexView::presence), repeats last
+  kRarest,    // rarest first (IndexView::rank), repeats last
   kCyclic,    // rarest first within row classes, 4 block-rotated copies (256-bin tiles)
   kLines,     // grouped by the 128-byte line of a bin vector that holds them, fullest line first
 };
@@ -141,16 +144,13 @@ enum class TokenOrder : uint32_t {
 // fix the counter depth from it); 0xFFFF = no limit.  max_bases: size of the
 // reads buffer when known (a read ending past it fails the batch with
 // kStatusArg), else ~0.  rv.copies token copies per read are written.  The
-// order is chosen from the mode: lists (`cand_mode`) or all bins.
+// order is chosen from the mode: lists (`cand_mode`) or all bins.  Leaves the
+// batch's extremes of D', slack and 16-token blocks in the control block.
 void launch_tokenise(const char* reads, const uint64_t* offsets, const uint32_t* lens,
                      const uint16_t* e, const IndexView& ix, ReadsView rv, uint16_t* tokens,
                      uint32_t* meta, Ctl* ctl, cudaStream_t st, bool cand_mode,
                      Live live = {false, 0}, uint32_t max_e = 0xFFFFu,
                      uint64_t max_bases = ~0ull);
-// ctl->blk_max / blk_lo: the most 16-token blocks of a read of the batch, and
-// 32 - the fewest
-void launch_block_spread(const uint32_t* lens, uint32_t n_reads, uint32_t q, Ctl* ctl,
-                         cudaStream_t st);
 // CSR offsets of the caller's lists: non-decreasing, ending at n_cand
 // (kStatusBadCsr otherwise); the ids themselves are checked by the
 // candidate kernel
@@ -311,7 +311,7 @@ struct grim_index {
   uint32_t* tm;
   uint32_t* bm;
   uint32_t* ctm;
-  uint32_t* presence;
+  uint32_t* presence;  // [4^q], followed by the ranks (uint16 [4^q])
   // the allocator the tables came from (grim_set_allocator), or null for
   // cudaMalloc / cudaFree
   grim_free_fn free_fn;
@@ -325,6 +325,11 @@ int index_alloc(uint64_t len, uint32_t B, uint32_t q, uint32_t max_read_len, uin
                 uint32_t f, grim_index** out);
 // Keep the CUDA error string for grim_last_cuda_error; the matching status.
 int record_cuda_error(cudaError_t e);
+
+// the ranks of IndexView::rank, behind the presence counts (null without them)
+inline uint16_t* index_rank(const grim_index* idx) {
+  return idx->presence ? reinterpret_cast<uint16_t*>(idx->presence + idx->v.r4) : nullptr;
+}
 
 // the all-bins filter can run coarse-then-exact when the index has both the
 // coarse table and the bin-major table

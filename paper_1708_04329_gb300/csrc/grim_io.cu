@@ -238,8 +238,10 @@ int grim_load(const char* path, uint32_t layouts, uint32_t flags, grim_index** o
     return GRIM_E_FORMAT;
   }
   // presence counts from the table the all-bins filter sweeps first, as in a build
-  if (ix->ctm) launch_row_popcount(ix->ctm, ix->cv.r4, ix->cv.wpad, ix->presence, sg.st);
-  else if (ix->tm) launch_row_popcount(ix->tm, ix->v.r4, ix->v.wpad, ix->presence, sg.st);
+  if (ix->ctm)
+    launch_presence(ix->ctm, ix->cv.r4, ix->cv.wpad, ix->presence, index_rank(ix), sg.st);
+  else if (ix->tm)
+    launch_presence(ix->tm, ix->v.r4, ix->v.wpad, ix->presence, index_rank(ix), sg.st);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(sg.st);
   prof_collect();

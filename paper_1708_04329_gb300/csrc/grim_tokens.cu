@@ -8,219 +8,288 @@ namespace {
 
 constexpr int kTokWarps = 8;
 constexpr uint32_t kMaxStride = 256;  // token stride: <= 255 tokens rounded up to 16
+constexpr int kTokRounds = 8;         // tokens per lane
+constexpr int kTokCtasPerSm = 5;      // of the persistent grid
+
+struct TokArgs {
+  const char* reads;
+  const uint64_t* offsets;
+  const uint32_t* lens;
+  const uint16_t* e;
+  uint32_t n_reads, q, max_read_len, r4, ts, copies;
+  const uint16_t* rank;  // IndexView::rank
+  uint16_t* tokens;
+  uint32_t* meta;
+  Ctl* ctl;
+  Live live;
+  uint32_t max_e;
+  uint64_t max_bases;
+};
 
 // One warp per read.  The read's tokens (row indices of the table: the token
 // value for a clean q-gram, rowInvalid for one holding a non-base -- it still
 // counts among the L-q+1 tokens and can never be found -- and rowPad after
-// the last token) are written to tokens[(r*copies + k)*ts ...].  With a
-// presence table they are written rarest first -- q-grams with a non-base,
-// which every bin misses, then ascending number of (super-)bins holding the
-// token, ties by position, and the repeats of a value already seen after all
-// distinct ones -- so that the all-bins kernels see misses as early as
-// possible; a sum does not depend on the order.  meta[r] = ntok | D' << 8
-// with D' = min(q*e, ntok): a bin passes iff at most D' of the read's tokens
-// are missing from it, which is sum >= (L-q+1) - q*e.
+// the last token) are written to tokens[(r*copies + k)*ts ...] in the order
+// the filter kernel wants (a sum does not depend on it).  meta[r] =
+// ntok | D' << 8 with D' = min(q*e, ntok): a bin passes iff at most D' of the
+// read's tokens are missing from it, which is sum >= (L-q+1) - q*e.
 //
-// copies = 4 (the 256-bin tiles of q = 6): a tile row is 32 bytes, so the
-// row's bank group in shared memory is row & 3, and 16 reads of a warp
-// loading random rows collide in bank groups.  The order is then made
-// class-cyclic -- position p holds a token of row class p & 3, each class
-// rarest first, for as long as every class has tokens left; the rest follow
-// rarest first -- and copy k rotates every 16-token block by k positions.  A
-// group g of the all-bins kernel reads copy g & 3, so at each load the
-// warp's 16 groups cover the four bank groups four times each.  Every block
-// holds the same tokens in every copy, so the per-block early exit and every
-// sum are unchanged.
+// The bases become bit planes (one ballot for each of the code's bits and one
+// for non-bases), so a lane cuts its q-grams out of registers with funnel
+// shifts.
 //
-// Candidate lists at q = 6 (TokenOrder::kLines): q-grams with a non-base
-// first (misses that need no look-up), then the tokens grouped by the
-// 128-byte line of a 512-byte bin vector that holds them (token >> 10), the
-// line with the most tokens first, so that the list kernel's first look-ups
-// touch as few lines of a vector as can rule the bin out.
-__global__ void __launch_bounds__(kTokWarps * 32) k_tokenise(
-    const char* __restrict__ reads, const uint64_t* __restrict__ offsets,
-    const uint32_t* __restrict__ lens, const uint16_t* __restrict__ e, uint32_t n_reads, uint32_t q,
-    uint32_t max_read_len, uint32_t r4, uint32_t ts, const uint32_t* __restrict__ presence,
-    uint16_t* __restrict__ tokens, uint32_t* __restrict__ meta, Ctl* ctl, Live live,
-    uint32_t max_e, uint64_t max_bases, uint32_t copies, TokenOrder order) {
-  __shared__ unsigned long long s_key[kTokWarps][kMaxStride];
-  __shared__ uint16_t s_row[kTokWarps][kMaxStride];
-  __shared__ uint16_t s_seq[kTokWarps][kMaxStride];
-  __shared__ uint8_t s_crank[kTokWarps][kMaxStride];
-  __shared__ uint8_t s_code[kTokWarps][kMaxStride + 16];  // per base: code | 4 if not a base
+// kRarest (all bins, up to q = 5): q-grams with a non-base, which every bin
+// misses, then the distinct tokens by ascending number of (super-)bins
+// holding them, so that the all-bins kernels see misses as early as possible,
+// then the repeats of a value already seen (a repeat misses exactly the bins
+// its first occurrence misses; 1024-bin tiles: 1.7% fewer bit tests at q = 5).
+// The order is a counting sort without counters: every distinct token sets
+// the bit of its rank in a bitmap of 4^q bits, and its place is the number of
+// bits below.
+//
+// kCyclic (the 256-bin tiles of q = 6, copies = 4): a tile row is 32 bytes, so
+// the row's bank group in shared memory is row & 3, and 16 reads of a warp
+// loading random rows collide in bank groups.  The distinct tokens are dealt
+// out round robin from the four row classes, each class rarest first (a
+// bitmap for each), and copy k rotates every 16-token block by k positions.  A
+// group g of the all-bins kernel reads copy g & 3, so at each load the warp's
+// 16 groups cover the four bank groups four times each.  Every block holds the
+// same tokens in every copy, so the per-block early exit and every sum are
+// unchanged.
+//
+// kLines (candidate lists at q = 6): q-grams with a non-base first (misses
+// that need no look-up), then the tokens grouped by the 128-byte line of a
+// 512-byte bin vector that holds them (token >> 10), the line with the most
+// tokens first, so that the list kernel's first look-ups touch as few lines
+// of a vector as can rule the bin out.
+//
+// Bound by instruction issue.  Measured on GB300 against coding the bases
+// through shared memory, q byte loads a token and a rank by comparing every
+// pair of keys: 250k reads of 100 bp at q = 5 0.77 -> 0.22 ms, 60k of 150 bp at
+// q = 6 0.91 -> 0.11 ms, 1M mixed reads in position order 0.85 -> 0.56 ms, a
+// lone read of 250 bp 67 -> 16 us.
+template <TokenOrder ORDER>
+__global__ void __launch_bounds__(kTokWarps * 32, kTokCtasPerSm) k_tokenise(TokArgs a) {
+  constexpr bool kRanked = ORDER == TokenOrder::kRarest || ORDER == TokenOrder::kCyclic;
+  constexpr uint32_t kBitWords = ORDER == TokenOrder::kCyclic ? 128 : 32;
+  __shared__ uint32_t s_bits[kRanked ? kTokWarps : 1][kBitWords];
+  __shared__ __align__(16) uint16_t s_seq[kTokWarps][kMaxStride];
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint64_t r = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
-  if (r >= live_reads(ctl, live, n_reads)) return;  // whole warps: warp syncs stay uniform
-  if (e[r] > max_e && lane == 0) atomicOr(&ctl->status, kStatusArg);
-  const uint32_t L = lens[r];
-  const uint64_t off = offsets[r];
-  uint16_t* out = tokens + r * copies * ts;
-  bool bad = false;
-  if (L < q) {
-    if (lane == 0) atomicOr(&ctl->status, kStatusShort);
-    bad = true;
-  } else if (L > max_read_len || L - q + 1 > kMaxTokens) {
-    if (lane == 0) atomicOr(&ctl->status, kStatusLong);
-    bad = true;
-  } else if (off > max_bases || L > max_bases - off) {  // past the end of the reads buffer
-    if (lane == 0) atomicOr(&ctl->status, kStatusArg);
-    bad = true;
-  }
-  const uint32_t ntok = bad ? 0 : L - q + 1;
-  // each base read once (coalesced) and coded into shared memory
-  for (uint32_t i = lane; i < (bad ? 0u : L); i += 32) {
-    const uint32_t u = (uint8_t)reads[off + i] & 0xDFu;  // fold lowercase letters
-    const bool ok = (u == 0x41u) | (u == 0x43u) | (u == 0x47u) | (u == 0x54u);
-    s_code[warp][i] = (uint8_t)((((u >> 1) ^ (u >> 2)) & 3u) | (ok ? 0u : 4u));  // A0 C1 G2 T3
-  }
-  __syncwarp();
-  for (uint32_t j = lane; j < ntok; j += 32) {
-    uint32_t v = 0, flags = 0;
-    for (uint32_t i = 0; i < q; ++i) {
-      const uint32_t c = s_code[warp][j + i];
-      v = (v << 2) | (c & 3u);
-      flags |= c;
+  const uint32_t below = (1u << lane) - 1u;
+  const uint32_t n_warps = gridDim.x * kTokWarps;
+  Ctl* ctl = a.ctl;
+  const uint32_t q = a.q, r4 = a.r4;
+  const uint32_t n_reads = live_reads(ctl, a.live, a.n_reads);
+  // the extremes of this warp's reads (as in Ctl); raised once at the end: a
+  // check of the shared words for every read is a load of one address for
+  // every read, which takes longer than the tokens
+  uint32_t max_d = 0, d_lo = 0, max_tight = 0, blk_max = 0, blk_lo = 0;
+  for (uint64_t r = blockIdx.x * (uint64_t)kTokWarps + warp; r < n_reads; r += n_warps) {
+    const uint32_t budget = a.e[r];
+    if (budget > a.max_e && lane == 0) atomicOr(&ctl->status, kStatusArg);
+    const uint32_t L = a.lens[r];
+    const uint64_t off = a.offsets[r];
+    bool bad = false;
+    if (L < q) {
+      if (lane == 0) atomicOr(&ctl->status, kStatusShort);
+      bad = true;
+    } else if (L > a.max_read_len || L - q + 1 > kMaxTokens) {
+      if (lane == 0) atomicOr(&ctl->status, kStatusLong);
+      bad = true;
+    } else if (off > a.max_bases || L > a.max_bases - off) {  // past the end of the reads buffer
+      if (lane == 0) atomicOr(&ctl->status, kStatusArg);
+      bad = true;
     }
-    const bool clean = (flags & 4u) == 0;
-    const uint32_t row = clean ? v : rowInvalid(r4);
-    if (order == TokenOrder::kPosition) {
-      out[j] = (uint16_t)row;
-      continue;
+    const uint32_t ntok = bad ? 0 : L - q + 1;
+    const uint32_t nb = bad ? 0 : L;
+
+    // each base read once; every row starts as padding
+    uint32_t ch[kTokRounds + 1];
+#pragma unroll
+    for (int i = 0; i <= kTokRounds; ++i)
+      ch[i] = 32u * i + lane < nb ? (uint8_t)a.reads[off + 32u * i + lane] : 0u;
+    const uint32_t pads = rowPad(r4) | (rowPad(r4) << 16);
+    reinterpret_cast<uint4*>(s_seq[warp])[lane] = make_uint4(pads, pads, pads, pads);
+    if constexpr (kRanked) {
+#pragma unroll
+      for (uint32_t w = 0; w < kBitWords; w += 32) s_bits[warp][w + lane] = 0;
     }
-    s_row[warp][j] = (uint16_t)row;
-    s_seq[warp][j] = (uint16_t)row;  // the order without a presence table
-  }
-  __syncwarp();
-  if (order == TokenOrder::kLines) {
-    // tokens per line (class 4: not a token), then each line's first position
-    uint32_t cnt[5] = {0, 0, 0, 0, 0};
-    for (uint32_t j0 = 0; j0 < ntok; j0 += 32) {
-      const uint32_t c = j0 + lane < ntok ? s_row[warp][j0 + lane] >> 10 : 5u;
+    __syncwarp();
+
+    // bit planes of 32 bases: code bits and not-a-base (A0 C1 G2 T3, case folded)
+    auto planes = [&](uint32_t c, uint32_t& lo, uint32_t& hi, uint32_t& inv) {
+      const uint32_t u = c & 0xDFu;
+      const bool ok = (u == 0x41u) | (u == 0x43u) | (u == 0x47u) | (u == 0x54u);
+      const uint32_t code = (u >> 1) ^ (u >> 2);
+      lo = __ballot_sync(0xFFFFFFFFu, code & 1u);
+      hi = __ballot_sync(0xFFFFFFFFu, code & 2u);
+      inv = __ballot_sync(0xFFFFFFFFu, !ok);
+    };
+    const uint32_t qmask = (1u << q) - 1u;
+    uint32_t row[kTokRounds], rk[kTokRounds], rep[kTokRounds];
+    uint32_t lo0, hi0, inv0, n_inv = 0, n_rep = 0;
+    uint32_t line_n[4] = {0, 0, 0, 0};  // kLines: tokens per line
+    planes(ch[0], lo0, hi0, inv0);
 #pragma unroll
-      for (uint32_t k = 0; k < 5; ++k) cnt[k] += __popc(__ballot_sync(0xFFFFFFFFu, c == k));
-    }
-    uint32_t at[5];
-    at[4] = 0;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      at[k] = cnt[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (cnt[i] > cnt[k] || (cnt[i] == cnt[k] && i < k)) at[k] += cnt[i];
-    }
-    for (uint32_t j0 = 0; j0 < ntok; j0 += 32) {
-      const uint32_t c = j0 + lane < ntok ? s_row[warp][j0 + lane] >> 10 : 5u;
-#pragma unroll
-      for (uint32_t k = 0; k < 5; ++k) {
-        const uint32_t m = __ballot_sync(0xFFFFFFFFu, c == k);
-        if (c == k) out[at[k] + __popc(m & ((1u << lane) - 1u))] = s_row[warp][j0 + lane];
-        at[k] += __popc(m);
+    for (int i = 0; i < kTokRounds; ++i) {
+      row[i] = rowPad(r4);
+      rk[i] = rep[i] = 0;
+      if (32u * i >= ntok) continue;  // the same for the warp
+      uint32_t lo1, hi1, inv1;
+      planes(ch[i + 1], lo1, hi1, inv1);
+      const uint32_t lo = __funnelshift_r(lo0, lo1, lane) & qmask;
+      const uint32_t hi = __funnelshift_r(hi0, hi1, lane) & qmask;
+      const bool unclean = __funnelshift_r(inv0, inv1, lane) & qmask;
+      lo0 = lo1;
+      hi0 = hi1;
+      inv0 = inv1;
+      // interleave the two planes, first base most significant
+      uint32_t z = __brev(lo | (hi << 16)) >> (16u - q);
+      z = (z | (z << 4)) & 0x0F0F0F0Fu;
+      z = (z | (z << 2)) & 0x33333333u;
+      z = (z | (z << 1)) & 0x55555555u;
+      const uint32_t t = ((z & 0xFFFFu) << 1) | (z >> 16);
+      const bool in = 32u * i + lane < ntok;
+      if (in) row[i] = unclean ? rowInvalid(r4) : t;
+      const uint32_t inv_mask = __ballot_sync(0xFFFFFFFFu, in && unclean);
+      if constexpr (ORDER == TokenOrder::kPosition) {
+        if (in) s_seq[warp][32u * i + lane] = (uint16_t)row[i];
+      } else {
+        if (in && unclean)
+          s_seq[warp][n_inv + __popc(inv_mask & below)] = (uint16_t)rowInvalid(r4);
       }
-    }
-  }
-  const bool ranked = order == TokenOrder::kRarest || order == TokenOrder::kCyclic;
-  for (uint32_t j = lane; j < ntok && ranked; j += 32) {
-    // a clean token whose value already occurred earlier in the read misses
-    // exactly the bins its first occurrence misses: it adds no new bins to
-    // the dead set, so repeats go after every distinct token (1024-bin
-    // tiles: 1.7% fewer bit tests at q = 5; at q = 6 repeats are rare and the
-    // scan did not pay for itself)
-    const uint32_t row = s_row[warp][j];
-    bool repeat = false;
-    if (copies == 1 && row != rowInvalid(r4))
-      for (uint32_t i = 0; i < j && !repeat; ++i) repeat = s_row[warp][i] == row;
-    const unsigned long long rare =
-        !presence ? 0ull : row != rowInvalid(r4) ? (unsigned long long)presence[row] + 1 : 0ull;
-    s_key[warp][j] = ((unsigned long long)repeat << 48) | (rare << 8) | j;
-  }
-  __syncwarp();
-  if (order == TokenOrder::kRarest) {
-    // rank = number of smaller keys (keys are distinct: position breaks ties)
-    for (uint32_t j = lane; j < ntok; j += 32) {
-      const unsigned long long mine = s_key[warp][j];
-      uint32_t rank = 0;
-      for (uint32_t i = 0; i < ntok; ++i) rank += s_key[warp][i] < mine;
-      out[rank] = s_row[warp][j];
-    }
-  } else if (order == TokenOrder::kCyclic) {
-    if (presence) {
-      // rank of each token within its row class, and the size of each class
-      uint32_t cnt = 0;  // 4 byte counters: tokens of class c counted by this lane
-      for (uint32_t j = lane; j < ntok; j += 32) {
-        const unsigned long long mine = s_key[warp][j];
-        const uint32_t c = s_row[warp][j] & 3u;
-        uint32_t rank = 0;
-        for (uint32_t i = 0; i < ntok; ++i)
-          rank += (s_row[warp][i] & 3u) == c && s_key[warp][i] < mine;
-        s_crank[warp][j] = (uint8_t)rank;
-        cnt += 1u << (8 * c);
+      n_inv += __popc(inv_mask);
+      if constexpr (ORDER == TokenOrder::kLines) {
+#pragma unroll
+        for (uint32_t k = 0; k < 4; ++k)
+          line_n[k] += __popc(__ballot_sync(0xFFFFFFFFu, row[i] < r4 && row[i] >> 10 == k));
       }
-      cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
-      const uint32_t m = min(min(cnt & 0xFFu, (cnt >> 8) & 0xFFu),
-                             min((cnt >> 16) & 0xFFu, cnt >> 24));  // complete cycles
-      __syncwarp();
-      // the first 4m positions cycle through the classes; the tokens left over
-      // follow, rarest first
-      for (uint32_t j = lane; j < ntok; j += 32) {
-        const uint32_t rc = s_crank[warp][j];
-        uint32_t pos;
-        if (rc < m) {
-          pos = 4u * rc + (s_row[warp][j] & 3u);
-        } else {
-          const unsigned long long mine = s_key[warp][j];
-          uint32_t rank = 0;
-          for (uint32_t i = 0; i < ntok; ++i) rank += s_crank[warp][i] >= m && s_key[warp][i] < mine;
-          pos = 4u * m + rank;
+      if constexpr (kRanked) {
+        const bool clean = row[i] < r4;
+        bool seen = false;
+        if (clean) {
+          rk[i] = a.rank[row[i]];
+          uint32_t w = rk[i] >> 5;
+          if (ORDER == TokenOrder::kCyclic) w += 32u * (row[i] & 3u);
+          seen = (atomicOr(&s_bits[warp][w], 1u << (rk[i] & 31u)) >> (rk[i] & 31u)) & 1u;
         }
-        s_seq[warp][pos] = s_row[warp][j];
+        // of equal tokens in this round that are new to the read, exactly one
+        // saw its bit clear, whichever came first; the lowest lane is taken as
+        // the first occurrence so that the order is always the same
+        uint32_t m = __ballot_sync(0xFFFFFFFFu, seen);
+        for (uint32_t left = m; left;) {
+          const uint32_t v = __shfl_sync(0xFFFFFFFFu, row[i], __ffs(left) - 1);
+          const uint32_t same = __ballot_sync(0xFFFFFFFFu, row[i] == v);
+          if (same & ~m) m = (m | same) & ~(same & (0u - same));
+          left &= ~same;
+        }
+        rep[i] = m;
+        n_rep += __popc(m);
+      }
+    }
+
+    if constexpr (ORDER == TokenOrder::kLines) {
+      uint32_t at[4];  // each line's first place
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        at[k] = n_inv;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (line_n[i] > line_n[k] || (line_n[i] == line_n[k] && i < k)) at[k] += line_n[i];
+      }
+#pragma unroll
+      for (int i = 0; i < kTokRounds; ++i) {
+        if (32u * i >= ntok) continue;
+#pragma unroll
+        for (uint32_t k = 0; k < 4; ++k) {
+          const bool mine = row[i] < r4 && row[i] >> 10 == k;
+          const uint32_t m = __ballot_sync(0xFFFFFFFFu, mine);
+          if (mine) s_seq[warp][at[k] + __popc(m & below)] = (uint16_t)row[i];
+          at[k] += __popc(m);
+        }
+      }
+    }
+    if constexpr (kRanked) {
+      __syncwarp();
+      // bits below each word of the bitmap; kCyclic: of the four classes, a byte
+      // each (at most 255 distinct tokens)
+      uint32_t n = 0;
+#pragma unroll
+      for (uint32_t w = 0; w < kBitWords; w += 32) n |= __popc(s_bits[warp][w + lane]) << (w / 4);
+      uint32_t incl = n;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+        if (lane >= (uint32_t)d) incl += t;
+      }
+      const uint32_t pre = incl - n, tot = __shfl_sync(0xFFFFFFFFu, incl, 31);
+      uint32_t rep_at = ntok - n_rep;
+#pragma unroll
+      for (int i = 0; i < kTokRounds; ++i) {
+        if (32u * i >= ntok) continue;
+        const uint32_t pw = __shfl_sync(0xFFFFFFFFu, pre, rk[i] >> 5);
+        if (row[i] < r4) {
+          uint32_t pos;
+          if (rep[i] >> lane & 1u) {
+            pos = rep_at + __popc(rep[i] & below);
+          } else if constexpr (ORDER == TokenOrder::kCyclic) {
+            const uint32_t c = row[i] & 3u;
+            const uint32_t word = s_bits[warp][32u * c + (rk[i] >> 5)];
+            const uint32_t x =
+                ((pw >> (8 * c)) & 0xFFu) + __popc(word & ((1u << (rk[i] & 31u)) - 1u));
+            // x rounds of the deal have passed, and the classes before c in this one
+            pos = n_inv;
+#pragma unroll
+            for (uint32_t k = 0; k < 4; ++k) {
+              const uint32_t tk = (tot >> (8 * k)) & 0xFFu;
+              pos += min(tk, x + (k < c ? 1u : 0u));
+            }
+          } else {
+            pos = n_inv + pw +
+                  __popc(s_bits[warp][rk[i] >> 5] & ((1u << (rk[i] & 31u)) - 1u));
+          }
+          s_seq[warp][pos] = (uint16_t)row[i];
+        }
+        rep_at += __popc(rep[i]);
       }
     }
     __syncwarp();
-    // copy k: every 16-token block rotated by k positions
-    for (uint32_t k = 0; k < copies; ++k) {
-      uint16_t* o = out + k * ts;
-      for (uint32_t p = lane; p < ts; p += 32) {
-        const uint32_t src = (p & ~15u) | ((p + k) & 15u);
-        o[p] = src < ntok ? s_seq[warp][src] : (uint16_t)rowPad(r4);
+    uint16_t* out = a.tokens + r * a.copies * a.ts;
+    if constexpr (ORDER == TokenOrder::kCyclic) {
+      // copy k: every 16-token block rotated by k positions
+      for (uint32_t k = 0; k < a.copies; ++k) {
+        uint32_t* o = reinterpret_cast<uint32_t*>(out + k * a.ts);
+        for (uint32_t w = lane; w < a.ts / 2; w += 32) {
+          const uint32_t p = 2u * w, blk = p & ~15u;
+          o[w] = (uint32_t)s_seq[warp][blk | ((p + k) & 15u)] |
+                 ((uint32_t)s_seq[warp][blk | ((p + 1u + k) & 15u)] << 16);
+        }
       }
+    } else {
+      if (8u * lane < a.ts)
+        reinterpret_cast<uint4*>(out)[lane] = reinterpret_cast<const uint4*>(s_seq[warp])[lane];
     }
-  }
-  if (copies == 1)
-    for (uint32_t j = ntok + lane; j < ts; j += 32) out[j] = (uint16_t)rowPad(r4);
-  if (lane == 0) {
-    uint32_t d = q * (uint32_t)e[r];
+    uint32_t d = q * budget;
     if (d > ntok) d = ntok;
-    meta[r] = ntok | (d << 8);
-    // most batches share one budget: skip the atomics once the max is reached
-    if (d > *reinterpret_cast<volatile uint32_t*>(&ctl->max_d)) atomicMax(&ctl->max_d, d);
-    if (255u - d > *reinterpret_cast<volatile uint32_t*>(&ctl->d_lo)) atomicMax(&ctl->d_lo, 255u - d);
-    const uint32_t tight = 255u - (ntok - d);
-    if (tight > *reinterpret_cast<volatile uint32_t*>(&ctl->max_tight))
-      atomicMax(&ctl->max_tight, tight);
-  }
-}
-
-// The spread of the reads' 16-token block counts (ctl->blk_max, blk_lo =
-// 32 - the fewest): the all-bins kernel can let a warp's lane groups take
-// their next reads together when every read spans as many blocks.  Reads
-// shorter than q are left out (the tokeniser fails the batch for them).
-__global__ void k_block_spread(const uint32_t* __restrict__ lens, uint32_t n_reads, uint32_t q,
-                               Ctl* ctl) {
-  uint32_t hi = 0, lo = 0;  // most blocks, 32 - fewest blocks
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n_reads;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint32_t L = lens[i];
-    if (L < q) continue;
-    const uint32_t ntok = min(L - q + 1, kMaxTokens);
+    if (lane == 0) a.meta[r] = ntok | (d << 8);
     const uint32_t nblk = (ntok + kBlockTokens - 1) / kBlockTokens;
-    hi = max(hi, nblk);
-    lo = max(lo, 32u - nblk);
+    max_d = max(max_d, d);
+    d_lo = max(d_lo, 255u - d);
+    max_tight = max(max_tight, 255u - (ntok - d));
+    blk_max = max(blk_max, nblk);
+    blk_lo = max(blk_lo, 32u - nblk);
+    __syncwarp();  // the row has been copied out
   }
-  hi = __reduce_max_sync(0xFFFFFFFFu, hi);
-  lo = __reduce_max_sync(0xFFFFFFFFu, lo);
-  if ((threadIdx.x & 31) == 0) {
-    if (hi) atomicMax(&ctl->blk_max, hi);
-    if (lo) atomicMax(&ctl->blk_lo, lo);
+  if (lane == 0) {
+    // (skip the atomics once the extremes are reached)
+    auto raise = [](uint32_t* p, uint32_t v) {
+      if (v > *reinterpret_cast<volatile uint32_t*>(p)) atomicMax(p, v);
+    };
+    raise(&ctl->max_d, max_d);
+    raise(&ctl->d_lo, d_lo);
+    raise(&ctl->max_tight, max_tight);
+    raise(&ctl->blk_max, blk_max);
+    raise(&ctl->blk_lo, blk_lo);
   }
 }
 
@@ -272,34 +341,24 @@ void launch_tokenise(const char* reads, const uint64_t* offsets, const uint32_t*
                      const uint16_t* e, const IndexView& ix, ReadsView rv, uint16_t* tokens,
                      uint32_t* meta, Ctl* ctl, cudaStream_t st, bool cand_mode, Live live,
                      uint32_t max_e, uint64_t max_bases) {
-  const uint32_t copies = rv.copies;
-  // lists read whole token rows in any order up to 128-byte vectors; larger
-  // ones (q = 6) are looked up line by line
-  const TokenOrder order = cand_mode ? (ix.wpb > 32 ? TokenOrder::kLines : TokenOrder::kPosition)
-                           : copies > 1   ? TokenOrder::kCyclic
-                           : ix.presence ? TokenOrder::kRarest
-                                         : TokenOrder::kPosition;
   if (rv.n_reads == 0) return;
   const uint32_t threads = kTokWarps * 32;
-  uint64_t grid = ((uint64_t)rv.n_reads * 32 + threads - 1) / threads;
-  ProfScope ps("tokenise", st);
-  k_tokenise<<<(unsigned)grid, threads, 0, st>>>(reads, offsets, lens, e, rv.n_reads, ix.q,
-                                                 ix.max_read_len, ix.r4, rv.ts, ix.presence, tokens,
-                                                 meta, ctl, live, max_e, max_bases, copies,
-                                                 order);
-}
-
-void launch_block_spread(const uint32_t* lens, uint32_t n_reads, uint32_t q, Ctl* ctl,
-                         cudaStream_t st) {
-  if (n_reads == 0) return;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const uint64_t need = ((uint64_t)n_reads + 255) / 256;
-  const uint64_t cap = (uint64_t)(sms > 0 ? sms : 1) * 4;
-  const uint32_t grid = (uint32_t)(need < cap ? need : cap);
-  ProfScope ps("block_spread", st);
-  k_block_spread<<<grid, 256, 0, st>>>(lens, n_reads, q, ctl);
+  const uint64_t need = ((uint64_t)rv.n_reads + kTokWarps - 1) / kTokWarps;
+  const uint64_t most = (uint64_t)(sms > 0 ? sms : 1) * kTokCtasPerSm;
+  const uint64_t grid = need < most ? need : most;
+  const TokArgs a{reads, offsets, lens,   e,    rv.n_reads, ix.q, ix.max_read_len, ix.r4,    rv.ts,
+                  rv.copies, ix.rank, tokens, meta, ctl,        live, max_e,           max_bases};
+  // lists read whole token rows in any order up to 128-byte vectors; larger
+  // ones (q = 6) are looked up line by line
+  auto kernel = cand_mode       ? (ix.wpb > 32 ? k_tokenise<TokenOrder::kLines>
+                                               : k_tokenise<TokenOrder::kPosition>)
+                : rv.copies > 1 ? k_tokenise<TokenOrder::kCyclic>
+                                : k_tokenise<TokenOrder::kRarest>;
+  ProfScope ps("tokenise", st);
+  kernel<<<(unsigned)grid, threads, 0, st>>>(a);
 }
 
 void launch_check_candidates(const uint64_t* cand_off, uint32_t n_reads, uint64_t n_cand, Ctl* ctl,
