@@ -220,11 +220,15 @@ __device__ __forceinline__ void load_ids(const int32_t* __restrict__ seg, uint32
 
 // Candidates per work claim: large enough that the search for a chunk's
 // first read and the planes of the reads split at chunk edges stay cheap,
-// small enough that every warp gets about 16 chunks (an even finish).
-constexpr uint64_t kChunkMin = 256, kChunkMax = 4096, kChunksPerWarp = 16;
+// small enough that every warp gets about 16 chunks (an even finish).  Below
+// that, calls too short to give every warp a chunk of 256 take smaller ones,
+// down to a batch of 32: a chunk is one warp's serial work, and there are
+// warps to spare (37 reads' lists, 10.8k candidates: 54 us at 256, 28 at 32).
+constexpr uint64_t kChunkFew = 32, kChunkMin = 256, kChunkMax = 4096, kChunksPerWarp = 16;
 __device__ __forceinline__ uint64_t chunk_size(uint64_t n_cand, uint64_t warps) {
   uint64_t c = kChunkMax;
   while (c > kChunkMin && c * kChunksPerWarp * warps > n_cand) c >>= 1;
+  while (c > kChunkFew && c * warps > n_cand) c >>= 1;
   return c;
 }
 
