@@ -398,13 +398,15 @@ constexpr int kRefineItems = 4;
 
 __global__ void __launch_bounds__(kWarps * 32, 4) k_refine(IndexView ix, ReadsView rv,
                                                            const unsigned long long* __restrict__ keys,
-                                                           uint64_t n_surv, uint32_t cbits, uint32_t f,
+                                                           const unsigned long long* n_surv_at,
+                                                           uint64_t room, uint32_t cbits, uint32_t f,
                                                            RecordsView rec, uint32_t bin_bits,
                                                            Ctl* ctl, Live live) {
   constexpr int U = kRefineItems;
   if (*(volatile uint32_t*)&ctl->status) return;
   if (gated_off(ctl, live)) return;
-  if (live.on) n_surv = ctl->n_surv;
+  const uint64_t n_surv = *n_surv_at;
+  if (n_surv > room) return;  // not all of them were kept: the call takes another way
   const uint32_t lane = threadIdx.x & 31;
   const uint64_t warp = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
   const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
@@ -462,7 +464,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_refine(IndexView ix, ReadsVi
     const uint32_t bal = __ballot_sync(0xFFFFFFFFu, found != 0);
     if (bal) {
       unsigned long long first = 0;
-      if (lane == 0) first = atomicAdd(&ctl->n_rec, (unsigned long long)__popc(bal));
+      if (lane == 0) first = atomicAdd(&ctl->n_final, (unsigned long long)__popc(bal));
       first = __shfl_sync(0xFFFFFFFFu, first, 0);
       const unsigned long long pos = first + __popc(bal & ((1u << lane) - 1u));
       if (found && pos < rec.cap) {
@@ -667,15 +669,15 @@ void launch_lookup(const CandArgs& a, cudaStream_t st) {
 
 template <int WPB, int U>
 void launch_u(const CandArgs& a, cudaStream_t st) {
+  // at most 14 KB a CTA, so the launch bounds set how many an SM holds
   const size_t smem = (size_t)kWarps * warp_smem_words(a.ix.r4, WPB) * sizeof(uint32_t);
-  cudaFuncSetAttribute(k_candidates<WPB, U>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int dev = 0, sms = 0, per_sm = 0;
+  static_assert(kWarps * warp_smem_words(1024, 32) * 4 * kCandCtasPerSm <= 227 * 1024,
+                "eight CTAs of the largest vectors fit an SM");
+  int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_candidates<WPB, U>, kWarps * 32, smem);
-  if (per_sm < 1) per_sm = 1;
   // persistent: warps that find no chunk left exit at once
-  const uint64_t grid = (uint64_t)sms * per_sm;
+  const uint64_t grid = (uint64_t)(sms > 0 ? sms : 1) * kCandCtasPerSm;
   ProfScope ps("candidates", st);
   k_candidates<WPB, U><<<(unsigned)grid, kWarps * 32, smem, st>>>(a);
 }
@@ -691,17 +693,17 @@ void launch_t(const CandArgs& a, cudaStream_t st, uint32_t unroll) {
 }  // namespace
 
 void launch_refine(const IndexView& ix, const ReadsView& rv, const unsigned long long* keys,
-                   uint64_t n_surv, uint32_t cbits, uint32_t f, RecordsView rec, uint32_t bin_bits,
-                   Ctl* ctl, cudaStream_t st, Live live) {
-  if (n_surv == 0) return;
+                   const unsigned long long* n_surv, uint64_t room, uint32_t cbits, uint32_t f,
+                   RecordsView rec, uint32_t bin_bits, Ctl* ctl, cudaStream_t st, Live live) {
+  if (room == 0) return;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const uint64_t need = (n_surv * f + 32 * kWarps - 1) / (32 * kWarps);
+  const uint64_t need = (room * f + 32 * kWarps - 1) / (32 * kWarps);
   const uint64_t most = (uint64_t)(sms > 0 ? sms : 1) * 4;
   ProfScope ps("candidates_refine", st);
   k_refine<<<(unsigned)(need < most ? need : most), kWarps * 32, 0, st>>>(
-      ix, rv, keys, n_surv, cbits, f, rec, bin_bits, ctl, live);
+      ix, rv, keys, n_surv, room, cbits, f, rec, bin_bits, ctl, live);
 }
 
 void launch_candidates(const IndexView& ix, const ReadsView& rv, const int32_t* cand,

@@ -184,16 +184,19 @@ __global__ void k_emit(const unsigned long long* __restrict__ keys,
 // n^2 compares instead of the radix sort's three launches per key byte.
 // Measured on GB300 (rank against radix with two-byte keys, events around each
 // launch, us): 64 records 7 / 31, 2,048 9.5 / 61, 8,192 27 / 77, 16,384 75 /
-// 78, 32,768 273 / 86: the line is drawn where the compares still hide behind
-// the launches they replace.
-constexpr uint64_t kRankMax = 8192;
+// 78, 32,768 273 / 86: the line (kRankMax) is drawn where the compares still
+// hide behind the launches they replace.  The number of records is read on the
+// device, so the launch need not wait for the host to learn it.
 constexpr uint32_t kRankThreads = 256;
 constexpr uint32_t kRankSplit = 16;    // threads per record
 constexpr uint32_t kRankChunk = 2048;  // keys in shared memory at a time
 __global__ void __launch_bounds__(kRankThreads) k_rank_emit(
-    const unsigned long long* __restrict__ keys, const uint8_t* __restrict__ counts, uint32_t n,
-    EmitArgs e) {
+    const unsigned long long* __restrict__ keys, const uint8_t* __restrict__ counts,
+    const unsigned long long* n_live, uint64_t limit, EmitArgs e, const Ctl* ctl) {
   __shared__ unsigned long long s_key[kRankChunk];
+  if (ctl->status || *n_live > limit) return;
+  const uint32_t n = (uint32_t)*n_live;
+  if (blockIdx.x * (kRankThreads / kRankSplit) >= n) return;
   const uint32_t i = (blockIdx.x * kRankThreads + threadIdx.x) / kRankSplit;
   const uint32_t part = threadIdx.x % kRankSplit;
   const unsigned long long key = i < n ? keys[i] : 0ull;
@@ -247,6 +250,18 @@ RecordsView sort_records(RecordsView a, RecordsView b, uint64_t n, uint32_t key_
   return src;
 }
 
+void rank_and_emit(const RecordsView& a, const unsigned long long* n_live, uint64_t limit,
+                   bool candidate_mode, uint32_t bin_bits, const int32_t* cand,
+                   const uint64_t* cand_off, uint32_t n_reads, uint32_t* out_read,
+                   uint32_t* out_bin, uint8_t* out_count, const Ctl* ctl, cudaStream_t st) {
+  if (limit > kRankMax) limit = kRankMax;
+  if (limit == 0) return;
+  const EmitArgs e{candidate_mode, bin_bits, cand, cand_off, n_reads, out_read, out_bin, out_count};
+  ProfScope ps("rank_emit", st);
+  k_rank_emit<<<(unsigned)((limit * kRankSplit + kRankThreads - 1) / kRankThreads), kRankThreads, 0,
+                st>>>(a.keys, a.counts, n_live, limit, e, ctl);
+}
+
 void sort_and_emit(RecordsView a, RecordsView b, uint64_t n, uint32_t key_bits, void* hist,
                    bool candidate_mode, uint32_t bin_bits, const int32_t* cand,
                    const uint64_t* cand_off, uint32_t n_reads, uint32_t* out_read,
@@ -254,12 +269,6 @@ void sort_and_emit(RecordsView a, RecordsView b, uint64_t n, uint32_t key_bits, 
                    const unsigned long long* n_live, const uint32_t* n_reads_live) {
   if (n == 0) return;
   const EmitArgs e{candidate_mode, bin_bits, cand, cand_off, n_reads, out_read, out_bin, out_count};
-  if (!n_live && n <= kRankMax) {
-    ProfScope ps("rank_emit", st);
-    k_rank_emit<<<(unsigned)((n * kRankSplit + kRankThreads - 1) / kRankThreads), kRankThreads, 0,
-                  st>>>(a.keys, a.counts, (uint32_t)n, e);
-    return;
-  }
   const RecordsView src = sort_records(a, b, n, key_bits, hist, st, n_live);
   ProfScope ps("emit", st);
   k_emit<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(src.keys, src.counts, n, e, n_live,

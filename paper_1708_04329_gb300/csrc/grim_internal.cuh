@@ -34,7 +34,7 @@ struct Ctl {
   unsigned long long live_cand;    // candidates in this batch
   unsigned long long live_bases;   // read bytes in this batch (host-memory plans)
   unsigned long long n_surv;       // survivors of the coarse pass
-  unsigned long long n_final;      // passing records of the batch
+  unsigned long long n_final;      // passing records (of the survivors' check; plans: of the batch)
   uint32_t blk_max;                // most 16-token blocks of a read in the batch
   uint32_t blk_lo;                 // 32 - the fewest 16-token blocks of a read
   unsigned long long tail_blocks;  // of `blocks`: applied to one word per lane (256 bins)
@@ -186,13 +186,14 @@ void launch_candidates(const IndexView& ix, const ReadsView& rv, const int32_t* 
                        const uint64_t* cand_off, RecordsView rec, Ctl* ctl, cudaStream_t st,
                        Live live = {false, 0}, uint32_t unroll = 0);
 // The exact check of the coarse pass's survivors (keys read << cbits |
-// super-bin, in any order): the members of each surviving super-bin of f
-// bins against the bin-major table; passing (read, bin) pairs become records
-// with keys read << bin_bits | bin.  With `live` on, the survivor count is
-// read from ctl->n_surv and n_surv only sizes the launch.
+// super-bin, in any order; *n_surv of them, on the device, none checked if
+// more than `room`): the members of each surviving super-bin of f bins against
+// the bin-major table; passing (read, bin) pairs become records with keys
+// read << bin_bits | bin, counted in ctl->n_final.
 void launch_refine(const IndexView& ix, const ReadsView& rv, const unsigned long long* keys,
-                   uint64_t n_surv, uint32_t cbits, uint32_t f, RecordsView rec, uint32_t bin_bits,
-                   Ctl* ctl, cudaStream_t st, Live live = {false, 0});
+                   const unsigned long long* n_surv, uint64_t room, uint32_t cbits, uint32_t f,
+                   RecordsView rec, uint32_t bin_bits, Ctl* ctl, cudaStream_t st,
+                   Live live = {false, 0});
 
 // Radix sort of n (key, count) records by the low key_bits bits of the key,
 // followed by the split into the caller's (read, bin, count) arrays.
@@ -201,6 +202,14 @@ uint64_t sort_workspace_bytes(uint64_t cap);
 // capped at n; n then only sizes the launches
 RecordsView sort_records(RecordsView a, RecordsView b, uint64_t n, uint32_t key_bits, void* hist,
                          cudaStream_t st, const unsigned long long* n_live = nullptr);
+// Lists of up to kRankMax records without the host knowing their number: does
+// the work of sort_and_emit if *n_live <= min(limit, kRankMax) and the batch
+// has no error, else nothing.  `limit`: the caller's capacity.
+constexpr uint64_t kRankMax = 8192;
+void rank_and_emit(const RecordsView& a, const unsigned long long* n_live, uint64_t limit,
+                   bool candidate_mode, uint32_t bin_bits, const int32_t* cand,
+                   const uint64_t* cand_off, uint32_t n_reads, uint32_t* out_read,
+                   uint32_t* out_bin, uint8_t* out_count, const Ctl* ctl, cudaStream_t st);
 void sort_and_emit(RecordsView a, RecordsView b, uint64_t n, uint32_t key_bits, void* hist,
                    bool candidate_mode, uint32_t bin_bits, const int32_t* cand,
                    const uint64_t* cand_off, uint32_t n_reads, uint32_t* out_read,

@@ -83,7 +83,7 @@ __global__ void k_plan_control(Ctl* c, uint32_t op, uint32_t capable, uint32_t h
     c->n_rec = 0;  // restart the record and work counters for the next pass
     c->item = 0;
   } else {
-    c->n_final = c->n_rec;
+    if (c->path != kPathCoarse) c->n_final = c->n_rec;  // (the survivors' check counts there itself)
   }
 }
 
@@ -173,7 +173,8 @@ int capture(grim_plan* p) {
       launch_exhaustive(idx->cv, rv, ra, cbits, max_d, p->ctl, st, "exhaustive_coarse", coarse,
                         idx->shape);
       k_plan_control<<<1, 1, 0, st>>>(p->ctl, kCtlAfterCoarse, 1, has_exact, rcap, 0);
-      launch_refine(v, rv, ra.keys, rcap, cbits, p->f, rb, bin_bits, p->ctl, st, coarse);
+      launch_refine(v, rv, ra.keys, &p->ctl->n_surv, rcap, cbits, p->f, rb, bin_bits, p->ctl, st,
+                    coarse);
     }
     if (has_exact) {
       const Live exact{true, kPathExact};
