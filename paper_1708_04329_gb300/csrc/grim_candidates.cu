@@ -265,7 +265,6 @@ __global__ void __launch_bounds__(kWarps * 32, kCandCtasPerSm) k_candidates(Cand
   const uint32_t sub = lane % G;     // this lane's slice of a bin vector
   const uint32_t slot = lane / G;    // which of the warp's CPW candidates
   if (*(volatile uint32_t*)&a.ctl->status) return;
-  if (gated_off(a.ctl, a.live)) return;  // the batch takes the other path
   const uint32_t n_reads = live_reads(a.ctl, a.live, a.rv.n_reads);
   if (n_reads == 0) return;
   // the batch's lists span candidates [c_begin, c_end); warps claim chunks
@@ -404,7 +403,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_refine(IndexView ix, ReadsVi
                                                            Ctl* ctl, Live live) {
   constexpr int U = kRefineItems;
   if (*(volatile uint32_t*)&ctl->status) return;
-  if (gated_off(ctl, live)) return;
+  if (routed_off(ctl, live)) return;
   const uint64_t n_surv = *n_surv_at;
   if (n_surv > room) return;  // not all of them were kept: the call takes another way
   const uint32_t lane = threadIdx.x & 31;
@@ -533,7 +532,6 @@ __global__ void __launch_bounds__(kWarps * 32, 6) k_candidates_lookup(CandArgs a
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t r4 = a.ix.r4, wpb = a.ix.wpb;
   if (*(volatile uint32_t*)&a.ctl->status) return;
-  if (gated_off(a.ctl, a.live)) return;
   const uint32_t n_reads = live_reads(a.ctl, a.live, a.rv.n_reads);
   if (n_reads == 0) return;
   const uint64_t c_begin = a.cand_off[0], c_end = a.cand_off[n_reads];

@@ -194,8 +194,49 @@ struct ExhArgs {
   uint32_t c_row, c_hi, c_lo;  // TW*4, 65536, -65536: multipliers of the address math
   uint64_t range_bytes;        // token-row bytes of one read range (the read tile)
   uint32_t switch_lanes;       // WS, 256-bin tiles: waiting lanes that make the warp switch
+  uint32_t few_reads;          // batches of up to this many reads are k_exhaustive_few's
   Ctl* ctl;
 };
+
+// the carries of a 16-token block between its quads
+template <int NW>
+struct CsaTemps {
+  uint32_t t2a[NW], t2b[NW], t4a[NW], t4b[NW], t8a[NW], t8b[NW], t16[NW];
+};
+
+// Add the misses of four tokens, the quad-th of a 16-token block, whose
+// existence words are a0..a3; the block's last quad carries into the upper
+// planes.
+template <int P, int NW>
+__device__ __forceinline__ void add_quad(Counters<P>& c, CsaTemps<NW>& t, int quad,
+                                         const uint32_t (&a0)[NW], const uint32_t (&a1)[NW],
+                                         const uint32_t (&a2)[NW], const uint32_t (&a3)[NW]) {
+#pragma unroll
+  for (int w = 0; w < NW; ++w) {
+    uint32_t* t4 = (quad & 1) ? t.t4b : t.t4a;
+    fa_miss(c.s1[w], a0[w], a1[w], c.s1[w], t.t2a[w]);
+    fa_miss(c.s1[w], a2[w], a3[w], c.s1[w], t.t2b[w]);
+    fa(c.s2[w], t.t2a[w], t.t2b[w], c.s2[w], t4[w]);
+    if (quad == 1) fa(c.s4[w], t.t4a[w], t.t4b[w], c.s4[w], t.t8a[w]);
+    if (quad == 3) {
+      fa(c.s4[w], t.t4a[w], t.t4b[w], c.s4[w], t.t8b[w]);
+      fa(c.s8[w], t.t8a[w], t.t8b[w], c.s8[w], t.t16[w]);
+      // ripple the weight-16 carry through the upper planes; the carry out
+      // of the top plane (counter >= 2^P: misses > D') sticks in `dead`
+      uint32_t k = t.t16[w];
+#pragma unroll
+      for (int i = 0; i < P - 5; ++i) {
+        const uint32_t nk = c.up[i][w] & k;
+        c.up[i][w] ^= k;
+        k = nk;
+      }
+      uint32_t d;
+      LOP3(d, c.dead[w], c.up[P - 5][w], k, 0xF8);  // dead | (top & k)
+      c.up[P - 5][w] ^= k;
+      c.dead[w] = d;
+    }
+  }
+}
 
 // Add the misses of one 16-token block.  tw holds 16 table row indices as
 // uint16 pairs; base is the shared address of this lane's words in row 0.
@@ -611,6 +652,112 @@ __global__ void __launch_bounds__(NT, 1) k_exhaustive(ExhArgs a) {
   }
 }
 
+// The same count for a handful of reads, straight from the token-major table.
+// Staging every tile reads the whole table however few reads there are (4^q
+// rows: 1 GB for the 3.1 Gbp coarse table at q = 5, 0.24 ms); here a warp holds
+// one read and 4096 bins, loads only the rows that the read's tokens name,
+// 512 contiguous bytes of each, and stops once all its bins are dead.  Warps
+// on the same 4096 bins (all the reads) run side by side, so rows that reads
+// share come from L2.  Bound by DRAM: 16 16-byte loads in flight a lane.
+constexpr uint32_t kFewThreads = 256;
+constexpr uint64_t kFewMinTable = 64ull << 20;  // bytes
+
+template <int P>
+__global__ void __launch_bounds__(kFewThreads, 2) k_exhaustive_few(ExhArgs a) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t n_warps = gridDim.x * (kFewThreads / 32);
+  const uint32_t r4 = a.ix.r4;
+  if (*(volatile uint32_t*)&a.ctl->status) return;
+  if (routed_off(a.ctl, a.live)) return;
+  const uint32_t n_reads = live_reads(a.ctl, a.live, a.rv.n_reads);
+  if (n_reads > a.few_reads) return;
+  const uint64_t n_items = (a.ix.wpad + 127) / 128 * n_reads;
+  for (uint64_t item = blockIdx.x * (kFewThreads / 32) + (threadIdx.x >> 5); item < n_items;
+       item += n_warps) {
+    const uint32_t r = (uint32_t)(item % n_reads);
+    const uint64_t word0 = item / n_reads * 128 + lane * 4;  // this lane's words of a row
+    const bool on = word0 < a.ix.wpad;                       // (rows are whole 1024-bin tiles)
+    const uint32_t* col = a.ix.tm + (on ? word0 : 0);
+    const uint32_t m = a.rv.meta[r];
+    const uint32_t ntok = m & 0xFFu, d = (m >> 8) & 0xFFu;
+    const uint32_t bias = (1u << P) - (d + 1u);
+    const uint32_t nblk = (ntok + kBlockTokens - 1) / kBlockTokens;
+    const uint4* tok =
+        reinterpret_cast<const uint4*>(a.rv.tokens + (uint64_t)r * a.rv.copies * a.rv.ts);
+    Counters<P> c;
+    c.init(bias);
+    uint32_t alive = 0;  // blocks after which this lane had a live bin
+    bool ldead = !on;
+    uint4 t0 = __ldg(tok), t1 = __ldg(tok + 1);
+    for (uint32_t b = 0; b < nblk; ++b) {
+      const uint32_t tw[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
+      if (b + 1 < nblk) {
+        t0 = __ldg(tok + 2 * b + 2);
+        t1 = __ldg(tok + 2 * b + 3);
+      }
+      // (the token is the same for the warp: no divergence)
+      uint32_t x[16][4];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const uint32_t row = (j & 1) ? tw[j >> 1] >> 16 : tw[j >> 1] & 0xFFFFu;
+        const uint32_t fill = row == rowPad(r4) ? ~0u : 0u;
+        uint4 v = make_uint4(fill, fill, fill, fill);
+        if (row < r4) v = __ldg(reinterpret_cast<const uint4*>(col + (uint64_t)row * a.ix.wpad));
+        x[j][0] = v.x; x[j][1] = v.y; x[j][2] = v.z; x[j][3] = v.w;
+      }
+      CsaTemps<4> t;
+#pragma unroll
+      for (int quad = 0; quad < 4; ++quad)
+        add_quad<P, 4>(c, t, quad, x[4 * quad], x[4 * quad + 1], x[4 * quad + 2], x[4 * quad + 3]);
+      ldead = !on || (c.dead[0] & c.dead[1] & c.dead[2] & c.dead[3]) == ~0u;
+      alive += ldead ? 0u : 1u;
+      if (__all_sync(0xFFFFFFFFu, ldead)) break;
+    }
+    // blocks each 1024-bin tile needed, as the staged kernel counts them
+    uint32_t used = alive;
+    used = max(used, __shfl_xor_sync(0xFFFFFFFFu, used, 1));
+    used = max(used, __shfl_xor_sync(0xFFFFFFFFu, used, 2));
+    used = max(used, __shfl_xor_sync(0xFFFFFFFFu, used, 4));
+    used = (lane & 7u) == 0 && on ? min(nblk, used + 1u) : 0u;
+    used = __reduce_add_sync(0xFFFFFFFFu, used);
+    if (lane == 0) atomicAdd(&a.ctl->blocks, (unsigned long long)used);
+    if (__all_sync(0xFFFFFFFFu, ldead)) continue;
+    uint32_t pm[4], cnt = 0;
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      const uint64_t b0 = (word0 + w) * 32;
+      const uint64_t left = on && b0 < a.ix.num_bins ? a.ix.num_bins - b0 : 0;
+      pm[w] = ~c.dead[w] & (left >= 32 ? ~0u : (1u << left) - 1u);
+      cnt += __popc(pm[w]);
+    }
+    uint32_t incl = cnt;
+#pragma unroll
+    for (int dd = 1; dd < 32; dd <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, dd);
+      if (lane >= (uint32_t)dd) incl += t;
+    }
+    const uint32_t tot = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    unsigned long long base = 0;
+    if (lane == 0 && tot) base = atomicAdd(&a.ctl->n_rec, (unsigned long long)tot);
+    base = __shfl_sync(0xFFFFFFFFu, base, 0);
+    if (base >= a.rec.cap) continue;  // counted only
+    unsigned long long pos = base + incl - cnt;
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      uint32_t mask = pm[w];
+      while (mask) {
+        const uint32_t bit = __ffs(mask) - 1;
+        mask &= mask - 1;
+        if (pos < a.rec.cap) {
+          a.rec.keys[pos] = ((unsigned long long)r << a.bin_bits) | ((word0 + w) * 32 + bit);
+          a.rec.counts[pos] = (uint8_t)(ntok - (c.value(w, bit) - bias));
+        }
+        ++pos;
+      }
+    }
+  }
+}
+
 template <int P, int TW, int NT, bool WS>
 void launch_p(const ExhArgs& a, size_t smem, uint32_t threads, uint32_t grid, cudaStream_t st,
               const char* name) {
@@ -675,6 +822,17 @@ bool exhaustive_shape_ok(const ExhShape& s) {
   return t_ok && r_ok && w_ok;
 }
 
+// A handful of reads go to k_exhaustive_few: it loads about n_reads * tokens
+// rows, the staged kernel all 4^q, each once.  Measured on GB300 (few /
+// staged, us): 3.1 Gbp coarse table at q = 5, mixed reads of an index for
+// 250 bp, 1 read 14 / 230, 8 97 / 273, 16 153 / 279, 24 197 / 325, 32 372 /
+// 341; 100 bp, 16 135 / 263, 48 290 / 321, 64 374 / 354; its fine table, 16
+// 218 / 449, 64 607 / 603; q = 6, 64 165 / 361.  Tables that L2 holds stage
+// as fast (50 Mbp: 18 / 15 at 16 reads).
+uint32_t exhaustive_few_reads(const IndexView& ix, uint32_t ts) {
+  return (uint64_t)ix.r4 * ix.wpad * 4u >= kFewMinTable ? 4u * ix.r4 / ts : 0u;
+}
+
 void launch_exhaustive(const IndexView& ix, const ReadsView& rv, RecordsView rec, uint32_t bin_bits,
                        uint32_t max_d, Ctl* ctl, cudaStream_t st, const char* prof_name,
                        Live live, ExhShape shape) {
@@ -721,6 +879,23 @@ void launch_exhaustive(const IndexView& ix, const ReadsView& rv, RecordsView rec
   a.c_lo = 0u - 65536u;
   a.range_bytes = shape.range_kb ? (uint64_t)shape.range_kb << 10 : kDefaultRangeBytes;
   a.ctl = ctl;
+  // A graph launch decides by the batch's own count (k_plan_control leaves
+  // ctl->path 0 for a few reads), so it enqueues both kernels.  (A count check
+  // inside the staged kernel itself cost it 2.4% of its loop's schedule.)
+  a.few_reads = exhaustive_few_reads(ix, rv.ts);
+  if (a.few_reads && (live.on || rv.n_reads <= a.few_reads)) {
+    const uint64_t n = min(rv.n_reads, a.few_reads);
+    const uint64_t items = (ix.wpad + 127) / 128 * n;
+    const uint64_t need = (items + kFewThreads / 32 - 1) / (kFewThreads / 32);
+    const uint64_t most = (uint64_t)sms * 2;
+    const unsigned grid = (unsigned)(need < most ? need : most);
+    {
+      ProfScope ps(prof_name, st);
+      if (max_d < 32) k_exhaustive_few<5><<<grid, kFewThreads, 0, st>>>(a);
+      else k_exhaustive_few<8><<<grid, kFewThreads, 0, st>>>(a);
+    }
+    if (!live.on || rv.n_reads <= a.few_reads) return;
+  }
   const bool ws = shape.read_switch == GRIM_SWITCH_WARP;
   if (ix.r4 <= 1024) launch_tw<32>(a, ix, max_d, (uint32_t)sms, nt, ws, st, prof_name);
   else launch_tw<8>(a, ix, max_d, (uint32_t)sms, nt, ws, st, prof_name);

@@ -30,7 +30,7 @@ struct Ctl {
   // graph launches (grim_plan): the batch's counts and the path taken live
   // on the device, so no launch depends on a host read-back
   uint32_t live_reads;             // reads in this batch
-  uint32_t path;                   // kPathCoarse / kPathExact
+  uint32_t path;                   // kPathCoarse / kPathExact for the staged all-bins kernel (0: not its batch)
   unsigned long long live_cand;    // candidates in this batch
   unsigned long long live_bases;   // read bytes in this batch (host-memory plans)
   unsigned long long n_surv;       // survivors of the coarse pass
@@ -39,7 +39,8 @@ struct Ctl {
   uint32_t blk_lo;                 // 32 - the fewest 16-token blocks of a read
   unsigned long long tail_blocks;  // of `blocks`: applied to one word per lane (256 bins)
   uint32_t d_lo;                   // 255 - the smallest miss budget D' of the batch
-  uint32_t pad[41];
+  uint32_t route;                  // the batch's path, whichever kernel sweeps it
+  uint32_t pad[40];
 };
 static_assert(sizeof(Ctl) == 256, "Ctl is one 256-byte slot");
 static_assert(offsetof(Ctl, live_reads) == 32, "live counts follow the per-pass counters");
@@ -48,7 +49,8 @@ constexpr uint32_t kPathExact = 2u;   // one exact pass over every bin
 
 // Counts a kernel works on: fixed by the host (grim_filter), or read from
 // the control block at run time (graph launches).  `gate`, when nonzero, is
-// the path the kernel belongs to: it returns at once unless ctl->path == gate.
+// the path the kernel belongs to: it returns at once unless the batch takes
+// that path (ctl->path for the staged all-bins kernel, ctl->route for others).
 struct Live {
   bool on;
   uint32_t gate;
@@ -60,6 +62,10 @@ __device__ __forceinline__ uint32_t live_reads(const Ctl* c, const Live& l, uint
 }
 __device__ __forceinline__ bool gated_off(const Ctl* c, const Live& l) {
   return l.on && l.gate && c->path != l.gate;
+}
+
+__device__ __forceinline__ bool routed_off(const Ctl* c, const Live& l) {
+  return l.on && l.gate && c->route != l.gate;
 }
 
 constexpr uint32_t kStatusShort = 1u;     // read with L < q
@@ -173,6 +179,9 @@ struct ExhShape {
   uint32_t read_switch;
   uint32_t path;
 };
+// batches of up to this many reads go to the all-bins kernel for few reads (0:
+// none), which needs no tiles (see launch_exhaustive)
+uint32_t exhaustive_few_reads(const IndexView& ix, uint32_t ts);
 // the launch shape's threads, range and read switch are ones the kernel builds
 bool exhaustive_shape_ok(const ExhShape& s);
 // max_d: the batch's largest miss budget (sizes the bit-sliced counters)

@@ -67,23 +67,30 @@ __global__ void k_copy_in(CopyIn a, const Ctl* c) {
 enum : uint32_t { kCtlDecide = 1, kCtlAfterCoarse = 2, kCtlFinal = 3 };
 
 // One thread: the per-batch decisions that grim_filter takes on the host.
+// few_coarse / few_exact: batches of up to this many reads are swept by the
+// all-bins kernel for few reads on that table, not by the staged one.
 __global__ void k_plan_control(Ctl* c, uint32_t op, uint32_t capable, uint32_t has_exact,
-                               unsigned long long rcap, uint32_t forced) {
+                               unsigned long long rcap, uint32_t forced, uint32_t few_coarse,
+                               uint32_t few_exact) {
+  auto take = [&](uint32_t route) {
+    c->route = route;
+    c->path = c->live_reads <= (route == kPathCoarse ? few_coarse : few_exact) ? 0u : route;
+  };
   if (op == kCtlDecide) {
     const uint32_t min_slack = 255u - c->max_tight;
-    c->path = (capable && (forced || min_slack >= 24 || !has_exact)) ? kPathCoarse : kPathExact;
+    take((capable && (forced || min_slack >= 24 || !has_exact)) ? kPathCoarse : kPathExact);
   } else if (op == kCtlAfterCoarse) {
-    if (c->path == kPathCoarse) {
+    if (c->route == kPathCoarse) {
       c->n_surv = c->n_rec;
       if (c->n_rec > rcap) {  // too many survivors to hold
-        if (has_exact) c->path = kPathExact;
+        if (has_exact) take(kPathExact);
         else c->status |= kStatusSurv;
       }
     }
     c->n_rec = 0;  // restart the record and work counters for the next pass
     c->item = 0;
   } else {
-    if (c->path != kPathCoarse) c->n_final = c->n_rec;  // (the survivors' check counts there itself)
+    if (c->route != kPathCoarse) c->n_final = c->n_rec;  // (the survivors' check counts there itself)
   }
 }
 
@@ -156,14 +163,17 @@ int capture(grim_plan* p) {
   if (p->cand_mode) {
     launch_check_candidates(B.cand_off, d.max_reads, d.max_cand, p->ctl, st, live);
     launch_candidates(v, rv, B.cand, B.cand_off, ra, p->ctl, st, live, d.cand_unroll);
-    k_plan_control<<<1, 1, 0, st>>>(p->ctl, kCtlFinal, 0, 0, 0, 0);
+    k_plan_control<<<1, 1, 0, st>>>(p->ctl, kCtlFinal, 0, 0, 0, 0, 0, 0);
     sort_and_emit(ra, rb, d.cap, bit_length(d.max_cand ? d.max_cand - 1 : 0), ws + L.hist, true,
                   bin_bits, B.cand, B.cand_off, d.max_reads, B.out_read,
                   B.out_bin, B.out_count, st, &p->ctl->n_final, &p->ctl->live_reads);
   } else {
     bool forced = false;
     all_bins_path(idx, &forced);
-    k_plan_control<<<1, 1, 0, st>>>(p->ctl, kCtlDecide, p->f != 0, has_exact, rcap, forced);
+    const uint32_t few_coarse = exhaustive_few_reads(idx->cv, rv.ts);
+    const uint32_t few_exact = exhaustive_few_reads(v, rv.ts);
+    k_plan_control<<<1, 1, 0, st>>>(p->ctl, kCtlDecide, p->f != 0, has_exact, rcap, forced,
+                                    few_coarse, few_exact);
     const uint32_t cbits =
         idx->cv.num_bins > 1 ? bit_length(idx->cv.num_bins - 1) : 0;
     // both paths leave their records in rb: the coarse pass's survivors are
@@ -172,7 +182,8 @@ int capture(grim_plan* p) {
       const Live coarse{true, kPathCoarse};
       launch_exhaustive(idx->cv, rv, ra, cbits, max_d, p->ctl, st, "exhaustive_coarse", coarse,
                         idx->shape);
-      k_plan_control<<<1, 1, 0, st>>>(p->ctl, kCtlAfterCoarse, 1, has_exact, rcap, 0);
+      k_plan_control<<<1, 1, 0, st>>>(p->ctl, kCtlAfterCoarse, 1, has_exact, rcap, 0, few_coarse,
+                                      few_exact);
       launch_refine(v, rv, ra.keys, &p->ctl->n_surv, rcap, cbits, p->f, rb, bin_bits, p->ctl, st,
                     coarse);
     }
@@ -180,7 +191,7 @@ int capture(grim_plan* p) {
       const Live exact{true, kPathExact};
       launch_exhaustive(v, rv, rb, bin_bits, max_d, p->ctl, st, "exhaustive", exact, idx->shape);
     }
-    k_plan_control<<<1, 1, 0, st>>>(p->ctl, kCtlFinal, 0, 0, 0, 0);
+    k_plan_control<<<1, 1, 0, st>>>(p->ctl, kCtlFinal, 0, 0, 0, 0, 0, 0);
     sort_and_emit(rb, ra, d.cap, bin_bits + read_bits, ws + L.hist, false, bin_bits, nullptr,
                   nullptr, d.max_reads, B.out_read, B.out_bin, B.out_count, st, &p->ctl->n_final,
                   &p->ctl->live_reads);

@@ -691,3 +691,41 @@ def test_one_pass_build_shapes(q, B, mrl, factor, n, layouts, shift):
         coarse = oracle.token_major(oracle.bin_vectors(g, factor * B, q, mrl))
         assert np.array_equal(idx.coarse_token_major().cpu().numpy().view(np.uint32), coarse)
     idx.close()
+
+
+@pytest.mark.parametrize("q,B,mrl,layouts", [(5, 50, 250, 7), (5, 50, 100, 1), (6, 100, 150, 6)])
+def test_few_reads_on_a_large_table(q, B, mrl, layouts):
+    """Batches of a few reads load table rows instead of staging tiles: counts
+    up to the rule's line (4 * 4^q rows' worth of tokens) and past it, a last
+    tile group cut by the row end, reads of one token, with non-bases and of
+    every budget, through the plain call and a plan that holds more reads."""
+    from paper_1708_04329_gb300 import grim, synth
+
+    n = 70_000_003
+    g = synth.human_genome(n, seed=q)
+    ts = -(-(mrl - q + 1) // 16) * 16
+    line = 4 * 4 ** q // ts
+    rs = synth.reads(g, line + 1, seed=9, lengths=(q, 80, mrl), probs=(0.05, 0.45, 0.5),
+                     e_frac=(5, 100), max_edits=None)
+    rs.seq[int(rs.offsets[2]) + 3] = ord("N")
+    rs.e[rs.lens == q] = 0
+    ix = build(g, B, q, mrl, layouts)
+    grim.grim_index_set_shape(ix, all_bins_path=0 if layouts != 7 else grim.GRIM_PATH_TWO_LEVEL)
+    oix = oracle.bin_vectors(g, B, q, mrl)
+    short = int((rs.lens == q).sum())
+    cap = 40_000 * (short + 1) + 200_000
+    want = oracle.filter(oix, rs)
+    for k in (1, 3, line, line + 1):
+        sub = rs.subset(range(k))
+        keep = want[0] < k
+        assert_same(gpu_filter(ix, sub, cap=len(want[0]) + cap), tuple(x[keep] for x in want))
+    plan = grim.grim_plan_create(ix, max_reads=line + 5, max_bases=len(rs.seq) + 64,
+                                 max_e=mrl // 20, cap=len(want[0]) + cap)
+    for k in (2, line + 1):
+        sub = rs.subset(range(k))
+        got = plan.run(**dev_reads(sub))
+        keep = want[0] < k
+        assert_same((got[0].cpu().numpy().view(np.uint32), got[1].cpu().numpy().view(np.uint32),
+                     got[2].cpu().numpy()), tuple(x[keep] for x in want))
+    plan.close()
+    ix.close()
