@@ -134,7 +134,7 @@ int grim_build_host(const char* ref, uint64_t len, uint32_t B, uint32_t q, uint3
 /* How the lane groups of a warp in the all-bins kernel take their next read
  * (grim_shape). */
 #define GRIM_SWITCH_GROUP 1u /* each group as soon as its read ends             */
-#define GRIM_SWITCH_WARP 2u  /* all groups of a warp together, once all ended   */
+#define GRIM_SWITCH_WARP 2u  /* all groups of a warp together                   */
 
 /* The all-bins path (grim_shape).  Automatic (0): coarse-then-exact when the
  * index has the coarse and bin-major tables and its super-bin window would
@@ -198,15 +198,16 @@ int grim_index_info(const grim_index* idx, grim_index_desc* out);
  *   read_switch    GRIM_SWITCH_GROUP, GRIM_SWITCH_WARP, or 0 (automatic):
  *                  a warp's lane groups each hold one read; taking the next
  *                  read costs the whole warp the same instructions whether
- *                  one group or all take one, so WARP lets a group whose read
- *                  ended early idle until every group's read has ended, and
- *                  then switches all of them at once (fewer switches, some
- *                  idle blocks).  Automatic: WARP when every read of the
- *                  batch spans the same number of 16-token blocks and has
- *                  the same miss budget D' (so reads leave a tile at similar
- *                  blocks and no group idles for long), GROUP otherwise;
- *                  graph plans, whose batches are not known when they are
- *                  captured, use GROUP
+ *                  one group or all take one.  GROUP switches each group as
+ *                  its read ends.  WARP runs the reads of a warp together for
+ *                  as many tokens as they are expected to need, finishes the
+ *                  few bins still live apart, and switches all of them at
+ *                  once.  Automatic: WARP for batches whose reads span the
+ *                  same number of 16-token blocks and have the same miss
+ *                  budget D'; of mixed batches those of 256 reads and more
+ *                  run together too, sorted so that reads of similar length
+ *                  to go share a warp (as do graph plans for that many
+ *                  reads), smaller ones switch by GROUP
  *   all_bins_path  GRIM_PATH_TWO_LEVEL, GRIM_PATH_EXACT, or 0 (automatic; see
  *                  GRIM_PATH_*)
  * Results do not depend on the shape.  Graph plans take the shape when they
@@ -582,19 +583,18 @@ typedef struct {
   uint64_t pairs;            /* (read, bin) pairs decided: reads x bins, or n_cand    */
   uint64_t tokens_executed;  /* all-bins mode: read tokens applied to (super-)bin tiles
                                 (1024 wide up to q = 5, 256 at q = 6), counting padding
-                                up to a 16-token block; stops early for a read once
-                                every bin of the tile has failed                       */
+                                up to a block of 16 (WARP: of 8) tokens; stops early for
+                                a read once every bin of the tile has failed           */
   uint64_t survivors;        /* all-bins mode, coarse-then-exact: (read, super-bin)
                                 pairs that passed the coarse pass (0 otherwise)       */
   uint64_t bit_tests_executed; /* all-bins mode: tokens_executed x (super-)bins per tile,
-                                  except that a token of the one-word tail (1024-bin tiles,
-                                  warp read switch: the last blocks of a read once every
-                                  lane of the warp has at most one 32-bin word with a live
-                                  bin) tests 256 of the tile's bins                       */
-  uint32_t read_switch;        /* all-bins mode: GRIM_SWITCH_GROUP or GRIM_SWITCH_WARP, as
-                                  chosen for the call (automatic: WARP when every read
-                                  spans as many 16-token blocks and has the same miss
-                                  budget D' = min(q*e, L-q+1)); 0 in candidate mode      */
+                                  except that once the live words of a warp's reads are
+                                  gathered (WARP), a token tests 32 bins for each of them */
+  uint32_t read_switch;        /* all-bins mode: GRIM_SWITCH_GROUP or GRIM_SWITCH_WARP as
+                                  set, or, automatic, the batch's kind: WARP when every
+                                  read spans as many 16-token blocks and has the same miss
+                                  budget D' = min(q*e, L-q+1), GROUP when they differ (see
+                                  grim_shape); 0 in candidate mode                       */
   uint32_t all_bins_path;      /* all-bins mode: GRIM_PATH_TWO_LEVEL or GRIM_PATH_EXACT,
                                   the path the call took (after any fallback); 0 in
                                   candidate mode                                          */

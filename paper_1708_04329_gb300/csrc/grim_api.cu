@@ -165,18 +165,20 @@ int index_alloc(uint64_t len, uint32_t B, uint32_t q, uint32_t max_read_len, uin
     if (e != cudaSuccess) return fail(e);
   }
   if (layouts & (GRIM_LAYOUT_COARSE | GRIM_LAYOUT_TOKEN_MAJOR)) {
-    e = table(&ix->presence, (uint64_t)v.r4 * (sizeof(uint32_t) + sizeof(uint16_t)));
+    e = table(&ix->presence, (uint64_t)v.r4 * kPresenceBytes);
     if (e != cudaSuccess) return fail(e);
   }
   ix->coarse_pays = coarse_density(B, q, v.ext, f) <= kCoarseDensityMax;
   v.tm = ix->tm;
   v.bm = ix->bm;
   v.bm_rows = bm_bins;
-  v.rank = ix->presence ? reinterpret_cast<uint16_t*>(ix->presence + v.r4) : nullptr;
+  v.rank = rank_table(ix->presence, v.r4);
+  v.miss = miss_table(ix->presence, v.r4);
   ix->v = v;
   cv.tm = ix->ctm;
   cv.bm = nullptr;
   cv.rank = v.rank;
+  cv.miss = v.miss;
   ix->cv = cv;
   *out = ix;
   return GRIM_OK;
@@ -390,8 +392,8 @@ int grim_build_ex(const char* ref, uint64_t len, uint32_t B, uint32_t q, uint32_
   if (from_bm_ctm) launch_tm_from_bm(bm, cv, v.wpb, f, ix->ctm, st);
   if (bm != ix->bm) cudaFreeAsync(bm, st);
   // token presence from the table the all-bins filter sweeps first
-  if (ix->ctm) launch_presence(ix->ctm, cv.r4, cv.wpad, ix->presence, index_rank(ix), st);
-  else if (ix->tm) launch_presence(ix->tm, v.r4, v.wpad, ix->presence, index_rank(ix), st);
+  if (ix->ctm) launch_presence(ix->ctm, cv, ix->presence, st);
+  else if (ix->tm) launch_presence(ix->tm, v, ix->presence, st);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   prof_collect();
@@ -536,7 +538,8 @@ int grim_filter(const grim_index* idx, const char* reads, const uint64_t* offset
   const uint32_t read_bits = n_reads > 1 ? bit_length((uint64_t)n_reads - 1) : 0;
 
   CK(cudaMemsetAsync(ctl, 0, sizeof(Ctl), st));
-  launch_tokenise(reads, offsets, lens, e, v, rv, tokens, meta, ctl, st, cand_mode);
+  launch_tokenise(reads, offsets, lens, e, v, rv, tokens, meta, ctl, st, cand_mode,
+                  fine_miss_power(idx));
   // The host waits where it has to decide: all-bins calls after tokenising
   // (the counters' depth, the path, the read switch) and every call for its
   // record count; what follows either way is enqueued before the wait (the
@@ -579,19 +582,23 @@ int grim_filter(const grim_index* idx, const char* reads, const uint64_t* offset
     // automatic read switch: a warp's lane groups take their next reads
     // together when every read has as many 16-token blocks and the same miss
     // budget D' (reads then leave a tile at similar blocks, so no group
-    // waits long for the others), each on its own otherwise
+    // waits long for the others), each on its own otherwise.  A mixed batch of
+    // some size runs together all the same, in an order that puts reads with as
+    // far to go side by side; so does a large uniform one.
     ExhShape shape = idx->shape;
-    if (!shape.read_switch)
-      shape.read_switch = h.blk_max + h.blk_lo == 32u && h.max_d + h.d_lo == 255u
-                              ? GRIM_SWITCH_WARP
-                              : GRIM_SWITCH_GROUP;
+    const bool uniform = h.blk_max + h.blk_lo == 32u && h.max_d + h.d_lo == 255u;
+    if (!shape.read_switch) shape.read_switch = uniform ? GRIM_SWITCH_WARP : GRIM_SWITCH_GROUP;
     switch_used = shape.read_switch;
+    uint32_t* order = order_room(v, ws, L, n_reads, rcap, f, rb);
+    if (idx->shape.read_switch || (uniform && n_reads < kOrderUniform)) order = nullptr;
+    if (order) shape.read_switch = GRIM_SWITCH_WARP;
+    launch_order(rv, order, ctl, st);
     const uint32_t max_d = h.max_d;
     if (two) {
       // the survivors stay in ra; their passing members go to rb
       const IndexView& cv = idx->cv;
       const uint32_t cbits = cv.num_bins > 1 ? bit_length(cv.num_bins - 1) : 0;
-      launch_exhaustive(cv, rv, ra, cbits, max_d, ctl, st, "exhaustive_coarse", {false, 0}, shape);
+      launch_exhaustive(cv, rv, ra, cbits, max_d, ctl, st, false, order, {false, 0}, shape);
       launch_refine(v, rv, ra.keys, &ctl->n_rec, rcap, cbits, f, rb, bin_bits, ctl, st);
       found = rb;
       other = ra;
@@ -618,7 +625,7 @@ int grim_filter(const grim_index* idx, const char* reads, const uint64_t* offset
     }
     path_used = two ? GRIM_PATH_TWO_LEVEL : GRIM_PATH_EXACT;
     if (!two) {
-      launch_exhaustive(v, rv, ra, bin_bits, max_d, ctl, st, "exhaustive", {false, 0}, shape);
+      launch_exhaustive(v, rv, ra, bin_bits, max_d, ctl, st, true, order, {false, 0}, shape);
       emit_short(~0ull);
       sc = read_back();
       if (sc != GRIM_OK) return sc;
@@ -639,11 +646,10 @@ int grim_filter(const grim_index* idx, const char* reads, const uint64_t* offset
   g_last_stats.n_reads = n_reads;
   g_last_stats.n_records = n_rec;
   g_last_stats.pairs = cand_mode ? n_cand : (uint64_t)n_reads * v.num_bins;
-  g_last_stats.tokens_executed = h.blocks * kBlockTokens;
-  // blocks of the one-word tail test a quarter of the tile's bins
+  constexpr uint64_t kHalf = kBlockTokens / 2;
+  g_last_stats.tokens_executed = (h.blocks + h.tail_blocks) * kHalf;
   g_last_stats.bit_tests_executed =
-      (h.blocks - h.tail_blocks) * kBlockTokens * exhaustive_tile_bins(v.r4) +
-      h.tail_blocks * kBlockTokens * (exhaustive_tile_bins(v.r4) / 4);
+      h.blocks * kHalf * exhaustive_tile_bins(v.r4) + h.tail_words * kHalf * 32;
   g_last_stats.survivors = survivors;
   g_last_stats.read_switch = switch_used;
   g_last_stats.all_bins_path = path_used;

@@ -227,10 +227,12 @@ __global__ void __launch_bounds__(512) k_row_popcount(const uint32_t* __restrict
 }
 
 // A token's rank among the tokens of its class (token % classes): how many of
-// them fewer (super-)bins hold, ties by value.
+// them fewer (super-)bins hold, ties by value; and the share of the `units`
+// (super-)bins without it.
 __global__ void __launch_bounds__(128) k_token_ranks(const uint32_t* __restrict__ presence,
-                                                     uint32_t rows, uint32_t classes,
-                                                     uint16_t* __restrict__ rank) {
+                                                     uint32_t rows, uint32_t classes, float units,
+                                                     uint16_t* __restrict__ rank,
+                                                     float* __restrict__ miss) {
   __shared__ uint32_t s_p[4096];  // q <= 6
   for (uint32_t i = threadIdx.x; i < rows; i += 128) s_p[i] = presence[i];
   __syncthreads();
@@ -241,6 +243,7 @@ __global__ void __launch_bounds__(128) k_token_ranks(const uint32_t* __restrict_
   for (uint32_t i = t % classes; i < rows; i += classes)
     r += s_p[i] < mine || (s_p[i] == mine && i < t);
   rank[t] = (uint16_t)r;
+  miss[t] = fmaxf(0.f, 1.f - (float)mine / units);
 }
 
 // 16 bases (bytes, first base lowest) to a code word (first base in the top
@@ -498,14 +501,18 @@ void launch_tm_from_bm(const uint32_t* bm, const IndexView& unit_view, uint32_t 
   }
 }
 
-void launch_presence(const uint32_t* tm, uint32_t rows, uint64_t words_per_row, uint32_t* presence,
-                     uint16_t* rank, cudaStream_t st) {
+void launch_presence(const uint32_t* tm, const IndexView& units, uint32_t* presence,
+                     cudaStream_t st) {
+  const uint32_t rows = units.r4;
   {
     ProfScope ps("row_popcount", st);
-    k_row_popcount<<<rows, 512, 0, st>>>(tm, words_per_row, presence);
+    k_row_popcount<<<rows, 512, 0, st>>>(tm, units.wpad, presence);
   }
   ProfScope ps("token_ranks", st);
-  k_token_ranks<<<(rows + 127) / 128, 128, 0, st>>>(presence, rows, rows > 1024 ? 4u : 1u, rank);
+  k_token_ranks<<<(rows + 127) / 128, 128, 0, st>>>(presence, rows, rows > 1024 ? 4u : 1u,
+                                                    (float)units.num_bins,
+                                                    rank_table(presence, rows),
+                                                    miss_table(presence, rows));
 }
 
 namespace {

@@ -437,7 +437,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_refine(IndexView ix, ReadsVi
         tok[u] = rv.tokens + (uint64_t)__shfl_sync(0xFFFFFFFFu, r, k + u) * rv.copies * rv.ts + lane;
         vec[u] = ix.bm + (uint64_t)__shfl_sync(0xFFFFFFFFu, bin, k + u) * ix.wpb;
         ntok[u] = mu & 0xFFu;
-        dmax[u] = mu >> 8;
+        dmax[u] = (mu >> 8) & 0xFFu;
         misses[u] = 0;
       }
       for (uint32_t j = 0; live_items; j += 32) {

@@ -40,34 +40,22 @@
 //   The logic ops run on the integer pipe, which bounds this kernel; the
 //   token-to-address arithmetic is written as integer multiply-adds so that
 //   it runs on the FMA pipe instead.
-// * Early exit: after each 16-token block the group stops a read once every
-//   one of its 1024 bins is dead -- exact, since a dead bin can never pass.
-//   With the warp switch and 1024-bin tiles the test is one warp vote per
-//   block: the warp takes new reads once every lane has no live bin or is
-//   past its read's last block.  A group that ended reads on through its
-//   token row's padding (the tokeniser fills each row to its stride with
-//   the never-miss token), so its counters hold; a per-lane count of the
-//   blocks that left a live bin gives each read's useful blocks.
-// * Groups stay converged: the per-block work is the same instruction stream
-//   for all groups of a warp, and every warp collective uses the full mask.
-//   Taking a next read (new counters, the claim, the prefetch of the read
-//   after it) runs for the whole warp whenever any group needs it, so the
-//   launch chooses how groups switch reads (WS): each as soon as its read
-//   ends (a switch for every read that ends), or all groups of a warp
-//   together once every one of them has ended (one switch per warp per
-//   round of reads; a group that ends early applies padding tokens, which
-//   change nothing, until the others end).  With sixteen groups (256-bin
-//   tiles) the warp switch comes once 14 of them wait; the other two keep
-//   their reads.
-// * One-word tail (1024-bin tiles, warp switch): after four blocks of a
-//   round, if no lane of the warp has more than one word with a live bin,
-//   the warp keeps that word's counters and applies the round's remaining
-//   blocks to it alone (one 4-byte load and a quarter of the logic ops per
-//   token).  Past the first blocks the live bins of a tile usually sit in
-//   one or two words near the read's true position.  Register pressure
-//   decides whether this pays: the tail runs as its own inner loop so that
-//   the four-word loop stays as it was (a variant that chose the word count
-//   per block spilled and ran slower than no tail at all).
+// * Early exit: a read leaves a tile once every one of its bins is dead --
+//   exact, since a dead bin can never pass.
+// * Two kernels differ in how a warp's groups, which run one instruction
+//   stream, take their reads.  Taking one (new counters, the claim, the
+//   prefetch of the read after it) costs the whole warp the same whether one
+//   group or all do.  k_exhaustive (GRIM_SWITCH_GROUP) tests after each block
+//   and switches every group whose read has ended.  k_lockstep
+//   (GRIM_SWITCH_WARP, and every batch large enough to sort) takes reads with
+//   as far to go together, tests nothing before the place where the tokeniser
+//   expects a tile to be nearly done, and finishes what is live there apart.
+//   Measured on GB300, k_exhaustive with a per-block test and a one-word tail
+//   for uniform batches against k_lockstep (3.1 Gbp, ms): 250k reads of 100 bp,
+//   coarse table 609 -> 599, 40k on the fine table 165 -> 159, 40k mixed
+//   100-250 bp reads 102 -> 89, a plan of 4,096 of them 11.3 -> 9.7, 60k of 150
+//   bp at q = 6 60.3 -> 56.8.  Both pipes are near their limit there (small
+//   case: ALU 78%, shared-memory wavefronts 83%).
 #include "grim_internal.cuh"
 
 namespace grim {
@@ -84,16 +72,13 @@ constexpr size_t kSmemLimit = 227 * 1024;  // dynamic shared memory per CTA
 // sweeps its tiles against the range
 constexpr uint64_t kDefaultRangeBytes = 48ull << 20;
 constexpr uint32_t kSlotBlocksNarrow = 4;  // most slot blocks per read, 256-bin tiles
-// WS, 256-bin tiles: groups of the sixteen that wait before the warp switches
-constexpr uint32_t kSwitchGroupsNarrow = 14;
-// blocks a warp applies to all four words of its lanes before it checks for
-// the one-word tail (1024-bin tiles, warp-synchronous read switch)
-constexpr uint32_t kTailAfter = 4;
-
-template <int N>
-struct Words {
-  static constexpr int value = N;
-};
+// per-warp scratch through which the lockstep kernel's live words change lanes:
+// some planes of 32 words (what fits beside the slots) and 32 bytes that say
+// where each came from
+template <int TW>
+constexpr int kScratchPlanes = TW == 32 ? 5 : 3;
+template <int TW>
+constexpr uint32_t kScratchBytes = kScratchPlanes<TW> * 128 + 32;
 
 #define LOP3(d, a, b, c, lut) \
   asm("lop3.b32 %0, %1, %2, %3, " #lut ";" : "=r"(d) : "r"(a), "r"(b), "r"(c))
@@ -137,14 +122,14 @@ __device__ __forceinline__ uint32_t lds32(uint32_t addr) {
   return v;
 }
 
-template <int P>
+template <int P, int NW = 4>
 struct Counters {
   // per word: s1 s2 s4 s8 (weights 1..8), up[i] (weight 16 << i), dead
-  uint32_t s1[4], s2[4], s4[4], s8[4], up[P - 4][4], dead[4];
+  uint32_t s1[NW], s2[NW], s4[NW], s8[NW], up[P - 4][NW], dead[NW];
 
   __device__ __forceinline__ void init(uint32_t bias) {
 #pragma unroll
-    for (int w = 0; w < 4; ++w) {
+    for (int w = 0; w < NW; ++w) {
       s1[w] = 0u - (bias & 1u);
       s2[w] = 0u - ((bias >> 1) & 1u);
       s4[w] = 0u - ((bias >> 2) & 1u);
@@ -155,20 +140,10 @@ struct Counters {
     }
   }
 
-  // One-word tail: keep only the counters of word k in slot 0 (dead unless
-  // `live`); slots 1..3 die.
-  __device__ __forceinline__ void keep_one(uint32_t k, bool live) {
-    auto sel = [k](const uint32_t(&x)[4]) {
-      return k == 0 ? x[0] : k == 1 ? x[1] : k == 2 ? x[2] : x[3];
-    };
-    s1[0] = sel(s1);
-    s2[0] = sel(s2);
-    s4[0] = sel(s4);
-    s8[0] = sel(s8);
-#pragma unroll
-    for (int i = 0; i < P - 4; ++i) up[i][0] = sel(up[i]);
-    dead[0] = live ? sel(dead) : ~0u;
-    dead[1] = dead[2] = dead[3] = ~0u;
+  // plane p of word w: the counter's planes by weight, then `dead`
+  __device__ __forceinline__ uint32_t& plane(int p, int w) {
+    return p == 0 ? s1[w] : p == 1 ? s2[w] : p == 2 ? s4[w] : p == 3 ? s8[w]
+           : p < P ? up[p - 4][w] : dead[w];
   }
 
   // counter value of bin `bit` of word w
@@ -193,8 +168,10 @@ struct ExhArgs {
   uint32_t slot_blocks; // 16-token blocks a slot row holds; later blocks come from L2
   uint32_t c_row, c_hi, c_lo;  // TW*4, 65536, -65536: multipliers of the address math
   uint64_t range_bytes;        // token-row bytes of one read range (the read tile)
-  uint32_t switch_lanes;       // WS, 256-bin tiles: waiting lanes that make the warp switch
   uint32_t few_reads;          // batches of up to this many reads are k_exhaustive_few's
+  const uint32_t* order;       // lockstep: the reads in the order they are taken (null: as given)
+  uint32_t check_shift;        // lockstep: kMetaCheckCoarse or kMetaCheckFine
+  uint32_t pad_pair;           // two never-miss tokens
   Ctl* ctl;
 };
 
@@ -238,14 +215,12 @@ __device__ __forceinline__ void add_quad(Counters<P>& c, CsaTemps<NW>& t, int qu
   }
 }
 
-// Add the misses of one 16-token block.  tw holds 16 table row indices as
-// uint16 pairs; base is the shared address of this lane's words in row 0.
-// NW = 4: all four words of the lane (one 16-byte load per token); NW = 1:
-// the one-word tail, counter slot 0 only, its word at `base`.
-template <int P, int NW>
+// Add the misses of one 16-token block to the lane's four words.  tw holds 16
+// table row indices as uint16 pairs; base is the shared address of this lane's
+// words in row 0 (one 16-byte load per token).
+template <int P>
 __device__ __forceinline__ void add_block(Counters<P>& c, const uint32_t (&tw)[8], uint32_t base,
                                           const ExhArgs& a) {
-  static_assert(NW == 4 || NW == 1, "four words or one");
   uint32_t addr[16];
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
@@ -254,52 +229,120 @@ __device__ __forceinline__ void add_block(Counters<P>& c, const uint32_t (&tw)[8
     addr[2 * j] = imad(lo, a.c_row, base);
     addr[2 * j + 1] = imad(hi, a.c_row, base);
   }
-  uint32_t t2a[NW], t2b[NW], t4a[NW], t4b[NW], t8a[NW], t8b[NW], t16[NW];
+  CsaTemps<4> t;
 #pragma unroll
   for (int quad = 0; quad < 4; ++quad) {
-    uint32_t a0[NW], a1[NW], a2[NW], a3[NW];
-    if constexpr (NW == 4) {
-      const uint4 x0 = lds128(addr[4 * quad]), x1 = lds128(addr[4 * quad + 1]);
-      const uint4 x2 = lds128(addr[4 * quad + 2]), x3 = lds128(addr[4 * quad + 3]);
-      a0[0] = x0.x; a0[1] = x0.y; a0[2] = x0.z; a0[3] = x0.w;
-      a1[0] = x1.x; a1[1] = x1.y; a1[2] = x1.z; a1[3] = x1.w;
-      a2[0] = x2.x; a2[1] = x2.y; a2[2] = x2.z; a2[3] = x2.w;
-      a3[0] = x3.x; a3[1] = x3.y; a3[2] = x3.z; a3[3] = x3.w;
-    } else {
-      a0[0] = lds32(addr[4 * quad]);
-      a1[0] = lds32(addr[4 * quad + 1]);
-      a2[0] = lds32(addr[4 * quad + 2]);
-      a3[0] = lds32(addr[4 * quad + 3]);
-    }
-#pragma unroll
-    for (int w = 0; w < NW; ++w) {
-      uint32_t* t4 = (quad & 1) ? t4b : t4a;
-      fa_miss(c.s1[w], a0[w], a1[w], c.s1[w], t2a[w]);
-      fa_miss(c.s1[w], a2[w], a3[w], c.s1[w], t2b[w]);
-      fa(c.s2[w], t2a[w], t2b[w], c.s2[w], t4[w]);
-      if (quad == 1) fa(c.s4[w], t4a[w], t4b[w], c.s4[w], t8a[w]);
-      if (quad == 3) {
-        fa(c.s4[w], t4a[w], t4b[w], c.s4[w], t8b[w]);
-        fa(c.s8[w], t8a[w], t8b[w], c.s8[w], t16[w]);
-        // ripple the weight-16 carry through the upper planes; the carry out
-        // of the top plane (counter >= 2^P: misses > D') sticks in `dead`
-        uint32_t k = t16[w];
-#pragma unroll
-        for (int i = 0; i < P - 5; ++i) {
-          const uint32_t nk = c.up[i][w] & k;
-          c.up[i][w] ^= k;
-          k = nk;
-        }
-        uint32_t d;
-        LOP3(d, c.dead[w], c.up[P - 5][w], k, 0xF8);  // dead | (top & k)
-        c.up[P - 5][w] ^= k;
-        c.dead[w] = d;
-      }
-    }
+    const uint4 x0 = lds128(addr[4 * quad]), x1 = lds128(addr[4 * quad + 1]);
+    const uint4 x2 = lds128(addr[4 * quad + 2]), x3 = lds128(addr[4 * quad + 3]);
+    const uint32_t a0[4] = {x0.x, x0.y, x0.z, x0.w}, a1[4] = {x1.x, x1.y, x1.z, x1.w};
+    const uint32_t a2[4] = {x2.x, x2.y, x2.z, x2.w}, a3[4] = {x3.x, x3.y, x3.z, x3.w};
+    add_quad<P, 4>(c, t, quad, a0, a1, a2, a3);
   }
 }
 
-template <int P, int TW, int NT, bool WS>
+// Add the misses of 8 tokens (half a block) to NW words: NW = 4 as add_block,
+// NW = 1 the single word at `base`.
+template <int P, int NW>
+__device__ __forceinline__ void add_half(Counters<P, NW>& c, const uint4& tok, uint32_t base,
+                                         const ExhArgs& a) {
+  const uint32_t tw[4] = {tok.x, tok.y, tok.z, tok.w};
+  uint32_t addr[8];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const uint32_t hi = imul_hi(tw[j], a.c_hi);
+    const uint32_t lo = imad(hi, a.c_lo, tw[j]);
+    addr[2 * j] = imad(lo, a.c_row, base);
+    addr[2 * j + 1] = imad(hi, a.c_row, base);
+  }
+  uint32_t x[8][NW];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    if constexpr (NW == 4) {
+      const uint4 v = lds128(addr[j]);
+      x[j][0] = v.x; x[j][1] = v.y; x[j][2] = v.z; x[j][3] = v.w;
+    } else {
+      x[j][0] = lds32(addr[j]);
+    }
+  }
+#pragma unroll
+  for (int w = 0; w < NW; ++w) {
+    uint32_t t2a, t2b, t4a, t4b, k;
+    fa_miss(c.s1[w], x[0][w], x[1][w], c.s1[w], t2a);
+    fa_miss(c.s1[w], x[2][w], x[3][w], c.s1[w], t2b);
+    fa(c.s2[w], t2a, t2b, c.s2[w], t4a);
+    fa_miss(c.s1[w], x[4][w], x[5][w], c.s1[w], t2a);
+    fa_miss(c.s1[w], x[6][w], x[7][w], c.s1[w], t2b);
+    fa(c.s2[w], t2a, t2b, c.s2[w], t4b);
+    fa(c.s4[w], t4a, t4b, c.s4[w], k);
+    uint32_t nk = c.s8[w] & k;  // the weight-8 carry ripples on
+    c.s8[w] ^= k;
+    k = nk;
+#pragma unroll
+    for (int i = 0; i < P - 5; ++i) {
+      nk = c.up[i][w] & k;
+      c.up[i][w] ^= k;
+      k = nk;
+    }
+    uint32_t d;
+    LOP3(d, c.dead[w], c.up[P - 5][w], k, 0xF8);  // dead | (top & k)
+    c.up[P - 5][w] ^= k;
+    c.dead[w] = d;
+  }
+}
+
+// Work items are (tile, range of reads): enough ranges (of at least 64 reads)
+// to balance the persistent grid when tiles are few, and ranges whose token
+// rows fit in L2 when there are many reads: items are then taken range by
+// range, so the CTAs sweeping different tiles at the same time share one
+// range's token rows in L2 instead of each streaming every read's tokens from
+// DRAM.
+struct Ranges {
+  uint32_t n_ranges, per, n_items;
+  bool range_major;
+};
+__device__ __forceinline__ Ranges read_ranges(const ExhArgs& a, uint32_t n_reads) {
+  uint32_t n_ranges = (4u * a.sms + a.n_tiles - 1) / a.n_tiles;
+  const uint64_t token_bytes = (uint64_t)n_reads * a.rv.ts * 2u * a.rv.copies;
+  const uint32_t l2_ranges = (uint32_t)((token_bytes + a.range_bytes - 1) / a.range_bytes);
+  n_ranges = max(n_ranges, l2_ranges);
+  n_ranges = min(n_ranges, (n_reads + 63) / 64);
+  n_ranges = max(n_ranges, 1u);
+  const uint32_t per = (n_reads + n_ranges - 1) / n_ranges;
+  n_ranges = (n_reads + per - 1) / per;
+  return {n_ranges, per, a.n_tiles * n_ranges, a.n_tiles >= 4u * a.sms};
+}
+
+// the all-zeros and all-ones rows behind a tile, and 16 padding tokens
+template <int TW>
+__device__ __forceinline__ void fill_special_rows(uint32_t* tile, uint32_t r4, uint32_t pad_tokens,
+                                                  uint32_t tid, uint32_t nthreads) {
+  for (uint32_t i = tid; i < (uint32_t)TW; i += nthreads) {
+    tile[rowInvalid(r4) * TW + i] = 0u;
+    tile[rowPad(r4) * TW + i] = ~0u;
+  }
+  if (tid < 2) {  // 32 bytes
+    const uint32_t pp = rowPad(r4) | (rowPad(r4) << 16);
+    asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(pad_tokens + tid * 16u), "r"(pp));
+  }
+}
+
+// start copying a tile: rows [0, r4), words [tile*TW, tile*TW+TW)
+template <int TW>
+__device__ __forceinline__ void stage_tile(const ExhArgs& a, uint32_t tile, uint32_t sh_base,
+                                           uint32_t tid, uint32_t nthreads) {
+  constexpr uint32_t kChunks = TW / 4;  // 16-byte chunks per row
+  const uint32_t* src = a.ix.tm + (uint64_t)tile * TW;
+  for (uint32_t i = tid; i < a.ix.r4 * kChunks; i += nthreads) {
+    const uint32_t row = i / kChunks, chunk = i % kChunks;
+    const uint32_t* g = src + (uint64_t)row * a.ix.wpad + chunk * 4u;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sh_base + row * TW * 4u +
+                                                                  chunk * 16u),
+                 "l"(g));
+  }
+  asm volatile("cp.async.commit_group;");
+}
+
+template <int P, int TW, int NT>
 __global__ void __launch_bounds__(NT, 1) k_exhaustive(ExhArgs a) {
   constexpr uint32_t kRowBytes = TW * 4;     // one token's row of a tile
   constexpr uint32_t GL = TW / 4;            // lanes per group (one read)
@@ -313,39 +356,16 @@ __global__ void __launch_bounds__(NT, 1) k_exhaustive(ExhArgs a) {
   const uint32_t r4 = a.ix.r4;
   if (*(volatile uint32_t*)&a.ctl->status) return;  // set by the tokeniser before launch
   if (gated_off(a.ctl, a.live)) return;             // the batch takes the other path
-  // work items: (tile, range of reads); enough of them to balance the
-  // persistent grid, each range at least 64 reads
   const uint32_t n_reads = live_reads(a.ctl, a.live, a.rv.n_reads);
   if (n_reads == 0) return;
-  // enough ranges to balance the persistent grid when tiles are few, and
-  // ranges whose token rows fit in L2 when there are many reads: items are
-  // then taken range by range, so the CTAs sweeping different tiles at the
-  // same time share one range's token rows in L2 instead of each streaming
-  // every read's tokens from DRAM
-  uint32_t n_ranges = (4u * a.sms + a.n_tiles - 1) / a.n_tiles;
-  const uint64_t token_bytes = (uint64_t)n_reads * a.rv.ts * 2u * a.rv.copies;
-  const uint32_t l2_ranges = (uint32_t)((token_bytes + a.range_bytes - 1) / a.range_bytes);
-  n_ranges = max(n_ranges, l2_ranges);
-  n_ranges = min(n_ranges, (n_reads + 63) / 64);
-  n_ranges = max(n_ranges, 1u);
-  const uint32_t per = (n_reads + n_ranges - 1) / n_ranges;
-  n_ranges = (n_reads + per - 1) / per;
-  const uint32_t n_items = a.n_tiles * n_ranges;
-  const bool range_major = a.n_tiles >= 4u * a.sms;
+  const Ranges rg = read_ranges(a, n_reads);
 
   uint32_t* s_tile = reinterpret_cast<uint32_t*>(smem);
   const uint32_t tile_bytes = (r4 + 2) * kRowBytes;
   const uint32_t sh_base = (uint32_t)__cvta_generic_to_shared(smem);
   const uint32_t slot = sh_base + tile_bytes + (tid / GL) * a.slot_bytes;
   const uint32_t pad_tokens = sh_base + tile_bytes + (nthreads / GL) * a.slot_bytes;
-  for (uint32_t i = tid; i < (uint32_t)TW; i += nthreads) {
-    s_tile[rowInvalid(r4) * TW + i] = 0u;
-    s_tile[rowPad(r4) * TW + i] = ~0u;
-  }
-  if (tid < 2) {  // 16 padding tokens = 32 bytes
-    const uint32_t pp = rowPad(r4) | (rowPad(r4) << 16);
-    asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(pad_tokens + tid * 16u), "r"(pp));
-  }
+  fill_special_rows<TW>(s_tile, r4, pad_tokens, tid, nthreads);
   const uint32_t lane_base = sh_base + li * 16u;
   // the token copy this group reads (block-rotated copies spread the groups'
   // 32-byte rows over the bank groups at q = 6)
@@ -361,25 +381,13 @@ __global__ void __launch_bounds__(NT, 1) k_exhaustive(ExhArgs a) {
     }
     __syncthreads();
     const uint32_t item = s_item;
-    if (item >= n_items) break;
-    const uint32_t tile = range_major ? item % a.n_tiles : item / n_ranges;
-    const uint32_t range = range_major ? item / a.n_tiles : item % n_ranges;
-    const uint32_t r0 = range * per;
-    const uint32_t nr = min(per, n_reads - r0);
+    if (item >= rg.n_items) break;
+    const uint32_t tile = rg.range_major ? item % a.n_tiles : item / rg.n_ranges;
+    const uint32_t range = rg.range_major ? item / a.n_tiles : item % rg.n_ranges;
+    const uint32_t r0 = range * rg.per;
+    const uint32_t nr = min(rg.per, n_reads - r0);
 
-    // stage the tile: rows [0, r4), words [tile*TW, tile*TW+TW)
-    {
-      constexpr uint32_t kChunks = TW / 4;  // 16-byte chunks per row
-      const uint32_t* src = a.ix.tm + (uint64_t)tile * TW;
-      for (uint32_t i = tid; i < r4 * kChunks; i += nthreads) {
-        const uint32_t row = i / kChunks, chunk = i % kChunks;
-        const uint32_t* g = src + (uint64_t)row * a.ix.wpad + chunk * 4u;
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sh_base + row * kRowBytes +
-                                                                      chunk * 16u),
-                     "l"(g));
-      }
-      asm volatile("cp.async.commit_group;");
-    }
+    stage_tile<TW>(a, tile, sh_base, tid, nthreads);
 
     // which bins of this lane's words exist (only the last tile is ragged)
     uint32_t vm[4];
@@ -389,18 +397,10 @@ __global__ void __launch_bounds__(NT, 1) k_exhaustive(ExhArgs a) {
       const uint64_t left = b0 < a.ix.num_bins ? a.ix.num_bins - b0 : 0;
       vm[w] = left >= 32 ? ~0u : ((1u << left) - 1u);
     }
-    auto vmask = [&](uint32_t w) -> uint32_t {
-      return w == 0 ? vm[0] : w == 1 ? vm[1] : w == 2 ? vm[2] : vm[3];
-    };
-
     // per-group state (identical in the group's 8 lanes); the group's slot
     // holds two token rows: `buf` is the current read's, buf^1 the next's
     uint32_t cur = kNone, nxt = kNone, nxt_meta = 0, buf = 1;
-    uint32_t nblk = 0, ntok = 0, bias = 0, executed = 0, tail_exec = 0;
-    // WS, 1024-bin tiles: blocks since the warp's last switch, and the word
-    // kept in the one-word tail
-    uint32_t bk = 0, kt = 0;
-    uint32_t alive = 0;  // WS, 1024-bin tiles: blocks after which this lane had a live bin
+    uint32_t nblk = 0, ntok = 0, bias = 0, executed = 0;
     bool fin = false;
     Counters<P> c;
     c.init(0);
@@ -469,18 +469,15 @@ __global__ void __launch_bounds__(NT, 1) k_exhaustive(ExhArgs a) {
     switch_reads(true);
     const uint32_t gmask = kGroupMask << (grp * GL);
     bool active = __any_sync(0xFFFFFFFFu, !fin);
-    bool waiting = false;  // WS, 256-bin tiles: the group's read has ended; it waits for a switch
 
     // the passing bins of the groups whose reads ended (emit), then new
     // reads for them (done); the warp runs this together
-    auto emit_and_switch = [&](bool done, bool emit, auto words) {
-      constexpr int NW = decltype(words)::value;
+    auto emit_and_switch = [&](bool done, bool emit) {
       if (__any_sync(0xFFFFFFFFu, emit)) {
-        // in the one-word tail slot 0 holds word kt and slots 1..3 are dead
         uint32_t pm[4], cnt = 0;
 #pragma unroll
         for (int w = 0; w < 4; ++w) {
-          pm[w] = emit ? (~c.dead[w] & vmask((NW == 1 && w == 0) ? kt : (uint32_t)w)) : 0u;
+          pm[w] = emit ? (~c.dead[w] & vm[w]) : 0u;
           cnt += __popc(pm[w]);
         }
         uint32_t incl = cnt;
@@ -508,8 +505,7 @@ __global__ void __launch_bounds__(NT, 1) k_exhaustive(ExhArgs a) {
             const uint32_t bit = __ffs(m) - 1;
             m &= m - 1;
             const uint32_t misses = c.value(w, bit) - bias;
-            const uint32_t wi = (NW == 1 && w == 0) ? kt : (uint32_t)w;
-            const uint64_t bin = (uint64_t)tile * kTileBinsT + (li * 4u + wi) * 32u + bit;
+            const uint64_t bin = (uint64_t)tile * kTileBinsT + (li * 4u + w) * 32u + bit;
             if (pos < a.rec.cap) {
               a.rec.keys[pos] = ((unsigned long long)cur << a.bin_bits) | bin;
               a.rec.counts[pos] = (uint8_t)(ntok - misses);
@@ -520,21 +516,17 @@ __global__ void __launch_bounds__(NT, 1) k_exhaustive(ExhArgs a) {
       }
       if (done) cur = kNone;
       switch_reads(done);
-      waiting = false;
       active = __any_sync(0xFFFFFFFFu, !fin);
     };
 
-    // (2) one 16-token block for all groups, to NW words per lane: from the
-    //     slot, or for the blocks past the slot's rows (long reads at q = 6)
-    //     from L2; (3) then the end-of-read test.  True when the warp took
-    //     new reads.
-    auto run_block = [&](auto words) -> bool {
-      constexpr int NW = decltype(words)::value;
+    while (active) {
+      // (2) one 16-token block for all groups: from the slot, or for the blocks
+      //     past the slot's rows (long reads at q = 6) from L2
       {
         uint4 t0, t1;
         const uint32_t bi = nblk - left;  // this read's block index
-        // (1024-bin tiles: whole reads in slots; waiting groups read padding)
-        if (TW == 32 || fin || waiting || bi < a.slot_blocks) {
+        // (1024-bin tiles: whole reads in slots)
+        if (TW == 32 || fin || bi < a.slot_blocks) {
           t0 = lds128(tp);
           t1 = lds128(tp + 16u);
         } else {
@@ -544,110 +536,303 @@ __global__ void __launch_bounds__(NT, 1) k_exhaustive(ExhArgs a) {
           t1 = __ldg(g + 1);
         }
         const uint32_t tw[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
-        if constexpr (NW == 1) add_block<P, 1>(c, tw, lane_base + kt * 4u, a);
-        else add_block<P, 4>(c, tw, lane_base, a);
+        add_block<P>(c, tw, lane_base, a);
       }
       tp += step;
       --left;
 
-      // a read ends when every bin of its tile is dead or its tokens are
-      // used up
+      // (3) a read ends when every bin of its tile is dead or its tokens are
+      //     used up
       const uint32_t all_dead = c.dead[0] & c.dead[1] & c.dead[2] & c.dead[3];
-      if constexpr (WS && TW == 32) {
-        // lockstep: one vote per block.  The warp takes new reads once every
-        // lane has no live bin or is past its read's last block (a group
-        // without a read has left = ~0).  A group whose read ended reads on
-        // through its token row's padding (never a miss), so its counters
-        // keep their values; a dead group may apply its remaining tokens
-        // (dead bins stay dead).
-        const bool ldead = all_dead == ~0u;
-        alive += ldead ? 0u : 1u;
-        if (!__all_sync(0xFFFFFFFFu, ldead || (int)left <= 0)) return false;
-        const bool gdead = (__ballot_sync(0xFFFFFFFFu, ldead) & gmask) == gmask;
-        // blocks the read needed: up to the one after which its last live
-        // lane died, or all of them
-        uint32_t m = alive;
-        m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 1));
-        m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 2));
-        m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, 4));
-        const uint32_t used = min(nblk, m + 1u);
-        const bool done = !fin;
-        if (done) {
-          executed += used;
-          if (NW == 1 && used > kTailAfter) tail_exec += used - kTailAfter;
-        }
-        alive = 0;
-        emit_and_switch(done, done && !gdead, Words<NW>{});
-        return true;
-      }
       const uint32_t bal = __ballot_sync(0xFFFFFFFFu, all_dead == ~0u);
       const bool gdead = (bal & gmask) == gmask;
-      bool done = !fin && !waiting && (gdead || left == 0);
-      if (WS && done) {
-        // freeze the group's counters (padding adds no misses) until the
-        // warp switches
-        executed += nblk - left;
-        if (NW == 1) tail_exec += nblk - left;
-        waiting = true;
-        tp = pad_tokens;
-        step = 0;
-      }
-      bool take_next;
-      if constexpr (!WS) {
-        take_next = __any_sync(0xFFFFFFFFu, done);
-      } else if constexpr (TW == 32) {
-        take_next = __all_sync(0xFFFFFFFFu, fin || waiting);
-      } else {
-        // sixteen groups: switch once enough of them wait, so that a few
-        // long reads do not hold the rest (the others keep their reads)
-        take_next = __popc(__ballot_sync(0xFFFFFFFFu, fin || waiting)) >= a.switch_lanes;
-      }
-      if (!take_next) return false;
-      if (WS) {
-        done = waiting;
-      } else if (done) {
-        executed += nblk - left;
-      }
-      emit_and_switch(done, done && !gdead, Words<NW>{});
-      return true;
-    };
-
-    while (active) {
-      if (run_block(Words<4>{})) {
-        bk = 0;
-        continue;
-      }
-      if constexpr (WS && TW == 32) {
-        if (++bk != kTailAfter) continue;
-        // one-word tail: once every lane of the warp has at most one word
-        // with a live bin (typically only near a read's true position), the
-        // warp applies the rest of the round's blocks to that word alone: a
-        // quarter of the logic ops, one 4-byte load per token.  Exact: a
-        // word dropped here has no live bin (or only bins past the table's
-        // end), and dead bins never pass.
-        uint32_t lm = 0;
-        if (!fin) {
-#pragma unroll
-          for (int w = 0; w < 4; ++w)
-            if (~c.dead[w] & vmask(w)) lm |= 1u << w;
-        }
-        if (__all_sync(0xFFFFFFFFu, (lm & (lm - 1u)) == 0u)) {
-          kt = lm ? (uint32_t)__ffs(lm) - 1u : 0u;
-          c.keep_one(kt, lm != 0u);
-          while (!run_block(Words<1>{})) {
-          }
-          bk = 0;
-        }
-      }
+      const bool done = !fin && (gdead || left == 0);
+      if (!__any_sync(0xFFFFFFFFu, done)) continue;
+      if (done) executed += nblk - left;
+      emit_and_switch(done, done && !gdead);
     }
     // one count per group (its lanes agree), one atomic per warp and item
     uint32_t ex = li == 0 ? executed : 0u;
     ex = __reduce_add_sync(0xFFFFFFFFu, ex);
-    if (lane == 0 && ex) atomicAdd(&a.ctl->blocks, (unsigned long long)ex);
-    if constexpr (WS && TW == 32) {
-      uint32_t tx = li == 0 ? tail_exec : 0u;
-      tx = __reduce_add_sync(0xFFFFFFFFu, tx);
-      if (lane == 0 && tx) atomicAdd(&a.ctl->tail_blocks, (unsigned long long)tx);
+    if (lane == 0 && ex) atomicAdd(&a.ctl->blocks, 2ull * ex);  // (counted in halves)
+  }
+}
+
+// The lockstep kernel: the lane groups of a warp (4 on 1024-bin tiles, 16 on
+// 256-bin tiles) take reads of similar length to go (ExhArgs::order) together,
+// run them for
+// as many tokens as the tokeniser expects a tile to need, gather what is still
+// live and finish that.
+//
+// * No end-of-read test until the check point (kMetaCheck*, the least of the
+//   reads): whole 16-token blocks, and a half block where it is odd.
+// * Then the warp counts the words (of its 128) that still hold a live bin.
+//   As long as more than 32 do, it applies half blocks to all of them; 32 or
+//   fewer are dealt out, one to a lane, through a scratch in shared memory
+//   (planes, and where the word came from), and only those get the rest of
+//   their reads' tokens: a quarter of the logic ops.  Exact: a word left
+//   behind has no live bin, and a dead bin can never pass.
+// * A read's last half blocks run into its row's padding (never a miss), so
+//   shorter reads of a warp hold their counters.
+// * Claims are a warp's: one shared atomic for its reads, two rounds ahead,
+//   so the order's index and then the token row (cp.async) arrive in time.
+template <int P, int TW, int NT>
+__global__ void __launch_bounds__(NT, 1) k_lockstep(ExhArgs a) {
+  constexpr uint32_t kRowBytes = TW * 4, kTileBinsT = TW * 32, GL = TW / 4, kGroups = 32 / GL;
+  constexpr int kPlanes = kScratchPlanes<TW>;
+  // [tile: (r4 + 2) rows x TW words][group slots][16 padding tokens][warp scratch]
+  extern __shared__ __align__(128) uint8_t smem[];
+  __shared__ uint32_t s_item, s_next;
+  const uint32_t tid = threadIdx.x, lane = tid & 31, grp = lane / GL, li = lane % GL;
+  const uint32_t nthreads = blockDim.x;
+  const uint32_t r4 = a.ix.r4;
+  if (*(volatile uint32_t*)&a.ctl->status) return;
+  if (gated_off(a.ctl, a.live)) return;
+  const uint32_t n_reads = live_reads(a.ctl, a.live, a.rv.n_reads);
+  if (n_reads == 0) return;
+  const Ranges rg = read_ranges(a, n_reads);
+
+  const uint32_t tile_bytes = (r4 + 2) * kRowBytes;
+  const uint32_t sh_base = (uint32_t)__cvta_generic_to_shared(smem);
+  const uint32_t slot = sh_base + tile_bytes + (tid / GL) * a.slot_bytes;
+  const uint32_t pad_tokens = sh_base + tile_bytes + (nthreads / GL) * a.slot_bytes;
+  const uint32_t scratch = pad_tokens + 32u + (tid >> 5) * kScratchBytes<TW>;
+  fill_special_rows<TW>(reinterpret_cast<uint32_t*>(smem), r4, pad_tokens, tid, nthreads);
+  const uint32_t lane_base = sh_base + li * 16u;
+  const uint32_t row_chunks = a.row_stride / 16u;
+  // 256-bin tiles: the token copy a group reads, and the halves its slot holds
+  // (a read's later tokens come from L2)
+  const uint32_t copies = TW == 32 ? 1u : a.rv.copies;
+  const uint32_t slot_halves = TW == 32 ? ~0u : 2u * a.slot_blocks;
+  auto token_row = [&](uint32_t r, uint32_t g) {
+    return a.rv.tokens + ((uint64_t)r * copies + (TW == 32 ? 0u : g % copies)) * a.rv.ts;
+  };
+
+  for (;;) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();  // previous item finished with the tile and the slots
+    if (tid == 0) {
+      s_item = atomicAdd(&a.ctl->item, 1u);
+      s_next = 0;
+    }
+    __syncthreads();
+    const uint32_t item = s_item;
+    if (item >= rg.n_items) break;
+    const uint32_t tile = rg.range_major ? item % a.n_tiles : item / rg.n_ranges;
+    const uint32_t range = rg.range_major ? item / a.n_tiles : item % rg.n_ranges;
+    const uint32_t r0 = range * rg.per;
+    const uint32_t nr = min(rg.per, n_reads - r0);
+    stage_tile<TW>(a, tile, sh_base, tid, nthreads);
+    // the last tile may be ragged: bins past the table's end start out dead
+    const bool ragged = (uint64_t)(tile + 1) * kTileBinsT > a.ix.num_bins;
+
+    auto claim = [&]() {
+      uint32_t k = 0;
+      if (lane == 0) k = atomicAdd(&s_next, kGroups);
+      k = __shfl_sync(0xFFFFFFFFu, k, 0) + grp;
+      return k >= nr ? kNone : a.order ? __ldg(a.order + r0 + k) : r0 + k;
+    };
+    auto fetch = [&](uint32_t r, uint32_t buf) {
+      uint32_t m = 0;
+      if (r != kNone) {
+        m = __ldg(a.rv.meta + r);
+        const char* src = reinterpret_cast<const char*>(token_row(r, grp));
+        for (uint32_t ch = li; ch < row_chunks; ch += GL)
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(
+                           slot + buf * a.row_stride + ch * 16u),
+                       "l"(src + ch * 16u));
+      }
+      asm volatile("cp.async.commit_group;");
+      return m;
+    };
+    uint32_t nxt = claim(), buf = 0;
+    uint32_t nxt_meta = fetch(nxt, 0);
+    uint32_t nxt2 = claim();
+    uint32_t ex = 0, tail_ex = 0, tail_words = 0;
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();  // tile staged
+
+    for (;;) {
+      const uint32_t cur = nxt, m = nxt_meta;
+      const bool have = cur != kNone;
+      if (!__any_sync(0xFFFFFFFFu, have)) break;
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncwarp();
+      uint32_t tp = have ? slot + buf * a.row_stride : pad_tokens;
+      const uint32_t step = have ? 16u : 0u;
+      buf ^= 1u;
+      nxt = nxt2;
+      nxt_meta = fetch(nxt, buf);
+      nxt2 = claim();
+
+      // 0 without a read; rotated copies spread a block's tokens over both halves
+      const uint32_t halves =
+          TW == 32 ? ((m & 0xFFu) + 7u) >> 3 : ((m & 0xFFu) + 15u) >> 4 << 1;
+      const uint32_t hmax = __reduce_max_sync(0xFFFFFFFFu, halves);
+      uint32_t h = __reduce_min_sync(0xFFFFFFFFu, have ? (m >> a.check_shift) & 31u : 31u);
+      h = min(h, hmax);
+      const uint32_t bias = (1u << P) - (((m >> 8) & 0xFFu) + 1u);
+      Counters<P> c;
+      c.init(bias);
+      if (!have || ragged) {
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+          const uint64_t b0 = (uint64_t)tile * kTileBinsT + (li * 4u + w) * 32u;
+          const uint64_t left = b0 < a.ix.num_bins ? a.ix.num_bins - b0 : 0;
+          c.dead[w] = !have ? ~0u : left >= 32 ? 0u : ~((1u << left) - 1u);
+        }
+      }
+      // eight tokens of the group's read: half block `at`
+      const uint4* far = reinterpret_cast<const uint4*>(token_row(have ? cur : 0u, grp));
+      const uint4 pads = make_uint4(a.pad_pair, a.pad_pair, a.pad_pair, a.pad_pair);
+      auto tokens_at = [&](uint32_t at, uint32_t near, const uint4* from, bool mine) {
+        if (TW == 32 || at < slot_halves) return lds128(near);
+        return mine ? __ldg(from + at) : pads;
+      };
+      for (uint32_t b = 0; b < h >> 1; ++b) {
+        const uint4 t0 = tokens_at(2 * b, tp, far, have);
+        const uint4 t1 = tokens_at(2 * b + 1, tp + 16u, far, have);
+        const uint32_t tw[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
+        tp += 2u * step;
+        add_block<P>(c, tw, lane_base, a);
+      }
+      if (h & 1u) {
+        const uint4 t0 = tokens_at(h - 1u, tp, far, have);
+        tp += step;
+        add_half<P, 4>(c, t0, lane_base, a);
+      }
+      // live words, until few enough to gather, none, or the tokens are used up
+      uint32_t live[4], n[4], total;
+      for (;;) {
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+          live[w] = __ballot_sync(0xFFFFFFFFu, c.dead[w] != ~0u);
+          n[w] = __popc(live[w]);
+        }
+        total = n[0] + n[1] + n[2] + n[3];
+        if (total <= 32u || h >= hmax) break;
+        const uint4 t0 = tokens_at(h, tp, far, have);
+        tp += step;
+        add_half<P, 4>(c, t0, lane_base, a);
+        ++h;
+      }
+      ex += min(h, halves);
+      if (total == 0) continue;
+
+      // passing bins of NW words: their records, at consecutive places
+      auto emit = [&](const uint32_t(&pm)[4], auto&& value, uint32_t read, uint32_t rm,
+                      uint32_t bin0, uint32_t bin_step) {
+        const uint32_t cnt = __popc(pm[0]) + __popc(pm[1]) + __popc(pm[2]) + __popc(pm[3]);
+        uint32_t incl = cnt;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+          if (lane >= (uint32_t)d) incl += t;
+        }
+        const uint32_t tot = __shfl_sync(0xFFFFFFFFu, incl, 31);
+        unsigned long long base = 0;
+        if (lane == 0 && tot) base = atomicAdd(&a.ctl->n_rec, (unsigned long long)tot);
+        base = __shfl_sync(0xFFFFFFFFu, base, 0);
+        if (base >= a.rec.cap) return;  // counted only
+        unsigned long long pos = base + incl - cnt;
+        const uint32_t ntok = rm & 0xFFu, bs = (1u << P) - (((rm >> 8) & 0xFFu) + 1u);
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+          uint32_t mask = pm[w];
+          while (mask) {
+            const uint32_t bit = __ffs(mask) - 1;
+            mask &= mask - 1;
+            if (pos < a.rec.cap) {
+              a.rec.keys[pos] = ((unsigned long long)read << a.bin_bits) |
+                                ((uint64_t)tile * kTileBinsT + bin0 + w * bin_step + bit);
+              a.rec.counts[pos] = (uint8_t)(ntok - (value(w, bit) - bs));
+            }
+            ++pos;
+          }
+        }
+      };
+      if (h >= hmax) {
+        const uint32_t pm[4] = {~c.dead[0], ~c.dead[1], ~c.dead[2], ~c.dead[3]};
+        emit(pm, [&](int w, uint32_t bit) { return c.value(w, bit); }, cur, m, li * 128u, 32u);
+        continue;
+      }
+
+      // gather: word w of this lane goes to lane at[w]
+      const uint32_t below = (1u << lane) - 1u;
+      uint32_t at[4], off = 0;
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        at[w] = off + __popc(live[w] & below);
+        off += n[w];
+      }
+      Counters<P, 1> g;
+      uint32_t info = 0;
+#pragma unroll
+      for (int p0 = 0; p0 <= P; p0 += kPlanes) {
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+          if (c.dead[w] != ~0u) {
+#pragma unroll
+            for (int p = p0; p < p0 + kPlanes && p <= P; ++p)
+              asm volatile("st.shared.u32 [%0], %1;" ::"r"(scratch + (p - p0) * 128u + at[w] * 4u),
+                           "r"(c.plane(p, w)));
+            if (p0 == 0)
+              asm volatile("st.shared.u8 [%0], %1;" ::"r"(scratch + kPlanes * 128u + at[w]),
+                           "r"(lane * 4u + w));
+          }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int p = p0; p < p0 + kPlanes && p <= P; ++p)
+          g.plane(p, 0) = lds32(scratch + (p - p0) * 128u + lane * 4u);
+        if (p0 == 0)
+          asm volatile("ld.shared.u8 %0, [%1];" : "=r"(info) : "r"(scratch + kPlanes * 128u + lane));
+        __syncwarp();
+      }
+      const bool on = lane < total;
+      const uint32_t src = on ? info >> 2 : lane;  // the lane whose read and bins these are
+      const uint32_t bin0 = (src % GL) * 128u + (info & 3u) * 32u;
+      if (!on) g.dead[0] = ~0u;
+      uint32_t gtp = __shfl_sync(0xFFFFFFFFu, tp, src);
+      const uint32_t gstep = __shfl_sync(0xFFFFFFFFu, step, src);
+      const uint32_t gbase = sh_base + (on ? bin0 >> 3 : 0u);
+      {  // reads with a word left
+        const uint32_t any = live[0] | live[1] | live[2] | live[3];
+        if (TW == 32)
+          off = ((any & 0xFFu) != 0) + ((any & 0xFF00u) != 0) + ((any & 0xFF0000u) != 0) +
+                ((any & 0xFF000000u) != 0);
+        else
+          off = __popc((any | any >> 1) & 0x55555555u);
+      }
+      const uint4* gfar = far;
+      if (TW != 32) {
+        const uint32_t read = __shfl_sync(0xFFFFFFFFu, cur, src);
+        gfar = reinterpret_cast<const uint4*>(token_row(on ? read : 0u, src / GL));
+      }
+      do {
+        tail_words += g.dead[0] != ~0u;
+        tail_ex += off;
+        const uint4 t0 = tokens_at(h, gtp, gfar, on);
+        gtp += gstep;
+        add_half<P, 1>(g, t0, gbase, a);
+        ++h;
+      } while (h < hmax && __any_sync(0xFFFFFFFFu, g.dead[0] != ~0u));
+      if (__any_sync(0xFFFFFFFFu, g.dead[0] != ~0u)) {
+        const uint32_t pm[4] = {~g.dead[0], 0u, 0u, 0u};
+        const uint32_t read = __shfl_sync(0xFFFFFFFFu, cur, src);
+        const uint32_t rm = __shfl_sync(0xFFFFFFFFu, m, src);
+        emit(pm, [&](int, uint32_t bit) { return g.value(0, bit); }, read, rm, bin0, 0u);
+      }
+    }
+    // one count per group (its lanes agree), one atomic per warp and item
+    ex = __reduce_add_sync(0xFFFFFFFFu, li == 0 ? ex : 0u);
+    tail_words = __reduce_add_sync(0xFFFFFFFFu, tail_words);
+    if (lane == 0) {
+      atomicAdd(&a.ctl->blocks, (unsigned long long)ex);
+      if (tail_ex) {
+        atomicAdd(&a.ctl->tail_blocks, (unsigned long long)tail_ex);
+        atomicAdd(&a.ctl->tail_words, (unsigned long long)tail_words);
+      }
     }
   }
 }
@@ -720,7 +905,7 @@ __global__ void __launch_bounds__(kFewThreads, 2) k_exhaustive_few(ExhArgs a) {
     used = max(used, __shfl_xor_sync(0xFFFFFFFFu, used, 4));
     used = (lane & 7u) == 0 && on ? min(nblk, used + 1u) : 0u;
     used = __reduce_add_sync(0xFFFFFFFFu, used);
-    if (lane == 0) atomicAdd(&a.ctl->blocks, (unsigned long long)used);
+    if (lane == 0) atomicAdd(&a.ctl->blocks, 2ull * used);  // (counted in halves)
     if (__all_sync(0xFFFFFFFFu, ldead)) continue;
     uint32_t pm[4], cnt = 0;
 #pragma unroll
@@ -758,30 +943,31 @@ __global__ void __launch_bounds__(kFewThreads, 2) k_exhaustive_few(ExhArgs a) {
   }
 }
 
-template <int P, int TW, int NT, bool WS>
-void launch_p(const ExhArgs& a, size_t smem, uint32_t threads, uint32_t grid, cudaStream_t st,
-              const char* name) {
-  cudaFuncSetAttribute(k_exhaustive<P, TW, NT, WS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)smem);
+template <typename Kernel>
+void launch_k(Kernel kernel, const ExhArgs& a, size_t smem, uint32_t threads, uint32_t grid,
+              cudaStream_t st, const char* name) {
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   ProfScope ps(name, st);
-  k_exhaustive<P, TW, NT, WS><<<grid, threads, smem, st>>>(a);
+  kernel<<<grid, threads, smem, st>>>(a);
 }
 
-template <int TW, int NT, bool WS>
-void launch_ws(const ExhArgs& a, size_t smem, uint32_t threads, uint32_t grid, uint32_t max_d,
-               cudaStream_t st, const char* name) {
-  // the counters need 2^P > D' (D' <= 255)
-  if (max_d < 32) launch_p<5, TW, NT, WS>(a, smem, threads, grid, st, name);
-  else if (max_d < 64) launch_p<6, TW, NT, WS>(a, smem, threads, grid, st, name);
-  else if (max_d < 128) launch_p<7, TW, NT, WS>(a, smem, threads, grid, st, name);
-  else launch_p<8, TW, NT, WS>(a, smem, threads, grid, st, name);
-}
-
+// the counters need 2^P > D' (D' <= 255)
 template <int TW, int NT>
 void launch_nt(const ExhArgs& a, size_t smem, uint32_t threads, uint32_t grid, uint32_t max_d,
-               bool warp_switch, cudaStream_t st, const char* name) {
-  if (warp_switch) launch_ws<TW, NT, true>(a, smem, threads, grid, max_d, st, name);
-  else launch_ws<TW, NT, false>(a, smem, threads, grid, max_d, st, name);
+               bool lockstep, cudaStream_t st, const char* name) {
+  auto run = [&](auto kernel) { launch_k(kernel, a, smem, threads, grid, st, name); };
+  const int p = max_d < 32 ? 5 : max_d < 64 ? 6 : max_d < 128 ? 7 : 8;
+  if (lockstep) {
+    if (p == 5) run(k_lockstep<5, TW, NT>);
+    else if (p == 6) run(k_lockstep<6, TW, NT>);
+    else if (p == 7) run(k_lockstep<7, TW, NT>);
+    else run(k_lockstep<8, TW, NT>);
+    return;
+  }
+  if (p == 5) run(k_exhaustive<5, TW, NT>);
+  else if (p == 6) run(k_exhaustive<6, TW, NT>);
+  else if (p == 7) run(k_exhaustive<7, TW, NT>);
+  else run(k_exhaustive<8, TW, NT>);
 }
 
 template <int TW>
@@ -795,9 +981,12 @@ void launch_tw(ExhArgs& a, const IndexView& ix, uint32_t max_d, uint32_t sms, ui
   // shared memory
   const size_t tile_bytes = (size_t)(ix.r4 + 2) * kRowBytes;
   uint32_t threads = nt;
-  while (threads > 64 && tile_bytes + (size_t)(threads / GL) * a.slot_bytes + 32 > kSmemLimit)
-    threads -= 32;
-  const size_t smem = tile_bytes + (size_t)(threads / GL) * a.slot_bytes + 32;
+  const size_t scratch = warp_switch ? kScratchBytes<TW> : 0;  // per warp
+  auto smem_of = [&](uint32_t t) {
+    return tile_bytes + (size_t)(t / GL) * a.slot_bytes + 32 + t / 32 * scratch;
+  };
+  while (threads > 64 && smem_of(threads) > kSmemLimit) threads -= 32;
+  const size_t smem = smem_of(threads);
   // small batches on few tiles need fewer CTAs (graph launches size for the
   // largest batch and let surplus CTAs find no work)
   uint32_t grid = sms;
@@ -834,9 +1023,10 @@ uint32_t exhaustive_few_reads(const IndexView& ix, uint32_t ts) {
 }
 
 void launch_exhaustive(const IndexView& ix, const ReadsView& rv, RecordsView rec, uint32_t bin_bits,
-                       uint32_t max_d, Ctl* ctl, cudaStream_t st, const char* prof_name,
+                       uint32_t max_d, Ctl* ctl, cudaStream_t st, bool fine, const uint32_t* order,
                        Live live, ExhShape shape) {
   if (rv.n_reads == 0) return;
+  const char* prof_name = fine ? "exhaustive" : "exhaustive_coarse";
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -867,14 +1057,14 @@ void launch_exhaustive(const IndexView& ix, const ReadsView& rv, RecordsView rec
     const uint32_t groups = nt / 2u;  // 2-lane groups
     a.slot_blocks = 1;
     for (uint32_t sb = min(blocks, kSlotBlocksNarrow); sb > 1; --sb)
-      if (tile_bytes + (size_t)groups * slot_bytes_of(sb) + 32 <= kSmemLimit) {
+      if (tile_bytes + (size_t)groups * slot_bytes_of(sb) + 32 + nt / 32 * kScratchBytes<8> <=
+          kSmemLimit) {
         a.slot_blocks = sb;
         break;
       }
   }
   a.row_stride = a.slot_blocks * kBlockTokens * 2u;
   a.slot_bytes = slot_bytes_of(a.slot_blocks);
-  a.switch_lanes = kSwitchGroupsNarrow * 2u;
   a.c_hi = 65536u;
   a.c_lo = 0u - 65536u;
   a.range_bytes = shape.range_kb ? (uint64_t)shape.range_kb << 10 : kDefaultRangeBytes;
@@ -896,6 +1086,9 @@ void launch_exhaustive(const IndexView& ix, const ReadsView& rv, RecordsView rec
     }
     if (!live.on || rv.n_reads <= a.few_reads) return;
   }
+  a.order = order;
+  a.pad_pair = rowPad(ix.r4) | (rowPad(ix.r4) << 16);
+  a.check_shift = fine ? kMetaCheckFine : kMetaCheckCoarse;
   const bool ws = shape.read_switch == GRIM_SWITCH_WARP;
   if (ix.r4 <= 1024) launch_tw<32>(a, ix, max_d, (uint32_t)sms, nt, ws, st, prof_name);
   else launch_tw<8>(a, ix, max_d, (uint32_t)sms, nt, ws, st, prof_name);

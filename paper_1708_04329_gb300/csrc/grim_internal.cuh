@@ -24,7 +24,9 @@ struct Ctl {
   unsigned long long n_rec;   // passing records found (may exceed cap)
   uint32_t status;            // kStatus* bits
   uint32_t item;              // work-item counter of the persistent filter kernels
-  unsigned long long blocks;  // 16-token blocks applied to (super-)bin tiles (all-bins mode)
+  // all-bins mode, in 8-token halves of a block applied for a read: to whole
+  // (super-)bin tiles, and (tail_*) after a read's live words were gathered
+  unsigned long long blocks;
   uint32_t max_d;             // largest miss budget D' = min(q*e, L-q+1) of the batch
   uint32_t max_tight;         // 255 - the smallest slack (L-q+1) - D' of the batch
   // graph launches (grim_plan): the batch's counts and the path taken live
@@ -37,10 +39,11 @@ struct Ctl {
   unsigned long long n_final;      // passing records (of the survivors' check; plans: of the batch)
   uint32_t blk_max;                // most 16-token blocks of a read in the batch
   uint32_t blk_lo;                 // 32 - the fewest 16-token blocks of a read
-  unsigned long long tail_blocks;  // of `blocks`: applied to one word per lane (256 bins)
+  unsigned long long tail_blocks;  // halves applied to a read's gathered words only
   uint32_t d_lo;                   // 255 - the smallest miss budget D' of the batch
   uint32_t route;                  // the batch's path, whichever kernel sweeps it
-  uint32_t pad[40];
+  unsigned long long tail_words;   // the words (32 bins) those halves were applied to
+  uint32_t pad[38];
 };
 static_assert(sizeof(Ctl) == 256, "Ctl is one 256-byte slot");
 static_assert(offsetof(Ctl, live_reads) == 32, "live counts follow the per-pass counters");
@@ -94,11 +97,23 @@ struct IndexView {
   // that the all-bins kernels apply the rarest tokens first and every bin of a
   // tile fails as early as possible
   const uint16_t* rank;
+  const float* miss;  // [r4] share of the (super-)bins without each token, beside rank
 };
 
 // Reads after tokenising: token j of read r (copy k) at
 // tokens[(r * copies + k) * ts + j], meta[r] = ntok | D' << 8 where
-// D' = min(q*e, ntok) is the number of misses a passing bin may have.
+// D' = min(q*e, ntok) is the number of misses a passing bin may have.  In the
+// all-bins orders two further fields, kMetaCheckCoarse and kMetaCheckFine, hold the number of 8-token halves after which few bins of a
+// tile are expected to be live, on the coarse and on the fine table.
+constexpr uint32_t kMetaCheckCoarse = 16, kMetaCheckFine = 21;  // shifts of 5-bit fields
+// The order in which the lockstep kernel takes a batch's reads: by that check
+// point (kMetaOrder, in steps of 4 tokens), longest first, as given within a
+// key.  In device memory: the reads, then the reads of each key in every block
+// of kOrderBlock.
+constexpr uint32_t kMetaOrder = 26, kOrderKeys = 64, kOrderBlock = 1024;
+constexpr uint64_t order_bytes(uint64_t n_reads) {
+  return (n_reads + (n_reads + kOrderBlock - 1) / kOrderBlock * kOrderKeys) * sizeof(uint32_t);
+}
 struct ReadsView {
   const uint16_t* tokens;  // read r, copy k: tokens + (r * copies + k) * ts
   const uint32_t* meta;
@@ -132,10 +147,18 @@ void launch_build_token_major(const uint32_t* codes, const uint32_t* invalid, co
 // bin-major table bm [units * f][wpb]; q >= 5
 void launch_tm_from_bm(const uint32_t* bm, const IndexView& unit_view, uint32_t wpb, uint32_t f,
                        uint32_t* tm, cudaStream_t st);
-// presence[t] = popcount of row t of a token-major table, and the tokens'
-// ranks by it (IndexView::rank)
-void launch_presence(const uint32_t* tm, uint32_t rows, uint64_t words_per_row, uint32_t* presence,
-                     uint16_t* rank, cudaStream_t st);
+// presence[t] = popcount of row t of a token-major table over `units`, and the
+// tokens' ranks and miss shares by it (IndexView::rank, miss)
+void launch_presence(const uint32_t* tm, const IndexView& units, uint32_t* presence,
+                     cudaStream_t st);
+// the tables behind the 4^q presence counts, in one allocation
+constexpr uint32_t kPresenceBytes = sizeof(uint32_t) + sizeof(uint16_t) + sizeof(float);
+inline uint16_t* rank_table(uint32_t* presence, uint32_t r4) {
+  return presence ? reinterpret_cast<uint16_t*>(presence + r4) : nullptr;
+}
+inline float* miss_table(uint32_t* presence, uint32_t r4) {
+  return presence ? reinterpret_cast<float*>(rank_table(presence, r4) + r4) : nullptr;
+}
 
 void launch_reverse_complement(const char* reads, const uint64_t* offsets, const uint32_t* lens,
                                uint32_t n_reads, char* out, cudaStream_t st);
@@ -154,9 +177,12 @@ enum class TokenOrder : uint32_t {
 // batch's extremes of D', slack and 16-token blocks in the control block.
 void launch_tokenise(const char* reads, const uint64_t* offsets, const uint32_t* lens,
                      const uint16_t* e, const IndexView& ix, ReadsView rv, uint16_t* tokens,
-                     uint32_t* meta, Ctl* ctl, cudaStream_t st, bool cand_mode,
+                     uint32_t* meta, Ctl* ctl, cudaStream_t st, bool cand_mode, float fine_power,
                      Live live = {false, 0}, uint32_t max_e = 0xFFFFu,
                      uint64_t max_bases = ~0ull);
+// the reads' order from the keys the tokeniser left in meta
+void launch_order(const ReadsView& rv, uint32_t* order, const Ctl* ctl, cudaStream_t st,
+                  Live live = {false, 0});
 // CSR offsets of the caller's lists: non-decreasing, ending at n_cand
 // (kStatusBadCsr otherwise); the ids themselves are checked by the
 // candidate kernel
@@ -184,11 +210,12 @@ struct ExhShape {
 uint32_t exhaustive_few_reads(const IndexView& ix, uint32_t ts);
 // the launch shape's threads, range and read switch are ones the kernel builds
 bool exhaustive_shape_ok(const ExhShape& s);
-// max_d: the batch's largest miss budget (sizes the bit-sliced counters)
+// max_d: the batch's largest miss budget (sizes the bit-sliced counters).
+// fine: the bins' table, not the super-bins'.  order: the reads in the order
+// in which warps should take them, or null
 void launch_exhaustive(const IndexView& ix, const ReadsView& rv, RecordsView rec, uint32_t bin_bits,
-                       uint32_t max_d, Ctl* ctl, cudaStream_t st,
-                       const char* prof_name = "exhaustive", Live live = {false, 0},
-                       ExhShape shape = {0, 0, 0, 0});
+                       uint32_t max_d, Ctl* ctl, cudaStream_t st, bool fine, const uint32_t* order,
+                       Live live, ExhShape shape);
 // unroll: candidate gathers in flight per lane group (1, 2, 4 or 8; 0 =
 // default).  An id outside [0, num_bins) sets kStatusBadCand.
 void launch_candidates(const IndexView& ix, const ReadsView& rv, const int32_t* cand,
@@ -271,6 +298,19 @@ inline uint64_t record_capacity(uint32_t n_reads, uint64_t cap, uint32_t coarse_
   return s > cap ? s : cap;
 }
 
+// Where a call's read order goes, or null: the spare words of
+// a two-level workspace, else the record buffer that the one exact pass does
+// not write (`idle`), if it is large enough.
+constexpr uint32_t kOrderMinReads = 256;
+constexpr uint32_t kOrderUniform = 32768;  // reads of one length and budget worth ordering
+inline uint32_t* order_room(const IndexView& v, char* ws, const Layout& L, uint32_t n_reads,
+                            uint64_t rcap, uint32_t coarse_factor, const RecordsView& idle) {
+  if (n_reads < kOrderMinReads) return nullptr;
+  if (coarse_factor) return reinterpret_cast<uint32_t*>(ws + L.spare);
+  if (rcap * sizeof(unsigned long long) < order_bytes(n_reads)) return nullptr;
+  return reinterpret_cast<uint32_t*>(idle.keys);
+}
+
 // coarse_factor > 0: room for the coarse pass's survivors, and per survivor
 // the coarse_factor words that grim_filter_workspace_size has always counted
 // Token copies per read: the all-bins kernel's 256-bin tiles (q = 6) read
@@ -329,7 +369,7 @@ struct grim_index {
   uint32_t* tm;
   uint32_t* bm;
   uint32_t* ctm;
-  uint32_t* presence;  // [4^q], followed by the ranks (uint16 [4^q])
+  uint32_t* presence;  // [4^q], followed by the ranks and miss shares (rank_table, miss_table)
   // the allocator the tables came from (grim_set_allocator), or null for
   // cudaMalloc / cudaFree
   grim_free_fn free_fn;
@@ -344,9 +384,13 @@ int index_alloc(uint64_t len, uint32_t B, uint32_t q, uint32_t max_read_len, uin
 // Keep the CUDA error string for grim_last_cuda_error; the matching status.
 int record_cuda_error(cudaError_t e);
 
-// the ranks of IndexView::rank, behind the presence counts (null without them)
-inline uint16_t* index_rank(const grim_index* idx) {
-  return idx->presence ? reinterpret_cast<uint16_t*>(idx->presence + idx->v.r4) : nullptr;
+// IndexView::miss is of the coarse table when there is one: a fine bin misses a
+// token about this power of that as often (q-grams of a window, as in a random
+// sequence); 1 without a coarse table
+inline float fine_miss_power(const grim_index* idx) {
+  if (!(idx->layouts & GRIM_LAYOUT_COARSE)) return 1.f;
+  const float rest = (float)idx->v.ext - (float)idx->v.q + 1.f;
+  return ((float)idx->v.B + rest) / ((float)idx->cv.B + rest);
 }
 
 // the all-bins filter can run coarse-then-exact when the index has both the

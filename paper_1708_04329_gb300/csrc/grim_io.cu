@@ -238,10 +238,8 @@ int grim_load(const char* path, uint32_t layouts, uint32_t flags, grim_index** o
     return GRIM_E_FORMAT;
   }
   // presence counts from the table the all-bins filter sweeps first, as in a build
-  if (ix->ctm)
-    launch_presence(ix->ctm, ix->cv.r4, ix->cv.wpad, ix->presence, index_rank(ix), sg.st);
-  else if (ix->tm)
-    launch_presence(ix->tm, ix->v.r4, ix->v.wpad, ix->presence, index_rank(ix), sg.st);
+  if (ix->ctm) launch_presence(ix->ctm, ix->cv, ix->presence, sg.st);
+  else if (ix->tm) launch_presence(ix->tm, ix->v, ix->presence, sg.st);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(sg.st);
   prof_collect();

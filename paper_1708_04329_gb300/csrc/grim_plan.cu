@@ -147,6 +147,15 @@ int capture(grim_plan* p) {
   if (max_d > ntok_max) max_d = ntok_max;
   const Live live{true, 0};
 
+  // all bins: with a coarse pass both paths leave their records in rb (the
+  // survivors are in ra while their members are checked), else in ra
+  const RecordsView dst = p->f ? rb : ra, tmp = p->f ? ra : rb;
+  uint32_t* order = p->cand_mode || idx->shape.read_switch
+                        ? nullptr
+                        : order_room(v, ws, L, d.max_reads, rcap, p->f, tmp);
+  ExhShape shape = idx->shape;
+  if (order) shape.read_switch = GRIM_SWITCH_WARP;
+
   prof_suspend(true);
   cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) {
@@ -159,7 +168,7 @@ int capture(grim_plan* p) {
   if (p->hio) k_copy_in<<<dim3(64, kCopySegs), 256, 0, st>>>(p->copy, p->ctl);
   launch_tokenise(B.reads, B.offsets, B.lens, B.e, v, rv,
                   reinterpret_cast<uint16_t*>(ws + L.tok), reinterpret_cast<uint32_t*>(ws + L.meta),
-                  p->ctl, st, p->cand_mode, live, d.max_e, d.max_bases);
+                  p->ctl, st, p->cand_mode, fine_miss_power(idx), live, d.max_e, d.max_bases);
   if (p->cand_mode) {
     launch_check_candidates(B.cand_off, d.max_reads, d.max_cand, p->ctl, st, live);
     launch_candidates(v, rv, B.cand, B.cand_off, ra, p->ctl, st, live, d.cand_unroll);
@@ -176,23 +185,22 @@ int capture(grim_plan* p) {
                                     few_coarse, few_exact);
     const uint32_t cbits =
         idx->cv.num_bins > 1 ? bit_length(idx->cv.num_bins - 1) : 0;
-    // both paths leave their records in rb: the coarse pass's survivors are
-    // in ra while their members are checked
+    launch_order(rv, order, p->ctl, st, live);
     if (p->f) {
       const Live coarse{true, kPathCoarse};
-      launch_exhaustive(idx->cv, rv, ra, cbits, max_d, p->ctl, st, "exhaustive_coarse", coarse,
-                        idx->shape);
+      launch_exhaustive(idx->cv, rv, ra, cbits, max_d, p->ctl, st, false, order, coarse,
+                        shape);
       k_plan_control<<<1, 1, 0, st>>>(p->ctl, kCtlAfterCoarse, 1, has_exact, rcap, 0, few_coarse,
                                       few_exact);
-      launch_refine(v, rv, ra.keys, &p->ctl->n_surv, rcap, cbits, p->f, rb, bin_bits, p->ctl, st,
+      launch_refine(v, rv, ra.keys, &p->ctl->n_surv, rcap, cbits, p->f, dst, bin_bits, p->ctl, st,
                     coarse);
     }
     if (has_exact) {
       const Live exact{true, kPathExact};
-      launch_exhaustive(v, rv, rb, bin_bits, max_d, p->ctl, st, "exhaustive", exact, idx->shape);
+      launch_exhaustive(v, rv, dst, bin_bits, max_d, p->ctl, st, true, order, exact, shape);
     }
     k_plan_control<<<1, 1, 0, st>>>(p->ctl, kCtlFinal, 0, 0, 0, 0, 0, 0);
-    sort_and_emit(rb, ra, d.cap, bin_bits + read_bits, ws + L.hist, false, bin_bits, nullptr,
+    sort_and_emit(dst, tmp, d.cap, bin_bits + read_bits, ws + L.hist, false, bin_bits, nullptr,
                   nullptr, d.max_reads, B.out_read, B.out_bin, B.out_count, st, &p->ctl->n_final,
                   &p->ctl->live_reads);
   }

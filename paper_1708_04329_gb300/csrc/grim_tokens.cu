@@ -10,6 +10,14 @@ constexpr int kTokWarps = 8;
 constexpr uint32_t kMaxStride = 256;  // token stride: <= 255 tokens rounded up to 16
 constexpr int kTokRounds = 8;         // tokens per lane
 constexpr int kTokCtasPerSm = 5;      // of the persistent grid
+// A bin is out once it misses more than D' tokens.  After j tokens the misses
+// of a random bin are about normal with mean S_j, the sum of the tokens' miss
+// shares, and variance S_j (j - S_j) / j; the check comes at the first j whose
+// mean is kCheckZ deviations past D'.
+// (3 / 4 / 5 / 6 deviations: 250k reads of 100 bp, coarse table 602 / 599 / 610
+// / 695 ms, 40k on the fine table 163 / 159 / 155 / 155, 40k mixed reads 89.6 /
+// 89.2 / 90.5 / 101.8, 60k of 150 bp at q = 6 57.6 / 56.8 / 57.3 / 63.9.)
+constexpr float kCheckZ = 4.0f;
 
 struct TokArgs {
   const char* reads;
@@ -18,6 +26,8 @@ struct TokArgs {
   const uint16_t* e;
   uint32_t n_reads, q, max_read_len, r4, ts, copies;
   const uint16_t* rank;  // IndexView::rank
+  const float* miss;     // IndexView::miss
+  float fine_power;      // fine_miss_power
   uint16_t* tokens;
   uint32_t* meta;
   Ctl* ctl;
@@ -43,6 +53,10 @@ struct TokArgs {
 // holding them, so that the all-bins kernels see misses as early as possible,
 // then the repeats of a value already seen (a repeat misses exactly the bins
 // its first occurrence misses; 1024-bin tiles: 1.7% fewer bit tests at q = 5).
+// meta also gets the place in that order where a tile's bins are expected to
+// be out but for a few (kCheckZ below): over 240 reads the number of tokens a
+// tile really takes follows it with a correlation of 0.96 (reads of one length
+// and budget) and 0.999 (mixed ones).
 // The order is a counting sort without counters: every distinct token sets
 // the bit of its rank in a bitmap of 4^q bits, and its place is the number of
 // bits below.
@@ -271,7 +285,38 @@ __global__ void __launch_bounds__(kTokWarps * 32, kTokCtasPerSm) k_tokenise(TokA
     }
     uint32_t d = q * budget;
     if (d > ntok) d = ntok;
-    if (lane == 0) a.meta[r] = ntok | (d << 8);
+    uint32_t meta = ntok | (d << 8);
+    if constexpr (kRanked) {
+      // (s_seq is complete: it was copied out above)
+      const float over = (float)(d + 1u);
+      float sum[2] = {0.f, 0.f};
+      uint32_t at[2] = {0, 0};  // 1 + the check's place, coarse and fine
+      const bool both = a.fine_power != 1.f;
+      for (uint32_t j0 = 0; j0 < ntok && !(at[0] && at[1]); j0 += 32) {
+        const uint32_t t = s_seq[warp][j0 + lane];
+        const float miss = t < r4 ? a.miss[t] : t == rowInvalid(r4) ? 1.f : 0.f;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          if (k == 1 && !both) break;
+          float incl = k == 0 ? miss : __powf(miss, a.fine_power);
+#pragma unroll
+          for (int dd = 1; dd < 32; dd <<= 1) {
+            const float up = __shfl_up_sync(0xFFFFFFFFu, incl, dd);
+            if (lane >= (uint32_t)dd) incl += up;
+          }
+          const float s = sum[k] + incl, n = (float)(j0 + lane + 1u), x = s - over;
+          const bool ok = j0 + lane < ntok && x > 0.f && x * x * n >= kCheckZ * kCheckZ * s * (n - s);
+          const uint32_t hit = __ballot_sync(0xFFFFFFFFu, ok);
+          if (hit && !at[k]) at[k] = j0 + __ffs(hit);
+          sum[k] += __shfl_sync(0xFFFFFFFFu, incl, 31);
+        }
+        if (!both) at[1] = at[0];
+      }
+      meta |= ((at[0] ? at[0] : ntok) >> 3) << kMetaCheckCoarse;
+      meta |= ((at[1] ? at[1] : ntok) >> 3) << kMetaCheckFine;
+      meta |= ((at[0] ? at[0] : ntok) >> 2) << kMetaOrder;
+    }
+    if (lane == 0) a.meta[r] = meta;
     const uint32_t nblk = (ntok + kBlockTokens - 1) / kBlockTokens;
     max_d = max(max_d, d);
     d_lo = max(d_lo, 255u - d);
@@ -290,6 +335,64 @@ __global__ void __launch_bounds__(kTokWarps * 32, kTokCtasPerSm) k_tokenise(TokA
     raise(&ctl->max_tight, max_tight);
     raise(&ctl->blk_max, blk_max);
     raise(&ctl->blk_lo, blk_lo);
+  }
+}
+
+// Reads by descending order key, as given within a key (so that a batch is
+// always grouped the same way): the keys of every block of reads are counted,
+// then each block finds its places from the counts before it.
+__global__ void __launch_bounds__(kOrderBlock) k_order_count(const uint32_t* __restrict__ meta,
+                                                             uint32_t n_reads, uint32_t most,
+                                                             uint32_t* __restrict__ order,
+                                                             const Ctl* ctl, Live live) {
+  __shared__ uint32_t s_n[kOrderKeys];
+  if (ctl->status) return;
+  n_reads = live_reads(ctl, live, n_reads);
+  const uint32_t t = threadIdx.x, r = blockIdx.x * kOrderBlock + t;
+  if (blockIdx.x * kOrderBlock >= n_reads) return;
+  if (t < kOrderKeys) s_n[t] = 0;
+  __syncthreads();
+  if (r < n_reads) atomicAdd(&s_n[meta[r] >> kMetaOrder], 1u);
+  __syncthreads();
+  if (t < kOrderKeys) order[most + blockIdx.x * kOrderKeys + t] = s_n[t];
+}
+
+__global__ void __launch_bounds__(kOrderBlock) k_order_place(const uint32_t* __restrict__ meta,
+                                                             uint32_t n_reads, uint32_t most,
+                                                             uint32_t* __restrict__ order,
+                                                             const Ctl* ctl, Live live) {
+  constexpr uint32_t kWarps = kOrderBlock / 32;
+  __shared__ uint32_t s_all[kOrderKeys], s_before[kOrderKeys];  // reads of a key; in earlier blocks
+  __shared__ uint32_t s_warp[kWarps][kOrderKeys];
+  if (ctl->status) return;
+  n_reads = live_reads(ctl, live, n_reads);
+  if (blockIdx.x * kOrderBlock >= n_reads) return;
+  const uint32_t t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const uint32_t r = blockIdx.x * kOrderBlock + t;
+  const uint32_t blocks = (n_reads + kOrderBlock - 1) / kOrderBlock;
+  if (t < kOrderKeys) s_all[t] = s_before[t] = 0;
+  for (uint32_t i = t; i < kWarps * kOrderKeys; i += kOrderBlock) (&s_warp[0][0])[i] = 0;
+  __syncthreads();
+  {
+    uint32_t all = 0, before = 0;
+    for (uint32_t b = t / kOrderKeys; b < blocks; b += kOrderBlock / kOrderKeys) {
+      const uint32_t n = order[most + b * kOrderKeys + t % kOrderKeys];
+      all += n;
+      if (b < blockIdx.x) before += n;
+    }
+    atomicAdd(&s_all[t % kOrderKeys], all);
+    atomicAdd(&s_before[t % kOrderKeys], before);
+  }
+  const uint32_t key = r < n_reads ? meta[r] >> kMetaOrder : kOrderKeys;
+  const uint32_t same = __match_any_sync(0xFFFFFFFFu, key);
+  const uint32_t rank = __popc(same & ((1u << lane) - 1u));
+  if (r < n_reads && rank == 0) s_warp[warp][key] = __popc(same);
+  __syncthreads();
+  if (r < n_reads) {
+    uint32_t at = s_before[key] + rank;
+    for (uint32_t k = key + 1; k < kOrderKeys; ++k) at += s_all[k];  // longer reads come first
+    for (uint32_t w = 0; w < warp; ++w) at += s_warp[w][key];
+    order[at] = r;
   }
 }
 
@@ -339,8 +442,8 @@ void launch_reverse_complement(const char* reads, const uint64_t* offsets, const
 
 void launch_tokenise(const char* reads, const uint64_t* offsets, const uint32_t* lens,
                      const uint16_t* e, const IndexView& ix, ReadsView rv, uint16_t* tokens,
-                     uint32_t* meta, Ctl* ctl, cudaStream_t st, bool cand_mode, Live live,
-                     uint32_t max_e, uint64_t max_bases) {
+                     uint32_t* meta, Ctl* ctl, cudaStream_t st, bool cand_mode,
+                     float fine_power, Live live, uint32_t max_e, uint64_t max_bases) {
   if (rv.n_reads == 0) return;
   const uint32_t threads = kTokWarps * 32;
   int dev = 0, sms = 0;
@@ -350,7 +453,7 @@ void launch_tokenise(const char* reads, const uint64_t* offsets, const uint32_t*
   const uint64_t most = (uint64_t)(sms > 0 ? sms : 1) * kTokCtasPerSm;
   const uint64_t grid = need < most ? need : most;
   const TokArgs a{reads, offsets, lens,   e,    rv.n_reads, ix.q, ix.max_read_len, ix.r4,    rv.ts,
-                  rv.copies, ix.rank, tokens, meta, ctl,        live, max_e,           max_bases};
+                  rv.copies, ix.rank, ix.miss, fine_power, tokens, meta, ctl, live, max_e, max_bases};
   // lists read whole token rows in any order up to 128-byte vectors; larger
   // ones (q = 6) are looked up line by line
   auto kernel = cand_mode       ? (ix.wpb > 32 ? k_tokenise<TokenOrder::kLines>
@@ -359,6 +462,15 @@ void launch_tokenise(const char* reads, const uint64_t* offsets, const uint32_t*
                                 : k_tokenise<TokenOrder::kRarest>;
   ProfScope ps("tokenise", st);
   kernel<<<(unsigned)grid, threads, 0, st>>>(a);
+}
+
+void launch_order(const ReadsView& rv, uint32_t* order, const Ctl* ctl, cudaStream_t st,
+                  Live live) {
+  if (!order) return;
+  const uint32_t grid = (rv.n_reads + kOrderBlock - 1) / kOrderBlock;
+  ProfScope ps("order", st);
+  k_order_count<<<grid, kOrderBlock, 0, st>>>(rv.meta, rv.n_reads, rv.n_reads, order, ctl, live);
+  k_order_place<<<grid, kOrderBlock, 0, st>>>(rv.meta, rv.n_reads, rv.n_reads, order, ctl, live);
 }
 
 void launch_check_candidates(const uint64_t* cand_off, uint32_t n_reads, uint64_t n_cand, Ctl* ctl,

@@ -729,3 +729,36 @@ def test_few_reads_on_a_large_table(q, B, mrl, layouts):
                      got[2].cpu().numpy()), tuple(x[keep] for x in want))
     plan.close()
     ix.close()
+
+
+@pytest.mark.parametrize("q,layouts", [(4, 1), (5, 7), (5, 1), (6, 7)])
+@pytest.mark.parametrize("n", [255, 256, 1025, 2500])
+def test_mixed_batches_in_lockstep(q, layouts, n):
+    """Mixed batches around the size from which they are sorted and run in
+    lockstep, and around the sort's blocks of 1024 reads: reads of one token up
+    to 255, budgets from 0 to T <= 0, non-bases, a repeat family that leaves
+    more live words than a gather takes, a ragged last tile; the plain call, a
+    plan, and output capacities that leave no room for the order."""
+    from paper_1708_04329_gb300 import grim, synth
+
+    rng = np.random.default_rng(n + q)
+    g = synth.human_genome(400_000, seed=q)
+    g[100_000:160_000] = np.resize(g[1000:1400], 60_000)
+    rs = synth.reads(g, n, seed=n, lengths=(q, 40, 100, 254 + q), probs=(0.02, 0.28, 0.4, 0.3),
+                     e_frac=(6, 100), max_edits=None)
+    rs.e[rng.integers(0, n, 3)] = 200
+    rs.e[rs.lens == q] = 0
+    for r in rng.integers(0, n, 5):
+        rs.seq[int(rs.offsets[r])] = ord("N")
+    ix = build(g, 150, q, 254 + q, layouts)
+    want = oracle.filter(oracle.bin_vectors(g, 150, q, 254 + q), rs)
+    assert_same(gpu_filter(ix, rs, cap=len(want[0])), want)
+    with pytest.raises(grim.GrimError):
+        grim.grim_filter(ix, **dev_reads(rs), cap=10, retry=False)
+    plan = grim.grim_plan_create(ix, max_reads=n + 3, max_bases=len(rs.seq), max_e=200,
+                                 cap=len(want[0]) + 5)
+    got = plan.run(**dev_reads(rs))
+    assert_same((got[0].cpu().numpy().view(np.uint32), got[1].cpu().numpy().view(np.uint32),
+                 got[2].cpu().numpy()), want)
+    plan.close()
+    ix.close()
