@@ -52,8 +52,8 @@
 //   expects a tile to be nearly done, and finishes what is live there apart.
 //   Measured on GB300, k_exhaustive with a per-block test and a one-word tail
 //   for uniform batches against k_lockstep (3.1 Gbp, ms): 250k reads of 100 bp,
-//   coarse table 609 -> 599, 40k on the fine table 165 -> 159, 40k mixed
-//   100-250 bp reads 102 -> 89, a plan of 4,096 of them 11.3 -> 9.7, 60k of 150
+//   coarse table 609 -> 589, 40k on the fine table 165 -> 156, 40k mixed
+//   100-250 bp reads 102 -> 88, a plan of 4,096 of them 11.3 -> 9.6, 60k of 150
 //   bp at q = 6 60.3 -> 56.8.  Both pipes are near their limit there (small
 //   case: ALU 78%, shared-memory wavefronts 83%).
 #include "grim_internal.cuh"
@@ -76,7 +76,7 @@ constexpr uint32_t kSlotBlocksNarrow = 4;  // most slot blocks per read, 256-bin
 // some planes of 32 words (what fits beside the slots) and 32 bytes that say
 // where each came from
 template <int TW>
-constexpr int kScratchPlanes = TW == 32 ? 5 : 3;
+constexpr int kScratchPlanes = TW == 32 ? 6 : 3;
 template <int TW>
 constexpr uint32_t kScratchBytes = kScratchPlanes<TW> * 128 + 32;
 
@@ -102,6 +102,17 @@ __device__ __forceinline__ uint32_t imad(uint32_t a, uint32_t b, uint32_t c) {
   uint32_t d;
   asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
   return d;
+}
+// The full adder with its sum on the FMA pipe: as integers a + b + c is the sum
+// word plus twice the carry word, so three multiply-adds stand in for one of
+// the two logic ops.  Used for the adders of weight 4 and 8 of a block (12 of
+// 60): 250k reads of 100 bp 593 -> 589.5 ms; with weight 2 as well 627.
+__device__ __forceinline__ void fa_fma(uint32_t a, uint32_t b, uint32_t c, uint32_t& s, uint32_t& k,
+                                       uint32_t one, uint32_t minus_two) {
+  uint32_t m;
+  LOP3(m, a, b, c, 0xE8);
+  s = imad(m, minus_two, imad(c, one, imad(b, one, a)));
+  k = m;
 }
 __device__ __forceinline__ uint32_t imul_hi(uint32_t a, uint32_t b) {
   uint32_t d;
@@ -171,6 +182,7 @@ struct ExhArgs {
   uint32_t few_reads;          // batches of up to this many reads are k_exhaustive_few's
   const uint32_t* order;       // lockstep: the reads in the order they are taken (null: as given)
   uint32_t check_shift;        // lockstep: kMetaCheckCoarse or kMetaCheckFine
+  uint32_t c_one, c_minus_two;  // multipliers of fa_fma
   uint32_t pad_pair;           // two never-miss tokens
   Ctl* ctl;
 };
@@ -187,17 +199,18 @@ struct CsaTemps {
 template <int P, int NW>
 __device__ __forceinline__ void add_quad(Counters<P>& c, CsaTemps<NW>& t, int quad,
                                          const uint32_t (&a0)[NW], const uint32_t (&a1)[NW],
-                                         const uint32_t (&a2)[NW], const uint32_t (&a3)[NW]) {
+                                         const uint32_t (&a2)[NW], const uint32_t (&a3)[NW],
+                                         uint32_t one, uint32_t m2) {
 #pragma unroll
   for (int w = 0; w < NW; ++w) {
     uint32_t* t4 = (quad & 1) ? t.t4b : t.t4a;
     fa_miss(c.s1[w], a0[w], a1[w], c.s1[w], t.t2a[w]);
     fa_miss(c.s1[w], a2[w], a3[w], c.s1[w], t.t2b[w]);
     fa(c.s2[w], t.t2a[w], t.t2b[w], c.s2[w], t4[w]);
-    if (quad == 1) fa(c.s4[w], t.t4a[w], t.t4b[w], c.s4[w], t.t8a[w]);
+    if (quad == 1) fa_fma(c.s4[w], t.t4a[w], t.t4b[w], c.s4[w], t.t8a[w], one, m2);
     if (quad == 3) {
-      fa(c.s4[w], t.t4a[w], t.t4b[w], c.s4[w], t.t8b[w]);
-      fa(c.s8[w], t.t8a[w], t.t8b[w], c.s8[w], t.t16[w]);
+      fa_fma(c.s4[w], t.t4a[w], t.t4b[w], c.s4[w], t.t8b[w], one, m2);
+      fa_fma(c.s8[w], t.t8a[w], t.t8b[w], c.s8[w], t.t16[w], one, m2);
       // ripple the weight-16 carry through the upper planes; the carry out
       // of the top plane (counter >= 2^P: misses > D') sticks in `dead`
       uint32_t k = t.t16[w];
@@ -236,7 +249,7 @@ __device__ __forceinline__ void add_block(Counters<P>& c, const uint32_t (&tw)[8
     const uint4 x2 = lds128(addr[4 * quad + 2]), x3 = lds128(addr[4 * quad + 3]);
     const uint32_t a0[4] = {x0.x, x0.y, x0.z, x0.w}, a1[4] = {x1.x, x1.y, x1.z, x1.w};
     const uint32_t a2[4] = {x2.x, x2.y, x2.z, x2.w}, a3[4] = {x3.x, x3.y, x3.z, x3.w};
-    add_quad<P, 4>(c, t, quad, a0, a1, a2, a3);
+    add_quad<P, 4>(c, t, quad, a0, a1, a2, a3, a.c_one, a.c_minus_two);
   }
 }
 
@@ -893,7 +906,8 @@ __global__ void __launch_bounds__(kFewThreads, 2) k_exhaustive_few(ExhArgs a) {
       CsaTemps<4> t;
 #pragma unroll
       for (int quad = 0; quad < 4; ++quad)
-        add_quad<P, 4>(c, t, quad, x[4 * quad], x[4 * quad + 1], x[4 * quad + 2], x[4 * quad + 3]);
+        add_quad<P, 4>(c, t, quad, x[4 * quad], x[4 * quad + 1], x[4 * quad + 2], x[4 * quad + 3],
+                       a.c_one, a.c_minus_two);
       ldead = !on || (c.dead[0] & c.dead[1] & c.dead[2] & c.dead[3]) == ~0u;
       alive += ldead ? 0u : 1u;
       if (__all_sync(0xFFFFFFFFu, ldead)) break;
@@ -1065,6 +1079,8 @@ void launch_exhaustive(const IndexView& ix, const ReadsView& rv, RecordsView rec
   }
   a.row_stride = a.slot_blocks * kBlockTokens * 2u;
   a.slot_bytes = slot_bytes_of(a.slot_blocks);
+  a.c_one = 1u;
+  a.c_minus_two = 0u - 2u;
   a.c_hi = 65536u;
   a.c_lo = 0u - 65536u;
   a.range_bytes = shape.range_kb ? (uint64_t)shape.range_kb << 10 : kDefaultRangeBytes;

@@ -14,10 +14,10 @@ constexpr int kTokCtasPerSm = 5;      // of the persistent grid
 // of a random bin are about normal with mean S_j, the sum of the tokens' miss
 // shares, and variance S_j (j - S_j) / j; the check comes at the first j whose
 // mean is kCheckZ deviations past D'.
-// (3 / 4 / 5 / 6 deviations: 250k reads of 100 bp, coarse table 602 / 599 / 610
-// / 695 ms, 40k on the fine table 163 / 159 / 155 / 155, 40k mixed reads 89.6 /
-// 89.2 / 90.5 / 101.8, 60k of 150 bp at q = 6 57.6 / 56.8 / 57.3 / 63.9.)
-constexpr float kCheckZ = 4.0f;
+// (3 / 4 / 4.5 / 5 / 6 deviations: 250k reads of 100 bp, coarse table 602 / 599
+// / 595 / 610 / 695 ms, 40k mixed reads 89.6 / 89.2 / 88.5 / 90.5 / 101.8, 60k of
+// 150 bp at q = 6 57.6 / 56.8 / 56.9 / 57.3 / 63.9.)
+constexpr float kCheckZ = 4.5f;
 
 struct TokArgs {
   const char* reads;
