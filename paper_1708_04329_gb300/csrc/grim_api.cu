@@ -538,8 +538,8 @@ int grim_filter(const grim_index* idx, const char* reads, const uint64_t* offset
   const uint32_t read_bits = n_reads > 1 ? bit_length((uint64_t)n_reads - 1) : 0;
 
   CK(cudaMemsetAsync(ctl, 0, sizeof(Ctl), st));
-  launch_tokenise(reads, offsets, lens, e, v, rv, tokens, meta, ctl, st, cand_mode,
-                  fine_miss_power(idx));
+  launch_tokenise(reads, offsets, lens, e, v, rv, tokens, meta, ctl, st,
+                  cand_mode ? cand_off : nullptr, n_cand, fine_miss_power(idx));
   // The host waits where it has to decide: all-bins calls after tokenising
   // (the counters' depth, the path, the read switch) and every call for its
   // record count; what follows either way is enqueued before the wait (the
@@ -564,8 +564,7 @@ int grim_filter(const grim_index* idx, const char* reads, const uint64_t* offset
   int sc;
   uint64_t n_rec;
   if (cand_mode) {
-    launch_check_candidates(cand_off, n_reads, n_cand, ctl, st);
-    launch_candidates(v, rv, cand, cand_off, ra, ctl, st);
+    launch_candidates(v, rv, cand, cand_off, n_cand, ra, ctl, st);
     emit_short(n_cand);
     sc = read_back();
     if (sc != GRIM_OK) return sc;

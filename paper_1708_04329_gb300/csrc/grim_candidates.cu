@@ -486,8 +486,8 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_refine(IndexView ix, ReadsVi
 // `stage` groups of 32 -- as many as leave more than D' misses expected -- in
 // U candidates at once; one redux per candidate counts the tokens present.
 // Only a bin that could still pass has the rest of its tokens looked up.
-// Measured on GB300 (300k reads of 150 bp, e = 7, 98.9M candidates): 3.83 ms,
-// 0.97 of the two-line rate; ANDing whole vectors with bit planes of the read
+// Measured on GB300 (300k reads of 150 bp, e = 7, 98.9M candidates): 4.0 ms,
+// 0.93 of the two-line rate; ANDing whole vectors with bit planes of the read
 // took 9.48 ms at 91 warp instructions a candidate.  The same look-ups over
 // 128-byte vectors (q = 5, mixed reads) lost to the planes, 9.8 against 8.6
 // ms: one line is read either way, and a quarter warp per vector issues less.
@@ -656,8 +656,17 @@ __global__ void __launch_bounds__(kWarps * 32, 6) k_candidates_lookup(CandArgs a
   if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) atomicOr(&a.ctl->status, kStatusBadCand);
 }
 
+// CTAs of a list kernel: persistent, up to `most`, but no more warps than the
+// smallest chunks that n_cand candidates make (every warp claims from one
+// counter before it can know that none is left: 9,728 warps took 28 us over
+// 338 chunks, 344 took 21)
+uint64_t list_grid(uint64_t n_cand, uint64_t most) {
+  const uint64_t need = n_cand / (kChunkFew * kWarps) + 1;
+  return need < most ? need : most;
+}
+
 template <int U>
-void launch_lookup(const CandArgs& a, cudaStream_t st) {
+void launch_lookup(const CandArgs& a, uint64_t n_cand, cudaStream_t st) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -665,12 +674,13 @@ void launch_lookup(const CandArgs& a, cudaStream_t st) {
   const double grams = (double)a.ix.B + a.ix.ext - a.ix.q + 1;
   const double miss = exp(-grams / (double)a.ix.r4);
   const uint32_t miss256 = miss * 256.0 < 16.0 ? 16u : (uint32_t)(miss * 256.0);
+  const uint64_t grid = list_grid(n_cand, (uint64_t)(sms > 0 ? sms : 1) * 6u);
   ProfScope ps("candidates", st);
-  k_candidates_lookup<U><<<(unsigned)(sms > 0 ? sms : 1) * 6u, kWarps * 32, 0, st>>>(a, miss256);
+  k_candidates_lookup<U><<<(unsigned)grid, kWarps * 32, 0, st>>>(a, miss256);
 }
 
 template <int WPB, int U>
-void launch_u(const CandArgs& a, cudaStream_t st) {
+void launch_u(const CandArgs& a, uint64_t n_cand, cudaStream_t st) {
   // at most 14 KB a CTA, so the launch bounds set how many an SM holds
   const size_t smem = (size_t)kWarps * warp_smem_words(a.ix.r4, WPB) * sizeof(uint32_t);
   static_assert(kWarps * warp_smem_words(1024, 32) * 4 * kCandCtasPerSm <= 227 * 1024,
@@ -678,18 +688,17 @@ void launch_u(const CandArgs& a, cudaStream_t st) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // persistent: warps that find no chunk left exit at once
-  const uint64_t grid = (uint64_t)(sms > 0 ? sms : 1) * kCandCtasPerSm;
+  const uint64_t grid = list_grid(n_cand, (uint64_t)(sms > 0 ? sms : 1) * kCandCtasPerSm);
   ProfScope ps("candidates", st);
   k_candidates<WPB, U><<<(unsigned)grid, kWarps * 32, smem, st>>>(a);
 }
 
 template <int WPB>
-void launch_t(const CandArgs& a, cudaStream_t st, uint32_t unroll) {
-  if (unroll >= 8) launch_u<WPB, 8>(a, st);
-  else if (unroll >= 4) launch_u<WPB, 4>(a, st);
-  else if (unroll >= 2) launch_u<WPB, 2>(a, st);
-  else launch_u<WPB, 1>(a, st);
+void launch_t(const CandArgs& a, uint64_t n_cand, cudaStream_t st, uint32_t unroll) {
+  if (unroll >= 8) launch_u<WPB, 8>(a, n_cand, st);
+  else if (unroll >= 4) launch_u<WPB, 4>(a, n_cand, st);
+  else if (unroll >= 2) launch_u<WPB, 2>(a, n_cand, st);
+  else launch_u<WPB, 1>(a, n_cand, st);
 }
 
 }  // namespace
@@ -709,21 +718,21 @@ void launch_refine(const IndexView& ix, const ReadsView& rv, const unsigned long
 }
 
 void launch_candidates(const IndexView& ix, const ReadsView& rv, const int32_t* cand,
-                       const uint64_t* cand_off, RecordsView rec, Ctl* ctl, cudaStream_t st,
-                       Live live, uint32_t unroll) {
+                       const uint64_t* cand_off, uint64_t n_cand, RecordsView rec, Ctl* ctl,
+                       cudaStream_t st, Live live, uint32_t unroll) {
   if (unroll == 0) unroll = ix.wpb > 32 ? kDefaultLookupUnroll : kDefaultCandUnroll;
   if (rv.n_reads == 0) return;
   CandArgs a{ix, rv, cand, cand_off, rec, ctl, live};
   switch (ix.wpb) {
-    case 1: launch_t<1>(a, st, unroll); break;
-    case 2: launch_t<2>(a, st, unroll); break;
-    case 8: launch_t<8>(a, st, unroll); break;
-    case 32: launch_t<32>(a, st, unroll); break;
+    case 1: launch_t<1>(a, n_cand, st, unroll); break;
+    case 2: launch_t<2>(a, n_cand, st, unroll); break;
+    case 8: launch_t<8>(a, n_cand, st, unroll); break;
+    case 32: launch_t<32>(a, n_cand, st, unroll); break;
     case 128:
-      if (unroll >= 8) launch_lookup<8>(a, st);
-      else if (unroll >= 4) launch_lookup<4>(a, st);
-      else if (unroll >= 2) launch_lookup<2>(a, st);
-      else launch_lookup<1>(a, st);
+      if (unroll >= 8) launch_lookup<8>(a, n_cand, st);
+      else if (unroll >= 4) launch_lookup<4>(a, n_cand, st);
+      else if (unroll >= 2) launch_lookup<2>(a, n_cand, st);
+      else launch_lookup<1>(a, n_cand, st);
       break;
     default: break;  // q outside 2..6 is rejected by grim_build
   }

@@ -173,21 +173,19 @@ enum class TokenOrder : uint32_t {
 // fix the counter depth from it); 0xFFFF = no limit.  max_bases: size of the
 // reads buffer when known (a read ending past it fails the batch with
 // kStatusArg), else ~0.  rv.copies token copies per read are written.  The
-// order is chosen from the mode: lists (`cand_mode`) or all bins.  Leaves the
+// order is chosen from the mode: lists (cand_off set: their CSR offsets, checked
+// here to be non-decreasing and to end at n_cand, else kStatusBadCsr; the ids
+// themselves are checked by the list kernels) or all bins.  Leaves the
 // batch's extremes of D', slack and 16-token blocks in the control block.
 void launch_tokenise(const char* reads, const uint64_t* offsets, const uint32_t* lens,
                      const uint16_t* e, const IndexView& ix, ReadsView rv, uint16_t* tokens,
-                     uint32_t* meta, Ctl* ctl, cudaStream_t st, bool cand_mode, float fine_power,
+                     uint32_t* meta, Ctl* ctl, cudaStream_t st, const uint64_t* cand_off,
+                     uint64_t n_cand, float fine_power,
                      Live live = {false, 0}, uint32_t max_e = 0xFFFFu,
                      uint64_t max_bases = ~0ull);
 // the reads' order from the keys the tokeniser left in meta
 void launch_order(const ReadsView& rv, uint32_t* order, const Ctl* ctl, cudaStream_t st,
                   Live live = {false, 0});
-// CSR offsets of the caller's lists: non-decreasing, ending at n_cand
-// (kStatusBadCsr otherwise); the ids themselves are checked by the
-// candidate kernel
-void launch_check_candidates(const uint64_t* cand_off, uint32_t n_reads, uint64_t n_cand, Ctl* ctl,
-                             cudaStream_t st, Live live = {false, 0});
 
 // bins per tile of the all-bins kernel for a table of r4 = 4^q rows
 uint32_t exhaustive_tile_bins(uint32_t r4);
@@ -217,10 +215,11 @@ void launch_exhaustive(const IndexView& ix, const ReadsView& rv, RecordsView rec
                        uint32_t max_d, Ctl* ctl, cudaStream_t st, bool fine, const uint32_t* order,
                        Live live, ExhShape shape);
 // unroll: candidate gathers in flight per lane group (1, 2, 4 or 8; 0 =
-// default).  An id outside [0, num_bins) sets kStatusBadCand.
+// default).  n_cand sizes the launch (graph launches: the most candidates).  An
+// id outside [0, num_bins) sets kStatusBadCand.
 void launch_candidates(const IndexView& ix, const ReadsView& rv, const int32_t* cand,
-                       const uint64_t* cand_off, RecordsView rec, Ctl* ctl, cudaStream_t st,
-                       Live live = {false, 0}, uint32_t unroll = 0);
+                       const uint64_t* cand_off, uint64_t n_cand, RecordsView rec, Ctl* ctl,
+                       cudaStream_t st, Live live = {false, 0}, uint32_t unroll = 0);
 // The exact check of the coarse pass's survivors (keys read << cbits |
 // super-bin, in any order; *n_surv of them, on the device, none checked if
 // more than `room`): the members of each surviving super-bin of f bins against

@@ -168,10 +168,10 @@ int capture(grim_plan* p) {
   if (p->hio) k_copy_in<<<dim3(64, kCopySegs), 256, 0, st>>>(p->copy, p->ctl);
   launch_tokenise(B.reads, B.offsets, B.lens, B.e, v, rv,
                   reinterpret_cast<uint16_t*>(ws + L.tok), reinterpret_cast<uint32_t*>(ws + L.meta),
-                  p->ctl, st, p->cand_mode, fine_miss_power(idx), live, d.max_e, d.max_bases);
+                  p->ctl, st, p->cand_mode ? B.cand_off : nullptr, d.max_cand, fine_miss_power(idx),
+                  live, d.max_e, d.max_bases);
   if (p->cand_mode) {
-    launch_check_candidates(B.cand_off, d.max_reads, d.max_cand, p->ctl, st, live);
-    launch_candidates(v, rv, B.cand, B.cand_off, ra, p->ctl, st, live, d.cand_unroll);
+    launch_candidates(v, rv, B.cand, B.cand_off, d.max_cand, ra, p->ctl, st, live, d.cand_unroll);
     k_plan_control<<<1, 1, 0, st>>>(p->ctl, kCtlFinal, 0, 0, 0, 0, 0, 0);
     sort_and_emit(ra, rb, d.cap, bit_length(d.max_cand ? d.max_cand - 1 : 0), ws + L.hist, true,
                   bin_bits, B.cand, B.cand_off, d.max_reads, B.out_read,

@@ -34,6 +34,8 @@ struct TokArgs {
   Live live;
   uint32_t max_e;
   uint64_t max_bases;
+  const uint64_t* cand_off;  // list modes: the lists' CSR offsets
+  uint64_t n_cand;
 };
 
 // One warp per read.  The read's tokens (row indices of the table: the token
@@ -94,6 +96,10 @@ __global__ void __launch_bounds__(kTokWarps * 32, kTokCtasPerSm) k_tokenise(TokA
   Ctl* ctl = a.ctl;
   const uint32_t q = a.q, r4 = a.r4;
   const uint32_t n_reads = live_reads(ctl, a.live, a.n_reads);
+  // (an empty graph batch has lists to end somewhere too)
+  if (n_reads == 0 && a.cand_off && blockIdx.x == 0 && threadIdx.x == 0 &&
+      a.cand_off[0] != (a.live.on ? ctl->live_cand : a.n_cand))
+    atomicOr(&ctl->status, kStatusBadCsr);
   // the extremes of this warp's reads (as in Ctl); raised once at the end: a
   // check of the shared words for every read is a load of one address for
   // every read, which takes longer than the tokens
@@ -101,6 +107,11 @@ __global__ void __launch_bounds__(kTokWarps * 32, kTokCtasPerSm) k_tokenise(TokA
   for (uint64_t r = blockIdx.x * (uint64_t)kTokWarps + warp; r < n_reads; r += n_warps) {
     const uint32_t budget = a.e[r];
     if (budget > a.max_e && lane == 0) atomicOr(&ctl->status, kStatusArg);
+    if (a.cand_off && lane == 0) {
+      const uint64_t c0 = a.cand_off[r], c1 = a.cand_off[r + 1];
+      if (c0 > c1 || (r + 1 == n_reads && c1 != (a.live.on ? ctl->live_cand : a.n_cand)))
+        atomicOr(&ctl->status, kStatusBadCsr);
+    }
     const uint32_t L = a.lens[r];
     const uint64_t off = a.offsets[r];
     bool bad = false;
@@ -396,17 +407,6 @@ __global__ void __launch_bounds__(kOrderBlock) k_order_place(const uint32_t* __r
   }
 }
 
-__global__ void k_check_csr(const uint64_t* __restrict__ cand_off, uint32_t n_reads,
-                            uint64_t n_cand, Ctl* ctl, Live live) {
-  const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  if (live.on) {
-    n_reads = ctl->live_reads;
-    n_cand = ctl->live_cand;
-  }
-  if (i < n_reads && cand_off[i] > cand_off[i + 1]) atomicOr(&ctl->status, kStatusBadCsr);
-  if (i == 0 && cand_off[n_reads] != n_cand) atomicOr(&ctl->status, kStatusBadCsr);
-}
-
 // Reverse complement, one warp per read: out[off + L-1-j] = comp(reads[off + j])
 // with A<->T and C<->G in either case (case kept); other bytes unchanged.
 __global__ void k_reverse_complement(const char* __restrict__ reads,
@@ -442,8 +442,9 @@ void launch_reverse_complement(const char* reads, const uint64_t* offsets, const
 
 void launch_tokenise(const char* reads, const uint64_t* offsets, const uint32_t* lens,
                      const uint16_t* e, const IndexView& ix, ReadsView rv, uint16_t* tokens,
-                     uint32_t* meta, Ctl* ctl, cudaStream_t st, bool cand_mode,
-                     float fine_power, Live live, uint32_t max_e, uint64_t max_bases) {
+                     uint32_t* meta, Ctl* ctl, cudaStream_t st, const uint64_t* cand_off,
+                     uint64_t n_cand, float fine_power, Live live, uint32_t max_e,
+                     uint64_t max_bases) {
   if (rv.n_reads == 0) return;
   const uint32_t threads = kTokWarps * 32;
   int dev = 0, sms = 0;
@@ -453,10 +454,11 @@ void launch_tokenise(const char* reads, const uint64_t* offsets, const uint32_t*
   const uint64_t most = (uint64_t)(sms > 0 ? sms : 1) * kTokCtasPerSm;
   const uint64_t grid = need < most ? need : most;
   const TokArgs a{reads, offsets, lens,   e,    rv.n_reads, ix.q, ix.max_read_len, ix.r4,    rv.ts,
-                  rv.copies, ix.rank, ix.miss, fine_power, tokens, meta, ctl, live, max_e, max_bases};
+                  rv.copies, ix.rank, ix.miss, fine_power, tokens, meta, ctl, live, max_e, max_bases,
+                  cand_off, n_cand};
   // lists read whole token rows in any order up to 128-byte vectors; larger
   // ones (q = 6) are looked up line by line
-  auto kernel = cand_mode       ? (ix.wpb > 32 ? k_tokenise<TokenOrder::kLines>
+  auto kernel = cand_off        ? (ix.wpb > 32 ? k_tokenise<TokenOrder::kLines>
                                                : k_tokenise<TokenOrder::kPosition>)
                 : rv.copies > 1 ? k_tokenise<TokenOrder::kCyclic>
                                 : k_tokenise<TokenOrder::kRarest>;
@@ -471,13 +473,6 @@ void launch_order(const ReadsView& rv, uint32_t* order, const Ctl* ctl, cudaStre
   ProfScope ps("order", st);
   k_order_count<<<grid, kOrderBlock, 0, st>>>(rv.meta, rv.n_reads, rv.n_reads, order, ctl, live);
   k_order_place<<<grid, kOrderBlock, 0, st>>>(rv.meta, rv.n_reads, rv.n_reads, order, ctl, live);
-}
-
-void launch_check_candidates(const uint64_t* cand_off, uint32_t n_reads, uint64_t n_cand, Ctl* ctl,
-                             cudaStream_t st, Live live) {
-  const uint64_t n = (uint64_t)n_reads + 1;
-  ProfScope ps("check_candidates", st);
-  k_check_csr<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(cand_off, n_reads, n_cand, ctl, live);
 }
 
 }  // namespace grim
