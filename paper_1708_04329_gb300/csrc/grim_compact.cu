@@ -6,8 +6,8 @@
 // the order is restored by a least-significant-digit radix sort on the record
 // key -- (read << bin_bits | bin) in all-bins mode, the global candidate index
 // in candidate mode; keys are unique, so the output order is unique too.
-// Each 8-bit pass is a per-block digit histogram, one exclusive scan over
-// all blocks' histograms, and a stable scatter (per-warp ranks from
+// Each 8-bit pass is a per-block digit histogram, a scan of each digit over
+// the blocks, and a stable scatter (per-warp ranks from
 // __match_any_sync, then warp order, then round order).  A last kernel splits
 // the keys into the caller's read / bin / count arrays.  Short lists skip the
 // radix sort: one kernel places each record by counting the smaller keys.
@@ -45,56 +45,40 @@ __global__ void __launch_bounds__(kSortThreads) k_rs_hist(const unsigned long lo
   hist[(uint64_t)threadIdx.x * nb + blockIdx.x] = cnt[threadIdx.x];
 }
 
-// Exclusive scan, with one block, of the digit-major histogram of the live
-// blocks: entry (d, blk) at h[d * nb + blk] for blk < nb_live, scanned in
-// the logical order i = d * nb_live + blk.  Warp w owns the logical range
-// [w*S, (w+1)*S): it sums the range (32 consecutive entries per step, so the
-// loads coalesce), the 32 warp totals are scanned, and each warp rescans its
-// range with shuffles, carrying its running offset.
-__device__ __forceinline__ uint64_t hist_at(uint32_t i, uint32_t nb_live, uint64_t nb) {
-  return (uint64_t)(i / nb_live) * nb + (i % nb_live);
+// Inclusive scan over the live blocks of each digit's row of the histogram
+// (entry (d, blk) at h[d * nb + blk]), a CTA per digit; the scatter adds the
+// smaller digits' totals, the rows' last entries.  One CTA scanning all 256
+// rows took 35 us a pass at 1M records, this 6.
+__device__ __forceinline__ uint32_t block_inclusive(uint32_t v, uint32_t* s_warp) {
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t incl = v;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+    if (lane >= (uint32_t)d) incl += t;
+  }
+  if (lane == 31) s_warp[warp] = incl;
+  __syncthreads();
+  for (uint32_t w = 0; w < warp; ++w) incl += s_warp[w];
+  __syncthreads();
+  return incl;
 }
 
-__global__ void __launch_bounds__(1024) k_rs_scan(uint32_t* __restrict__ h, uint64_t nb, uint64_t n,
-                                                  const unsigned long long* n_live) {
-  __shared__ uint32_t s_warp[32];
+__global__ void __launch_bounds__(kSortThreads) k_rs_scan(uint32_t* __restrict__ h, uint64_t nb,
+                                                          uint64_t n,
+                                                          const unsigned long long* n_live) {
+  __shared__ uint32_t s_warp[kSortThreads / 32], s_carry;
   n = live_n(n_live, n);
   const uint32_t nb_live = (uint32_t)((n + kSortTile - 1) / kSortTile);
-  if (nb_live == 0) return;
-  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t m = 256u * nb_live;
-  const uint32_t span = (m + 31) / 32;
-  const uint32_t lo = min(warp * span, m), hi = min(lo + span, m);
-  uint32_t total = 0;
-  for (uint32_t i = lo + lane; i < hi; i += 32) total += h[hist_at(i, nb_live, nb)];
-  total = __reduce_add_sync(0xFFFFFFFFu, total);
-  if (lane == 0) s_warp[warp] = total;
-  __syncthreads();
-  if (warp == 0) {
-    const uint32_t v = s_warp[lane];
-    uint32_t incl = v;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-      if (lane >= (uint32_t)d) incl += t;
-    }
-    s_warp[lane] = incl - v;  // exclusive
-  }
-  __syncthreads();
-  uint32_t carry = s_warp[warp];
-  for (uint32_t c = lo; c < hi; c += 32) {
-    const uint32_t i = c + lane;
-    const bool in = i < hi;
-    const uint64_t j = in ? hist_at(i, nb_live, nb) : 0;
-    const uint32_t v = in ? h[j] : 0u;
-    uint32_t incl = v;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-      if (lane >= (uint32_t)d) incl += t;
-    }
-    if (in) h[j] = carry + incl - v;
-    carry += __shfl_sync(0xFFFFFFFFu, incl, 31);
+  uint32_t* row = h + blockIdx.x * nb;
+  uint32_t carry = 0;
+  for (uint32_t c = 0; c < nb_live; c += kSortThreads) {
+    const uint32_t i = c + threadIdx.x;
+    const uint32_t incl = carry + block_inclusive(i < nb_live ? row[i] : 0u, s_warp);
+    if (i < nb_live) row[i] = incl;
+    if (threadIdx.x == kSortThreads - 1) s_carry = incl;
+    __syncthreads();
+    carry = s_carry;
   }
 }
 
@@ -108,7 +92,13 @@ __global__ void __launch_bounds__(kSortThreads) k_rs_scatter(
   n = live_n(n_live, n);
   if ((uint64_t)blockIdx.x * kSortTile >= n) return;  // past the live records
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  s_base[tid] = hist[(uint64_t)tid * nb + blockIdx.x];
+  {  // places of this block's first record of each digit
+    static_assert(kSortThreads == 256, "a thread per digit");
+    const uint32_t* row = hist + (uint64_t)tid * nb;
+    const uint32_t all = row[(n + kSortTile - 1) / kSortTile - 1];
+    const uint32_t before = block_inclusive(all, &s_wcnt[0][0]) - all;
+    s_base[tid] = before + (blockIdx.x ? row[blockIdx.x - 1] : 0u);
+  }
   const uint64_t base = (uint64_t)blockIdx.x * kSortTile;
   for (uint32_t round = 0; round < kSortItems; ++round) {
     for (uint32_t i = tid; i < kW * 256; i += kSortThreads) (&s_wcnt[0][0])[i] = 0;
@@ -236,7 +226,7 @@ RecordsView sort_records(RecordsView a, RecordsView b, uint64_t n, uint32_t key_
     }
     {
       ProfScope ps("sort_scan", st);
-      k_rs_scan<<<1, 1024, 0, st>>>(h, nb, n, n_live);
+      k_rs_scan<<<256, kSortThreads, 0, st>>>(h, nb, n, n_live);
     }
     {
       ProfScope ps("sort_scatter", st);

@@ -762,3 +762,21 @@ def test_mixed_batches_in_lockstep(q, layouts, n):
                  got[2].cpu().numpy()), want)
     plan.close()
     ix.close()
+
+
+@pytest.mark.parametrize("n", [4096 * 2 + 1, 4096 * 256, 4096 * 256 + 1])
+def test_radix_sort_block_counts(n):
+    """Pass lists of two and of 256 sort blocks and one record more (the scan
+    of a digit's row takes a second step): every listed bin passes (T <= 0)."""
+    rng = np.random.default_rng(n)
+    g = rng.choice(np.frombuffer(b"ACGT", np.uint8), 30_000)
+    nr = 300
+    rs = Reads([g[p:p + 30].tobytes().decode() for p in rng.integers(0, 29_000, nr)], [15] * nr)
+    cand = rng.integers(0, 600, n).astype(np.int32)
+    off = np.sort(rng.integers(0, n + 1, nr + 1)).astype(np.uint64)
+    off[0], off[-1] = 0, n
+    ix = build(g, 50, 5, 30, layouts=2)
+    r, b, _ = gpu_filter(ix, rs, off, cand, cap=n)
+    assert np.array_equal(b.view(np.int32), cand)
+    assert np.array_equal(r, np.repeat(np.arange(nr), np.diff(off.astype(np.int64))))
+    ix.close()
