@@ -596,6 +596,7 @@ __global__ void __launch_bounds__(NT, 1) k_lockstep(ExhArgs a) {
   // [tile: (r4 + 2) rows x TW words][group slots][16 padding tokens][warp scratch]
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ uint32_t s_item, s_next;
+  __shared__ unsigned long long s_counted;  // calls without room for records: passing bins
   const uint32_t tid = threadIdx.x, lane = tid & 31, grp = lane / GL, li = lane % GL;
   const uint32_t nthreads = blockDim.x;
   const uint32_t r4 = a.ix.r4;
@@ -610,6 +611,7 @@ __global__ void __launch_bounds__(NT, 1) k_lockstep(ExhArgs a) {
   const uint32_t slot = sh_base + tile_bytes + (tid / GL) * a.slot_bytes;
   const uint32_t pad_tokens = sh_base + tile_bytes + (nthreads / GL) * a.slot_bytes;
   const uint32_t scratch = pad_tokens + 32u + (tid >> 5) * kScratchBytes<TW>;
+  if (tid == 0) s_counted = 0;
   fill_special_rows<TW>(reinterpret_cast<uint32_t*>(smem), r4, pad_tokens, tid, nthreads);
   const uint32_t lane_base = sh_base + li * 16u;
   const uint32_t row_chunks = a.row_stride / 16u;
@@ -627,6 +629,10 @@ __global__ void __launch_bounds__(NT, 1) k_lockstep(ExhArgs a) {
     if (tid == 0) {
       s_item = atomicAdd(&a.ctl->item, 1u);
       s_next = 0;
+      if (a.rec.cap == 0) {
+        if (s_counted) atomicAdd(&a.ctl->n_rec, s_counted);
+        s_counted = 0;
+      }
     }
     __syncthreads();
     const uint32_t item = s_item;
@@ -736,6 +742,13 @@ __global__ void __launch_bounds__(NT, 1) k_lockstep(ExhArgs a) {
       auto emit = [&](const uint32_t(&pm)[4], auto&& value, uint32_t read, uint32_t rm,
                       uint32_t bin0, uint32_t bin_step) {
         const uint32_t cnt = __popc(pm[0]) + __popc(pm[1]) + __popc(pm[2]) + __popc(pm[3]);
+        if (a.rec.cap == 0) {
+          // one global atomic per CTA and item instead of one per round, which
+          // all warps would queue for when most bins pass
+          const uint32_t all = __reduce_add_sync(0xFFFFFFFFu, cnt);
+          if (lane == 0) atomicAdd(&s_counted, (unsigned long long)all);
+          return;
+        }
         uint32_t incl = cnt;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
