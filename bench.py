@@ -315,9 +315,9 @@ def alu_roofline(executed: int, per_launch_ms: float, n_sm: int, sm_mhz: float, 
     return {"bound": "alu", "achieved": round(achieved, 2), "peak": round(peak, 2),
             "unit": "Tbit-tests/s", "frac": round(achieved / peak, 4), "kernel": kernel,
             "kernel_ms": round(per_launch_ms, 3),
-            "work": ("bit tests the kernel executed: 16-token blocks applied to (super-)bin "
-                     "tiles x bins per tile (early exit skips the rest; a block of the "
-                     "one-word tail counts a quarter of the 1024-bin tile)"),
+            "work": ("bit tests the kernel executed: blocks of 8 tokens applied to (super-)bin "
+                     "tiles x bins per tile (early exit skips the rest; once a warp's live "
+                     "words are gathered a block counts 32 bins for each of them)"),
             "executed_bit_tests": int(executed),
             "peak_basis": (f"ALU pipe: {n_sm} SMs x 64 lanes/clk x 32 bins per logic op / 2 "
                            f"LOP3 per token per 32-bin word (carry-save minimum) x {sm_mhz:.0f} "
@@ -513,16 +513,20 @@ def run_native(args, rank, world, local):
 
 def candidate_roofline(n_cand: int, k_ms: float, nb: int, vec: int, st, peaks: dict, args,
                        traffic_key: str, headline: bool = False) -> dict:
-    """The candidate kernel (one bin-vector gather per pair): algorithmic bytes
-    (vector + id per pair) over its CUDA-event time, against the copy
-    bandwidth and against this GPU's random-gather ceiling for such rows."""
-    gbytes = n_cand * (vec + 4) / 1e9
+    """The candidate kernel: algorithmic bytes (what it reads of a vector, and an
+    id, per pair) over its CUDA-event time, against the copy bandwidth and, where
+    whole vectors are gathered, this GPU's random-gather ceiling for such rows.
+    Of a 512-byte vector (q = 6) the two 128-byte lines with most of the read's
+    tokens are looked up: they hold more than D' = 42 of the 145 tokens of a
+    150 bp read with e = 7."""
+    gbytes = n_cand * (min(vec, 256) + 4) / 1e9
     hbm = float(peaks.get("hbm_gbs", 6800.0))
     leg = {"bound": "hbm", "kernel": "k_candidates", "kernel_ms": k_ms,
            "algorithmic_bytes": round(gbytes * 1e9), "achieved": round(gbytes / (k_ms / 1e3), 1),
            "peak": hbm, "unit": "GB/s", "frac": round(gbytes / (k_ms / 1e3) / hbm, 4),
            "traffic": traffic_for(args, traffic_key, "grim_candidates.cu", headline)}
-    ceiling = gather_ceiling(nb, vec, n_cand, st)
+    ceiling = (gather_ceiling(nb, vec, n_cand, st) if vec <= 256 else
+               {"unavailable": "two of a vector's four 128-byte lines are read, not whole rows"})
     if ceiling.get("gbs"):
         ceiling["frac_of_hbm"] = round(ceiling["gbs"] / hbm, 4)
         leg["frac_of_gather_ceiling"] = round(n_cand / (k_ms / 1e3) / ceiling["rows_per_s"], 4)
