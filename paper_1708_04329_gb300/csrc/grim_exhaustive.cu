@@ -76,7 +76,7 @@ constexpr uint32_t kSlotBlocksNarrow = 4;  // most slot blocks per read, 256-bin
 // some planes of 32 words (what fits beside the slots) and 32 bytes that say
 // where each came from
 template <int TW>
-constexpr int kScratchPlanes = TW == 32 ? 6 : 3;
+constexpr int kScratchPlanes = TW == 8 ? 3 : 6;
 template <int TW>
 constexpr uint32_t kScratchBytes = kScratchPlanes<TW> * 128 + 32;
 
@@ -347,6 +347,8 @@ __device__ __forceinline__ void stage_tile(const ExhArgs& a, uint32_t tile, uint
   const uint32_t* src = a.ix.tm + (uint64_t)tile * TW;
   for (uint32_t i = tid; i < a.ix.r4 * kChunks; i += nthreads) {
     const uint32_t row = i / kChunks, chunk = i % kChunks;
+    // (rows end on 1024 bins; the bins of a larger tile past them start out dead)
+    if (TW > 32 && (uint64_t)tile * TW + chunk * 4u >= a.ix.wpad) continue;
     const uint32_t* g = src + (uint64_t)row * a.ix.wpad + chunk * 4u;
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sh_base + row * TW * 4u +
                                                                   chunk * 16u),
@@ -572,7 +574,7 @@ __global__ void __launch_bounds__(NT, 1) k_exhaustive(ExhArgs a) {
 }
 
 // The lockstep kernel: the lane groups of a warp (4 on 1024-bin tiles, 16 on
-// 256-bin tiles) take reads of similar length to go (ExhArgs::order) together,
+// 256-bin tiles, 1 on the 4096-bin tiles of q <= 4) take reads of similar length to go (ExhArgs::order) together,
 // run them for
 // as many tokens as the tokeniser expects a tile to need, gather what is still
 // live and finish that.
@@ -617,10 +619,10 @@ __global__ void __launch_bounds__(NT, 1) k_lockstep(ExhArgs a) {
   const uint32_t row_chunks = a.row_stride / 16u;
   // 256-bin tiles: the token copy a group reads, and the halves its slot holds
   // (a read's later tokens come from L2)
-  const uint32_t copies = TW == 32 ? 1u : a.rv.copies;
-  const uint32_t slot_halves = TW == 32 ? ~0u : 2u * a.slot_blocks;
+  const uint32_t copies = TW == 8 ? a.rv.copies : 1u;
+  const uint32_t slot_halves = TW == 8 ? 2u * a.slot_blocks : ~0u;
   auto token_row = [&](uint32_t r, uint32_t g) {
-    return a.rv.tokens + ((uint64_t)r * copies + (TW == 32 ? 0u : g % copies)) * a.rv.ts;
+    return a.rv.tokens + ((uint64_t)r * copies + (TW == 8 ? g % copies : 0u)) * a.rv.ts;
   };
 
   for (;;) {
@@ -686,7 +688,7 @@ __global__ void __launch_bounds__(NT, 1) k_lockstep(ExhArgs a) {
 
       // 0 without a read; rotated copies spread a block's tokens over both halves
       const uint32_t halves =
-          TW == 32 ? ((m & 0xFFu) + 7u) >> 3 : ((m & 0xFFu) + 15u) >> 4 << 1;
+          TW == 8 ? ((m & 0xFFu) + 15u) >> 4 << 1 : ((m & 0xFFu) + 7u) >> 3;
       const uint32_t hmax = __reduce_max_sync(0xFFFFFFFFu, halves);
       uint32_t h = __reduce_min_sync(0xFFFFFFFFu, have ? (m >> a.check_shift) & 31u : 31u);
       h = min(h, hmax);
@@ -705,7 +707,7 @@ __global__ void __launch_bounds__(NT, 1) k_lockstep(ExhArgs a) {
       const uint4* far = reinterpret_cast<const uint4*>(token_row(have ? cur : 0u, grp));
       const uint4 pads = make_uint4(a.pad_pair, a.pad_pair, a.pad_pair, a.pad_pair);
       auto tokens_at = [&](uint32_t at, uint32_t near, const uint4* from, bool mine) {
-        if (TW == 32 || at < slot_halves) return lds128(near);
+        if (TW != 8 || at < slot_halves) return lds128(near);
         return mine ? __ldg(from + at) : pads;
       };
       for (uint32_t b = 0; b < h >> 1; ++b) {
@@ -824,14 +826,16 @@ __global__ void __launch_bounds__(NT, 1) k_lockstep(ExhArgs a) {
       const uint32_t gbase = sh_base + (on ? bin0 >> 3 : 0u);
       {  // reads with a word left
         const uint32_t any = live[0] | live[1] | live[2] | live[3];
-        if (TW == 32)
+        if (TW == 128)
+          off = 1;
+        else if (TW == 32)
           off = ((any & 0xFFu) != 0) + ((any & 0xFF00u) != 0) + ((any & 0xFF0000u) != 0) +
                 ((any & 0xFF000000u) != 0);
         else
           off = __popc((any | any >> 1) & 0x55555555u);
       }
       const uint4* gfar = far;
-      if (TW != 32) {
+      if (TW == 8) {
         const uint32_t read = __shfl_sync(0xFFFFFFFFu, cur, src);
         gfar = reinterpret_cast<const uint4*>(token_row(on ? read : 0u, src / GL));
       }
@@ -851,12 +855,14 @@ __global__ void __launch_bounds__(NT, 1) k_lockstep(ExhArgs a) {
       }
     }
     // one count per group (its lanes agree), one atomic per warp and item
-    ex = __reduce_add_sync(0xFFFFFFFFu, li == 0 ? ex : 0u);
+    // (4096-bin tiles count as four)
+    constexpr uint32_t kUnits = TW == 128 ? 4 : 1;
+    ex = __reduce_add_sync(0xFFFFFFFFu, li == 0 ? ex * kUnits : 0u);
     tail_words = __reduce_add_sync(0xFFFFFFFFu, tail_words);
     if (lane == 0) {
       atomicAdd(&a.ctl->blocks, (unsigned long long)ex);
       if (tail_ex) {
-        atomicAdd(&a.ctl->tail_blocks, (unsigned long long)tail_ex);
+        atomicAdd(&a.ctl->tail_blocks, (unsigned long long)tail_ex * kUnits);
         atomicAdd(&a.ctl->tail_words, (unsigned long long)tail_words);
       }
     }
@@ -991,17 +997,19 @@ void launch_nt(const ExhArgs& a, size_t smem, uint32_t threads, uint32_t grid, u
     else run(k_lockstep<8, TW, NT>);
     return;
   }
-  if (p == 5) run(k_exhaustive<5, TW, NT>);
-  else if (p == 6) run(k_exhaustive<6, TW, NT>);
-  else if (p == 7) run(k_exhaustive<7, TW, NT>);
-  else run(k_exhaustive<8, TW, NT>);
+  if constexpr (TW != 128) {
+    if (p == 5) run(k_exhaustive<5, TW, NT>);
+    else if (p == 6) run(k_exhaustive<6, TW, NT>);
+    else if (p == 7) run(k_exhaustive<7, TW, NT>);
+    else run(k_exhaustive<8, TW, NT>);
+  }
 }
 
 template <int TW>
 void launch_tw(ExhArgs& a, const IndexView& ix, uint32_t max_d, uint32_t sms, uint32_t nt,
                bool warp_switch, cudaStream_t st, const char* name) {
   constexpr uint32_t kRowBytes = TW * 4, GL = TW / 4, kTileBinsT = TW * 32;
-  a.n_tiles = (uint32_t)(ix.num_bins_pad / kTileBinsT);
+  a.n_tiles = (uint32_t)((ix.num_bins_pad + kTileBinsT - 1) / kTileBinsT);
   a.sms = sms;
   a.c_row = kRowBytes;
   // the largest CTA up to the built size whose tile and group slots fit in
@@ -1119,7 +1127,14 @@ void launch_exhaustive(const IndexView& ix, const ReadsView& rv, RecordsView rec
   a.pad_pair = rowPad(ix.r4) | (rowPad(ix.r4) << 16);
   a.check_shift = fine ? kMetaCheckFine : kMetaCheckCoarse;
   const bool ws = shape.read_switch == GRIM_SWITCH_WARP;
-  if (ix.r4 <= 1024) launch_tw<32>(a, ix, max_d, (uint32_t)sms, nt, ws, st, prof_name);
+  // q <= 4: four times the bins fit a tile, a warp runs one read over all of
+  // them, and a CTA has four times the rounds between two waits for a tile (500
+  // reads at q = 4 are 6.25 rounds of its warps on 1024 bins, run as 7).  Where
+  // there are tiles enough for every SM.  Existence counts of 500 reads against
+  // 6.6M bins, six budgets: 9.3 -> 8.9 ms.
+  if (ws && ix.r4 <= 256 && ix.num_bins_pad / 4096 >= (uint64_t)sms)
+    launch_tw<128>(a, ix, max_d, (uint32_t)sms, nt, ws, st, prof_name);
+  else if (ix.r4 <= 1024) launch_tw<32>(a, ix, max_d, (uint32_t)sms, nt, ws, st, prof_name);
   else launch_tw<8>(a, ix, max_d, (uint32_t)sms, nt, ws, st, prof_name);
 }
 

@@ -780,3 +780,24 @@ def test_radix_sort_block_counts(n):
     assert np.array_equal(b.view(np.int32), cand)
     assert np.array_equal(r, np.repeat(np.arange(nr), np.diff(off.astype(np.int64))))
     ix.close()
+
+
+@pytest.mark.parametrize("q,n,tail", [(4, 300, 1), (4, 70, 1025), (3, 257, 3 * 1024), (2, 300, 4095)])
+def test_wide_tiles_of_small_q(q, n, tail):
+    """q <= 4 with tiles enough for every SM: 4096-bin tiles, the last of them
+    cut by the table's rows (which end on 1024 bins), mixed and uniform reads,
+    non-bases, T <= 0; records and counts alone."""
+    from paper_1708_04329_gb300 import grim, synth
+
+    B = 9
+    g = synth.genome(B * (4096 * 160 + tail), seed=q)
+    rs = synth.reads(g, n, seed=n, lengths=(40, 60) if n > 70 else (40,),
+                     probs=(0.5, 0.5) if n > 70 else (1.0,), e=1, max_edits=1)
+    rs.seq[int(rs.offsets[3]) + 7] = ord("N")
+    if n > 70:
+        rs.e[5] = 60
+    ix = build(g, B, q, 60, layouts=1)
+    want = oracle.filter(oracle.bin_vectors(g, B, q, 60), rs)
+    assert_same(gpu_filter(ix, rs, cap=len(want[0])), want)
+    assert grim.grim_filter_count(ix, **dev_reads(rs)) == len(want[0])
+    ix.close()
