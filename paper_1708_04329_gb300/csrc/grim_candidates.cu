@@ -40,8 +40,11 @@ struct Cfg {
 template <int WL>
 __device__ __forceinline__ void load_words(const uint32_t* p, uint32_t (&v)[WL]) {
   if constexpr (WL == 4) {
-    const uint4 x = __ldg(reinterpret_cast<const uint4*>(p));
-    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+    // a vector is read once: it need not displace the ids and token rows in L1
+    // (330M candidates: 8.66 -> 8.58 ms)
+    asm("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+        : "l"(p));
   } else if constexpr (WL == 2) {
     const uint2 x = __ldg(reinterpret_cast<const uint2*>(p));
     v[0] = x.x; v[1] = x.y;
