@@ -81,8 +81,8 @@ struct TokArgs {
 //
 // Bound by instruction issue.  Measured on GB300 against coding the bases
 // through shared memory, q byte loads a token and a rank by comparing every
-// pair of keys: 250k reads of 100 bp at q = 5 0.77 -> 0.22 ms, 60k of 150 bp at
-// q = 6 0.91 -> 0.11 ms, 1M mixed reads in position order 0.85 -> 0.56 ms, a
+// pair of keys: 250k reads of 100 bp at q = 5 0.77 -> 0.29 ms, 60k of 150 bp at
+// q = 6 0.91 -> 0.12 ms, 1M mixed reads in position order 0.85 -> 0.55 ms, a
 // lone read of 250 bp 67 -> 16 us.
 template <TokenOrder ORDER>
 __global__ void __launch_bounds__(kTokWarps * 32, kTokCtasPerSm) k_tokenise(TokArgs a) {
@@ -144,8 +144,8 @@ __global__ void __launch_bounds__(kTokWarps * 32, kTokCtasPerSm) k_tokenise(TokA
     // bit planes of 32 bases: code bits and not-a-base (A0 C1 G2 T3, case folded)
     auto planes = [&](uint32_t c, uint32_t& lo, uint32_t& hi, uint32_t& inv) {
       const uint32_t u = c & 0xDFu;
-      const bool ok = (u == 0x41u) | (u == 0x43u) | (u == 0x47u) | (u == 0x54u);
-      const uint32_t code = (u >> 1) ^ (u >> 2);
+      const uint32_t code = ((u >> 1) ^ (u >> 2)) & 3u;
+      const bool ok = __byte_perm(0x54474341u, 0u, code | 0x4440u) == u;  // the code's letter
       lo = __ballot_sync(0xFFFFFFFFu, code & 1u);
       hi = __ballot_sync(0xFFFFFFFFu, code & 2u);
       inv = __ballot_sync(0xFFFFFFFFu, !ok);
@@ -176,14 +176,14 @@ __global__ void __launch_bounds__(kTokWarps * 32, kTokCtasPerSm) k_tokenise(TokA
       const uint32_t t = ((z & 0xFFFFu) << 1) | (z >> 16);
       const bool in = 32u * i + lane < ntok;
       if (in) row[i] = unclean ? rowInvalid(r4) : t;
-      const uint32_t inv_mask = __ballot_sync(0xFFFFFFFFu, in && unclean);
       if constexpr (ORDER == TokenOrder::kPosition) {
         if (in) s_seq[warp][32u * i + lane] = (uint16_t)row[i];
       } else {
+        const uint32_t inv_mask = __ballot_sync(0xFFFFFFFFu, in && unclean);
         if (in && unclean)
           s_seq[warp][n_inv + __popc(inv_mask & below)] = (uint16_t)rowInvalid(r4);
+        n_inv += __popc(inv_mask);
       }
-      n_inv += __popc(inv_mask);
       if constexpr (ORDER == TokenOrder::kLines) {
 #pragma unroll
         for (uint32_t k = 0; k < 4; ++k)
