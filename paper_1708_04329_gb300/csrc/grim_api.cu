@@ -352,9 +352,14 @@ int grim_build_ex(const char* ref, uint64_t len, uint32_t B, uint32_t q, uint32_
   // index keeps none), those of q < 5 come from the packed reference
   const uint32_t fused = build_fused_layouts(v, f);
   const bool from_bm_tm = v.q >= 5 && ix->tm && !(fused & GRIM_LAYOUT_TOKEN_MAJOR);
-  const bool from_bm_ctm = v.q >= 5 && ix->ctm && !(fused & GRIM_LAYOUT_COARSE);
+  // q = 6: super-bins' rows leave the one pass a word at a time, 1.1 ms of 6.4
+  // at 1.5 Gbp, B = 100 where it reads the vectors back for the bins' rows anyway
+  // (1.4 as a pass of their own); without those rows 1.5 against 1.4
+  const bool from_bm_ctm = v.q >= 5 && ix->ctm &&
+                           (!(fused & GRIM_LAYOUT_COARSE) || (v.q > 5 && !ix->tm));
   uint32_t* bm = ix->bm;
-  if (!bm && (from_bm_tm || from_bm_ctm)) {
+  // (q = 6: the one pass reads its vectors back for the token rows)
+  if (!bm && (from_bm_tm || from_bm_ctm || (v.q > 5 && ix->tm))) {
     e = scratch_alloc(reinterpret_cast<void**>(&bm), bm_bins * v.wpb * sizeof(uint32_t), st);
     if (e != cudaSuccess) return fail(cuda_fail(e));
   }

@@ -283,12 +283,16 @@ __device__ __forceinline__ void pack16(const uint4& v, uint32_t& code, uint32_t&
 //      for each of the bins whose windows overlap there;
 //   3. (q = 5) the run's 32 vectors, one word a lane, are a 32 x 32 bit
 //      transpose away from the token rows; both token-major tables leave
-//      through shared memory in row pieces of 64 and 64 / f bytes.
+//      through shared memory in row pieces of 64 and 64 / f bytes.  At q = 6
+//      the tile's 256 KB of vectors do not fit there: each thread reads the
+//      words it has just written back from L2, 1024 tokens a pass.
 // Bound by instruction issue (about 250 warp instructions a bin, 71% of the
 // issue slots; the shared atomics take 23% of their pipe), not by its 8.1 GB
 // of letters and tables at 3.1 Gbp, B = 200, q = 5: 4.3 ms there.  Packing the
 // reference, setting each bin's bits from the codes and two transposes from
-// DRAM took 16.0 ms.
+// DRAM took 16.0 ms.  q = 6, 1.5 Gbp, B = 100: 6.4 ms for all tables (17.6 GB,
+// 2.6 ms of copying; half is the 64-byte row pieces), 13.5 with the token rows
+// and the super-bins' as transposes from DRAM, 2.7 for the vectors alone.
 constexpr uint32_t kFusedBins = 512, kFusedWarps = kFusedBins / 32, kFusedMaxK = 3;
 constexpr uint32_t kFusedGroups = kFusedBins / 32;  // tile words of a token row
 
@@ -297,31 +301,32 @@ struct FusedArgs {
   uint64_t n, num_bins, wpad, cwpad;
   uint32_t B, q, k, rem;
   uint32_t code_words;  // code words of the tile in shared memory (16 bases each)
-  uint32_t f;           // coarse factor (ctm set: 2, 4, 8 or 16)
+  uint32_t region_words;  // shared memory before the warps' vectors
+  uint32_t f;           // coarse factor (ctm set: 2, 4, 8 or 16; q = 6: 8 or 16)
   uint32_t* bm;
   uint32_t* tm;
   uint32_t* ctm;
 };
 
-// shared memory, in words: row pieces / vectors of the tile (q = 5), then
-// codes and mask, later the coarse row pieces, then a vector per warp
-__host__ __device__ constexpr uint32_t fused_rows_words(uint32_t wpl) {
-  return wpl == 1 ? 1024u * kFusedGroups + 32u : 0u;
-}
-__host__ __device__ constexpr uint32_t fused_code_words(uint32_t wpl, uint32_t code_words) {
-  const uint32_t c = code_words + (code_words + 1) / 2 + 2;
-  const uint32_t coarse = wpl == 1 ? 1024u * (kFusedGroups / 2) + 32u : 0u;
-  return c > coarse ? c : coarse;
+// shared memory, in words.  q = 5: the tile's vectors, later row pieces; codes
+// and mask, later the coarse row pieces; a vector per warp.  q = 6: codes and
+// mask, later the row pieces of a token chunk and the super-bins' vectors; a
+// vector per warp.
+constexpr uint32_t kFusedRowWords = 1024u * kFusedGroups + 32u;
+__host__ __device__ constexpr uint32_t fused_super_words(uint32_t f) {  // q = 6
+  return f ? 4u * 32u * (kFusedBins / f) : 0u;
 }
 
-// WPL: words of a vector per lane, 1 (q = 5) or 4 (q = 6); K >= k
-template <uint32_t WPL, uint32_t K>
+// WPL: words of a vector per lane, 1 (q = 5) or 4 (q = 6); K >= k; ROWS: the
+// token rows too (at q = 6 a kernel of its own: their shared memory and code
+// cost the vectors alone 7%)
+template <uint32_t WPL, uint32_t K, bool ROWS>
 __global__ void __launch_bounds__(kFusedWarps * 32, 2) k_build_fused(FusedArgs a) {
   extern __shared__ uint32_t s_fused[];
   uint32_t* s_rows = s_fused;
-  uint32_t* s_code = s_fused + fused_rows_words(WPL);
+  uint32_t* s_code = s_fused + (WPL == 1 ? kFusedRowWords : 0u);
   uint16_t* inv16 = reinterpret_cast<uint16_t*>(s_code + a.code_words);  // 16 positions each
-  uint32_t* s_vec = s_code + fused_code_words(WPL, a.code_words);
+  uint32_t* s_vec = s_fused + a.region_words;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint64_t bin0 = (uint64_t)blockIdx.x * kFusedBins;
   const uint64_t p0 = bin0 * a.B;  // a multiple of 512: 16-byte aligned in an aligned reference
@@ -433,7 +438,61 @@ __global__ void __launch_bounds__(kFusedWarps * 32, 2) k_build_fused(FusedArgs a
     }
     __syncwarp();
   }
-  if (WPL != 1 || (!a.tm && !a.ctm)) return;
+  if (!ROWS || (!a.tm && !a.ctm)) return;
+
+  // 3. (q = 6) 1024 tokens at a time, a thread's words of its run's vectors
+  // come back from L2, where it has just written them
+  if constexpr (WPL == 4 && ROWS) {
+    uint32_t* s_super = s_rows + kFusedRowWords;  // [chunk][super-bin of the tile][lane]
+    const uint32_t supers = a.ctm ? kFusedBins / a.f : 0u;
+    const uint32_t* in = a.bm + (bin0 + first) * 128 + lane;
+    const uint64_t col0 = (uint64_t)blockIdx.x * kFusedGroups;
+#pragma unroll 1
+    for (uint32_t c = 0; c < 4; ++c) {
+      uint32_t x[32];
+#pragma unroll
+      for (uint32_t k = 0; k < 32; ++k) x[k] = k < rows ? __ldcg(in + k * 128 + c * 32) : 0u;
+      __syncthreads();  // codes, or the last chunk's rows, are no longer read
+      if (supers) {
+        uint32_t* to = s_super + (c * supers + first / a.f) * 32 + lane;
+        uint32_t w = 0;
+#pragma unroll
+        for (uint32_t k = 0; k < 32; ++k) {
+          w |= x[k];
+          if (((k + 1) & (a.f - 1)) == 0) {
+            *to = w;
+            to += 32;
+            w = 0;
+          }
+        }
+      }
+      if (col0 >= a.wpad) continue;
+      transpose32(x);
+#pragma unroll
+      for (uint32_t j = 0; j < 32; ++j) s_rows[(32u * lane + j) * kFusedGroups + warp + lane] = x[j];
+      __syncthreads();
+      uint32_t* dst = a.tm + (1024u * c + tid / kFusedGroups) * a.wpad + col0 + tid % kFusedGroups;
+#pragma unroll 8
+      for (uint32_t j = 0; j < 32; ++j, dst += 32 * a.wpad)
+        *dst = s_rows[tid + j * (32 * kFusedGroups + 1)];
+    }
+    __syncthreads();
+    const uint32_t words = supers / 32;  // of a coarse row
+    const uint64_t ccol0 = (uint64_t)blockIdx.x * words;
+    if (ccol0 < a.cwpad) {
+      for (uint32_t i = warp; i < 4 * words; i += kFusedWarps) {
+        uint32_t x[32];
+#pragma unroll
+        for (uint32_t k = 0; k < 32; ++k)
+          x[k] = s_super[(i / words * supers + i % words * 32 + k) * 32 + lane];
+        transpose32(x);
+        uint32_t* dst = a.ctm + (1024u * (i / words) + 32u * lane) * a.cwpad + ccol0 + i % words;
+#pragma unroll
+        for (uint32_t j = 0; j < 32; ++j, dst += a.cwpad) *dst = x[j];
+      }
+    }
+    return;
+  }
 
   // 3. token rows: the coarse table's from the ORs of f vectors, then the bins'
   __syncthreads();  // vectors complete, codes no longer read
@@ -520,23 +579,29 @@ uint64_t fused_tile_words(const IndexView& v) {  // code words of a tile
   const uint32_t span = v.ext - v.q + 1;
   return ((uint64_t)(kFusedBins + span / v.B) * v.B + span % v.B + v.q + 15) / 16 + 1;
 }
-size_t fused_smem(const IndexView& v) {
-  const uint32_t wpl = v.wpb / 32;
-  return sizeof(uint32_t) * (fused_rows_words(wpl) +
-                             fused_code_words(wpl, (uint32_t)fused_tile_words(v)) +
-                             kFusedWarps * 32 * wpl);
+uint32_t fused_super_factor(uint32_t q, uint32_t f) {  // 0: not this kernel's
+  // whole row words of super-bins in a tile; at q = 6 their vectors of all
+  // 4096 tokens wait in shared memory (16 KB at f = 16, 128 KB at f = 2)
+  return f > (q == 5 ? 1u : 7u) && kFusedGroups % f == 0 ? f : 0u;
+}
+uint32_t fused_region_words(const IndexView& v, uint32_t f, bool rows) {
+  const uint32_t words = (uint32_t)fused_tile_words(v);
+  const uint32_t codes = words + (words + 1) / 2 + 2;
+  if (v.q == 5) return kFusedRowWords + std::max(codes, 1024u * (kFusedGroups / 2) + 32u);
+  if (!rows) return codes;
+  return std::max(codes, kFusedRowWords + fused_super_words(fused_super_factor(v.q, f)));
+}
+size_t fused_smem(const IndexView& v, uint32_t f, bool rows) {
+  return sizeof(uint32_t) * (fused_region_words(v, f, rows) + kFusedWarps * v.wpb);
 }
 }  // namespace
 
 uint32_t build_fused_layouts(const IndexView& v, uint32_t f) {
   if (v.q < 5 || (v.ext - v.q + 1) / v.B > kFusedMaxK || fused_tile_words(v) > 65536 ||
-      fused_smem(v) > 227 * 1024)
+      fused_smem(v, f, true) > 227 * 1024)
     return 0;
-  uint32_t can = GRIM_LAYOUT_BIN_MAJOR;
-  if (v.q == 5) can |= GRIM_LAYOUT_TOKEN_MAJOR;
-  // whole row words of super-bins in a tile
-  if (v.q == 5 && f > 1 && kFusedGroups % f == 0) can |= GRIM_LAYOUT_COARSE;
-  return can;
+  return GRIM_LAYOUT_BIN_MAJOR | GRIM_LAYOUT_TOKEN_MAJOR |
+         (fused_super_factor(v.q, f) ? GRIM_LAYOUT_COARSE : 0u);
 }
 
 void launch_build_fused(const char* ref, const IndexView& v, const IndexView& cv, uint32_t f,
@@ -561,14 +626,18 @@ void launch_build_fused(const char* ref, const IndexView& v, const IndexView& cv
   uint64_t grid = (v.num_bins + kFusedBins - 1) / kFusedBins;
   if (tm) grid = v.num_bins_pad / kFusedBins;
   if (ctm && cv.num_bins_pad * f / kFusedBins > grid) grid = cv.num_bins_pad * f / kFusedBins;
-  const size_t smem = fused_smem(v);
+  const bool rows = v.q == 5 || tm;
+  a.region_words = fused_region_words(v, f, rows);
+  const size_t smem = fused_smem(v, f, rows);
   ProfScope ps("build_fused", st);
   auto run = [&](auto kernel) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     kernel<<<(unsigned)grid, kFusedWarps * 32, smem, st>>>(a);
   };
-  if (v.q == 5) run(a.k <= 1 ? k_build_fused<1, 1> : k_build_fused<1, kFusedMaxK>);
-  else run(a.k <= 1 ? k_build_fused<4, 1> : k_build_fused<4, kFusedMaxK>);
+  const bool near = a.k <= 1;
+  if (v.q == 5) run(near ? k_build_fused<1, 1, true> : k_build_fused<1, kFusedMaxK, true>);
+  else if (rows) run(near ? k_build_fused<4, 1, true> : k_build_fused<4, kFusedMaxK, true>);
+  else run(near ? k_build_fused<4, 1, false> : k_build_fused<4, kFusedMaxK, false>);
 }
 
 void launch_pack_ref(const char* ref, uint64_t n, uint32_t* codes, uint32_t* invalid,

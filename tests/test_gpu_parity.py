@@ -693,6 +693,20 @@ def test_one_pass_build_shapes(q, B, mrl, factor, n, layouts, shift):
     idx.close()
 
 
+@pytest.mark.parametrize("B,mrl,factor,n,layouts,shift", [
+    (100, 150, 16, 1024 * 16 * 100 + 1, 7, 0),  # one coarse row pad and a base; full tiles
+    (100, 150, 8, 512 * 8 * 100 - 3, 7, 1),     # two coarse words a tile
+    (90, 250, 8, 200_003, 4, 0),                # super-bins alone, the vectors in scratch
+    (128, 150, 16, 70_000, 1, 3),               # rows alone
+    (61, 250, 16, 333_333, 6, 0),               # more cores than the one-pass build takes
+    (400, 100, 2, 450_000, 7, 0),               # a factor whose vectors have no room
+    (900, 6, 8, 512 * 900 + 5, 7, 0)])          # codes larger than the row pieces
+def test_one_pass_build_q6_rows(B, mrl, factor, n, layouts, shift):
+    """Token rows and super-bins of q = 6 from the one-pass build, against the
+    oracle."""
+    test_one_pass_build_shapes(6, B, mrl, factor, n, layouts, shift)
+
+
 @pytest.mark.parametrize("q,B,mrl,layouts", [(5, 50, 250, 7), (5, 50, 100, 1), (6, 100, 150, 6)])
 def test_few_reads_on_a_large_table(q, B, mrl, layouts):
     """Batches of a few reads load table rows instead of staging tiles: counts
