@@ -352,7 +352,7 @@ int grim_build_ex(const char* ref, uint64_t len, uint32_t B, uint32_t q, uint32_
   // index keeps none), those of q < 5 come from the packed reference
   const uint32_t fused = build_fused_layouts(v, f);
   const bool from_bm_tm = v.q >= 5 && ix->tm && !(fused & GRIM_LAYOUT_TOKEN_MAJOR);
-  // q = 6: super-bins' rows leave the one pass a word at a time, 1.1 ms of 6.4
+  // q = 6: super-bins' rows leave the one pass a word at a time, 1.1 ms of 6.2
   // at 1.5 Gbp, B = 100 where it reads the vectors back for the bins' rows anyway
   // (1.4 as a pass of their own); without those rows 1.5 against 1.4
   const bool from_bm_ctm = v.q >= 5 && ix->ctm &&

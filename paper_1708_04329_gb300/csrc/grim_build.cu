@@ -286,13 +286,15 @@ __device__ __forceinline__ void pack16(const uint4& v, uint32_t& code, uint32_t&
 //      through shared memory in row pieces of 64 and 64 / f bytes.  At q = 6
 //      the tile's 256 KB of vectors do not fit there: each thread reads the
 //      words it has just written back from L2, 1024 tokens a pass.
-// Bound by instruction issue (about 250 warp instructions a bin, 71% of the
-// issue slots; the shared atomics take 23% of their pipe), not by its 8.1 GB
-// of letters and tables at 3.1 Gbp, B = 200, q = 5: 4.3 ms there.  Packing the
-// reference, setting each bin's bits from the codes and two transposes from
-// DRAM took 16.0 ms.  q = 6, 1.5 Gbp, B = 100: 6.4 ms for all tables (17.6 GB,
-// 2.6 ms of copying; half is the 64-byte row pieces), 13.5 with the token rows
-// and the super-bins' as transposes from DRAM, 2.7 for the vectors alone.
+// Bound by instruction issue (235 warp instructions a bin, 70% of the issue
+// slots; the shared atomics take 29% of their pipe), not by its 8.1 GB of
+// letters and tables at 3.1 Gbp, B = 200, q = 5: 4.1 ms there (4.3 with the
+// runs' masks worked out for every core).  Packing the reference, setting each
+// bin's bits from the codes and two transposes from DRAM took 16.0 ms.
+// q = 6, 1.5 Gbp, B = 100: 6.2 ms for all tables (17.6 GB, 2.6 ms of copying;
+// 295 instructions a bin, 58% of the slots, and the 64-byte row pieces), 13.5
+// with the token rows and the super-bins' as transposes from DRAM, 2.6 for the
+// vectors alone.
 constexpr uint32_t kFusedBins = 512, kFusedWarps = kFusedBins / 32, kFusedMaxK = 3;
 constexpr uint32_t kFusedGroups = kFusedBins / 32;  // tile words of a token row
 
@@ -354,48 +356,58 @@ __global__ void __launch_bounds__(kFusedWarps * 32, 2) k_build_fused(FusedArgs a
   any = __syncthreads_or(any);
 
   // 2. tokens starting at tile positions [lo, lo + len) into the warp's
-  // vector: a lane takes `per` consecutive positions, whose per + q - 1 <= 16
-  // bases it aligns into one register, so a token costs two shifts for its
-  // bit, a shift and a mask for its word, and the atomic
+  // vector: a lane takes `per` consecutive positions (a run), whose
+  // per + q - 1 <= 16 bases it aligns into one register, so a token costs two
+  // shifts for its bit, a shift and a mask for its word, and the atomic
   constexpr uint32_t kQ = WPL == 1 ? 5u : 6u, kMost = 17u - kQ;  // positions per lane
   constexpr uint32_t kBitShift = 32u - 2u * kQ, kWordMask = ((1u << (2u * kQ - 5u)) - 1u) << 2;
   const uint32_t v_base = (uint32_t)__cvta_generic_to_shared(v);
-  auto set_tokens = [&](uint32_t lo, uint32_t len, uint32_t per) {
-    for (uint32_t at = lane * per; at < len; at += 32u * per) {
-      const uint32_t p = lo + at;
-      uint32_t ok = (1u << min(per, len - at)) - 1u;
-      const uint32_t* c = s_code + (p >> 4);
-      const uint32_t x = __funnelshift_l(c[1], c[0], 2u * p);
-      if (any) {
-        const uint16_t* m16 = inv16 + (p >> 4);
-        const uint32_t m = ((uint32_t)m16[0] | ((uint32_t)m16[1] << 16)) >> (p & 15u);
-        uint32_t bad = m;
+  auto set_run = [&](uint32_t p, uint32_t ok, uint32_t per) {
+    const uint32_t* c = s_code + (p >> 4);
+    const uint32_t x = __funnelshift_l(c[1], c[0], 2u * p);
+    if (any) {
+      const uint16_t* m16 = inv16 + (p >> 4);
+      const uint32_t m = ((uint32_t)m16[0] | ((uint32_t)m16[1] << 16)) >> (p & 15u);
+      uint32_t bad = m;
 #pragma unroll
-        for (uint32_t i = 1; i < kQ; ++i) bad |= m >> i;
-        ok &= ~bad;
-      }
-      auto set = [&](uint32_t i) {
-        asm volatile(
-            "{\n.reg .pred p;\nsetp.ne.u32 p, %2, 0;\n@p red.shared.or.b32 [%0], %1;\n}" ::"r"(
-                v_base + ((x >> (kBitShift + 3u - 2u * i)) & kWordMask)),
-            "r"(1u << ((x >> (kBitShift - 2u * i)) & 31u)), "r"(ok & (1u << i))
-            : "memory");
-      };
+      for (uint32_t i = 1; i < kQ; ++i) bad |= m >> i;
+      ok &= ~bad;
+    }
+    auto set = [&](uint32_t i) {
+      asm volatile(
+          "{\n.reg .pred p;\nsetp.ne.u32 p, %2, 0;\n@p red.shared.or.b32 [%0], %1;\n}" ::"r"(
+              v_base + ((x >> (kBitShift + 3u - 2u * i)) & kWordMask)),
+          "r"(1u << ((x >> (kBitShift - 2u * i)) & 31u)), "r"(ok & (1u << i))
+          : "memory");
+    };
 #pragma unroll
-      for (uint32_t i = 0; i < 4; ++i) set(i);
-      if (per > 4) {
+    for (uint32_t i = 0; i < 3; ++i) set(i);
+    if (per > 3) set(3);
+    if (per > 4) {
 #pragma unroll
-        for (uint32_t i = 4; i < 8; ++i) set(i);
-      }
-      if (per > 8) {
+      for (uint32_t i = 4; i < 8; ++i) set(i);
+    }
+    if (per > 8) {
 #pragma unroll
-        for (uint32_t i = 8; i < kMost; ++i) set(i);
-      }
+      for (uint32_t i = 8; i < kMost; ++i) set(i);
     }
   };
+  // a lane's first run in a core's first `rem` positions and in the rest: its
+  // offset (0 for a lane without one) and which of its tokens exist
   const uint32_t rest = a.B - a.rem;
   const uint32_t per_p = max(1u, min(kMost, (a.rem + 31u) / 32u));
   const uint32_t per_r = min(kMost, (rest + 31u) / 32u);
+  auto mask_of = [&](uint32_t at, uint32_t len, uint32_t per) {
+    return at < len ? (1u << min(per, len - at)) - 1u : 0u;
+  };
+  const uint32_t ok_p = mask_of(lane * per_p, a.rem, per_p), at_p = ok_p ? lane * per_p : 0u;
+  const uint32_t ok_r = mask_of(lane * per_r, rest, per_r), at_r = ok_r ? lane * per_r : 0u;
+  auto set_tokens = [&](uint32_t lo, uint32_t len, uint32_t per, uint32_t at, uint32_t ok) {
+    set_run(lo + at, ok, per);
+    if (len > 32u * per)  // (more than 32 lanes' runs)
+      for (at += 32u * per; at < len; at += 32u * per)
+        set_run(lo + at, mask_of(at, len, per), per);
+  };
   uint32_t pend[K + 1][WPL];  // bins c - k .. c so far (newest first)
 #pragma unroll
   for (uint32_t i = 0; i <= K; ++i)
@@ -409,7 +421,7 @@ __global__ void __launch_bounds__(kFusedWarps * 32, 2) k_build_fused(FusedArgs a
   uint32_t* out = a.bm + (bin0 + first) * (32 * WPL) + lane;
   uint32_t lo = first * a.B;
   for (uint32_t c = 0; c <= 32 + a.k; ++c, lo += a.B) {
-    set_tokens(lo, a.rem, per_p);
+    set_tokens(lo, a.rem, per_p, at_p, ok_p);
     __syncwarp();
     // core c's first positions complete bin c - k - 1
     if (c > a.k) {
@@ -426,7 +438,7 @@ __global__ void __launch_bounds__(kFusedWarps * 32, 2) k_build_fused(FusedArgs a
       out += 32 * WPL;
       if (done == 31) break;
     }
-    set_tokens(lo + a.rem, rest, per_r);
+    set_tokens(lo + a.rem, rest, per_r, at_r, ok_r);
     __syncwarp();
 #pragma unroll
     for (uint32_t w = 0; w < WPL; ++w) {
