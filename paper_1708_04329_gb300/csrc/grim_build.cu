@@ -1,7 +1,7 @@
 // Index build (§GRIM-Filter: the reference is scanned once and every bin's
 // bit vector is set from the tokens that occur in it; Fig. 2):
-//   k_build_fused       q = 5, 6: ASCII straight to bin-major vectors and, at
-//                       q = 5, both token-major tables in one pass
+//   k_build_fused       q = 5, 6: ASCII straight to bin-major vectors and both
+//                       token-major tables in one pass
 //   k_pack_ref          ASCII -> 2-bit codes + not-a-base mask (the kernels below)
 //   k_build_bin_major   one warp per bin, bit vector in shared memory
 //   k_build_token_major one CTA per 1024-bin tile, the tile's [4^q rows x tile

@@ -135,7 +135,8 @@ void launch_pack_ref(const char* ref, uint64_t n, uint32_t* codes, uint32_t* inv
 // One pass from the letters to the tables.  build_fused_layouts: the tables
 // (GRIM_LAYOUT_*) it can write for an index's shape and coarse factor f, 0
 // when the shape is left to the kernels below (q < 5, windows of more than
-// four cores, a tile past shared memory).
+// four cores, a tile past shared memory).  At q = 6 the token rows need bm,
+// and ctm needs tm.
 uint32_t build_fused_layouts(const IndexView& v, uint32_t f);
 void launch_build_fused(const char* ref, const IndexView& v, const IndexView& cv, uint32_t f,
                         uint32_t* bm, uint32_t* tm, uint32_t* ctm, cudaStream_t st);
