@@ -437,6 +437,7 @@ __global__ void __launch_bounds__(kFusedWarps * 32, 2) k_build_fused(FusedArgs a
       }
       out += 32 * WPL;
       if (done == 31) break;
+      __syncwarp();  // the vector is read: the core's other tokens may be set
     }
     set_tokens(lo + a.rem, rest, per_r, at_r, ok_r);
     __syncwarp();
