@@ -563,11 +563,11 @@ void launch_tm_from_bm(const uint32_t* bm, const IndexView& unit_view, uint32_t 
   const uint64_t grid = unit_view.num_bins_pad / (tw * 32);
   ProfScope ps("transpose_token_major", st);
   if (tw == 32) {
-    cudaFuncSetAttribute(k_tm_from_bm<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(k_tm_from_bm<32>);
     k_tm_from_bm<32><<<(unsigned)grid, 1024, smem, st>>>(bm, wpb, f, unit_view.num_bins, r4,
                                                          unit_view.wpad, tm);
   } else {
-    cudaFuncSetAttribute(k_tm_from_bm<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(k_tm_from_bm<8>);
     k_tm_from_bm<8><<<(unsigned)grid, 1024, smem, st>>>(bm, wpb, f, unit_view.num_bins, r4,
                                                         unit_view.wpad, tm);
   }
@@ -611,7 +611,7 @@ size_t fused_smem(const IndexView& v, uint32_t f, bool rows) {
 
 uint32_t build_fused_layouts(const IndexView& v, uint32_t f) {
   if (v.q < 5 || (v.ext - v.q + 1) / v.B > kFusedMaxK || fused_tile_words(v) > 65536 ||
-      fused_smem(v, f, true) > 227 * 1024)
+      fused_smem(v, f, true) > kSmemMost)
     return 0;
   return GRIM_LAYOUT_BIN_MAJOR | GRIM_LAYOUT_TOKEN_MAJOR |
          (fused_super_factor(v.q, f) ? GRIM_LAYOUT_COARSE : 0u);
@@ -644,7 +644,7 @@ void launch_build_fused(const char* ref, const IndexView& v, const IndexView& cv
   const size_t smem = fused_smem(v, f, rows);
   ProfScope ps("build_fused", st);
   auto run = [&](auto kernel) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(kernel);
     kernel<<<(unsigned)grid, kFusedWarps * 32, smem, st>>>(a);
   };
   const bool near = a.k <= 1;
@@ -678,8 +678,7 @@ void launch_build_token_major(const uint32_t* codes, const uint32_t* invalid, co
   // 8 words (256 bins) at q = 6
   uint32_t tile_words = ix.r4 <= 1024 ? 32u : 32768u / ix.r4;
   size_t smem = (size_t)ix.r4 * tile_words * sizeof(uint32_t);
-  cudaFuncSetAttribute(k_build_token_major, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)smem);
+  allow_smem(k_build_token_major);
   uint64_t grid = (ix.num_bins_pad / 32) / tile_words;
   ProfScope ps("build_token_major", st);
   k_build_token_major<<<(unsigned)grid, 512, smem, st>>>(codes, invalid, ix, tile_words, tm);

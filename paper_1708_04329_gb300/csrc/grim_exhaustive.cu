@@ -67,7 +67,7 @@ namespace {
 // 2.4% at q = 6, and 512 by 2.6%; the autotuner can pick another.
 constexpr uint32_t kDefaultThreads = 640;
 constexpr uint32_t kNone = 0xFFFFFFFFu;
-constexpr size_t kSmemLimit = 227 * 1024;  // dynamic shared memory per CTA
+constexpr size_t kSmemLimit = kSmemMost - 128;  // dynamic shared memory per CTA (128 bytes are static)
 // token rows of one read range: small enough to stay in L2 while every CTA
 // sweeps its tiles against the range
 constexpr uint64_t kDefaultRangeBytes = 48ull << 20;
@@ -979,7 +979,7 @@ __global__ void __launch_bounds__(kFewThreads, 2) k_exhaustive_few(ExhArgs a) {
 template <typename Kernel>
 void launch_k(Kernel kernel, const ExhArgs& a, size_t smem, uint32_t threads, uint32_t grid,
               cudaStream_t st, const char* name) {
-  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem(kernel, kSmemLimit);
   ProfScope ps(name, st);
   kernel<<<grid, threads, smem, st>>>(a);
 }

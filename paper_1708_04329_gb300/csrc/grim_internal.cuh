@@ -127,6 +127,15 @@ struct RecordsView {
   uint64_t cap;
 };
 
+// Shared memory of a CTA, static and dynamic.  How much of it launches may ask
+// for dynamically is kept with the function, for all threads: every launch of a
+// kernel allows the same, so that none takes away what another is about to use.
+constexpr size_t kSmemMost = 227 * 1024;
+template <typename Kernel>
+inline void allow_smem(Kernel kernel, size_t most = kSmemMost) {
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // ---------------------------------------------------------------------------
 // launchers (each enqueues on `st`; errors surface through cudaGetLastError)
 // ---------------------------------------------------------------------------
