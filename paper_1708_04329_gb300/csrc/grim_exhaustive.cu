@@ -931,12 +931,16 @@ __global__ void __launch_bounds__(kFewThreads, 2) k_exhaustive_few(ExhArgs a) {
       alive += ldead ? 0u : 1u;
       if (__all_sync(0xFFFFFFFFu, ldead)) break;
     }
-    // blocks each 1024-bin tile needed, as the staged kernel counts them
+    // blocks each tile (of 1024 bins, 256 at q = 6) needed, as the staged kernel
+    // counts them
+    const uint32_t tile_lanes = r4 <= 1024 ? 8u : 2u;
     uint32_t used = alive;
     used = max(used, __shfl_xor_sync(0xFFFFFFFFu, used, 1));
-    used = max(used, __shfl_xor_sync(0xFFFFFFFFu, used, 2));
-    used = max(used, __shfl_xor_sync(0xFFFFFFFFu, used, 4));
-    used = (lane & 7u) == 0 && on ? min(nblk, used + 1u) : 0u;
+    if (tile_lanes == 8) {
+      used = max(used, __shfl_xor_sync(0xFFFFFFFFu, used, 2));
+      used = max(used, __shfl_xor_sync(0xFFFFFFFFu, used, 4));
+    }
+    used = lane % tile_lanes == 0 && on ? min(nblk, used + 1u) : 0u;
     used = __reduce_add_sync(0xFFFFFFFFu, used);
     if (lane == 0) atomicAdd(&a.ctl->blocks, 2ull * used);  // (counted in halves)
     if (__all_sync(0xFFFFFFFFu, ldead)) continue;
