@@ -228,22 +228,28 @@ __global__ void __launch_bounds__(512) k_row_popcount(const uint32_t* __restrict
 
 // A token's rank among the tokens of its class (token % classes): how many of
 // them fewer (super-)bins hold, ties by value; and the share of the `units`
-// (super-)bins without it.
-__global__ void __launch_bounds__(128) k_token_ranks(const uint32_t* __restrict__ presence,
-                                                     uint32_t rows, uint32_t classes, float units,
-                                                     uint16_t* __restrict__ rank,
-                                                     float* __restrict__ miss) {
-  __shared__ uint32_t s_p[4096];  // q <= 6
-  for (uint32_t i = threadIdx.x; i < rows; i += 128) s_p[i] = presence[i];
-  __syncthreads();
-  const uint32_t t = blockIdx.x * 128 + threadIdx.x;
+// (super-)bins without it.  A warp per token, bound by the latency of its loads:
+// with a thread per token the walk over the class took 37 us at q = 5, longer
+// than the other kernels of a small build, this 12 (a launch that does nothing
+// reads 5; 1 Mbp, B = 200, whole call 241 -> 211 us).
+constexpr uint32_t kRanksWarps = 8;
+__global__ void __launch_bounds__(kRanksWarps * 32) k_token_ranks(
+    const uint32_t* __restrict__ presence, uint32_t rows, uint32_t classes, float units,
+    uint16_t* __restrict__ rank, float* __restrict__ miss) {
+  const uint32_t t = blockIdx.x * kRanksWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (t >= rows) return;
-  const uint32_t mine = s_p[t];
+  const uint32_t mine = __ldg(presence + t);
   uint32_t r = 0;
-  for (uint32_t i = t % classes; i < rows; i += classes)
-    r += s_p[i] < mine || (s_p[i] == mine && i < t);
-  rank[t] = (uint16_t)r;
-  miss[t] = fmaxf(0.f, 1.f - (float)mine / units);
+#pragma unroll 16
+  for (uint32_t i = t % classes + lane * classes; i < rows; i += 32 * classes) {
+    const uint32_t p = __ldg(presence + i);
+    r += p < mine || (p == mine && i < t);
+  }
+  r = __reduce_add_sync(0xFFFFFFFFu, r);
+  if (lane == 0) {
+    rank[t] = (uint16_t)r;
+    miss[t] = fmaxf(0.f, 1.f - (float)mine / units);
+  }
 }
 
 // 16 bases (bytes, first base lowest) to a code word (first base in the top
@@ -581,10 +587,9 @@ void launch_presence(const uint32_t* tm, const IndexView& units, uint32_t* prese
     k_row_popcount<<<rows, 512, 0, st>>>(tm, units.wpad, presence);
   }
   ProfScope ps("token_ranks", st);
-  k_token_ranks<<<(rows + 127) / 128, 128, 0, st>>>(presence, rows, rows > 1024 ? 4u : 1u,
-                                                    (float)units.num_bins,
-                                                    rank_table(presence, rows),
-                                                    miss_table(presence, rows));
+  k_token_ranks<<<(rows + kRanksWarps - 1) / kRanksWarps, kRanksWarps * 32, 0, st>>>(
+      presence, rows, rows > 1024 ? 4u : 1u, (float)units.num_bins, rank_table(presence, rows),
+      miss_table(presence, rows));
 }
 
 namespace {
