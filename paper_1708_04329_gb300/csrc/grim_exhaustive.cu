@@ -195,8 +195,10 @@ struct CsaTemps {
 
 // Add the misses of four tokens, the quad-th of a 16-token block, whose
 // existence words are a0..a3; the block's last quad carries into the upper
-// planes.
-template <int P, int NW>
+// planes.  FMA: fa_fma for the adders of weight 4 and 8.  k_exhaustive does
+// without and is handed the row count in stage_tile, or it spills at P = 5: 4,000
+// reads of 100 bp in one pass over 1.5M bins, GROUP, 2.32 -> 2.16 ms.
+template <int P, int NW, bool FMA>
 __device__ __forceinline__ void add_quad(Counters<P>& c, CsaTemps<NW>& t, int quad,
                                          const uint32_t (&a0)[NW], const uint32_t (&a1)[NW],
                                          const uint32_t (&a2)[NW], const uint32_t (&a3)[NW],
@@ -207,10 +209,14 @@ __device__ __forceinline__ void add_quad(Counters<P>& c, CsaTemps<NW>& t, int qu
     fa_miss(c.s1[w], a0[w], a1[w], c.s1[w], t.t2a[w]);
     fa_miss(c.s1[w], a2[w], a3[w], c.s1[w], t.t2b[w]);
     fa(c.s2[w], t.t2a[w], t.t2b[w], c.s2[w], t4[w]);
-    if (quad == 1) fa_fma(c.s4[w], t.t4a[w], t.t4b[w], c.s4[w], t.t8a[w], one, m2);
+    auto fa_high = [&](uint32_t a, uint32_t b, uint32_t x, uint32_t& s, uint32_t& k) {
+      if constexpr (FMA) fa_fma(a, b, x, s, k, one, m2);
+      else fa(a, b, x, s, k);
+    };
+    if (quad == 1) fa_high(c.s4[w], t.t4a[w], t.t4b[w], c.s4[w], t.t8a[w]);
     if (quad == 3) {
-      fa_fma(c.s4[w], t.t4a[w], t.t4b[w], c.s4[w], t.t8b[w], one, m2);
-      fa_fma(c.s8[w], t.t8a[w], t.t8b[w], c.s8[w], t.t16[w], one, m2);
+      fa_high(c.s4[w], t.t4a[w], t.t4b[w], c.s4[w], t.t8b[w]);
+      fa_high(c.s8[w], t.t8a[w], t.t8b[w], c.s8[w], t.t16[w]);
       // ripple the weight-16 carry through the upper planes; the carry out
       // of the top plane (counter >= 2^P: misses > D') sticks in `dead`
       uint32_t k = t.t16[w];
@@ -231,7 +237,7 @@ __device__ __forceinline__ void add_quad(Counters<P>& c, CsaTemps<NW>& t, int qu
 // Add the misses of one 16-token block to the lane's four words.  tw holds 16
 // table row indices as uint16 pairs; base is the shared address of this lane's
 // words in row 0 (one 16-byte load per token).
-template <int P>
+template <int P, bool FMA>
 __device__ __forceinline__ void add_block(Counters<P>& c, const uint32_t (&tw)[8], uint32_t base,
                                           const ExhArgs& a) {
   uint32_t addr[16];
@@ -249,7 +255,7 @@ __device__ __forceinline__ void add_block(Counters<P>& c, const uint32_t (&tw)[8
     const uint4 x2 = lds128(addr[4 * quad + 2]), x3 = lds128(addr[4 * quad + 3]);
     const uint32_t a0[4] = {x0.x, x0.y, x0.z, x0.w}, a1[4] = {x1.x, x1.y, x1.z, x1.w};
     const uint32_t a2[4] = {x2.x, x2.y, x2.z, x2.w}, a3[4] = {x3.x, x3.y, x3.z, x3.w};
-    add_quad<P, 4>(c, t, quad, a0, a1, a2, a3, a.c_one, a.c_minus_two);
+    add_quad<P, 4, FMA>(c, t, quad, a0, a1, a2, a3, a.c_one, a.c_minus_two);
   }
 }
 
@@ -341,11 +347,11 @@ __device__ __forceinline__ void fill_special_rows(uint32_t* tile, uint32_t r4, u
 
 // start copying a tile: rows [0, r4), words [tile*TW, tile*TW+TW)
 template <int TW>
-__device__ __forceinline__ void stage_tile(const ExhArgs& a, uint32_t tile, uint32_t sh_base,
-                                           uint32_t tid, uint32_t nthreads) {
+__device__ __forceinline__ void stage_tile(const ExhArgs& a, uint32_t r4, uint32_t tile,
+                                           uint32_t sh_base, uint32_t tid, uint32_t nthreads) {
   constexpr uint32_t kChunks = TW / 4;  // 16-byte chunks per row
   const uint32_t* src = a.ix.tm + (uint64_t)tile * TW;
-  for (uint32_t i = tid; i < a.ix.r4 * kChunks; i += nthreads) {
+  for (uint32_t i = tid; i < r4 * kChunks; i += nthreads) {
     const uint32_t row = i / kChunks, chunk = i % kChunks;
     // (rows end on 1024 bins; the bins of a larger tile past them start out dead)
     if (TW > 32 && (uint64_t)tile * TW + chunk * 4u >= a.ix.wpad) continue;
@@ -402,7 +408,7 @@ __global__ void __launch_bounds__(NT, 1) k_exhaustive(ExhArgs a) {
     const uint32_t r0 = range * rg.per;
     const uint32_t nr = min(rg.per, n_reads - r0);
 
-    stage_tile<TW>(a, tile, sh_base, tid, nthreads);
+    stage_tile<TW>(a, r4, tile, sh_base, tid, nthreads);
 
     // which bins of this lane's words exist (only the last tile is ragged)
     uint32_t vm[4];
@@ -551,7 +557,7 @@ __global__ void __launch_bounds__(NT, 1) k_exhaustive(ExhArgs a) {
           t1 = __ldg(g + 1);
         }
         const uint32_t tw[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
-        add_block<P>(c, tw, lane_base, a);
+        add_block<P, false>(c, tw, lane_base, a);
       }
       tp += step;
       --left;
@@ -643,7 +649,7 @@ __global__ void __launch_bounds__(NT, 1) k_lockstep(ExhArgs a) {
     const uint32_t range = rg.range_major ? item / a.n_tiles : item % rg.n_ranges;
     const uint32_t r0 = range * rg.per;
     const uint32_t nr = min(rg.per, n_reads - r0);
-    stage_tile<TW>(a, tile, sh_base, tid, nthreads);
+    stage_tile<TW>(a, r4, tile, sh_base, tid, nthreads);
     // the last tile may be ragged: bins past the table's end start out dead
     const bool ragged = (uint64_t)(tile + 1) * kTileBinsT > a.ix.num_bins;
 
@@ -715,7 +721,7 @@ __global__ void __launch_bounds__(NT, 1) k_lockstep(ExhArgs a) {
         const uint4 t1 = tokens_at(2 * b + 1, tp + 16u, far, have);
         const uint32_t tw[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
         tp += 2u * step;
-        add_block<P>(c, tw, lane_base, a);
+        add_block<P, true>(c, tw, lane_base, a);
       }
       if (h & 1u) {
         const uint4 t0 = tokens_at(h - 1u, tp, far, have);
@@ -925,7 +931,7 @@ __global__ void __launch_bounds__(kFewThreads, 2) k_exhaustive_few(ExhArgs a) {
       CsaTemps<4> t;
 #pragma unroll
       for (int quad = 0; quad < 4; ++quad)
-        add_quad<P, 4>(c, t, quad, x[4 * quad], x[4 * quad + 1], x[4 * quad + 2], x[4 * quad + 3],
+        add_quad<P, 4, true>(c, t, quad, x[4 * quad], x[4 * quad + 1], x[4 * quad + 2], x[4 * quad + 3],
                        a.c_one, a.c_minus_two);
       ldead = !on || (c.dead[0] & c.dead[1] & c.dead[2] & c.dead[3]) == ~0u;
       alive += ldead ? 0u : 1u;
