@@ -18,6 +18,13 @@ constexpr int kTokCtasPerSm = 5;      // of the persistent grid
 // / 595 / 610 / 695 ms, 40k mixed reads 89.6 / 89.2 / 88.5 / 90.5 / 101.8, 60k of
 // 150 bp at q = 6 57.6 / 56.8 / 56.9 / 57.3 / 63.9.)
 constexpr float kCheckZ = 4.5f;
+// The place is rounded to half blocks of 8 tokens: to the nearest, and of short
+// ones most of them up, since a half block too many is cheaper there than looking
+// again after each.  Uniform 100 bp reads, 600 Mbp, q = 5, sweeps in ms (rounded
+// down / to the nearest / all up): one pass e = 0 2.85 / 2.82 / 2.85, e = 2 5.81 /
+// 5.42 / 5.27, e = 5 9.20 / 9.05 / 8.93; coarse e = 0 1.80 / 1.78 / 1.68, e = 2 3.31 /
+// 3.25 / 3.25, e = 5 5.99 / 6.01 / 6.06; 24 bp e = 0 3.73 / 3.68 / 3.42.
+constexpr uint32_t kCheckShort = 48;
 
 struct TokArgs {
   const char* reads;
@@ -323,8 +330,13 @@ __global__ void __launch_bounds__(kTokWarps * 32, kTokCtasPerSm) k_tokenise(TokA
         }
         if (!both) at[1] = at[0];
       }
-      meta |= ((at[0] ? at[0] : ntok) >> 3) << kMetaCheckCoarse;
-      meta |= ((at[1] ? at[1] : ntok) >> 3) << kMetaCheckFine;
+      // to halves: the nearest, or up where one makes a difference
+      auto check = [&](uint32_t place) {
+        const uint32_t p = place ? place : ntok;
+        return min((p + (p < kCheckShort ? 6u : 3u)) >> 3, 31u);
+      };
+      meta |= check(at[0]) << kMetaCheckCoarse;
+      meta |= check(at[1]) << kMetaCheckFine;
       meta |= ((at[0] ? at[0] : ntok) >> 2) << kMetaOrder;
     }
     if (lane == 0) a.meta[r] = meta;
