@@ -23,8 +23,6 @@
 //   instead, few lines of a vector at a time.
 // * The path is random reads of 128-byte lines per (read, bin) pair: bound by
 //   HBM, not by arithmetic.
-#include <math.h>
-
 #include "grim_internal.cuh"
 
 namespace grim {
@@ -382,6 +380,92 @@ __global__ void __launch_bounds__(kWarps * 32, kCandCtasPerSm) k_candidates(Cand
   if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) atomicOr(&a.ctl->status, kStatusBadCand);
 }
 
+// Whole vectors of 512 bytes (q = 6) against a read, for budgets so large that
+// a bin is ruled out only by a hundred or more tokens that it lacks: a vector is
+// ANDed with the set of the read's tokens and with the set of those it holds
+// twice; the few it holds more often are looked up.  Bound by HBM's rate of random
+// 512-byte rows: 20k reads of 250 bp, 6.6M candidates, 0.55 ms whatever the budget
+// (12e9 rows/s of 13.7e9).  A binary plane for each bit of the multiplicity, from a
+// histogram of the tokens, took 0.78; the look-ups 0.51 at e = 18, 0.88 at e = 20,
+// 1.47 at e = 33.
+constexpr uint32_t kPlaneWords = 128;
+struct __align__(16) Planes {  // a warp's, in shared memory; a lane takes 4 words of each
+  uint32_t once[kPlaneWords], twice[kPlaneWords];
+  uint16_t more[256];  // a token for every further occurrence
+};
+
+// Sets the planes of a token row; the number of further occurrences.
+// Warp-collective.
+__device__ __forceinline__ uint32_t set_planes(Planes& p, const uint16_t* tok, uint32_t ntok,
+                                               uint32_t r4, uint32_t lane) {
+  constexpr int kRounds = 8;  // up to 255 tokens
+  uint32_t t[kRounds];
+#pragma unroll
+  for (int i = 0; i < kRounds; ++i)
+    t[i] = 32u * i + lane < ntok ? tok[32u * i + lane] : rowPad(r4);
+  __syncwarp();  // the last read's planes are no longer read
+  reinterpret_cast<uint4*>(p.once)[lane] = make_uint4(0u, 0u, 0u, 0u);
+  reinterpret_cast<uint4*>(p.twice)[lane] = make_uint4(0u, 0u, 0u, 0u);
+  __syncwarp();
+  uint32_t n = 0;
+#pragma unroll
+  for (int i = 0; i < kRounds; ++i) {
+    const uint32_t w = t[i] >> 5, bit = 1u << (t[i] & 31u);
+    const bool further = t[i] < r4 && (atomicOr(p.once + w, bit) & bit) &&
+                         (atomicOr(p.twice + w, bit) & bit);
+    const uint32_t m = __ballot_sync(0xFFFFFFFFu, further);
+    if (further) p.more[n + __popc(m & ((1u << lane) - 1u))] = (uint16_t)t[i];
+    n += __popc(m);
+  }
+  __syncwarp();
+  return n;
+}
+
+// popc(v & a) + popc(v & b) over the warp's 128 words, through a carry-save tree
+// (4 POPC instead of 8)
+__device__ __forceinline__ uint32_t planes_present(const uint4& v, const uint4& a, const uint4& b) {
+  const uint32_t x0 = v.x & a.x, x1 = v.y & a.y, x2 = v.z & a.z, x3 = v.w & a.w;
+  const uint32_t y0 = v.x & b.x, y1 = v.y & b.y, y2 = v.z & b.z, y3 = v.w & b.w;
+  const uint32_t s0 = x0 ^ x1 ^ x2, c0 = (x0 & x1) | (x2 & (x0 ^ x1));
+  const uint32_t s1 = x3 ^ y0 ^ y1, c1 = (x3 & y0) | (y1 & (x3 ^ y0));
+  const uint32_t s2 = s0 ^ s1 ^ y2, c2 = (s0 & s1) | (y2 & (s0 ^ s1));
+  const uint32_t s3 = s2 ^ y3, c3 = s2 & y3;                            // weight 1; carries of 2
+  const uint32_t s4 = c0 ^ c1 ^ c2, c4 = (c0 & c1) | (c2 & (c0 ^ c1));  // weights 2, 4
+  const uint32_t s5 = s4 ^ c3, c5 = s4 & c3;                            // weights 2, 4
+  return __reduce_add_sync(0xFFFFFFFFu, __popc(s3) + 2u * __popc(s5) + 4u * __popc(c4 ^ c5) +
+                                            8u * __popc(c4 & c5));
+}
+
+// Up to 32 bins (lane k < n: its bin's row) against the read: the lane's sum + 1
+// where it is at least thr, else 0.  Warp-collective.
+template <int U>
+__device__ __forceinline__ uint32_t planes_check(const uint32_t* bm, const Planes& p,
+                                                 uint32_t n_more, uint32_t thr, uint32_t row,
+                                                 uint32_t n, uint32_t lane) {
+  const uint4 p0 = reinterpret_cast<const uint4*>(p.once)[lane];
+  const uint4 p1 = reinterpret_cast<const uint4*>(p.twice)[lane];
+  const uint4* vecs = reinterpret_cast<const uint4*>(bm) + lane;
+  uint32_t sum = 0;  // of the lane's bin
+  for (uint32_t k = 0; k < n; k += U) {
+    uint4 v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      v[u] = __ldg(vecs + (uint64_t)__shfl_sync(0xFFFFFFFFu, row, k + u) * (kPlaneWords / 4));
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint32_t present = planes_present(v[u], p0, p1);
+      sum = lane == k + u ? present : sum;
+    }
+  }
+  // a lane's bin and one token at a time
+  const uint32_t* mine = bm + (uint64_t)row * kPlaneWords;
+  for (uint32_t i = 0; i < n_more; ++i) {
+    const uint32_t t = p.more[i];
+    sum += (__ldg(mine + (t >> 5)) >> (t & 31u)) & 1u;
+  }
+  return lane < n && sum >= thr ? sum + 1u : 0u;
+}
+
 // Exact check of the coarse pass's survivors, one (survivor, member bin) item
 // at a time by a whole warp: lane j looks up the read's tokens j, j + 32, ...
 // in the member's vector and a ballot counts the misses; the item ends once
@@ -494,7 +578,11 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_refine(IndexView ix, ReadsVi
 // took 9.48 ms at 91 warp instructions a candidate.  The same look-ups over
 // 128-byte vectors (q = 5, mixed reads) lost to the planes, 9.8 against 8.6
 // ms: one line is read either way, and a quarter warp per vector issues less.
-constexpr int kStageMax = 4;
+// Batches of which a third of the reads or more have budgets too large to be
+// settled by the first groups (Ctl::n_far) are checked with planes, whose time does
+// not depend on the budget: 0.55 ms where the look-ups take 0.26 to 0.52 for the
+// reads before that line and 0.82 to 1.47 for those past it.
+constexpr uint32_t kFarShare = 3;
 
 struct StageTokens {
   const char* at[kStageMax];  // the token's word in row 0, or a zero word
@@ -534,6 +622,54 @@ __device__ __forceinline__ uint32_t stage_scan(const StageTokens& st, uint32_t i
   return alive;
 }
 
+// The lists of a batch of reads with large budgets, in whole vectors.
+__device__ __forceinline__ void lists_by_planes(const CandArgs& a, Planes& planes,
+                                                uint32_t n_reads, uint32_t lane) {
+  const uint64_t c_begin = a.cand_off[0], c_end = a.cand_off[n_reads];
+  const uint64_t chunk = chunk_size(c_end - c_begin, (uint64_t)gridDim.x * kWarps);
+  const uint64_t n_chunks = (c_end - c_begin + chunk - 1) / chunk;
+  const uint32_t num_bins = (uint32_t)a.ix.num_bins, r4 = a.ix.r4;
+  uint32_t cur = 0xFFFFFFFFu, thr = 0, n_more = 0;  // the read whose planes are set
+  bool bad = false;
+  for (;;) {
+    uint32_t cj = 0;
+    if (lane == 0) cj = atomicAdd(&a.ctl->item, 1u);
+    cj = __shfl_sync(0xFFFFFFFFu, cj, 0);
+    if (cj >= n_chunks) break;
+    const uint64_t base = c_begin + (uint64_t)cj * chunk;
+    const uint32_t clen = (uint32_t)min(chunk, c_end - base);
+    uint32_t r = read_of(a.cand_off, n_reads, base, lane);
+    for (uint32_t p = 0; p < clen; ++r) {
+      const uint32_t c1 = (uint32_t)min(a.cand_off[r + 1] - base, (uint64_t)clen);
+      if (c1 > p && r != cur) {
+        cur = r;
+        const uint32_t m = a.rv.meta[r], ntok = m & 0xFFu;
+        thr = ntok - ((m >> 8) & 0xFFu);
+        n_more = set_planes(planes, a.rv.tokens + (uint64_t)r * a.rv.copies * a.rv.ts, ntok, r4, lane);
+      }
+      for (; p < c1; p += 32) {
+        const uint32_t n = min(c1 - p, 32u);
+        const uint32_t id = lane < n ? (uint32_t)__ldg(a.cand + base + p + lane) : 0u;
+        const bool ok = id < num_bins;
+        bad |= !ok;
+        uint32_t found = planes_check<4>(a.ix.bm, planes, n_more, thr, ok ? id : 0u, n, lane);
+        if (!ok) found = 0;
+        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, found != 0);
+        if (!bal) continue;
+        unsigned long long at = 0;
+        if (lane == 0) at = atomicAdd(&a.ctl->n_rec, (unsigned long long)__popc(bal));
+        at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(bal & ((1u << lane) - 1u));
+        if (found && at < a.rec.cap) {
+          a.rec.keys[at] = base + p + lane;
+          a.rec.counts[at] = (uint8_t)(found - 1u);
+        }
+      }
+      p = c1;
+    }
+  }
+  if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) atomicOr(&a.ctl->status, kStatusBadCand);
+}
+
 template <int U>
 __global__ void __launch_bounds__(kWarps * 32, 6) k_candidates_lookup(CandArgs a, uint32_t miss256) {
   const uint32_t lane = threadIdx.x & 31;
@@ -543,6 +679,11 @@ __global__ void __launch_bounds__(kWarps * 32, 6) k_candidates_lookup(CandArgs a
   if (n_reads == 0) return;
   const uint64_t c_begin = a.cand_off[0], c_end = a.cand_off[n_reads];
   if (c_end <= c_begin) return;
+  __shared__ Planes s_planes[kWarps];
+  if ((uint64_t)a.ctl->n_far * kFarShare >= n_reads) {
+    lists_by_planes(a, s_planes[threadIdx.x >> 5], n_reads, lane);
+    return;
+  }
   const uint64_t chunk = chunk_size(c_end - c_begin, (uint64_t)gridDim.x * kWarps);
   const uint64_t n_chunks = (c_end - c_begin + chunk - 1) / chunk;
   const uint32_t num_bins = (uint32_t)a.ix.num_bins;
@@ -577,8 +718,7 @@ __global__ void __launch_bounds__(kWarps * 32, 6) k_candidates_lookup(CandArgs a
         dmax = (m >> 8) & 0xFFu;
         tok = a.rv.tokens + (uint64_t)r * a.rv.copies * a.rv.ts;
         // groups of 32 tokens that leave D' + 6 misses expected
-        stage = min(min(((dmax + 6u) * 8u + miss256 - 1u) / miss256, (ntok + 31u) / 32u),
-                    (uint32_t)kStageMax);
+        stage = min(min(lookup_groups(dmax, miss256), (ntok + 31u) / 32u), (uint32_t)kStageMax);
 #pragma unroll
         for (int s = 0; s < kStageMax; ++s) {
           const uint32_t t = s * 32u + lane < ntok ? tok[s * 32u + lane] : rowPad(r4);
@@ -673,13 +813,9 @@ void launch_lookup(const CandArgs& a, uint64_t n_cand, cudaStream_t st) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // share of a window's tokens that a random one misses, in 1/256
-  const double grams = (double)a.ix.B + a.ix.ext - a.ix.q + 1;
-  const double miss = exp(-grams / (double)a.ix.r4);
-  const uint32_t miss256 = miss * 256.0 < 16.0 ? 16u : (uint32_t)(miss * 256.0);
   const uint64_t grid = list_grid(n_cand, (uint64_t)(sms > 0 ? sms : 1) * 6u);
   ProfScope ps("candidates", st);
-  k_candidates_lookup<U><<<(unsigned)grid, kWarps * 32, 0, st>>>(a, miss256);
+  k_candidates_lookup<U><<<(unsigned)grid, kWarps * 32, 0, st>>>(a, lookup_miss256(a.ix));
 }
 
 template <int WPB, int U>

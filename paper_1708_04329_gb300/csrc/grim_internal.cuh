@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stddef.h>
 #include <stdint.h>
 
@@ -43,7 +44,8 @@ struct Ctl {
   uint32_t d_lo;                   // 255 - the smallest miss budget D' of the batch
   uint32_t route;                  // the batch's path, whichever kernel sweeps it
   unsigned long long tail_words;   // the words (32 bins) those halves were applied to
-  uint32_t pad[38];
+  uint32_t n_far;                  // lists at q = 6: reads that look-ups are not for (lookup_far)
+  uint32_t pad[37];
 };
 static_assert(sizeof(Ctl) == 256, "Ctl is one 256-byte slot");
 static_assert(offsetof(Ctl, live_reads) == 32, "live counts follow the per-pass counters");
@@ -120,6 +122,24 @@ struct ReadsView {
   uint32_t n_reads, ts;
   uint32_t copies;  // 1, or 4 block-rotated copies for the 256-bin tiles (q = 6)
 };
+
+// Lists at q = 6 look up the first groups of 32 of a read's tokens in a bin's
+// vector, as many as leave more than D' misses expected, up to kStageMax groups.
+constexpr int kStageMax = 4;
+// share of a window's tokens that a random one misses, in 1/256
+inline uint32_t lookup_miss256(const IndexView& v) {
+  const double grams = (double)v.B + v.ext - v.q + 1;
+  const double miss = exp(-grams / (double)v.r4) * 256.0;
+  return miss < 16.0 ? 16u : (uint32_t)miss;
+}
+// groups of 32 tokens that leave D' + 6 misses expected
+__host__ __device__ inline uint32_t lookup_groups(uint32_t d, uint32_t miss256) {
+  return ((d + 6u) * 8u + miss256 - 1u) / miss256;
+}
+// a read that the first groups cannot settle (Ctl::n_far)
+__host__ __device__ inline bool lookup_far(uint32_t ntok, uint32_t d, uint32_t miss256) {
+  return ntok > 32u * kStageMax && lookup_groups(d, miss256) > (uint32_t)kStageMax;
+}
 
 struct RecordsView {
   unsigned long long* keys;  // sort keys of passing records

@@ -43,6 +43,7 @@ struct TokArgs {
   uint64_t max_bases;
   const uint64_t* cand_off;  // list modes: the lists' CSR offsets
   uint64_t n_cand;
+  uint32_t miss256;          // kLines: lookup_miss256
 };
 
 // One warp per read.  The read's tokens (row indices of the table: the token
@@ -111,6 +112,7 @@ __global__ void __launch_bounds__(kTokWarps * 32, kTokCtasPerSm) k_tokenise(TokA
   // check of the shared words for every read is a load of one address for
   // every read, which takes longer than the tokens
   uint32_t max_d = 0, d_lo = 0, max_tight = 0, blk_max = 0, blk_lo = 0;
+  uint32_t n_far = 0;  // kLines: reads past the look-ups
   for (uint64_t r = blockIdx.x * (uint64_t)kTokWarps + warp; r < n_reads; r += n_warps) {
     const uint32_t budget = a.e[r];
     if (budget > a.max_e && lane == 0) atomicOr(&ctl->status, kStatusArg);
@@ -341,6 +343,7 @@ __global__ void __launch_bounds__(kTokWarps * 32, kTokCtasPerSm) k_tokenise(TokA
     }
     if (lane == 0) a.meta[r] = meta;
     const uint32_t nblk = (ntok + kBlockTokens - 1) / kBlockTokens;
+    if constexpr (ORDER == TokenOrder::kLines) n_far += lookup_far(ntok, d, a.miss256);
     max_d = max(max_d, d);
     d_lo = max(d_lo, 255u - d);
     max_tight = max(max_tight, 255u - (ntok - d));
@@ -353,6 +356,7 @@ __global__ void __launch_bounds__(kTokWarps * 32, kTokCtasPerSm) k_tokenise(TokA
     auto raise = [](uint32_t* p, uint32_t v) {
       if (v > *reinterpret_cast<volatile uint32_t*>(p)) atomicMax(p, v);
     };
+    if (ORDER == TokenOrder::kLines && n_far) atomicAdd(&ctl->n_far, n_far);
     raise(&ctl->max_d, max_d);
     raise(&ctl->d_lo, d_lo);
     raise(&ctl->max_tight, max_tight);
@@ -467,7 +471,7 @@ void launch_tokenise(const char* reads, const uint64_t* offsets, const uint32_t*
   const uint64_t grid = need < most ? need : most;
   const TokArgs a{reads, offsets, lens,   e,    rv.n_reads, ix.q, ix.max_read_len, ix.r4,    rv.ts,
                   rv.copies, ix.rank, ix.miss, fine_power, tokens, meta, ctl, live, max_e, max_bases,
-                  cand_off, n_cand};
+                  cand_off, n_cand, cand_off && ix.wpb > 32 ? lookup_miss256(ix) : 0u};
   // lists read whole token rows in any order up to 128-byte vectors; larger
   // ones (q = 6) are looked up line by line
   auto kernel = cand_off        ? (ix.wpb > 32 ? k_tokenise<TokenOrder::kLines>
