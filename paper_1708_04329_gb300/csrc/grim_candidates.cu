@@ -466,6 +466,54 @@ __device__ __forceinline__ uint32_t planes_check(const uint32_t* bm, const Plane
   return lane < n && sum >= thr ? sum + 1u : 0u;
 }
 
+// Survivors of reads with D' >= far at q = 6, one at a time: its f members' vectors
+// are consecutive and share the read's planes.  3.4M survivors of 16 members, 250 bp,
+// e = 20: 5.0 ms (28 GB of vectors, 0.81 of the copy rate), 12.2 with k_refine's
+// look-ups; 5.1 + 1.1 for sorting and expanding them into lists.
+__device__ __forceinline__ void refine_by_planes(const IndexView& ix, const ReadsView& rv,
+                                                 const unsigned long long* __restrict__ keys,
+                                                 uint64_t n_surv, uint32_t cbits, uint32_t f,
+                                                 const RecordsView& rec, uint32_t bin_bits,
+                                                 uint32_t far, Ctl* ctl, Planes& planes) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint64_t warp = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
+  const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  uint32_t cur = 0xFFFFFFFFu, n_more = 0;  // the read whose planes are set
+  uint32_t batch = 32;  // survivors
+  while (batch > 1 && n_surv < n_warps * batch) batch >>= 1;
+  for (uint64_t base = warp * batch; base < n_surv; base += n_warps * batch) {
+    const bool in = lane < batch && base + lane < n_surv;
+    const unsigned long long key = in ? keys[base + lane] : 0ull;
+    const uint32_t mine = (uint32_t)(key >> cbits), m = in ? rv.meta[mine] : 0u;
+    uint32_t todo = __ballot_sync(0xFFFFFFFFu, in && ((m >> 8) & 0xFFu) >= far);
+    for (; todo; todo &= todo - 1u) {
+      const int s = __ffs(todo) - 1;
+      const uint32_t r = __shfl_sync(0xFFFFFFFFu, mine, s), mr = __shfl_sync(0xFFFFFFFFu, m, s);
+      const uint32_t ntok = mr & 0xFFu, dmax = (mr >> 8) & 0xFFu;
+      const uint32_t first = (uint32_t)(__shfl_sync(0xFFFFFFFFu, key, s) & ((1ull << cbits) - 1ull)) * f;
+      const uint32_t end = (uint32_t)min((uint64_t)first + f, ix.num_bins);
+      const uint16_t* tok = rv.tokens + (uint64_t)r * rv.copies * rv.ts;
+      if (r != cur) {
+        cur = r;
+        n_more = set_planes(planes, tok, ntok, ix.r4, lane);
+      }
+      for (uint32_t b = first; b < end; b += 32) {
+        const uint32_t n = min(end - b, 32u), row = b + min(lane, n - 1u);
+        const uint32_t found = planes_check<4>(ix.bm, planes, n_more, ntok - dmax, row, n, lane);
+        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, found != 0);
+        if (!bal) continue;
+        unsigned long long at = 0;
+        if (lane == 0) at = atomicAdd(&ctl->n_final, (unsigned long long)__popc(bal));
+        at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(bal & ((1u << lane) - 1u));
+        if (found && at < rec.cap) {
+          rec.keys[at] = ((unsigned long long)r << bin_bits) | (b + lane);
+          rec.counts[at] = (uint8_t)(found - 1u);
+        }
+      }
+    }
+  }
+}
+
 // Exact check of the coarse pass's survivors, one (survivor, member bin) item
 // at a time by a whole warp: lane j looks up the read's tokens j, j + 32, ...
 // in the member's vector and a ballot counts the misses; the item ends once
@@ -480,14 +528,21 @@ __device__ __forceinline__ uint32_t planes_check(const uint32_t* bm, const Plane
 // (19 chunks of short lists there, each one warp's serial work).  The chain of
 // loads (token, then word of the vector) bounds it, so kRefineItems items run
 // side by side in a warp.
+// WIDE (q = 6): the survivors of reads with D' >= far are left to a second loop,
+// refine_by_planes.  Look-ups cost with D', vectors do not (us, look-ups / vectors):
+// 100 bp, D' = 36, 562k survivors of 16 1124 / 1034; 150 bp, D' = 48, 13k 244 / 234;
+// D' = 60, 353k 1009 / 795, 2.0M of 8 2179 / 1218; with few members to share the
+// planes, f = 2, 8k survivors at D' = 48 206 / 213.
 constexpr int kRefineItems = 4;
+constexpr uint32_t kRefineFar = 32, kRefineFarMembers = 8;
 
+template <bool WIDE>
 __global__ void __launch_bounds__(kWarps * 32, 4) k_refine(IndexView ix, ReadsView rv,
                                                            const unsigned long long* __restrict__ keys,
                                                            const unsigned long long* n_surv_at,
                                                            uint64_t room, uint32_t cbits, uint32_t f,
                                                            RecordsView rec, uint32_t bin_bits,
-                                                           Ctl* ctl, Live live) {
+                                                           uint32_t far, Ctl* ctl, Live live) {
   constexpr int U = kRefineItems;
   if (*(volatile uint32_t*)&ctl->status) return;
   if (routed_off(ctl, live)) return;
@@ -514,6 +569,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_refine(IndexView ix, ReadsVi
       in = b < ix.num_bins;  // the last super-bin may have fewer members
       bin = (uint32_t)b;
       m = in ? rv.meta[r] : 0u;
+      if (WIDE) in = in && ((m >> 8) & 0xFFu) < far;
     }
     const uint32_t todo = __ballot_sync(0xFFFFFFFFu, in);
     for (uint32_t k = 0; k < batch; k += U) {
@@ -562,6 +618,12 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_refine(IndexView ix, ReadsVi
         rec.counts[pos] = (uint8_t)(found - 1u);
       }
     }
+  }
+  if constexpr (WIDE) {
+    __shared__ Planes s_planes[kWarps];
+    if (ctl->max_d >= far)
+      refine_by_planes(ix, rv, keys, n_surv, cbits, f, rec, bin_bits, far, ctl,
+                       s_planes[threadIdx.x >> 5]);
   }
 }
 
@@ -851,9 +913,11 @@ void launch_refine(const IndexView& ix, const ReadsView& rv, const unsigned long
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const uint64_t need = (room * f + 32 * kWarps - 1) / (32 * kWarps);
   const uint64_t most = (uint64_t)(sms > 0 ? sms : 1) * 4;
+  const bool planes = ix.wpb == kPlaneWords && f >= kRefineFarMembers;
+  auto kernel = planes ? k_refine<true> : k_refine<false>;
   ProfScope ps("candidates_refine", st);
-  k_refine<<<(unsigned)(need < most ? need : most), kWarps * 32, 0, st>>>(
-      ix, rv, keys, n_surv, room, cbits, f, rec, bin_bits, ctl, live);
+  kernel<<<(unsigned)(need < most ? need : most), kWarps * 32, 0, st>>>(
+      ix, rv, keys, n_surv, room, cbits, f, rec, bin_bits, kRefineFar, ctl, live);
 }
 
 void launch_candidates(const IndexView& ix, const ReadsView& rv, const int32_t* cand,

@@ -62,3 +62,22 @@ def test_lists_of_large_budgets(L, far):
         gpu_filter(ix, rs, off, bad, cap=4000)
     assert ei.value.code == grim.GRIM_E_BAD_CANDIDATE
     ix.close()
+
+
+@pytest.mark.parametrize("factor,L", [(7, 150), (8, 150), (16, 37), (16, 250), (33, 200), (64, 250)])
+def test_survivors_of_large_budgets(factor, L):
+    """Survivors of reads with D' below, at and past the line, up to where every
+    bin passes, and super-bins of fewer members at the end; one path forced."""
+    from paper_1708_04329_gb300 import grim
+
+    g = _genome(100 * factor * 41 + 11, factor)
+    reads = _reads(g, L, 60)
+    e = [(5, 6, L // 10, L // 8, L // 6 + 1, 2, L // 5)[i % 7] for i in range(60)]
+    rs = Reads(reads, e)
+    ix = build(g, 100, 6, 260, layouts=6, coarse_factor=factor)
+    nb = ix.desc.num_bins
+    want = oracle.filter(oracle.bin_vectors(g, 100, 6, 260), rs)
+    assert len(want[0]) > nb
+    assert_same(gpu_filter(ix, rs, cap=60 * nb), want)
+    assert grim.grim_last_filter_stats()["survivors"] > 0
+    ix.close()
