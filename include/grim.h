@@ -202,12 +202,14 @@ int grim_index_info(const grim_index* idx, grim_index_desc* out);
  *                  its read ends.  WARP runs the reads of a warp together for
  *                  as many tokens as they are expected to need, finishes the
  *                  few bins still live apart, and switches all of them at
- *                  once.  Automatic: WARP for batches whose reads span the
- *                  same number of 16-token blocks and have the same miss
- *                  budget D'; of mixed batches those of 256 reads and more
- *                  run together too, sorted so that reads of similar length
- *                  to go share a warp (as do graph plans for that many
- *                  reads), smaller ones switch by GROUP
+ *                  once; batches of 256 reads and more are sorted for it, so
+ *                  that reads of similar length to go share a warp (batches
+ *                  whose reads span the same number of 16-token blocks and
+ *                  have the same miss budget D' from 32768 reads on).
+ *                  Automatic: WARP, but GROUP for mixed batches of fewer
+ *                  than 256 reads, and where the sort finds no room: an index
+ *                  with the token-major table alone, 8 * cap bytes short of
+ *                  4.3 a read.  Graph plans decide by the most reads they hold
  *   all_bins_path  GRIM_PATH_TWO_LEVEL, GRIM_PATH_EXACT, or 0 (automatic; see
  *                  GRIM_PATH_*)
  * Results do not depend on the shape.  Graph plans take the shape when they

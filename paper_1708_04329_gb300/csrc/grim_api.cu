@@ -594,7 +594,8 @@ int grim_filter(const grim_index* idx, const char* reads, const uint64_t* offset
     if (!shape.read_switch) shape.read_switch = uniform ? GRIM_SWITCH_WARP : GRIM_SWITCH_GROUP;
     switch_used = shape.read_switch;
     uint32_t* order = order_room(v, ws, L, n_reads, rcap, f, rb);
-    if (idx->shape.read_switch || (uniform && n_reads < kOrderUniform)) order = nullptr;
+    if (idx->shape.read_switch == GRIM_SWITCH_GROUP || (uniform && n_reads < kOrderUniform))
+      order = nullptr;
     if (order) shape.read_switch = GRIM_SWITCH_WARP;
     launch_order(rv, order, ctl, st);
     const uint32_t max_d = h.max_d;

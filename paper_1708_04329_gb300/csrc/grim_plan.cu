@@ -150,7 +150,7 @@ int capture(grim_plan* p) {
   // all bins: with a coarse pass both paths leave their records in rb (the
   // survivors are in ra while their members are checked), else in ra
   const RecordsView dst = p->f ? rb : ra, tmp = p->f ? ra : rb;
-  uint32_t* order = p->cand_mode || idx->shape.read_switch
+  uint32_t* order = p->cand_mode || idx->shape.read_switch == GRIM_SWITCH_GROUP
                         ? nullptr
                         : order_room(v, ws, L, d.max_reads, rcap, p->f, tmp);
   ExhShape shape = idx->shape;
