@@ -25,6 +25,15 @@ constexpr float kCheckZ = 4.5f;
 // 5.42 / 5.27, e = 5 9.20 / 9.05 / 8.93; coarse e = 0 1.80 / 1.78 / 1.68, e = 2 3.31 /
 // 3.25 / 3.25, e = 5 5.99 / 6.01 / 6.06; 24 bp e = 0 3.73 / 3.68 / 3.42.
 constexpr uint32_t kCheckShort = 48;
+// Up to q = 4 most bins hold most tokens.  Where a token's share of misses is
+// small their number is nearer a Poisson's than a normal's, and kCheckZ deviations
+// put the check far too late: it comes there when the exponent of the tail
+// (over ln(over / S) + (j - over) ln((j - over) / (j - S)), as much as kCheckZ
+// deviations' kCheckZ^2 / 2) is large enough, cut down to halves.  Counts of 200
+// reads of 150 bp against 15.1M bins, e = 0 743 -> 541 us, e = 2 1631 -> 1379; of 500
+// reads of 80 bp against 19.7M, e = 0..5 17.8 -> 17.1 ms.  At q = 5 and 6 the two
+// rules differ by less than 0.5%.
+constexpr uint32_t kDenseRows = 256;
 
 struct TokArgs {
   const char* reads;
@@ -325,7 +334,13 @@ __global__ void __launch_bounds__(kTokWarps * 32, kTokCtasPerSm) k_tokenise(TokA
             if (lane >= (uint32_t)dd) incl += up;
           }
           const float s = sum[k] + incl, n = (float)(j0 + lane + 1u), x = s - over;
-          const bool ok = j0 + lane < ntok && x > 0.f && x * x * n >= kCheckZ * kCheckZ * s * (n - s);
+          bool ok = j0 + lane < ntok && x > 0.f;
+          if (r4 > kDenseRows)
+            ok = ok && x * x * n >= kCheckZ * kCheckZ * s * (n - s);
+          else  // (n - s is 0 for tokens that no bin holds)
+            ok = ok && over * __logf(over / s) +
+                               (n - over) * __logf((n - over) / fmaxf(n - s, 1e-6f)) >=
+                           0.5f * kCheckZ * kCheckZ;
           const uint32_t hit = __ballot_sync(0xFFFFFFFFu, ok);
           if (hit && !at[k]) at[k] = j0 + __ffs(hit);
           sum[k] += __shfl_sync(0xFFFFFFFFu, incl, 31);
@@ -335,7 +350,7 @@ __global__ void __launch_bounds__(kTokWarps * 32, kTokCtasPerSm) k_tokenise(TokA
       // to halves: the nearest, or up where one makes a difference
       auto check = [&](uint32_t place) {
         const uint32_t p = place ? place : ntok;
-        return min((p + (p < kCheckShort ? 6u : 3u)) >> 3, 31u);
+        return min((p + (r4 <= kDenseRows ? 0u : p < kCheckShort ? 6u : 3u)) >> 3, 31u);
       };
       meta |= check(at[0]) << kMetaCheckCoarse;
       meta |= check(at[1]) << kMetaCheckFine;
