@@ -23,17 +23,20 @@ reads with CUDA events:
   each lane group keeps in flight (1, 2, 4 or 8), timed through
   graph-captured plans.
 
-Results are cached in a JSON file keyed by the problem's shape and the GPU,
-so a service tunes once per (reference, parameters, device).
+Results are cached in a JSON file keyed by the problem's shape, the GPU and the
+library's kernels, so a service tunes once per (reference, parameters, device,
+library): a pick made for other kernels is not taken over.
 """
 from __future__ import annotations
 
+import functools
+import hashlib
 import json
 import os
 import statistics
 from pathlib import Path
 
-from . import grim
+from . import _build, grim
 
 DEFAULT_CACHE = Path(os.environ.get("GRIM_AUTOTUNE_CACHE",
                                     Path.home() / ".cache" / "grim_gb300" / "autotune.json"))
@@ -43,6 +46,15 @@ def _device_name() -> str:
     import torch
 
     return torch.cuda.get_device_name()
+
+
+@functools.cache
+def _kernels() -> str:
+    """A digest of the sources that the library's kernels are built from."""
+    h = hashlib.sha256()
+    for name in _build.GRIM_SOURCES + _build.GRIM_HEADERS:
+        h.update((_build.CSRC / name).read_bytes())
+    return h.hexdigest()[:16]
 
 
 def _load(cache: Path | None) -> dict:
@@ -105,7 +117,7 @@ def tune_all_bins(ref, B: int, q: int, max_read_len: int, sample: dict,
     """
     n = int(sample["lens"].numel())
     key = (f"allbins|{int(ref.numel())}|{B}|{q}|{max_read_len}|{n}|"
-           f"{tuple(threads)}|{tuple(ranges_kb)}|{tuple(switches)}|{_device_name()}")
+           f"{tuple(threads)}|{tuple(ranges_kb)}|{tuple(switches)}|{_device_name()}|{_kernels()}")
     table = _load(cache)
     if key in table:
         return table[key]
@@ -196,7 +208,7 @@ def tune_candidate_unroll(index, sample: dict, max_e: int, unrolls=(1, 2, 4, 8),
     n = int(sample["lens"].numel())
     nc = int(sample["cand"].numel())
     d = index.desc
-    key = f"cand|{d.num_bins}|{d.q}|{n}|{nc}|{_device_name()}"
+    key = f"cand|{d.num_bins}|{d.q}|{n}|{nc}|{_device_name()}|{_kernels()}"
     table = _load(cache)
     if key in table:
         return table[key]
