@@ -138,7 +138,7 @@ __host__ __device__ inline uint32_t lookup_groups(uint32_t d, uint32_t miss256) 
 }
 // a read that the first groups cannot settle (Ctl::n_far)
 __host__ __device__ inline bool lookup_far(uint32_t ntok, uint32_t d, uint32_t miss256) {
-  return ntok > 32u * kStageMax && lookup_groups(d, miss256) > (uint32_t)kStageMax;
+  return ntok > 32u * kStageMax && (d + 6u) * 8u > kStageMax * miss256;  // (lookup_groups > kStageMax)
 }
 
 struct RecordsView {
