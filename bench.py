@@ -450,7 +450,7 @@ def run_native(args, rank, world, local):
     sm_max = float(peaks.get("sm_max_mhz", 2070.0))
     n_sm = props.multi_processor_count
     roofline = alu_roofline(stats["bit_tests_executed"], per_launch_ms, n_sm, sm_max,
-                            f"k_exhaustive ({'super-bins' if dom == 'exhaustive_coarse' else 'bins'})")
+                            f"k_lockstep ({'super-bins' if dom == 'exhaustive_coarse' else 'bins'})")
     roofline["traffic"] = traffic_for(args, f"{args.workload}:{dom}", headline=True)
     decided = rs.n * units * ntok  # L-q+1 tests per (read, unit) decided, dense
     all_bins_ms = part_ms["all_bins"] / args.steps
@@ -521,7 +521,8 @@ def candidate_roofline(n_cand: int, k_ms: float, nb: int, vec: int, st, peaks: d
     150 bp read with e = 7."""
     gbytes = n_cand * (min(vec, 256) + 4) / 1e9
     hbm = float(peaks.get("hbm_gbs", 6800.0))
-    leg = {"bound": "hbm", "kernel": "k_candidates", "kernel_ms": k_ms,
+    leg = {"bound": "hbm", "kernel": "k_candidates_lookup" if vec > 256 else "k_candidates",
+           "kernel_ms": k_ms,
            "algorithmic_bytes": round(gbytes * 1e9), "achieved": round(gbytes / (k_ms / 1e3), 1),
            "peak": hbm, "unit": "GB/s", "frac": round(gbytes / (k_ms / 1e3) / hbm, 4),
            "traffic": traffic_for(args, traffic_key, "grim_candidates.cu", headline)}
@@ -581,7 +582,7 @@ def exact_leg(w, dev, ref, shape, st, n_sm, sm_max, args, steps: int = 2, warmup
     nb = idx.desc.num_bins
     idx.close()
     roof = alu_roofline(res["stats"]["bit_tests_executed"], prof["exhaustive"], n_sm, sm_max,
-                        "k_exhaustive (bins, one exact pass)")
+                        "k_lockstep (bins, one exact pass)")
     roof["traffic"] = traffic_for(args, "human:exhaustive_exact")
     ntok = w["read_len"] - w["q"] + 1
     roof["decided_bit_tests"] = rs.n * nb * ntok
@@ -641,7 +642,7 @@ def finer_leg(args, g, n_sm, sm_max, peaks, steps: int = 2, warmup: int = 1) -> 
     desc = res["desc"]
     dom = "exhaustive_coarse" if "exhaustive_coarse" in prof else "exhaustive"
     roof = alu_roofline(res["stats"]["bit_tests_executed"], prof[dom], n_sm, sm_max,
-                        f"k_exhaustive ({'super-bins' if dom == 'exhaustive_coarse' else 'bins'}, q = 6)")
+                        f"k_lockstep ({'super-bins' if dom == 'exhaustive_coarse' else 'bins'}, q = 6)")
     roof["traffic"] = traffic_for(args, "finer:" + dom)
     out = {"value": round(rs.n / (ms / 1e3), 1), "unit": UNIT, "ms_per_step": round(ms, 3),
            "steps": steps,

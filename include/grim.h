@@ -351,8 +351,8 @@ int grim_filter_host(const grim_index* idx, const char* reads, const uint64_t* o
  *     for the token copies of the all-bins mode at q = 6; then 18 bytes per
  *     record of capacity, which is cap, or max(cap, 320 * n_reads) for an
  *     index with the coarse layout (room for the coarse pass's survivors),
- *     whose records take another 4 * coarse_factor bytes each for the
- *     survivors' expanded candidate lists.
+ *     whose records take another 4 * coarse_factor bytes each (the order in
+ *     which the sweep takes the reads is kept there).
  *   - First call on a device: it looks up the array's device address (once
  *     per device, with that device current) and keeps it for the life of the
  *     process; make that first call before any stream capture.  The kept

@@ -4,7 +4,7 @@
 //
 // GB300 mapping
 // -------------
-// * Warps claim chunks of 256-4096 consecutive candidates of the flattened lists
+// * Warps claim chunks of 32-4096 consecutive candidates of the flattened lists
 //   from a global counter (a chunk may hold many short lists; a long list is
 //   spread over many warps, so no single 20,000-candidate list is left
 //   running alone at the end).  For each read in its chunk the warp turns the
@@ -20,7 +20,8 @@
 //   that halves the sums at each exchange), compared with
 //   T = (L-q+1) - q*e, and one ballot places the passes.
 // * At q = 6 (512-byte vectors) k_candidates_lookup looks up the read's tokens
-//   instead, few lines of a vector at a time.
+//   instead, few lines of a vector at a time, and batches of reads with large
+//   budgets go by whole vectors (lists_by_planes).
 // * The path is random reads of 128-byte lines per (read, bin) pair: bound by
 //   HBM, not by arithmetic.
 #include "grim_internal.cuh"

@@ -55,7 +55,7 @@
 //   coarse table 609 -> 589, 40k on the fine table 165 -> 156, 40k mixed
 //   100-250 bp reads 102 -> 88, a plan of 4,096 of them 11.3 -> 9.6, 60k of 150
 //   bp at q = 6 60.3 -> 56.8.  Both pipes are near their limit there (small
-//   case: ALU 78%, shared-memory wavefronts 83%).
+//   case: ALU 76%, shared-memory wavefronts 81%).
 #include "grim_internal.cuh"
 
 namespace grim {

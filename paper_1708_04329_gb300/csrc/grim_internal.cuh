@@ -329,9 +329,15 @@ inline uint64_t record_capacity(uint32_t n_reads, uint64_t cap, uint32_t coarse_
 
 // Where a call's read order goes, or null: the spare words of
 // a two-level workspace, else the record buffer that the one exact pass does
-// not write (`idle`), if it is large enough.
+// not write (`idle`), if it is large enough.  Batches of fewer than
+// kOrderMinReads are not sorted, nor uniform ones (one length, one budget) of
+// fewer than kOrderUniform.  Either side of the lines, 3.1 Gbp, ms: 255 mixed
+// reads by group switch 0.952 on the coarse table and 1.62 in one pass, 256
+// sorted in lockstep 0.785 and 1.32 (with the line at 64, 128 reads 0.616 ->
+// 0.508); 32,767 of 100 bp as given 243.6 and 147.0, 32,768 sorted 240.7 and
+// 145.0 (8,192 sorted 61.5 -> 60.7).
 constexpr uint32_t kOrderMinReads = 256;
-constexpr uint32_t kOrderUniform = 32768;  // reads of one length and budget worth ordering
+constexpr uint32_t kOrderUniform = 32768;
 inline uint32_t* order_room(const IndexView& v, char* ws, const Layout& L, uint32_t n_reads,
                             uint64_t rcap, uint32_t coarse_factor, const RecordsView& idle) {
   if (n_reads < kOrderMinReads) return nullptr;
@@ -340,14 +346,15 @@ inline uint32_t* order_room(const IndexView& v, char* ws, const Layout& L, uint3
   return reinterpret_cast<uint32_t*>(idle.keys);
 }
 
-// coarse_factor > 0: room for the coarse pass's survivors, and per survivor
-// the coarse_factor words that grim_filter_workspace_size has always counted
 // Token copies per read: the all-bins kernel's 256-bin tiles (q = 6) read
 // one of 4 block-rotated copies per lane group (see k_tokenise).
 inline uint32_t token_copies(const IndexView& v, bool cand_mode) {
   return !cand_mode && v.r4 > 1024 ? 4u : 1u;
 }
 
+// coarse_factor > 0: room for the coarse pass's survivors, and coarse_factor
+// words for each, of which the reads' order uses the first (the size is part of
+// the limits that grim_filter_noalloc and servers state)
 inline Layout layout(const IndexView& v, uint32_t n_reads, uint64_t cap, uint32_t coarse_factor,
                      uint32_t copies) {
   Layout L{};
@@ -392,7 +399,7 @@ struct grim_index {
   uint32_t layouts;
   grim::ExhShape shape;  // launch shape of the all-bins kernel (grim_index_set_shape)
   // the coarse table is sparse enough for the coarse pass to pay: its
-  // super-bin window would hold at most 40% of the 4^q tokens in a uniform
+  // super-bin window would hold at most half of the 4^q tokens in a uniform
   // random sequence (the rule that picks the default coarse factor)
   bool coarse_pays;
   uint32_t* tm;
