@@ -51,25 +51,24 @@ UNIT = "reads/s"
 TRAFFIC = {
     # all-bins kernel, 1M reads of 100 bp (4 read ranges), linear in the
     # tiles swept: captures at 0.4 and 0.8 Gbp (977 and 1,954 coarse tiles:
-    # 1.292 and 2.174 GB per launch) give 0.409 GB + 0.903 MB per tile;
+    # 2.096 and 3.915 GB per launch) give 0.277 GB + 1.862 MB per tile;
     # 7,569 coarse tiles of the 3.1 Gbp table
-    ("164bfabfb98b2648", "human:exhaustive_coarse"): 7_245_892_095,
+    ("814cc26706c8d301", "human:exhaustive_coarse"): 14_371_097_876,
     # the same rule for the one exact pass over bins (1,954 and 3,907 tiles:
-    # 1.995 and 3.578 GB; 0.411 GB + 0.811 MB per tile); 15,137 tiles
-    ("164bfabfb98b2648", "human:exhaustive_exact"): 12_680_709_263,
+    # 3.385 and 6.055 GB; 0.713 GB + 1.368 MB per tile); 15,137 tiles
+    ("814cc26706c8d301", "human:exhaustive_exact"): 21_412_794_554,
     # the all-bins kernel at q = 6 (finer index, 1M reads of 150 bp, 27 read
     # ranges), linear in the 256-bin coarse tiles: captures at 0.4 and 0.6 Gbp
-    # (977 and 1,465 tiles: 5.736 and 7.452 GB per launch) give 2.301 GB +
-    # 3.516 MB per tile; 7,569 tiles of the 3.1 Gbp coarse table
-    ("164bfabfb98b2648", "finer:exhaustive_coarse"): 28_913_063_934,
+    # (977 and 1,465 tiles: 3.813 and 5.536 GB per launch) give 0.364 GB +
+    # 3.530 MB per tile; 7,569 tiles of the 3.1 Gbp coarse table
+    ("814cc26706c8d301", "finer:exhaustive_coarse"): 27_085_531_468,
     # candidate kernel, in proportion to the pairs gathered: the 3.1 Gbp
     # bin-major table (1.98 GB, as at full size) with 100k ragged reads,
-    # 32,876,582 pairs, 4.314 GB (131.2 B per pair); 1,320,234,389 pairs
-    ("0b88d3370894bf47", "ragged:candidates"): 173_256_211_892,
-    # the same rule at q = 6: 0.4 Gbp (a 2 GB table, 6.4% L2 hits against
-    # ~1% on the full 15.9 GB one, so this is low by up to ~5%), 6,565,154
-    # pairs, 3.260 GB (496.6 B per pair); 329,738,997 pairs
-    ("0b88d3370894bf47", "finer:candidates"): 163_736_639_321,
+    # 32,876,582 pairs, 4.313 GB (131.2 B per pair); 1,320,234,389 pairs
+    ("86bd86ae4adec168", "ragged:candidates"): 173_211_099_515,
+    # the same rule for the look-ups at q = 6: 0.4 Gbp (a 2 GB table), 6,565,154
+    # pairs, 1.621 GB (246.8 B per pair); 329,738,997 pairs
+    ("86bd86ae4adec168", "finer:candidates"): 81_391_995_052,
 }
 
 
